@@ -814,7 +814,7 @@ tfjsb_status tfjsb_bias_backprop(tfjsb_ctx* ctx, const tfjsb_tensor* dz, tfjsb_t
         cudaError_t e = cudaMemsetAsync(dbias->data, 0, (size_t)C * 4, s);
         return e == cudaSuccess ? TFJSB_OK : cuda_fail(ctx, e, "cudaMemsetAsync");
     }
-    const int slices = backprop_slices(rows, ctx->sm_count);
+    const int slices = sum_rows_slices(rows, C, ctx->sm_count);
     if (slices > 1 && (st = ensure_scratch(ctx, &ctx->scratch_c, (size_t)slices * C * 4)) != TFJSB_OK) return st;
     cudaError_t e = launch_sum_rows(static_cast<const float*>(dz->data), static_cast<float*>(dbias->data), ctx->scratch_c.ptr, rows, C,
                                     slices, s, &ctx->launches);

@@ -100,34 +100,60 @@ conv2d_backprop_filter_partial_kernel(const float* __restrict__ x, const float* 
         partial[((int64_t)slice * g.fh * g.fw + tap) * g.C * g.Co + (int64_t)(ci0 + ty) * g.Co + co0 + tx] = acc;
 }
 
-// out[c] = sum over r < rows (in order) of in[r, c]
-__global__ void __launch_bounds__(BP_THREADS)
-sum_rows_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t rows, int64_t C) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    float acc = 0.f;
-    for (int64_t r = 0; r < rows; ++r) acc += in[r * C + c];
-    out[c] = acc;
-}
-
-// partial[slice, c] = sum over the rows of the slice of in[r, c]; block = 32 columns x 8 row lanes
-__global__ void __launch_bounds__(BP_THREADS)
-sum_rows_partial_kernel(const float* __restrict__ in, float* __restrict__ partial, int64_t rows, int64_t C,
-                        int64_t rows_per_slice) {
-    __shared__ float red[8][32];
-    const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
+// ---- column sums ------------------------------------------------------------------------------------
+// out[c] = sum over r < rows of in[r, c].  Block = blockDim.x column lanes (V columns each) x blockDim.y row
+// lanes; a lane adds every blockDim.y-th row (UNROLL of them in flight), the row lanes meet in shared memory in
+// lane order.  blockIdx.y cuts the rows into slices of `rows_per_slice`, one row of `out` per slice: the same
+// kernel makes the partial sums and adds them up.  The order of the additions depends on the shape alone.
+// Bound: memory.  One thread per column with a serial walk over 392 partial rows, and 4-byte loads with one in
+// flight per thread before that, took 24 + 26 us for [100352, 128] (51 MB); now 16 + 5 us with a cold cache.
+template <int V>
+__global__ void __launch_bounds__(1024)
+column_sums_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t rows, int64_t C, int64_t rows_per_slice) {
+    constexpr int UNROLL = 8;
+    __shared__ float red[1024 * V];
+    const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int64_t r_begin = (int64_t)blockIdx.y * rows_per_slice;
     const int64_t r_end = min(rows, r_begin + rows_per_slice);
-    float acc = 0.f;
-    if (c < C)
-        for (int64_t r = r_begin + threadIdx.y; r < r_end; r += 8) acc += __ldg(in + r * C + c);
-    red[threadIdx.y][threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.y == 0 && c < C) {
-        float v = red[0][threadIdx.x];
+    const int lanes = blockDim.y;
+    float acc[V];
 #pragma unroll
-        for (int k = 1; k < 8; ++k) v += red[k][threadIdx.x];
-        partial[(int64_t)blockIdx.y * C + c] = v;
+    for (int v = 0; v < V; ++v) acc[v] = 0.f;
+    if (c < C) {
+        const float* p = in + c;
+        // the last rows of a slice stay in the unrolled form (predicated): one by one, each would cost a memory latency
+        for (int64_t r = r_begin + threadIdx.y; r < r_end; r += (int64_t)UNROLL * lanes) {
+            float t[UNROLL][V];
+#pragma unroll
+            for (int u = 0; u < UNROLL; ++u) {
+                const int64_t row = r + (int64_t)u * lanes;
+#pragma unroll
+                for (int v = 0; v < V; ++v) t[u][v] = 0.f;
+                if (row < r_end) {
+                    if (V == 4) *reinterpret_cast<float4*>(t[u]) = __ldg(reinterpret_cast<const float4*>(p + row * C));
+                    else t[u][0] = __ldg(p + row * C);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < UNROLL; ++u)
+#pragma unroll
+                for (int v = 0; v < V; ++v) acc[v] += t[u][v];
+        }
+    }
+    // [row lane][V][column lane]: neighbouring threads of a warp write neighbouring words
+#pragma unroll
+    for (int v = 0; v < V; ++v) red[(threadIdx.y * V + v) * blockDim.x + threadIdx.x] = acc[v];
+    for (int half = lanes >> 1; half > 0; half >>= 1) {
+        __syncthreads();
+        if (threadIdx.y < half) {
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                red[(threadIdx.y * V + v) * blockDim.x + threadIdx.x] += red[((threadIdx.y + half) * V + v) * blockDim.x + threadIdx.x];
+        }
+    }
+    if (threadIdx.y == 0 && c < C) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) out[(int64_t)blockIdx.y * C + c + v] = red[v * blockDim.x + threadIdx.x];
     }
 }
 
@@ -195,15 +221,23 @@ depthwise_backprop_filter_partial_kernel(const float* __restrict__ x, const floa
 }
 
 // ---- epilogue ---------------------------------------------------------------------------------------
-// dz = dy where the activation passed its input through (judged by the forward output y), +0 elsewhere
+// dz = dy where the activation passed its input through (judged by the forward output y), +0 elsewhere.  Bound by
+// memory (two operands in, one out); four values per thread and step: 26 -> 24 us for 3 x 51 MB.
+__device__ __forceinline__ float act_grad(float y, float dy, int act) {
+    const bool pass = act == TFJSB_ACT_NONE || (y > 0.f && (act == TFJSB_ACT_RELU || y < 6.f));
+    return pass ? dy : 0.f;
+}
 __global__ void __launch_bounds__(BP_THREADS)
 act_backprop_kernel(const float* __restrict__ y, const float* __restrict__ dy, float* __restrict__ dz, int64_t n, int act) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const float v = y[i];
-        const bool pass = act == TFJSB_ACT_NONE || (v > 0.f && (act == TFJSB_ACT_RELU || v < 6.f));
-        dz[i] = pass ? dy[i] : 0.f;
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t n4 = n >> 2;
+    for (int64_t i = first; i < n4; i += stride) {
+        const float4 v = reinterpret_cast<const float4*>(y)[i], g = reinterpret_cast<const float4*>(dy)[i];
+        reinterpret_cast<float4*>(dz)[i] =
+            make_float4(act_grad(v.x, g.x, act), act_grad(v.y, g.y, act), act_grad(v.z, g.z, act), act_grad(v.w, g.w, act));
     }
+    if (first < (n & 3)) dz[4 * n4 + first] = act_grad(y[4 * n4 + first], dy[4 * n4 + first], act);
 }
 
 // out[b, c, r] = in[b, r, c] for B matrices of shape [rows, cols] stored one after the other
@@ -246,18 +280,48 @@ cudaError_t launch_conv2d_backprop_input(const float* dy, const float* f, float*
     return cudaGetLastError();
 }
 
+namespace {
+
+int pow2_at_least(int64_t v, int limit) {
+    int p = 1;
+    while (p < v && p < limit) p <<= 1;
+    return p;
+}
+
+// One launch of column_sums_kernel over `slices` slices of the rows.
+cudaError_t launch_column_sums(const float* in, float* out, int64_t rows, int64_t C, int slices, cudaStream_t s, int64_t* launches) {
+    const int64_t per = (rows + slices - 1) / slices;
+    // four columns per thread where rows start on 16 bytes and there are columns enough to fill the SMs that way
+    const bool vec = C % 4 == 0 && C * slices >= 8192;
+    const int64_t cols = vec ? C / 4 : C;
+    const int tx = pow2_at_least(cols, 32);
+    // eight rows per lane and pass, up to 1024 threads; one warp at least
+    int ty = pow2_at_least((per + 7) / 8, 1024 / tx);
+    if (ty * tx < 32) ty = 32 / tx;
+    const dim3 grid((unsigned)((cols + tx - 1) / tx), (unsigned)slices), block(tx, ty);
+    if (vec) column_sums_kernel<4><<<grid, block, 0, s>>>(in, out, rows, C, per);
+    else column_sums_kernel<1><<<grid, block, 0, s>>>(in, out, rows, C, per);
+    ++*launches;
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+int sum_rows_slices(int64_t rows, int64_t C, int sm_count) {
+    // One step while the 1024 threads of a block read their column strip in one pass.  Beyond that, slices of at least
+    // 128 rows and two blocks of 1024 threads per SM, one wave.
+    const int64_t strips = C % 4 == 0 ? (C + 127) / 128 : (C + 31) / 32;
+    if (rows <= 1024) return 1;
+    int64_t s = (2 * (int64_t)sm_count + strips - 1) / strips;
+    if (s > rows / 128) s = rows / 128;
+    return (int)(s < 1 ? 1 : (s > 65535 ? 65535 : s));
+}
+
 cudaError_t launch_sum_rows(const float* in, float* out, float* partial, int64_t rows, int64_t C, int slices, cudaStream_t s,
                             int64_t* launches) {
-    if (slices <= 1) {
-        sum_rows_kernel<<<(unsigned)((C + BP_THREADS - 1) / BP_THREADS), BP_THREADS, 0, s>>>(in, out, rows, C);
-        ++*launches;
-        return cudaGetLastError();
-    }
-    const int64_t per = (rows + slices - 1) / slices;
-    sum_rows_partial_kernel<<<dim3((unsigned)((C + 31) / 32), (unsigned)slices), dim3(32, 8), 0, s>>>(in, partial, rows, C, per);
-    sum_rows_kernel<<<(unsigned)((C + BP_THREADS - 1) / BP_THREADS), BP_THREADS, 0, s>>>(partial, out, slices, C);
-    *launches += 2;
-    return cudaGetLastError();
+    if (slices <= 1) return launch_column_sums(in, out, rows, C, 1, s, launches);
+    cudaError_t e = launch_column_sums(in, partial, rows, C, slices, s, launches);
+    return e != cudaSuccess ? e : launch_column_sums(partial, out, slices, C, 1, s, launches);
 }
 
 cudaError_t launch_conv2d_backprop_filter(const float* x, const float* dy, float* df, float* partial, int slices,
@@ -300,7 +364,7 @@ cudaError_t launch_depthwise_backprop_filter(const float* x, const float* dy, fl
 
 cudaError_t launch_act_backprop(const float* y, const float* dy, float* dz, int64_t n, int act, int sm_count, cudaStream_t s,
                                 int64_t* launches) {
-    act_backprop_kernel<<<blocks_for(n, sm_count), BP_THREADS, 0, s>>>(y, dy, dz, n, act);
+    act_backprop_kernel<<<blocks_for((n + 3) / 4, sm_count), BP_THREADS, 0, s>>>(y, dy, dz, n, act);
     ++*launches;
     return cudaGetLastError();
 }

@@ -299,6 +299,7 @@ cudaError_t launch_block_diagonal(const float* km, float* out, int64_t N, int64_
 // ---- gradients (backprop.cu) ----------------------------------------------------------------------
 // `g` is the geometry of the FORWARD op (H, W, C the forward input; Ho, Wo, Co the forward output).
 int backprop_slices(int64_t rows, int sm_count);
+int sum_rows_slices(int64_t rows, int64_t C, int sm_count);  // slices that launch_sum_rows wants for this shape
 cudaError_t launch_conv2d_backprop_input(const float* dy, const float* f, float* dx, const ConvGeom& g, int sm_count,
                                          cudaStream_t s, int64_t* launches);
 // `partial` holds slices * fh*fw*C*Co floats (unused when slices == 1)
