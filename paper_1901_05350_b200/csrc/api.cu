@@ -745,7 +745,19 @@ tfjsb_status tfjsb_depthwise_conv2d_backprop_input(tfjsb_ctx* ctx, const tfjsb_t
     if ((st = grad_geometry(ctx, dx, filter, dy, strides, pad, dilations, true, &g)) != TFJSB_OK) return st;
     if (overlaps(dx, dy) || overlaps(dx, filter)) return fail(ctx, TFJSB_ERR_INVALID_ARG, "dx aliases an input");
     if (numel(dx) == 0) return TFJSB_OK;
-    cudaError_t e = launch_depthwise_backprop_input(static_cast<const float*>(dy->data), static_cast<const float*>(filter->data),
+    cudaError_t e;
+    if (depthwise_backprop_is_forward(g)) {
+        // stride 1: the forward kernels over dy with the taps reversed and the padding mirrored
+        const ConvGeom t = depthwise_backprop_geometry(g);
+        DepthwisePlan plan;
+        if ((st = depthwise_plan(ctx, dy->data, t, &plan)) != TFJSB_OK) return st;
+        e = launch_depthwise(plan, static_cast<const float*>(dy->data), static_cast<const float*>(filter->data), nullptr,
+                             TFJSB_ACT_NONE, static_cast<float*>(dx->data), t, ctx->dev_status, static_cast<cudaStream_t>(stream),
+                             &ctx->launches);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "depthwise_backprop_input launch");
+        return TFJSB_OK;
+    }
+    e = launch_depthwise_backprop_input(static_cast<const float*>(dy->data), static_cast<const float*>(filter->data),
                                                     static_cast<float*>(dx->data), g, ctx->sm_count,
                                                     static_cast<cudaStream_t>(stream), &ctx->launches);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "depthwise_backprop_input launch");

@@ -185,6 +185,59 @@ depthwise_backprop_input_kernel(const float* __restrict__ dy, const float* __res
     }
 }
 
+// 3x3, stride 2, multiplier 1, C % 4 == 0.  In padded coordinates u = iy + pt, v = ix + pl the 2x2 group of samples
+// (u, v) = (2q, 2r) .. (2q+1, 2r+1) is reached from the four output pixels (q-1..q, r-1..r) only:
+//   (2q, 2r): four taps (corners), (2q, 2r+1) and (2q+1, 2r): two each, (2q+1, 2r+1): the centre tap.
+// Thread = 4 channels x one column pair x a strip of ROWS row pairs: 2 (ROWS + 1) 16-byte loads, all issued before
+// the first use, feed 4 ROWS 16-byte stores.  Bound by memory (dx is four times dy).
+template <int ROWS>
+__global__ void __launch_bounds__(BP_THREADS)
+depthwise3x3_s2_backprop_input_kernel(const float* __restrict__ dy, const float* __restrict__ f, float* __restrict__ dx, ConvGeom g,
+                                      int tc, int c4_tiles) {
+    const int C4 = g.C >> 2;
+    const int c4 = (blockIdx.x % c4_tiles) * tc + (threadIdx.x % tc);
+    const int r = (blockIdx.x / c4_tiles) * (BP_THREADS / tc) + threadIdx.x / tc;
+    const int q0 = blockIdx.y * ROWS;
+    const int ix = 2 * r - g.pl;
+    if (c4 >= C4 || ix >= g.W) return;
+    const int c = c4 * 4;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 w[9];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) w[t] = __ldg(reinterpret_cast<const float4*>(f + (int64_t)t * g.C + c));
+    const int64_t n = blockIdx.z;
+    const float* gy = dy + n * (int64_t)g.Ho * g.Wo * g.C + c;
+    float4 a[ROWS + 1], b[ROWS + 1];  // columns r - 1 and r of rows q0 - 1 .. q0 + ROWS - 1
+#pragma unroll
+    for (int j = 0; j <= ROWS; ++j) {
+        const int oy = q0 - 1 + j;
+        const bool row = oy >= 0 && oy < g.Ho;
+        const float* p = gy + ((int64_t)oy * g.Wo + r) * g.C;
+        a[j] = row && r >= 1 && r - 1 < g.Wo ? __ldg(reinterpret_cast<const float4*>(p - g.C)) : zero;
+        b[j] = row && r < g.Wo ? __ldg(reinterpret_cast<const float4*>(p)) : zero;
+    }
+    float* out = dx + n * (int64_t)g.H * g.W * g.C + c;
+#pragma unroll
+    for (int j = 1; j <= ROWS; ++j) {
+        const int iy = 2 * (q0 + j - 1) - g.pt;
+        float4 v00 = zero, v01 = zero, v10 = zero, v11 = zero;
+        fma4_packed(v00, b[j], w[0]); fma4_packed(v00, a[j], w[2]); fma4_packed(v00, b[j - 1], w[6]); fma4_packed(v00, a[j - 1], w[8]);
+        fma4_packed(v01, b[j], w[1]); fma4_packed(v01, b[j - 1], w[7]);
+        fma4_packed(v10, b[j], w[3]); fma4_packed(v10, a[j], w[5]);
+        fma4_packed(v11, b[j], w[4]);
+        float* o = out + ((int64_t)iy * g.W + ix) * g.C;
+        if (iy >= 0 && iy < g.H) {
+            if (ix >= 0) *reinterpret_cast<float4*>(o) = v00;
+            if (ix + 1 < g.W) *reinterpret_cast<float4*>(o + g.C) = v01;
+        }
+        if (iy + 1 < g.H) {
+            o += (int64_t)g.W * g.C;
+            if (ix >= 0) *reinterpret_cast<float4*>(o) = v10;
+            if (ix + 1 < g.W) *reinterpret_cast<float4*>(o + g.C) = v11;
+        }
+    }
+}
+
 // ---- depthwise, gradient with respect to the filter: partial sums ------------------------------------
 // Block = 32 output channels (tx) x 8 pixel lanes (ty) for one tap (blockIdx.z) and one slice of the
 // output pixels (blockIdx.y).
@@ -340,8 +393,36 @@ cudaError_t launch_conv2d_backprop_filter(const float* x, const float* dy, float
     return launch_sum_rows(partial, df, nullptr, slices, elems, 1, s, launches);
 }
 
+bool depthwise_backprop_is_forward(const ConvGeom& g) {
+    return g.fh == 3 && g.fw == 3 && g.mult == 1 && g.sh == 1 && g.sw == 1 && g.C % 4 == 0 && g.dh == g.dw &&
+           (g.dh == 1 || g.dh == 2 || g.dh == 4) && g.N <= 65535 && (g.H + 3) / 4 <= 65535;
+}
+
+ConvGeom depthwise_backprop_geometry(const ConvGeom& g) {
+    ConvGeom t = g;
+    t.H = g.Ho; t.W = g.Wo; t.Ho = g.H; t.Wo = g.W;
+    t.pt = (g.fh - 1) * g.dh - g.pt;  // dx[i] = sum over k of dy[i + pt - k d] f[k], k from last to first
+    t.pl = (g.fw - 1) * g.dw - g.pl;
+    t.reversed = 1;
+    return t;
+}
+
 cudaError_t launch_depthwise_backprop_input(const float* dy, const float* f, float* dx, const ConvGeom& g, int sm_count,
                                             cudaStream_t s, int64_t* launches) {
+    if (g.fh == 3 && g.fw == 3 && g.mult == 1 && g.sh == 2 && g.sw == 2 && g.dh == 1 && g.dw == 1 && g.C % 4 == 0 && g.N <= 65535) {
+        constexpr int ROWS = 4;
+        const int tc = pow2_at_least(g.C / 4, 32);
+        const int c4_tiles = (g.C / 4 + tc - 1) / tc;
+        const int cols = BP_THREADS / tc;
+        const int64_t gx = (int64_t)c4_tiles * (((g.W + g.pl + 1) / 2 + cols - 1) / cols);
+        const int gy = ((g.H + g.pt + 1) / 2 + ROWS - 1) / ROWS;
+        if (gx <= 2147483647LL && gy <= 65535) {
+            depthwise3x3_s2_backprop_input_kernel<ROWS>
+                <<<dim3((unsigned)gx, (unsigned)gy, (unsigned)g.N), BP_THREADS, 0, s>>>(dy, f, dx, g, tc, c4_tiles);
+            ++*launches;
+            return cudaGetLastError();
+        }
+    }
     const int64_t total = g.N * g.H * g.W * g.C;
     depthwise_backprop_input_kernel<<<blocks_for(total, sm_count), BP_THREADS, 0, s>>>(dy, f, dx, g, total);
     ++*launches;

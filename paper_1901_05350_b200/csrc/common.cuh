@@ -159,6 +159,9 @@ struct ConvGeom {
     int sh, sw, dh, dw; // strides, dilations
     int pt, pl;         // padding before (top, left)
     int Ho, Wo;
+    // 3x3 depthwise kernels: taps read last to first, which turns the forward pass over dy into the gradient with
+    // respect to the input (stride 1)
+    int reversed = 0;
 };
 
 // ---- launchers (each returns the CUDA launch error; `launches` is incremented per kernel) -----
@@ -305,6 +308,10 @@ cudaError_t launch_conv2d_backprop_input(const float* dy, const float* f, float*
 // `partial` holds slices * fh*fw*C*Co floats (unused when slices == 1)
 cudaError_t launch_conv2d_backprop_filter(const float* x, const float* dy, float* df, float* partial, int slices,
                                           const ConvGeom& g, cudaStream_t s, int64_t* launches);
+// The input gradient of a stride-1 3x3 depthwise convolution is a forward one over dy (taps reversed): whether the
+// 3x3 kernels of depthwise.cu can run it for this forward geometry, and the geometry that they get.
+bool depthwise_backprop_is_forward(const ConvGeom& g);
+ConvGeom depthwise_backprop_geometry(const ConvGeom& g);
 cudaError_t launch_depthwise_backprop_input(const float* dy, const float* f, float* dx, const ConvGeom& g, int sm_count,
                                             cudaStream_t s, int64_t* launches);
 // `partial` holds slices * fh*fw*Co floats (unused when slices == 1)

@@ -59,7 +59,7 @@ depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ f, co
 
     float4 w[9];
 #pragma unroll
-    for (int t = 0; t < 9; ++t) w[t] = ld4(f + (int64_t)t * g.C + c);
+    for (int t = 0; t < 9; ++t) w[t] = ld4(f + (int64_t)(g.reversed ? 8 - t : t) * g.C + c);
 
     float4 acc[ROWS];
 #pragma unroll
@@ -315,7 +315,8 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
         if (live) {
             if (cb != loaded_cb) {
 #pragma unroll
-                for (int k = 0; k < 9; ++k) w[k] = __ldg(reinterpret_cast<const float4*>(f + (int64_t)k * g.C + c));
+                for (int k = 0; k < 9; ++k)
+                    w[k] = __ldg(reinterpret_cast<const float4*>(f + (int64_t)(g.reversed ? 8 - k : k) * g.C + c));
                 if (bias) b = __ldg(reinterpret_cast<const float4*>(bias + c));
                 loaded_cb = cb;
             }
