@@ -35,6 +35,7 @@ SOURCES = [
     "dwpw_fused_tcgen05.cu",
     "bf16_storage.cu",
     "backprop.cu",
+    "depthwise_grad.cu",
 ]
 
 NVCC_FLAGS = [

@@ -782,6 +782,13 @@ tfjsb_status tfjsb_depthwise_conv2d_backprop_filter(tfjsb_ctx* ctx, const tfjsb_
         cudaError_t e = cudaMemsetAsync(dfilter->data, 0, (size_t)numel(dfilter) * 4, s);
         return e == cudaSuccess ? TFJSB_OK : cuda_fail(ctx, e, "cudaMemsetAsync");
     }
+    DepthwiseGradPlan plan;
+    if (depthwise_grad_plan(ctx, static_cast<const float*>(x->data), static_cast<const float*>(dy->data), g, &plan)) {
+        if (plan.slices > 1 && (st = ensure_scratch(ctx, &ctx->scratch_c, (size_t)plan.slices * numel(dfilter) * 4)) != TFJSB_OK) return st;
+        cudaError_t e = launch_depthwise_grad(plan, static_cast<float*>(dfilter->data), ctx->scratch_c.ptr, ctx->dev_status, s, &ctx->launches);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "depthwise_backprop_filter launch");
+        return TFJSB_OK;
+    }
     int slices = backprop_slices(pixels, ctx->sm_count);
     if (slices > 1 && (st = ensure_scratch(ctx, &ctx->scratch_c, (size_t)slices * numel(dfilter) * 4)) != TFJSB_OK) return st;
     cudaError_t e = launch_depthwise_backprop_filter(static_cast<const float*>(x->data), static_cast<const float*>(dy->data),

@@ -317,6 +317,17 @@ cudaError_t launch_depthwise_backprop_input(const float* dy, const float* f, flo
 // `partial` holds slices * fh*fw*Co floats (unused when slices == 1)
 cudaError_t launch_depthwise_backprop_filter(const float* x, const float* dy, float* df, float* partial, int slices,
                                              const ConvGeom& g, cudaStream_t s, int64_t* launches);
+// Pipelined filter gradient of the 3x3 depthwise convolution (depthwise_grad.cu); depthwise_grad_plan says whether the
+// shape is one of its own.  `partial` holds slices * 9 * C floats (unused when slices == 1).
+struct DepthwiseGradPlan {
+    CUtensorMap map_x, map_dy;
+    ConvGeom g{};
+    int variant = 0, th = 0, tw = 0, thin = 0, twin = 0, stage_bytes = 0, stages = 0;
+    int tiles_x = 0, tiles_y = 0, c_blocks = 0, num_tiles = 0, slices = 0;
+};
+bool depthwise_grad_plan(tfjsb_ctx* ctx, const float* x, const float* dy, const ConvGeom& g, DepthwiseGradPlan* plan);
+cudaError_t launch_depthwise_grad(const DepthwiseGradPlan& plan, float* df, float* partial, unsigned int* dev_status, cudaStream_t s,
+                                  int64_t* launches);
 cudaError_t launch_act_backprop(const float* y, const float* dy, float* dz, int64_t n, int act, int sm_count, cudaStream_t s,
                                 int64_t* launches);
 // out[c] = sum_r in[r, c]; with slices > 1 in two steps through `partial` (slices * C floats)

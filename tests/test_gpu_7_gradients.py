@@ -81,6 +81,44 @@ def test_depthwise_gradients(ctx, oracle, case, mult):
     assert rel_fro(df, oracle.depthwise_conv2d_backprop_filter(x, f.shape, g, (s, s), pad, (d, d))) <= 1e-5
 
 
+DEPTHWISE_3X3_CASES = [
+    # N, H, W, C, stride, dilation, pad: tile edges of the pipelined kernels and of the stride-2 column pairs
+    (1, 1, 1, 4, 1, 1, "same"),
+    (2, 7, 7, 100, 1, 1, "same"),      # 8-wide tiles, a ragged channel block
+    (3, 14, 17, 64, 1, 1, "same"),     # one column past a 16-wide tile
+    (2, 9, 33, 36, 1, 1, "valid"),     # mirrored padding of two
+    (1, 13, 20, 8, 1, 2, "same"),      # dilated: register kernel forward over dy, per-tap filter gradient
+    (2, 20, 18, 32, 1, 4, "same"),
+    (2, 1, 2, 4, 2, 1, "same"),
+    (2, 16, 16, 32, 2, 1, "same"),     # even size: padding after only
+    (3, 15, 31, 40, 2, 1, "same"),     # odd size: padding on both sides
+    (2, 18, 35, 68, 2, 1, "valid"),    # an input row that no output reads
+    (70, 28, 28, 128, 1, 1, "same"),   # several tiles per CTA
+    (70, 28, 29, 96, 2, 1, "same"),
+]
+
+
+@pytest.mark.parametrize("case", DEPTHWISE_3X3_CASES)
+def test_depthwise_3x3_gradients_at_tile_edges(ctx, oracle, case):
+    N, H, W, C, s, d, pad = case
+    Ho, Wo = geometry(oracle, H, W, 3, 3, s, d, pad)
+    # small integers: |df| <= 9 * N * Ho * Wo < 2^24, exact in any order
+    x = si.small_integers(91, 0, (N, H, W, C), -3, 3)
+    f = si.small_integers(91, 1, (3, 3, C, 1), -3, 3)
+    g = si.small_integers(91, 2, (N, Ho, Wo, C), -3, 3)
+    dx = host(ctx.depthwise_conv2d_backprop_input(x.shape, dev(f), dev(g), (s, s), pad, (d, d)))
+    df = host(ctx.depthwise_conv2d_backprop_filter(dev(x), f.shape, dev(g), (s, s), pad, (d, d)))
+    ctx.check_device_status()
+    assert same_bits(dx + 0.0, oracle.depthwise_conv2d_backprop_input(x.shape, f, g, (s, s), pad, (d, d)) + 0.0)
+    assert same_bits(df + 0.0, oracle.depthwise_conv2d_backprop_filter(x, f.shape, g, (s, s), pad, (d, d)) + 0.0)
+
+
+@pytest.mark.parametrize("shape", [(1, 1), (1024, 3), (1025, 32), (5000, 101), (3000, 8192), (40, 3, 7, 4), (1 << 17, 4), (70001, 36)])
+def test_bias_gradient_slices(ctx, oracle, shape):
+    dz = si.small_integers(92, 0, shape, -8, 8)  # |sums| <= 8 * 2^17: exact in any order
+    assert same_bits(host(ctx.bias_backprop(dev(dz))), oracle.bias_backprop(dz))
+
+
 POINTWISE_CASES = [
     # N, H, W, Cin, Cout: gradients of a 1x1 convolution as matrix products on the tensor cores
     (1, 8, 8, 32, 64),        # 64 pixels: a single slice, K = 64
