@@ -209,6 +209,12 @@ tfjsb_status tfjsb_init(int device, tfjsb_ctx** out) {
     e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
     if (e == cudaSuccess && qres == cudaDriverEntryPointSuccess) ctx->encode_tiled = reinterpret_cast<EncodeTiledFn>(fn);
     else (void)cudaGetLastError();
+    e = cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &fn, cudaEnableDefault, &qres);
+    if (e == cudaSuccess && qres == cudaDriverEntryPointSuccess) ctx->encode_im2col = reinterpret_cast<EncodeIm2colFn>(fn);
+    else {
+        (void)cudaGetLastError();
+        ctx->encode_tiled = nullptr;  // a driver with tensor maps has both calls
+    }
     *out = ctx;
     return TFJSB_OK;
 }
@@ -454,8 +460,7 @@ tfjsb_status tfjsb_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_ten
         // implicit GEMM on the tensor cores: the filter is packed [Cout, k_pad] into scratch first
         const int64_t k_pad = conv_igemm_k_pad(g);
         if ((st = ensure_scratch(ctx, &ctx->scratch_b, (size_t)Cout * k_pad * 4)) != TFJSB_OK) return st;
-        if ((e = launch_pack_filter(pf, ctx->scratch_b.ptr, (int64_t)g.fh * g.fw * g.C, Cout, k_pad, s, &ctx->launches)) !=
-            cudaSuccess)
+        if ((e = launch_pack_conv_filter(pf, ctx->scratch_b.ptr, g, s, &ctx->launches)) != cudaSuccess)
             return cuda_fail(ctx, e, "filter packing");
         if (conv_patch_supported(g) && !getenv("TFJSB_NO_PATCH_CONV")) {
             DwPwPlan pplan;

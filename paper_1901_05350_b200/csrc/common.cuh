@@ -72,6 +72,10 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+typedef CUresult (*EncodeIm2colFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                   const int*, const int*, cuuint32_t, cuuint32_t, const cuuint32_t*, CUtensorMapInterleave,
+                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
 struct Scratch {
     float* ptr = nullptr;
     size_t bytes = 0;
@@ -86,6 +90,7 @@ struct tfjsb_ctx {
     std::string last_error;
     unsigned int* dev_status = nullptr;  // device status word
     tfjsb::EncodeTiledFn encode_tiled = nullptr;
+    tfjsb::EncodeIm2colFn encode_im2col = nullptr;
     tfjsb::Scratch scratch_a, scratch_b;  // transposed operands of tfjsb_matmul
     tfjsb::Scratch scratch_c;             // partial sums of the filter / bias gradients
     std::vector<void*> retired;            // outgrown scratch blocks, freed at shutdown
@@ -228,8 +233,9 @@ struct GemmTf32Plan {
     bool cluster_split = false;
     int splits = 1, kb_per_split = 0;  // slices of the K loop (= cluster size) and k-blocks per slice
     float* c = nullptr;                // C, which that kernel stores directly
-    // implicit-GEMM convolution: A is gathered from x by the kernel instead of copied
+    // implicit-GEMM convolution: A is gathered from x by the kernel instead of copied, or copied by im2col loads
     bool gather = false;
+    bool im2col = false;
     const float* x = nullptr;
     ConvGeom g{};
 };
@@ -251,13 +257,16 @@ tfjsb_status gemm_tf32_splitk_plan(tfjsb_ctx* ctx, const float* a, const float* 
 cudaError_t launch_gemm_tf32_splitk(const GemmTf32Plan& plan, const float* bias, int act, unsigned int* dev_status,
                                     cudaStream_t s, int64_t* launches);
 // Implicit-GEMM convolution on the same kernel: M = N*Ho*Wo output pixels, K = fh*fw*Cin, N = Cout.
-// `bt` is the filter packed as [Cout, k_pad] (K-contiguous, zero padded to a multiple of 32).
+// `bt` is the filter packed as [Cout, k_pad] by launch_pack_conv_filter (K-contiguous, zero padded to whole k-blocks of
+// 32: each tap for itself where A comes by im2col loads, the whole window otherwise).
 bool conv_igemm_supported(const ConvGeom& g);
+bool conv_igemm_uses_im2col(const ConvGeom& g);
 int64_t conv_igemm_k_pad(const ConvGeom& g);
+cudaError_t launch_pack_conv_filter(const float* f, float* out, const ConvGeom& g, cudaStream_t s, int64_t* launches);
 tfjsb_status conv_igemm_plan(tfjsb_ctx* ctx, const float* x, const float* bt, float* y, const ConvGeom& g,
                              GemmTf32Plan* plan);
-// out[n, k] = k < K ? f[k, n] : 0 for f of shape [K, N], out of shape [N, k_pad]
-cudaError_t launch_pack_filter(const float* f, float* out, int64_t K, int64_t N, int64_t k_pad, cudaStream_t s,
+// out[n, t * c_pad + c] = c < C ? f[t, c, n] : 0 for f of shape [taps, C, N], out of shape [N, taps * c_pad]
+cudaError_t launch_pack_filter(const float* f, float* out, int64_t taps, int64_t C, int64_t N, int64_t c_pad, cudaStream_t s,
                                int64_t* launches);
 cudaError_t launch_gemm_tf32(const GemmTf32Plan& plan, const float* bias, int act, unsigned int* dev_status,
                              cudaStream_t s, int64_t* launches);

@@ -286,23 +286,30 @@ __global__ void transpose_kernel(const float* __restrict__ in, float* __restrict
 }
 
 // ---- filter packing for the implicit-GEMM convolution ------------------------------------------------
-__global__ void pack_filter_kernel(const float* __restrict__ f, float* __restrict__ out, int64_t K, int64_t N,
-                                   int64_t k_pad) {
-    const int64_t total = N * k_pad;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-        const int64_t n = i / k_pad, k = i - n * k_pad;
-        out[i] = k < K ? f[k * N + n] : 0.0f;
+// out[n, t * c_pad + c] = c < C ? f[t, c, n] : 0.  A 32 x 32 transpose through shared memory per block, so that both
+// sides are read and written in 128-byte runs.
+__global__ void pack_filter_kernel(const float* __restrict__ f, float* __restrict__ out, int64_t C, int64_t N, int64_t c_pad) {
+    __shared__ float tile[32][33];
+    const int64_t n0 = (int64_t)blockIdx.x * 32, c0 = (int64_t)blockIdx.y * 32, t = blockIdx.z;
+    for (int j = threadIdx.y; j < 32; j += 8) {
+        const int64_t c = c0 + j, n = n0 + threadIdx.x;
+        tile[j][threadIdx.x] = c < C && n < N ? f[(t * C + c) * N + n] : 0.0f;
+    }
+    __syncthreads();
+    for (int j = threadIdx.y; j < 32; j += 8) {
+        const int64_t n = n0 + j, c = c0 + threadIdx.x;
+        if (n < N && c < c_pad) out[(n * gridDim.z + t) * c_pad + c] = tile[threadIdx.x][j];
     }
 }
 
 }  // namespace
 
-cudaError_t launch_pack_filter(const float* f, float* out, int64_t K, int64_t N, int64_t k_pad, cudaStream_t s,
+cudaError_t launch_pack_filter(const float* f, float* out, int64_t taps, int64_t C, int64_t N, int64_t c_pad, cudaStream_t s,
                                int64_t* launches) {
-    const int64_t total = N * k_pad;
-    if (total == 0) return cudaSuccess;
-    pack_filter_kernel<<<grid_for(total, kThreads, current_sm_count() * 8), kThreads, 0, s>>>(f, out, K, N, k_pad);
+    if (taps * N * c_pad == 0) return cudaSuccess;
+    const int64_t gy = (c_pad + 31) / 32;
+    if (gy > 65535 || taps > 65535) return cudaErrorInvalidConfiguration;
+    pack_filter_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)gy, (unsigned)taps), dim3(32, 8), 0, s>>>(f, out, C, N, c_pad);
     ++*launches;
     return cudaGetLastError();
 }

@@ -538,8 +538,7 @@ tfjsb_status tfjsb_model_create(tfjsb_ctx* ctx, const tfjsb_layer_desc* layers, 
             // filter [fh*fw*Cin, Cout] -> [Cout, k_pad] once, on the device
             const int64_t k_pad = conv_igemm_k_pad(step.g);
             if ((st = dev_alloc(m, (size_t)(k_pad * step.g.Co), &step.filter_km)) != TFJSB_OK) return bail(st, ctx->last_error);
-            cudaError_t e = launch_pack_filter(step.filter, step.filter_km, (int64_t)step.g.fh * step.g.fw * step.g.C,
-                                               step.g.Co, k_pad, 0, &ctx->launches);
+            cudaError_t e = launch_pack_conv_filter(step.filter, step.filter_km, step.g, 0, &ctx->launches);
             if (e != cudaSuccess) return bail(TFJSB_ERR_CUDA, std::string("packing weights: ") + cudaGetErrorString(e));
         }
         if (step.kind == STEP_GEMM_NARROW) {
@@ -599,8 +598,7 @@ tfjsb_status tfjsb_model_create(tfjsb_ctx* ctx, const tfjsb_layer_desc* layers, 
                 conv_patch_supported(sp.g) && !getenv("TFJSB_NO_PATCH_CONV")) {
                 const int64_t k_pad = conv_igemm_k_pad(sp.g);
                 if ((st = dev_alloc(m, (size_t)(k_pad * sp.g.Co), &sp.filter_km)) != TFJSB_OK) return bail(st, ctx->last_error);
-                cudaError_t e = launch_pack_filter(sp.filter, sp.filter_km, (int64_t)sp.g.fh * sp.g.fw * sp.g.C, sp.g.Co, k_pad, 0,
-                                                   &ctx->launches);
+                cudaError_t e = launch_pack_conv_filter(sp.filter, sp.filter_km, sp.g, 0, &ctx->launches);
                 if (e != cudaSuccess) return bail(TFJSB_ERR_CUDA, std::string("packing weights: ") + cudaGetErrorString(e));
                 sp.conv_patch = true;
             }
@@ -881,7 +879,7 @@ tfjsb_status tfjsb_model_layer_kernel(tfjsb_model* m, int layer, char* name, int
         case STEP_GEMM_TF32:
             k = st.plan.pair ? "gemm_pair_kernel<false>" : st.plan.cluster_split ? "gemm_tf32_splitk_kernel" : "gemm_tf32_kernel<false>";
             break;
-        case STEP_CONV_TF32: k = st.conv_patch ? "dwpw_fused_kernel<true>" : "gemm_tf32_kernel<true>"; break;
+        case STEP_CONV_TF32: k = st.conv_patch ? "dwpw_fused_kernel<true>" : st.plan.im2col ? "gemm_tf32_im2col_kernel" : "gemm_tf32_kernel<true>"; break;
         case STEP_GEMM_FP32: k = "gemm_fp32_kernel"; break;
         case STEP_CONV_FP32: k = "conv2d_fp32_kernel"; break;
         case STEP_DEPTHWISE: k = st.dw_plan.variant >= 0 ? "depthwise3x3_tma_kernel" : "depthwise3x3_kernel"; break;

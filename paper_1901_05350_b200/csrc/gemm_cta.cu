@@ -159,6 +159,11 @@ __device__ __forceinline__ void gather_scalar(float (&v)[BLOCK_K], const float* 
     }
 }
 
+// where the rows of A come from: a matrix in memory, threads that gather windows, or im2col copies of an NHWC tensor
+constexpr int A_TILED = 0;
+constexpr int A_GATHER = 1;
+constexpr int A_IM2COL = 2;
+
 struct KernelArgs {
     int M, N, K;
     int block_n;
@@ -176,10 +181,11 @@ struct KernelArgs {
     ConvGeom g;
 };
 
-template <bool GATHER, int IO, bool BATCHED>
+template <int A_SOURCE, int IO, bool BATCHED>
 __device__ __forceinline__ void gemm_pipeline(const CUtensorMap& map_a, const CUtensorMap& map_b, const CUtensorMap& map_c,
                                               const KernelArgs& args) {
-    static_assert(!GATHER || IO == IO_F32, "the gathering producer builds fp32 tiles");
+    constexpr bool GATHER = A_SOURCE == A_GATHER, IM2COL = A_SOURCE == A_IM2COL;
+    static_assert(A_SOURCE == A_TILED || IO == IO_F32, "the convolutions read fp32");
     constexpr bool IN_BF16 = IO != IO_F32;
     constexpr bool OUT_BF16 = IO == IO_BF16;
     constexpr int BK = IN_BF16 ? 64 : BLOCK_K;        // elements per k-block: 128 bytes either way
@@ -258,6 +264,14 @@ __device__ __forceinline__ void gemm_pipeline(const CUtensorMap& map_a, const CU
                 const int m0 = (in_batch / args.n_tiles) * BLOCK_M;
                 const int n0 = (in_batch % args.n_tiles) * block_n;
                 (void)m0;
+                // im2col: the tile's first output pixel, and the filter tap and channel of the next k-block
+                int img = 0, h0 = 0, w0 = 0, c0 = 0, off_h = 0, off_w = 0;
+                if (IM2COL) {
+                    const int row = m0 / args.g.Wo;
+                    img = row / args.g.Ho;
+                    h0 = (row - img * args.g.Ho) * args.g.sh - args.g.pt;
+                    w0 = (m0 - row * args.g.Wo) * args.g.sw - args.g.pl;
+                }
                 for (int kb = 0; kb < num_k_blocks; ++kb) {
                     if (!bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag)) {
                         if (!*abort_flag) {
@@ -273,7 +287,13 @@ __device__ __forceinline__ void gemm_pipeline(const CUtensorMap& map_a, const CU
                         mbar_arrive_expect_tx(full, (uint32_t)(stage_bytes - A_STAGE_BYTES));
                     } else {
                         mbar_arrive_expect_tx(full, (uint32_t)stage_bytes);
-                        if (BATCHED) tma_load_3d(a_dst, &map_a, full, kb * BK, m0, batch);
+                        if (IM2COL) {
+                            tma_load_im2col(a_dst, &map_a, full, c0, w0, h0, img, off_w, off_h);
+                            if ((c0 += BK) >= args.g.C) {
+                                c0 = 0;
+                                if ((off_w += args.g.dw) == args.g.fw * args.g.dw) { off_w = 0; off_h += args.g.dh; }
+                            }
+                        } else if (BATCHED) tma_load_3d(a_dst, &map_a, full, kb * BK, m0, batch);
                         else tma_load_2d(a_dst, &map_a, full, kb * BK, m0);
                     }
                     if (BATCHED) tma_load_3d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BK, n0, batch);
@@ -526,7 +546,18 @@ template <bool GATHER>
 __global__ void __launch_bounds__(GATHER ? CONV_THREADS : GEMM_MAX_THREADS, 1)
 gemm_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                  const __grid_constant__ CUtensorMap map_c, const KernelArgs args) {
-    gemm_pipeline<GATHER, IO_F32, false>(map_a, map_b, map_c, args);
+    gemm_pipeline<GATHER ? A_GATHER : A_TILED, IO_F32, false>(map_a, map_b, map_c, args);
+}
+
+// conv2d with the A tiles fetched by im2col copies: a k-block is 32 channels of one filter tap for 128 successive output
+// pixels, which the copy unit collects across image rows and images and zero-fills outside them, in the layout of any
+// other A tile; no thread touches the input.  The threads of the gathering kernel spent their time on addresses and
+// shared-memory stores: [32,56,56,64] * 3x3x64x64 95 us against 43 here, [16,28,28,128] * 3x3x128x128 63 against 29.5.
+// What bounds it now is the copy unit, which delivers a pixel's 128 bytes about every five cycles (a matrix row every two).
+__global__ void __launch_bounds__(GEMM_MAX_THREADS, 1)
+gemm_tf32_im2col_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                        const __grid_constant__ CUtensorMap map_c, const KernelArgs args) {
+    gemm_pipeline<A_IM2COL, IO_F32, false>(map_a, map_b, map_c, args);
 }
 
 // A batch of independent products of one shape (rank-3 matMul): the tensor maps carry the batch as a third
@@ -534,14 +565,14 @@ gemm_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 __global__ void __launch_bounds__(GEMM_MAX_THREADS, 1)
 gemm_tf32_batched_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                          const __grid_constant__ CUtensorMap map_c, const KernelArgs args) {
-    gemm_pipeline<false, IO_F32, true>(map_a, map_b, map_c, args);
+    gemm_pipeline<A_TILED, IO_F32, true>(map_a, map_b, map_c, args);
 }
 
 template <bool OUT_BF16>
 __global__ void __launch_bounds__(GEMM_MAX_THREADS, 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                  const __grid_constant__ CUtensorMap map_c, const KernelArgs args) {
-    gemm_pipeline<false, OUT_BF16 ? IO_BF16 : IO_BF16_F32, false>(map_a, map_b, map_c, args);
+    gemm_pipeline<A_TILED, OUT_BF16 ? IO_BF16 : IO_BF16_F32, false>(map_a, map_b, map_c, args);
 }
 
 int choose_block_n(int64_t M, int64_t N, int sm_count, int64_t batches) {
@@ -631,15 +662,32 @@ tfjsb_status gemm_tf32_plan(tfjsb_ctx* ctx, const float* a, const float* bt, flo
     plan->pair = false;
     plan->cluster_split = false;
     plan->gather = false;
+    plan->im2col = false;
     plan->x = nullptr;
     tfjsb_status st;
     if ((st = plan_common(ctx, bt, K, c, plan, batches)) != TFJSB_OK) return st;
     return encode_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, BLOCK_M, "A", batches);
 }
 
+// im2col copies where the channels can be 128-byte rows at least half full (16-byte strides) and the window and padding
+// fit the tensor map's fields.  With fewer channels a k-block per tap is mostly padding and the gathering kernel, which
+// packs the taps, is the faster one.
+bool conv_igemm_uses_im2col(const ConvGeom& g) {
+    const int64_t upper_w = (int64_t)(g.Wo - 1) * g.sw - g.pl - (g.W - 1), upper_h = (int64_t)(g.Ho - 1) * g.sh - g.pt - (g.H - 1);
+    return !conv_patch_supported(g) && g.C % 4 == 0 && g.C >= 16 && g.sh <= 8 && g.sw <= 8 && (int64_t)(g.fh - 1) * g.dh <= 127 && (int64_t)(g.fw - 1) * g.dw <= 127 &&
+           g.pl <= 127 && g.pt <= 127 && upper_w >= -128 && upper_w <= 127 && upper_h >= -128 && upper_h <= 127;
+}
+
 int64_t conv_igemm_k_pad(const ConvGeom& g) {
-    const int64_t k = (int64_t)g.fh * g.fw * g.C;
-    return (k + BLOCK_K - 1) / BLOCK_K * BLOCK_K;
+    const int64_t taps = (int64_t)g.fh * g.fw;
+    if (conv_igemm_uses_im2col(g)) return taps * ((g.C + BLOCK_K - 1) / BLOCK_K * BLOCK_K);
+    return (taps * g.C + BLOCK_K - 1) / BLOCK_K * BLOCK_K;
+}
+
+cudaError_t launch_pack_conv_filter(const float* f, float* out, const ConvGeom& g, cudaStream_t s, int64_t* launches) {
+    const int64_t taps = (int64_t)g.fh * g.fw, k_pad = conv_igemm_k_pad(g);
+    if (conv_igemm_uses_im2col(g)) return launch_pack_filter(f, out, taps, g.C, g.Co, k_pad / taps, s, launches);
+    return launch_pack_filter(f, out, 1, taps * g.C, g.Co, k_pad, s, launches);
 }
 
 bool conv_igemm_supported(const ConvGeom& g) {
@@ -656,14 +704,29 @@ tfjsb_status conv_igemm_plan(tfjsb_ctx* ctx, const float* x, const float* bt, fl
     plan->M = g.N * g.Ho * g.Wo;
     plan->N = g.Co;
     plan->K = (int64_t)g.fh * g.fw * g.C;
-    plan->gather = true;
+    plan->im2col = conv_igemm_uses_im2col(g);
+    plan->gather = !plan->im2col;
     plan->pair = false;
     plan->cluster_split = false;
     plan->x = x;
     plan->g = g;
     tfjsb_status st = plan_common(ctx, bt, conv_igemm_k_pad(g), y, plan);
     if (st != TFJSB_OK) return st;
-    plan->map_a = plan->map_b;  // unused by the gathering kernel; kept initialised
+    if (!plan->im2col) {
+        plan->map_a = plan->map_b;  // unused by the gathering kernel; kept initialised
+        return TFJSB_OK;
+    }
+    plan->K = conv_igemm_k_pad(g);
+    // bounding box: the window's first sample for every output pixel, first to last along W and H
+    cuuint64_t dims[4] = {(cuuint64_t)g.C, (cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)g.N};
+    cuuint64_t strides[3] = {(cuuint64_t)g.C * 4, (cuuint64_t)g.W * g.C * 4, (cuuint64_t)g.H * g.W * g.C * 4};
+    const int lower[2] = {-g.pl, -g.pt};
+    const int upper[2] = {(g.Wo - 1) * g.sw - g.pl - (g.W - 1), (g.Ho - 1) * g.sh - g.pt - (g.H - 1)};
+    cuuint32_t elem[4] = {1u, (cuuint32_t)g.sw, (cuuint32_t)g.sh, 1u};
+    CUresult r = ctx->encode_im2col(&plan->map_a, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(x), dims, strides, lower, upper,
+                                    BLOCK_K, BLOCK_M, elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(ctx, TFJSB_ERR_CUDA, "cuTensorMapEncodeIm2col failed (CUresult " + std::to_string((int)r) + ")");
     return TFJSB_OK;
 }
 
@@ -676,6 +739,7 @@ cudaError_t launch_gemm_tf32(const GemmTf32Plan& plan, const float* bias, int ac
         if (ae == cudaSuccess) ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_tf32_kernel<false>), SMEM_LIMIT - 2048);
         if (ae == cudaSuccess) ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_tf32_kernel<true>), SMEM_LIMIT - 2048);
         if (ae == cudaSuccess) ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_tf32_batched_kernel), SMEM_LIMIT - 2048);
+        if (ae == cudaSuccess) ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_tf32_im2col_kernel), SMEM_LIMIT - 2048);
         if (ae != cudaSuccess) return ae;
     }
     cudaError_t e;
@@ -695,6 +759,9 @@ cudaError_t launch_gemm_tf32(const GemmTf32Plan& plan, const float* bias, int ac
     args.g = plan.g;
     if (plan.gather)
         e = launch_k(gemm_tf32_kernel<true>, dim3(plan.grid), dim3(CONV_THREADS), plan.smem_bytes, s, plan.map_a, plan.map_b,
+                     plan.map_c, args);
+    else if (plan.im2col)
+        e = launch_k(gemm_tf32_im2col_kernel, dim3(plan.grid), dim3(64 + 32 * args.epi_warps), plan.smem_bytes, s, plan.map_a, plan.map_b,
                      plan.map_c, args);
     else if (plan.batches > 1)
         e = launch_k(gemm_tf32_batched_kernel, dim3(plan.grid), dim3(64 + 32 * args.epi_warps), plan.smem_bytes, s, plan.map_a,

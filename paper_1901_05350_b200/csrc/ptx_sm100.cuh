@@ -177,6 +177,18 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// im2col load over an NHWC tensor (rank 4): `pixelsPerColumn` successive base positions of the map's bounding box,
+// starting at column w, row h of image n and running on through rows and images, each displaced by the filter tap
+// (off_w, off_h); channels c0 ..  Samples outside the image, and images past the last, read as zero.
+__device__ __forceinline__ void tma_load_im2col(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int w, int h, int n,
+                                                int off_w, int off_h) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], "
+        "{%7, %8};" ::"r"(dst),
+        "l"(map), "r"(bar), "r"(c0), "r"(w), "r"(h), "r"(n), "h"((uint16_t)off_w), "h"((uint16_t)off_h)
+        : "memory");
+}
+
 // ---- CTA pairs (cta_group::2) ----------------------------------------------------------------------
 // Two CTAs of a cluster (ranks 2i and 2i+1, on the two SMs of one pair) run one tensor-core tile
 // together: the even CTA issues the MMAs, each CTA's tensor core reads the A rows and half of the B

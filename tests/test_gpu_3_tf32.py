@@ -211,6 +211,42 @@ def test_tf32_result_is_deterministic(ctx):
     ctx.check_device_status()
 
 
+IM2COL_CASES = [
+    # N, H, W, Cin, fh, fw, Cout, strides, pad, dilations: A tiles fetched by im2col copies (Cin >= 16, Cin % 4 == 0)
+    (1, 16, 16, 32, 3, 3, 64, (1, 1), "same", (1, 1)),
+    (3, 9, 9, 16, 3, 3, 4, (1, 1), "same", (1, 1)),        # tiles run on from image to image; half-empty k-blocks
+    (2, 13, 21, 64, 3, 3, 68, (1, 1), "same", (1, 1)),     # height and width differ
+    (1, 1, 150, 20, 1, 3, 8, (1, 1), "same", (1, 1)),      # one row
+    (2, 150, 1, 20, 3, 1, 8, (1, 1), "valid", (1, 1)),     # one column
+    (2, 20, 20, 36, 3, 3, 32, (2, 2), "same", (1, 1)),     # even size: padding after only; a k-block of 4 channels
+    (2, 21, 15, 48, 3, 3, 36, (2, 2), "same", (1, 1)),
+    (1, 23, 19, 32, 5, 3, 12, (3, 2), "valid", (1, 1)),    # unequal window and strides, samples that nothing reads
+    (1, 18, 31, 32, 3, 3, 8, (1, 1), "same", (4, 4)),      # dilation
+    (2, 12, 10, 132, 2, 4, 260, (1, 1), "same", (1, 1)),   # even windows: padding after one more than before
+    (4, 9, 7, 64, 1, 1, 40, (2, 2), "same", (1, 1)),       # strided 1x1
+    (9, 30, 30, 64, 3, 3, 64, (1, 1), "same", (1, 1)),     # several tiles per CTA
+    # a large window.  The tensor core cuts its fp32 sums (2^-24 of the sum at most per MMA, 7e-9 seen on average): with
+    # 33 x 33 taps, 4356 MMAs long, that alone is 3e-5; 13 x 13 taps stay below the bar of 2e-5
+    (1, 40, 40, 16, 13, 13, 4, (1, 1), "valid", (1, 1)),
+]
+
+
+@pytest.mark.parametrize("case", IM2COL_CASES)
+def test_conv2d_im2col_copies(ctx, oracle, case):
+    N, H, W, Cin, fh, fw, Cout, strides, pad, dil = case
+    K = fh * fw * Cin
+    xi = si.small_integers(315, 0, (N, H, W, Cin), -4, 4)   # |sums| <= 16 K < 2^24: exact in any order
+    fi = si.small_integers(315, 1, (fh, fw, Cin, Cout), -4, 4)
+    got = host(ctx.conv2d(dev(xi), dev(fi), strides, pad, dil))
+    ctx.check_device_status()
+    assert same_bits(got, oracle.conv2d(xi, fi, strides, pad, dil))
+    x = si.uniform(316, 0, xi.shape, -1, 1)
+    f = si.normal(316, 1, fi.shape, 0, float(np.sqrt(2.0 / K)))
+    b = si.normal(316, 2, (Cout,), 0, 0.5)
+    got = host(ctx.conv2d(dev(x), dev(f), strides, pad, dil, dev(b), "relu"))
+    assert rel_fro(got, oracle.conv2d(x, f, strides, pad, dil, b, "relu", operand="tf32_rz")) <= MATCHED_TOL
+
+
 FUSED_BLOCK_CASES = [
     # N, H, W, C, Cout, pad: depthwise 3x3 stride 1 + pointwise, run by the executor as one fused kernel
     (1, 112, 112, 32, 64, "same"),     # config 2
