@@ -227,8 +227,10 @@ tfjsb_status tfjsb_bias_act(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_t
  * forward output's shape, which is checked.  Sums over pixels are taken in a fixed order: results do
  * not depend on scheduling.  1x1 / stride-1 convolutions run their two gradients as matrix products on
  * the tensor cores in TF32 mode (channel counts multiples of 4; for the filter gradient the pixel count
- * a multiple of 4); every other case runs on CUDA cores in fp32.  All enqueue on `stream` and return;
- * the filter and bias gradients use context-owned scratch (see tfjsb_reserve_scratch). */
+ * a multiple of 4).  Every other case is fp32 arithmetic: in TF32 mode on the tensor cores too where the
+ * channel counts are multiples of 4 (each operand as two TF32 values, which keeps fp32 accuracy), on CUDA
+ * cores otherwise and in FP32 mode.  All enqueue on `stream` and return;
+ * the gradients use context-owned scratch (see tfjsb_reserve_scratch). */
 
 /* dx[n,iy,ix,ci] = sum over (oy,ky), (ox,kx) with oy*sh - pt + ky*dh = iy and ox*sw - pl + kx*dw = ix, and co,
  *                  of dy[n,oy,ox,co] * filter[ky,kx,ci,co].

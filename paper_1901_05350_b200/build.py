@@ -36,6 +36,7 @@ SOURCES = [
     "bf16_storage.cu",
     "backprop.cu",
     "depthwise_grad.cu",
+    "conv_grad_tcgen05.cu",
 ]
 
 NVCC_FLAGS = [

@@ -666,7 +666,11 @@ tfjsb_status tfjsb_conv2d_backprop_input(tfjsb_ctx* ctx, const tfjsb_tensor* dy,
         cudaError_t e = cudaMemsetAsync(pdx, 0, (size_t)numel(dx) * 4, s);
         return e == cudaSuccess ? TFJSB_OK : cuda_fail(ctx, e, "cudaMemsetAsync");
     }
-    if (g.fh == 1 && g.fw == 1 && g.sh == 1 && g.sw == 1)
+    const bool pointwise = g.fh == 1 && g.fw == 1 && g.sh == 1 && g.sw == 1;
+    if (ctx->math == TFJSB_MATH_TF32 && ctx->encode_tiled && conv2d_grad_input_supported(g) &&
+        !(pointwise && gemm_tf32_supported(g.N * g.H * g.W, g.C, g.Co)))
+        return run_conv2d_grad_input(ctx, pg, pf, pdx, g, s);
+    if (pointwise)
         // dx [M, Cin] = dy [M, Cout] . f [Cin, Cout]^T: both operands already have the summed index contiguous
         return matmul_2d(ctx, pg, pf, pdx, g.N * g.H * g.W, g.Co, g.C, 0, 1, s);
     cudaError_t e = launch_conv2d_backprop_input(pg, pf, pdx, g, ctx->sm_count, s, &ctx->launches);
@@ -696,8 +700,11 @@ tfjsb_status tfjsb_conv2d_backprop_filter(tfjsb_ctx* ctx, const tfjsb_tensor* x,
         return e == cudaSuccess ? TFJSB_OK : cuda_fail(ctx, e, "cudaMemsetAsync");
     }
     const bool pointwise = g.fh == 1 && g.fw == 1 && g.sh == 1 && g.sw == 1;
+    if (ctx->math == TFJSB_MATH_TF32 && ctx->encode_tiled && conv2d_grad_filter_supported(g))
+        // plain TF32 for the products that tfjsb_matmul would take too, fp32 accuracy for the rest
+        return run_conv2d_grad_filter(ctx, px, pg, pdf, g, !(pointwise && pixels % 4 == 0), s);
     if (pointwise && ctx->math == TFJSB_MATH_TF32 && ctx->encode_tiled) {
-        // df [Cin, Cout] = x^T . dy, a product whose summed index is the pixel.  The pixels are cut into B
+        // input channels that are no multiple of 4: df [Cin, Cout] = x^T . dy, a product whose summed index is the pixel.  The pixels are cut into B
         // slices; slice b of x and of dy is transposed into scratch ([Cin, M/B] and [Cout, M/B]), the B small
         // products run as one batched launch of the tensor-core GEMM (their tiles share the SMs), and the B
         // partial results are added in slice order.

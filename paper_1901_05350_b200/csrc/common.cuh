@@ -326,6 +326,12 @@ cudaError_t launch_depthwise_backprop_input(const float* dy, const float* f, flo
 // `partial` holds slices * fh*fw*Co floats (unused when slices == 1)
 cudaError_t launch_depthwise_backprop_filter(const float* x, const float* dy, float* df, float* partial, int slices,
                                              const ConvGeom& g, cudaStream_t s, int64_t* launches);
+// Gradients of conv2d on the tensor cores (conv_grad_tcgen05.cu).  fp32 results: operands as two TF32 values each, except
+// the filter gradient with `split` false, which reads them as TF32.  Scratch for partial sums is the context's.
+bool conv2d_grad_input_supported(const ConvGeom& g);
+tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float* f, float* dx, const ConvGeom& g, cudaStream_t s);
+bool conv2d_grad_filter_supported(const ConvGeom& g);
+tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float* dy, float* df, const ConvGeom& g, bool split, cudaStream_t s);
 // Pipelined filter gradient of the 3x3 depthwise convolution (depthwise_grad.cu); depthwise_grad_plan says whether the
 // shape is one of its own.  `partial` holds slices * 9 * C floats (unused when slices == 1).
 struct DepthwiseGradPlan {

@@ -1,0 +1,753 @@
+// Gradients of conv2d on the tensor cores (tcgen05), for any window, stride and dilation with channel counts that are
+// multiples of 4.
+//
+// Precision.  These gradients are fp32 results: every fp32 operand v is used as two TF32 values, hi = v as the tensor
+// core reads it (it drops the low 13 bits) and lo = v - hi rounded to TF32, and a product is hi*hi + hi*lo + lo*hi.
+// What is dropped, lo*lo, is at most 2^-20 of the product and 1e-7 of it on average.  The large products and the two
+// small ones are summed in separate fp32 accumulators in tensor memory and added at the end, so the accumulator that
+// matters sees one addition per eight products.  (Infinite operands give NaN: inf - inf in lo.)  Against the CUDA-core kernels: 2.7e-6 relative for
+// K = 1152 and for 1024-pixel slices.
+// (The filter gradient of a pointwise convolution whose operands are read as plain TF32 runs on the same kernel
+// without the lo half.)
+//
+// Input gradient, conv2d_grad_input_kernel.  In padded coordinates u = iy + pt an input sample of residue a = u mod s
+// receives the taps ky = a + s j from the output rows oy = (u - a) / s - j: for each of the sh * sw residue classes a
+// stride-1 convolution of dy with the class's taps.  It is the implicit GEMM  dx[pixels, Cin] = dy_im2col . f^T  with
+// K = (tap, Cout): both operands have Cout contiguous in memory already, so neither is packed or transposed.
+//   warp 0      producer: A tile = im2col copy of 128 pixels x 32 channels of dy for one tap, B tile = block_n x 32
+//               box of f[tap]; both swizzled K-major operand tiles as they land.
+//   warp 1      MMA issuer: three products per 8 of K.
+//   warps 2-5   epilogue: both accumulators added, staged, and stored row by row to the class's pixels.
+//   warps 6-13  split: lo tile = elementwise function of the landed tile in the same layout (no index arithmetic).
+// All classes are tiles of one launch; with too few tiles for the SMs the K loop is cut and the parts are added
+// by a column sum.  Bound by shared memory: per k-block at block_n 128, 32 KB landed, 64 KB split and 96 KB read by the
+// MMAs are 1500 cycles (768 of MMAs, about 600 of im2col copy); measured 1900.
+// [16,28,28,128], 3x3, 128 channels: 6600 us with one CUDA-core thread per sample, 38 us here.
+//
+// Filter gradient, conv2d_grad_filter_kernel.  df[(tap, ci), co] = sum over pixels: the summed index is the row of
+// both x and dy, so both landed tiles ([32 pixels][32 channels] groups: im2col or matrix boxes) are transposed into
+// operand tiles by the eight converter warps: 4x4 blocks through registers, on diagonals of the group so that the
+// 16-byte reads and writes are both free of bank conflicts under the 128-byte swizzle.  M = four (tap, 32-channel)
+// groups, N = 32..128 channels of dy, one (M tile, N tile, slice of the pixels) per CTA, partial sums added in slice
+// order.  Bound by shared-memory bandwidth (about 1800 cycles per k-block with the lo half, 1000 without, against 768 /
+// 256 of MMAs).  [16,28,28,128], 3x3: 811 us with 32 x 32 tiles on CUDA cores, 36 us here.  Pointwise, plain TF32,
+// [32,56,56] 128 x 128: 36 + 36 us of transposes and 23 + 8 us of batched products, 25 + 6 us here.
+#include "common.cuh"
+#include "ptx_sm100.cuh"
+#include "umma_tile.cuh"
+
+namespace tfjsb {
+
+using namespace ptx;
+using namespace tile;
+
+namespace {
+
+constexpr int EPI_WARPS = 4, CVT_WARPS = 8;
+constexpr int CG_THREADS = (2 + EPI_WARPS + CVT_WARPS) * 32;
+constexpr int CG_MAX_STAGES = 4;
+constexpr int GROUP_BYTES = 4096;  // 32 pixels x 32 channels
+
+__device__ __forceinline__ float tf32_rest(float v) {
+    const float hi = __uint_as_float(__float_as_uint(v) & 0xffffe000u);
+    uint32_t lo;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(v - hi));
+    return __uint_as_float(lo);
+}
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, float w) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+
+// Raises the abort flag; the first role to do so reports the reason.
+__device__ __forceinline__ void give_up(volatile int* abort_flag, unsigned int* dev_status, unsigned int code) {
+    if (!*abort_flag) {
+        *abort_flag = 1;
+        atomicOr(dev_status, code);
+    }
+}
+// Waits (bounded) until the phase has completed, whatever the abort flag says.
+__device__ __forceinline__ void drain(uint32_t bar, uint32_t parity, unsigned int* dev_status) {
+    const unsigned long long t0 = global_ns();
+    while (!mbar_try_wait(bar, parity)) {
+        if (global_ns() - t0 > WAIT_LIMIT_NS) {
+            atomicOr(dev_status, DEV_STATUS_TIMEOUT_DRAIN);
+            break;
+        }
+    }
+}
+__device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t cols) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_free(uint32_t base, uint32_t cols) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
+}
+
+// ---- input gradient --------------------------------------------------------------------------------------
+struct GradInputArgs {
+    int H, W, Cin, Cout, fh, fw, sh, sw, dh, dw, pt, pl;  // the forward convolution's
+    int q0h, q0w, Qh, Qw;    // u / s of the first row / column, and how many
+    int reach_h, reach_w;    // (taps of the largest class - 1) * dilation
+    long long M;             // N * Qh * Qw
+    int m_tiles, n_tiles, block_n, stages, splits, num_tiles;
+    float* out;              // dx, or `splits` of them one after the other
+    long long out_elems;
+    unsigned int* dev_status;
+};
+
+struct GradInputTile {
+    int a, b, m0, n0, kb_begin, kb_end, c_blocks, taps_x, split;
+};
+__device__ __forceinline__ GradInputTile grad_input_tile(const GradInputArgs& g, int t) {
+    GradInputTile r;
+    r.split = t % g.splits;
+    t /= g.splits;
+    r.n0 = (t % g.n_tiles) * g.block_n;
+    t /= g.n_tiles;
+    r.m0 = (t % g.m_tiles) * BLOCK_M;
+    const int cls = t / g.m_tiles;
+    r.a = cls / g.sw;
+    r.b = cls - r.a * g.sw;
+    const int ny = r.a < g.fh ? (g.fh - r.a + g.sh - 1) / g.sh : 0;
+    r.taps_x = r.b < g.fw ? (g.fw - r.b + g.sw - 1) / g.sw : 0;
+    r.c_blocks = (g.Cout + BLOCK_K - 1) / BLOCK_K;
+    const int kbs = ny * r.taps_x * r.c_blocks;
+    r.kb_begin = (int)((long long)kbs * r.split / g.splits);
+    r.kb_end = (int)((long long)kbs * (r.split + 1) / g.splits);
+    return r;
+}
+
+__global__ void __launch_bounds__(CG_THREADS, 1)
+conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_f, const GradInputArgs g) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t bar_full[CG_MAX_STAGES], bar_split[CG_MAX_STAGES], bar_empty[CG_MAX_STAGES];
+    __shared__ __align__(8) uint64_t bar_acc_full[2], bar_acc_empty[2], bar_drain;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag_s;
+    volatile int* abort_flag = &abort_flag_s;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int raw_bytes = A_STAGE_BYTES + g.block_n * 128;
+    const uint32_t epi_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t stage_base = epi_base + EPI_WARPS * EPI_SLAB_BYTES;
+    auto stage_addr = [&](int s) { return stage_base + (uint32_t)s * (uint32_t)(2 * raw_bytes); };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < g.stages; ++s) {
+            mbar_init(smem_u32(&bar_full[s]), 1);
+            mbar_init(smem_u32(&bar_split[s]), CVT_WARPS);
+            mbar_init(smem_u32(&bar_empty[s]), 1);
+        }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(smem_u32(&bar_acc_full[s]), 1);
+            mbar_init(smem_u32(&bar_acc_empty[s]), EPI_WARPS);
+        }
+        mbar_init(smem_u32(&bar_drain), 1);
+        abort_flag_s = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    const uint32_t tmem_cols = (uint32_t)(4 * g.block_n);  // two stages of (large, small) accumulators; block_n 32, 64, 128
+    if (warp == 1) tmem_alloc(smem_u32(&tmem_slot), tmem_cols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int stage = 0, filled = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; ok && t < g.num_tiles; t += gridDim.x) {
+                const GradInputTile r = grad_input_tile(g, t);
+                const int row = r.m0 / g.Qw, img = row / g.Qh;
+                const int h0 = g.q0h + row - img * g.Qh - g.reach_h, w0 = g.q0w + r.m0 - row * g.Qw - g.reach_w;
+                int tap = r.kb_begin / r.c_blocks, cb = r.kb_begin - tap * r.c_blocks;
+                for (int kb = r.kb_begin; kb < r.kb_end; ++kb) {
+                    if (!bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag)) { ok = false; break; }
+                    const int jy = tap / r.taps_x, jx = tap - jy * r.taps_x;
+                    const uint32_t full = smem_u32(&bar_full[stage]), dst = stage_addr(stage);
+                    mbar_arrive_expect_tx(full, (uint32_t)raw_bytes);
+                    tma_load_im2col(dst, &map_dy, full, cb * BLOCK_K, w0, h0, img, g.reach_w - jx * g.dw, g.reach_h - jy * g.dh);
+                    tma_load_3d(dst + A_STAGE_BYTES, &map_f, full, cb * BLOCK_K, r.n0, (r.a + jy * g.sh) * g.fw + r.b + jx * g.sw);
+                    if (++cb == r.c_blocks) { cb = 0; ++tap; }
+                    ++filled;
+                    if (++stage == g.stages) { stage = 0; phase ^= 1u; }
+                }
+            }
+            if (!ok) {
+                give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
+                for (int k = filled > g.stages ? filled - g.stages : 0; k < filled; ++k)
+                    drain(smem_u32(&bar_full[k % g.stages]), (uint32_t)((k / g.stages) & 1), g.dev_status);
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = make_idesc_tf32(BLOCK_M, g.block_n);
+            int stage = 0, acc = 0;
+            uint32_t phase = 0, acc_phase = 0;
+            bool ok = true, issued = false;
+            for (int t = blockIdx.x; ok && t < g.num_tiles; t += gridDim.x) {
+                const GradInputTile r = grad_input_tile(g, t);
+                if (r.kb_begin == r.kb_end) continue;  // no tap reaches these samples
+                if (!bounded_wait(smem_u32(&bar_acc_empty[acc]), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t large = tmem + (uint32_t)(acc * 2 * g.block_n), small = large + (uint32_t)g.block_n;
+                for (int kb = r.kb_begin; kb < r.kb_end; ++kb) {
+                    if (!bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag) ||
+                        !bounded_wait(smem_u32(&bar_split[stage]), phase, abort_flag)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t hi = stage_addr(stage), lo = hi + (uint32_t)raw_bytes;
+                    const uint64_t ah = make_kmajor_sw128_desc(hi), bh = make_kmajor_sw128_desc(hi + A_STAGE_BYTES);
+                    const uint64_t al = make_kmajor_sw128_desc(lo), bl = make_kmajor_sw128_desc(lo + A_STAGE_BYTES);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint64_t o = (uint64_t)(2 * k);
+                        const uint32_t more = (kb != r.kb_begin || k != 0) ? 1u : 0u;
+                        tc_mma_tf32(large, ah + o, bh + o, idesc, more);
+                        tc_mma_tf32(small, ah + o, bl + o, idesc, more);
+                        tc_mma_tf32(small, al + o, bh + o, idesc, 1u);
+                    }
+                    issued = true;
+                    tc_commit(smem_u32(&bar_empty[stage]));
+                    if (++stage == g.stages) { stage = 0; phase ^= 1u; }
+                }
+                if (!ok) break;
+                tc_commit(smem_u32(&bar_acc_full[acc]));
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            }
+            if (!ok) {
+                give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_MMA);
+                if (issued) {
+                    tc_commit(smem_u32(&bar_drain));
+                    drain(smem_u32(&bar_drain), 0u, g.dev_status);
+                }
+            }
+        }
+    } else if (warp < 2 + EPI_WARPS) {
+        const int quad = warp & 3;
+        const uint32_t slab = epi_base + (uint32_t)(warp - 2) * EPI_SLAB_BYTES;
+        const bool vec = (g.Cin & 3) == 0;
+        int acc = 0;
+        uint32_t acc_phase = 0;
+        for (int t = blockIdx.x; t < g.num_tiles; t += gridDim.x) {
+            const GradInputTile r = grad_input_tile(g, t);
+            const bool any = r.kb_begin != r.kb_end;
+            // lane = one sample of dx: where its row of channels goes, or -1
+            long long at = -1;
+            const long long p = (long long)r.m0 + quad * 32 + lane;
+            if (p < g.M) {
+                const long long row = p / g.Qw;
+                const int qx = (int)(p - row * g.Qw);
+                const long long n = row / g.Qh;
+                const int qy = (int)(row - n * g.Qh);
+                const int iy = (g.q0h + qy) * g.sh + r.a - g.pt, ix = (g.q0w + qx) * g.sw + r.b - g.pl;
+                if (iy >= 0 && iy < g.H && ix >= 0 && ix < g.W) at = ((n * g.H + iy) * (long long)g.W + ix) * g.Cin;
+            }
+            if (any) {
+                const bool got = bounded_wait(smem_u32(&bar_acc_full[acc]), acc_phase, abort_flag);
+                if (!__all_sync(0xffffffffu, got)) {
+                    if (lane == 0) give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_EPILOGUE);
+                    break;
+                }
+                tc_fence_after();
+            }
+            float* out = g.out + (long long)r.split * g.out_elems;
+            const int live = min(g.block_n, g.Cin - r.n0);
+            for (int c0 = 0; c0 < live; c0 += 32) {
+                uint32_t u[32], v[32];
+                if (any) {
+                    const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 2 * g.block_n + c0);
+                    tc_ld_32x32(ta, u);
+                    tc_ld_32x32(ta + (uint32_t)g.block_n, v);
+                    tc_ld_wait();
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) u[e] = v[e] = 0u;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    sts4(slab + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4),
+                         __uint_as_float(u[4 * j]) + __uint_as_float(v[4 * j]), __uint_as_float(u[4 * j + 1]) + __uint_as_float(v[4 * j + 1]),
+                         __uint_as_float(u[4 * j + 2]) + __uint_as_float(v[4 * j + 2]),
+                         __uint_as_float(u[4 * j + 3]) + __uint_as_float(v[4 * j + 3]));
+                __syncwarp();
+                const int col0 = r.n0 + c0;
+                if (vec) {
+                    // four rows per step, eight lanes to a row's 128 bytes
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int rr = 4 * i + (lane >> 3), j = lane & 7;
+                        const long long o = __shfl_sync(0xffffffffu, at, rr);
+                        const float4 w = lds4(slab + (uint32_t)rr * 128u + (uint32_t)((j ^ (rr & 7)) << 4));
+                        if (o >= 0 && col0 + 4 * j < g.Cin) *reinterpret_cast<float4*>(out + o + col0 + 4 * j) = w;
+                    }
+                } else {
+                    for (int rr = 0; rr < 32; ++rr) {
+                        const long long o = __shfl_sync(0xffffffffu, at, rr);
+                        float w;
+                        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w) : "r"(slab + (uint32_t)rr * 128u + (uint32_t)((((lane >> 2) ^ (rr & 7)) << 4) + (lane & 3) * 4)) : "memory");
+                        if (o >= 0 && col0 + lane < g.Cin) out[o + col0 + lane] = w;
+                    }
+                }
+                __syncwarp();
+            }
+            if (any) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[acc]));
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            }
+        }
+    } else {
+        const uint32_t mine = (uint32_t)(threadIdx.x - (2 + EPI_WARPS) * 32) * 16u;
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; ok && t < g.num_tiles; t += gridDim.x) {
+            const GradInputTile r = grad_input_tile(g, t);
+            for (int kb = r.kb_begin; kb < r.kb_end; ++kb) {
+                const bool got = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag);
+                if (!__all_sync(0xffffffffu, got)) {
+                    if (lane == 0) give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
+                    ok = false;
+                    break;
+                }
+                const uint32_t src = stage_addr(stage) + mine, dst = src + (uint32_t)raw_bytes;
+                // 256 threads x 16 bytes = 4 KB per step; raw_bytes is a multiple of 4 KB
+#pragma unroll 4
+                for (int o = 0; o < raw_bytes; o += CVT_WARPS * 512) {
+                    const float4 v = lds4(src + (uint32_t)o);
+                    sts4(dst + (uint32_t)o, tf32_rest(v.x), tf32_rest(v.y), tf32_rest(v.z), tf32_rest(v.w));
+                }
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_split[stage]));
+                if (++stage == g.stages) { stage = 0; phase ^= 1u; }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_free(tmem, tmem_cols);
+    }
+}
+
+// ---- filter gradient ---------------------------------------------------------------------------------------
+struct GradFilterArgs {
+    int taps, fw, sh, sw, dh, dw, pt, pl, Ho, Wo;
+    int c_blocks;   // 32-channel blocks of x
+    int groups;     // taps * c_blocks
+    int n_tiles, block_n, raw_stages, op_stages;
+    int pixel_blocks, blocks_per_slice;  // blocks of 32 pixels
+    int m_tiles;
+    int tiled;      // x as a matrix [pixels, Cin] (1x1, stride 1) instead of im2col copies
+    unsigned int* dev_status;
+};
+
+template <bool SPLIT>
+__global__ void __launch_bounds__(CG_THREADS, 1)
+conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_dy,
+                          const __grid_constant__ CUtensorMap map_out, const GradFilterArgs g) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t bar_raw_full[CG_MAX_STAGES], bar_raw_empty[CG_MAX_STAGES];
+    __shared__ __align__(8) uint64_t bar_op_full[CG_MAX_STAGES], bar_op_empty[CG_MAX_STAGES];
+    __shared__ __align__(8) uint64_t bar_acc, bar_drain;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag_s;
+    volatile int* abort_flag = &abort_flag_s;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b_groups = g.block_n >> 5;
+    const int raw_bytes = (4 + b_groups) * GROUP_BYTES;  // A groups, then B groups; an operand stage has the same size
+    const uint32_t epi_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t raw_base = epi_base + EPI_WARPS * EPI_SLAB_BYTES;
+    const uint32_t op_base = raw_base + (uint32_t)(g.raw_stages * raw_bytes);
+    constexpr int HALVES = SPLIT ? 2 : 1;
+
+    int unit = blockIdx.x;
+    const int nt = unit % g.n_tiles;
+    unit /= g.n_tiles;
+    const int mt = unit % g.m_tiles, slice = unit / g.m_tiles;
+    const int g0 = mt * 4, live_groups = min(4, g.groups - g0), n0 = nt * g.block_n;
+    const int pb0 = slice * g.blocks_per_slice;
+    const int kbs = max(0, min(g.blocks_per_slice, g.pixel_blocks - pb0));  // never zero: the host makes no empty slice
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < g.raw_stages; ++s) {
+            mbar_init(smem_u32(&bar_raw_full[s]), 1);
+            mbar_init(smem_u32(&bar_raw_empty[s]), CVT_WARPS);
+        }
+        for (int s = 0; s < g.op_stages; ++s) {
+            mbar_init(smem_u32(&bar_op_full[s]), CVT_WARPS);
+            mbar_init(smem_u32(&bar_op_empty[s]), 1);
+        }
+        mbar_init(smem_u32(&bar_acc), 1);
+        mbar_init(smem_u32(&bar_drain), 1);
+        abort_flag_s = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    const uint32_t tmem_cols = (uint32_t)(HALVES * g.block_n);
+    if (warp == 1) tmem_alloc(smem_u32(&tmem_slot), tmem_cols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int tap_h[4], tap_w[4], ch[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int gi = g0 + i, tap = gi / g.c_blocks;
+                ch[i] = (gi - tap * g.c_blocks) * 32;
+                const int ky = tap / g.fw;
+                tap_h[i] = ky * g.dh;
+                tap_w[i] = (tap - ky * g.fw) * g.dw;
+            }
+            int stage = 0, filled = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int kb = 0; kb < kbs; ++kb) {
+                if (!bounded_wait(smem_u32(&bar_raw_empty[stage]), phase ^ 1u, abort_flag)) { ok = false; break; }
+                const uint32_t full = smem_u32(&bar_raw_full[stage]), dst = raw_base + (uint32_t)(stage * raw_bytes);
+                const int p0 = (pb0 + kb) * 32;
+                mbar_arrive_expect_tx(full, (uint32_t)((live_groups + b_groups) * GROUP_BYTES));
+                const int row = p0 / g.Wo, img = row / g.Ho;
+                const int h0 = (row - img * g.Ho) * g.sh - g.pt, w0 = (p0 - row * g.Wo) * g.sw - g.pl;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (i >= live_groups) break;
+                    if (g.tiled) tma_load_2d(dst + i * GROUP_BYTES, &map_x, full, ch[i], p0);
+                    else tma_load_im2col(dst + i * GROUP_BYTES, &map_x, full, ch[i], w0, h0, img, tap_w[i], tap_h[i]);
+                }
+                for (int i = 0; i < b_groups; ++i) tma_load_2d(dst + (4 + i) * GROUP_BYTES, &map_dy, full, n0 + i * 32, p0);
+                ++filled;
+                if (++stage == g.raw_stages) { stage = 0; phase ^= 1u; }
+            }
+            if (!ok) {
+                give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
+                for (int k = filled > g.raw_stages ? filled - g.raw_stages : 0; k < filled; ++k)
+                    drain(smem_u32(&bar_raw_full[k % g.raw_stages]), (uint32_t)((k / g.raw_stages) & 1), g.dev_status);
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = make_idesc_tf32(BLOCK_M, g.block_n);
+            const uint32_t large = tmem, small = tmem + (uint32_t)g.block_n;
+            int stage = 0;
+            uint32_t phase = 0;
+            bool ok = true, issued = false;
+            for (int kb = 0; kb < kbs; ++kb) {
+                if (!bounded_wait(smem_u32(&bar_op_full[stage]), phase, abort_flag)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t hi = op_base + (uint32_t)(stage * HALVES * raw_bytes), lo = hi + (uint32_t)raw_bytes;
+                const uint64_t ah = make_kmajor_sw128_desc(hi), bh = make_kmajor_sw128_desc(hi + A_STAGE_BYTES);
+                const uint64_t al = make_kmajor_sw128_desc(lo), bl = make_kmajor_sw128_desc(lo + A_STAGE_BYTES);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint64_t o = (uint64_t)(2 * k);
+                    const uint32_t more = (kb | k) != 0 ? 1u : 0u;
+                    tc_mma_tf32(large, ah + o, bh + o, idesc, more);
+                    if (SPLIT) {
+                        tc_mma_tf32(small, ah + o, bl + o, idesc, more);
+                        tc_mma_tf32(small, al + o, bh + o, idesc, 1u);
+                    }
+                }
+                issued = true;
+                tc_commit(smem_u32(&bar_op_empty[stage]));
+                if (++stage == g.op_stages) { stage = 0; phase ^= 1u; }
+            }
+            if (ok) tc_commit(smem_u32(&bar_acc));
+            else {
+                give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_MMA);
+                if (issued) {
+                    tc_commit(smem_u32(&bar_drain));
+                    drain(smem_u32(&bar_drain), 0u, g.dev_status);
+                }
+            }
+        }
+    } else if (warp < 2 + EPI_WARPS) {
+        const int quad = warp & 3;  // the M tile's group whose 32 rows this warp may read
+        const uint32_t slab = epi_base + (uint32_t)(warp - 2) * EPI_SLAB_BYTES;
+        const bool got = bounded_wait(smem_u32(&bar_acc), 0u, abort_flag);
+        if (!__all_sync(0xffffffffu, got)) {
+            if (lane == 0) give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_EPILOGUE);
+        } else if (quad < live_groups) {
+            tc_fence_after();
+            const int gi = g0 + quad, tap = gi / g.c_blocks, ci0 = (gi - tap * g.c_blocks) * 32;
+            for (int c0 = 0; c0 < g.block_n; c0 += 32) {
+                uint32_t u[32], v[32];
+                const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
+                tc_ld_32x32(ta, u);
+                if (SPLIT) tc_ld_32x32(ta + (uint32_t)g.block_n, v);
+                tc_ld_wait();
+                if (lane == 0) tma_store_wait_read<0>();
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    float w[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        w[e] = __uint_as_float(u[4 * j + e]);
+                        if (SPLIT) w[e] += __uint_as_float(v[4 * j + e]);
+                    }
+                    sts4(slab + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4), w[0], w[1], w[2], w[3]);
+                }
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    tma_store_3d(&map_out, slab, n0 + c0, ci0, slice * g.taps + tap);  // clipped at Cout and Cin
+                    tma_store_commit();
+                }
+            }
+            if (lane == 0) tma_store_wait_all();
+            __syncwarp();
+        }
+    } else {
+        const int w = warp - 2 - EPI_WARPS;
+        const int l = lane & 7, sub = lane >> 3;
+        int rs = 0, os = 0;
+        uint32_t rphase = 0, ophase = 0;
+        for (int kb = 0; kb < kbs; ++kb) {
+            const bool got = bounded_wait(smem_u32(&bar_raw_full[rs]), rphase, abort_flag) &&
+                             bounded_wait(smem_u32(&bar_op_empty[os]), ophase ^ 1u, abort_flag);
+            if (!__all_sync(0xffffffffu, got)) {
+                if (lane == 0) give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
+                break;
+            }
+            const uint32_t raw = raw_base + (uint32_t)(rs * raw_bytes), hi = op_base + (uint32_t)(os * HALVES * raw_bytes);
+            for (int step = w; step < 2 * (4 + b_groups); step += CVT_WARPS) {
+                const int grp = step >> 1;
+                if (grp >= live_groups && grp < 4) continue;  // rows that nothing reads
+                // eight lanes: pixel quad l and channel quad l ^ base, so that neither the reads (slot q ^ pixel % 8) nor
+                // the writes (slot l ^ channel % 8) of the eight meet in a bank
+                const int q = l ^ ((step & 1) * 4 + sub);
+                float4 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int px = 4 * l + i;
+                    v[i] = lds4(raw + (uint32_t)(grp * GROUP_BYTES + px * 128 + ((q ^ (px & 7)) << 4)));
+                }
+                const float* f = reinterpret_cast<const float*>(v);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int row = 4 * q + e;
+                    const uint32_t at = (uint32_t)(grp * GROUP_BYTES + row * 128 + ((l ^ (row & 7)) << 4));
+                    sts4(hi + at, f[e], f[4 + e], f[8 + e], f[12 + e]);
+                    if (SPLIT)
+                        sts4(hi + (uint32_t)raw_bytes + at, tf32_rest(f[e]), tf32_rest(f[4 + e]), tf32_rest(f[8 + e]), tf32_rest(f[12 + e]));
+                }
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(smem_u32(&bar_raw_empty[rs]));
+                mbar_arrive(smem_u32(&bar_op_full[os]));
+            }
+            if (++rs == g.raw_stages) { rs = 0; rphase ^= 1u; }
+            if (++os == g.op_stages) { os = 0; ophase ^= 1u; }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_free(tmem, tmem_cols);
+    }
+}
+
+constexpr int CG_SMEM = SMEM_LIMIT - 1024;  // beside the barriers
+
+tfjsb_status encode(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int rank, const int64_t* dims, const uint32_t* box, const char* what) {
+    cuuint64_t d[3], st[2];
+    cuuint32_t b[3], elem[3] = {1u, 1u, 1u};
+    cuuint64_t pitch = 4;
+    for (int i = 0; i < rank; ++i) {
+        d[i] = (cuuint64_t)dims[i];
+        b[i] = box[i];
+        pitch *= d[i];
+        if (i + 1 < rank) st[i] = pitch;
+    }
+    CUresult r = ctx->encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), d, st, b, elem,
+                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(ctx, TFJSB_ERR_CUDA, std::string("cuTensorMapEncodeTiled failed for ") + what + " (CUresult " + std::to_string((int)r) + ")");
+    return TFJSB_OK;
+}
+
+tfjsb_status encode_im2col(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int64_t n, int h, int w, int c, const int lower[2],
+                           const int upper[2], int sw, int sh, int pixels, const char* what) {
+    cuuint64_t d[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
+    cuuint64_t st[3] = {(cuuint64_t)c * 4, (cuuint64_t)w * c * 4, (cuuint64_t)h * w * c * 4};
+    cuuint32_t elem[4] = {1u, (cuuint32_t)sw, (cuuint32_t)sh, 1u};
+    CUresult r = ctx->encode_im2col(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(base), d, st, lower, upper, 32,
+                                    (cuuint32_t)pixels, elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(ctx, TFJSB_ERR_CUDA, std::string("cuTensorMapEncodeIm2col failed for ") + what + " (CUresult " + std::to_string((int)r) + ")");
+    return TFJSB_OK;
+}
+
+bool corner_ok(int64_t v) { return v >= -128 && v <= 127; }
+
+}  // namespace
+
+// u / s of the first sample along one dimension, and how many values it takes
+static void grad_rows(int size, int pad, int s, int* q0, int* count) {
+    *q0 = pad / s;
+    *count = (size - 1 + pad) / s - *q0 + 1;
+}
+
+bool conv2d_grad_input_supported(const ConvGeom& g) {
+    int q0h, q0w, Qh, Qw;
+    grad_rows(g.H, g.pt, g.sh, &q0h, &Qh);
+    grad_rows(g.W, g.pl, g.sw, &q0w, &Qw);
+    const int64_t reach_h = (int64_t)((g.fh - 1) / g.sh) * g.dh, reach_w = (int64_t)((g.fw - 1) / g.sw) * g.dw;
+    const int64_t m_tiles = (g.N * Qh * Qw + BLOCK_M - 1) / BLOCK_M;
+    return g.Co % 4 == 0 && reach_h <= 127 && reach_w <= 127 && corner_ok(q0h - reach_h) && corner_ok(q0w - reach_w) &&
+           corner_ok(q0h - reach_h + Qh - g.Ho) && corner_ok(q0w - reach_w + Qw - g.Wo) && g.Ho > 0 && g.Wo > 0 &&
+           g.N * Qh * Qw < (1LL << 31) - 256 && m_tiles * g.sh * g.sw * ((g.C + 31) / 32) * 16 < (1LL << 31) &&
+           (int64_t)g.fh * g.fw * ((g.Co + 31) / 32) < (1LL << 24);
+}
+
+tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float* f, float* dx, const ConvGeom& g, cudaStream_t s) {
+    GradInputArgs a{};
+    a.H = g.H; a.W = g.W; a.Cin = g.C; a.Cout = g.Co; a.fh = g.fh; a.fw = g.fw;
+    a.sh = g.sh; a.sw = g.sw; a.dh = g.dh; a.dw = g.dw; a.pt = g.pt; a.pl = g.pl;
+    grad_rows(g.H, g.pt, g.sh, &a.q0h, &a.Qh);
+    grad_rows(g.W, g.pl, g.sw, &a.q0w, &a.Qw);
+    a.reach_h = (g.fh - 1) / g.sh * g.dh;
+    a.reach_w = (g.fw - 1) / g.sw * g.dw;
+    a.M = g.N * a.Qh * a.Qw;
+    a.m_tiles = (int)((a.M + BLOCK_M - 1) / BLOCK_M);
+    // Tile width: the fewest rounds, each as long as the slower of the MMAs (6 cycles per column and k-block) and the
+    // im2col copy (about 600 cycles per k-block).
+    const int sms = ctx->sm_count;
+    const int classes = g.sh * g.sw;
+    int64_t best = INT64_MAX;
+    for (int bn = 32; bn <= 128; bn <<= 1) {
+        const int64_t tiles = (int64_t)a.m_tiles * ((g.C + bn - 1) / bn) * classes;
+        const int64_t cost = (tiles + sms - 1) / sms * (6 * bn > 600 ? 6 * bn : 600);
+        if (cost < best) { best = cost; a.block_n = bn; }
+        if (bn >= g.C) break;
+    }
+    a.n_tiles = (g.C + a.block_n - 1) / a.block_n;
+    const int64_t tiles = (int64_t)a.m_tiles * a.n_tiles * classes;
+    const int kbs = ((g.fh + g.sh - 1) / g.sh) * ((g.fw + g.sw - 1) / g.sw) * ((g.Co + 31) / 32);  // of the largest class
+    // fewer tiles than half the SMs: the K loop in parts of at least eight k-blocks
+    a.splits = 1;
+    if (2 * tiles <= sms) {
+        a.splits = (int)(sms / tiles);
+        if (a.splits > kbs / 8) a.splits = kbs / 8;
+        if (a.splits > 16) a.splits = 16;
+        if (a.splits < 1) a.splits = 1;
+    }
+    a.num_tiles = (int)(tiles * a.splits);
+    const int stage_bytes = 2 * (A_STAGE_BYTES + a.block_n * 128);
+    a.stages = (CG_SMEM - 1024 - EPI_WARPS * EPI_SLAB_BYTES) / stage_bytes;
+    if (a.stages > CG_MAX_STAGES) a.stages = CG_MAX_STAGES;
+    a.out_elems = (long long)g.N * g.H * g.W * g.C;
+    a.dev_status = ctx->dev_status;
+    tfjsb_status st;
+    a.out = dx;
+    if (a.splits > 1) {
+        if ((st = ensure_scratch(ctx, &ctx->scratch_c, (size_t)a.splits * a.out_elems * 4)) != TFJSB_OK) return st;
+        a.out = ctx->scratch_c.ptr;
+    }
+    CUtensorMap map_dy, map_f;
+    const int lower[2] = {a.q0w - a.reach_w, a.q0h - a.reach_h};
+    const int upper[2] = {lower[0] + a.Qw - g.Wo, lower[1] + a.Qh - g.Ho};
+    if ((st = encode_im2col(ctx, &map_dy, dy, g.N, g.Ho, g.Wo, g.Co, lower, upper, 1, 1, BLOCK_M, "dy")) != TFJSB_OK) return st;
+    const int64_t fd[3] = {g.Co, g.C, (int64_t)g.fh * g.fw};
+    const uint32_t fb[3] = {32u, (uint32_t)a.block_n, 1u};
+    if ((st = encode(ctx, &map_f, f, 3, fd, fb, "the filter")) != TFJSB_OK) return st;
+    cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(&conv2d_grad_input_kernel), CG_SMEM);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "shared-memory limit");
+    const size_t smem = 1024 + (size_t)EPI_WARPS * EPI_SLAB_BYTES + (size_t)a.stages * stage_bytes;
+    const int grid = a.num_tiles < sms ? a.num_tiles : sms;
+    if ((e = launch_k(conv2d_grad_input_kernel, dim3(grid), dim3(CG_THREADS), smem, s, map_dy, map_f, a)) != cudaSuccess)
+        return cuda_fail(ctx, e, "conv2d_grad_input launch");
+    ++ctx->launches;
+    if (a.splits > 1 && (e = launch_sum_rows(a.out, dx, nullptr, a.splits, a.out_elems, 1, s, &ctx->launches)) != cudaSuccess)
+        return cuda_fail(ctx, e, "partial-sum launch");
+    return TFJSB_OK;
+}
+
+bool conv2d_grad_filter_supported(const ConvGeom& g) {
+    const int64_t upper_w = (int64_t)(g.Wo - 1) * g.sw - g.pl - (g.W - 1), upper_h = (int64_t)(g.Ho - 1) * g.sh - g.pt - (g.H - 1);
+    const int64_t pixels = g.N * g.Ho * g.Wo, taps = (int64_t)g.fh * g.fw;
+    const bool tiled = taps == 1 && g.sh == 1 && g.sw == 1;
+    return g.C % 4 == 0 && g.Co % 4 == 0 && g.C > 0 && g.Co > 0 && pixels > 0 && pixels < (1LL << 31) - 256 &&
+           (tiled || (g.sh <= 8 && g.sw <= 8 && (int64_t)(g.fh - 1) * g.dh <= 127 && (int64_t)(g.fw - 1) * g.dw <= 127 && g.pl <= 127 &&
+                      g.pt <= 127 && corner_ok(upper_w) && corner_ok(upper_h))) &&
+           taps * ((g.C + 31) / 32) * ((g.Co + 31) / 32) < (1LL << 20);
+}
+
+tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float* dy, float* df, const ConvGeom& g, bool split, cudaStream_t s) {
+    GradFilterArgs a{};
+    const int64_t pixels = g.N * g.Ho * g.Wo;
+    a.taps = g.fh * g.fw; a.fw = g.fw; a.sh = g.sh; a.sw = g.sw; a.dh = g.dh; a.dw = g.dw; a.pt = g.pt; a.pl = g.pl;
+    a.Ho = g.Ho; a.Wo = g.Wo;
+    a.c_blocks = (g.C + 31) / 32;
+    a.groups = a.taps * a.c_blocks;
+    a.m_tiles = (a.groups + 3) / 4;
+    a.block_n = g.Co > 64 ? 128 : (g.Co > 32 ? 64 : 32);
+    a.n_tiles = (g.Co + a.block_n - 1) / a.block_n;
+    a.tiled = a.taps == 1 && g.sh == 1 && g.sw == 1;
+    a.pixel_blocks = (int)((pixels + 31) / 32);
+    a.dev_status = ctx->dev_status;
+    // One wave of CTAs; a slice has at least 4 blocks of 32 pixels, and at most 32 (1024 additions per 8 products keep
+    // the rounding of the accumulator below 1e-6), the latter while the partial sums stay smaller than the operands.
+    const int64_t units = (int64_t)a.m_tiles * a.n_tiles, elems = (int64_t)a.taps * g.C * g.Co;
+    int64_t slices = ctx->sm_count / units;
+    if (slices < (a.pixel_blocks + 31) / 32) {
+        int64_t more = (a.pixel_blocks + 31) / 32;
+        const int64_t most = pixels * (g.C + g.Co) / elems + 1;
+        if (more > most) more = most;
+        if (slices < more) slices = (more * units + ctx->sm_count - 1) / ctx->sm_count * ctx->sm_count / units;
+    }
+    if (slices > (a.pixel_blocks + 3) / 4) slices = (a.pixel_blocks + 3) / 4;
+    if (slices < 1) slices = 1;
+    a.blocks_per_slice = (int)((a.pixel_blocks + slices - 1) / slices);
+    slices = (a.pixel_blocks + a.blocks_per_slice - 1) / a.blocks_per_slice;
+    const int raw_bytes = (4 + a.block_n / 32) * GROUP_BYTES, halves = split ? 2 : 1;
+    a.op_stages = split ? 2 : 3;
+    a.raw_stages = (CG_SMEM - 1024 - EPI_WARPS * EPI_SLAB_BYTES - a.op_stages * halves * raw_bytes) / raw_bytes;
+    if (a.raw_stages > CG_MAX_STAGES) a.raw_stages = CG_MAX_STAGES;
+    tfjsb_status st;
+    float* out = df;
+    if (slices > 1) {
+        if ((st = ensure_scratch(ctx, &ctx->scratch_c, (size_t)slices * elems * 4)) != TFJSB_OK) return st;
+        out = ctx->scratch_c.ptr;
+    }
+    CUtensorMap map_x, map_dy, map_out;
+    const uint32_t box[3] = {32u, 32u, 1u};
+    if (a.tiled) {
+        const int64_t d[2] = {g.C, pixels};
+        if ((st = encode(ctx, &map_x, x, 2, d, box, "x")) != TFJSB_OK) return st;
+    } else {
+        const int lower[2] = {-g.pl, -g.pt};
+        const int upper[2] = {(g.Wo - 1) * g.sw - g.pl - (g.W - 1), (g.Ho - 1) * g.sh - g.pt - (g.H - 1)};
+        if ((st = encode_im2col(ctx, &map_x, x, g.N, g.H, g.W, g.C, lower, upper, g.sw, g.sh, 32, "x")) != TFJSB_OK) return st;
+    }
+    const int64_t dd[2] = {g.Co, pixels}, od[3] = {g.Co, g.C, slices * a.taps};
+    if ((st = encode(ctx, &map_dy, dy, 2, dd, box, "dy")) != TFJSB_OK) return st;
+    if ((st = encode(ctx, &map_out, out, 3, od, box, "the filter gradient")) != TFJSB_OK) return st;
+    auto kernel = split ? conv2d_grad_filter_kernel<true> : conv2d_grad_filter_kernel<false>;
+    cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kernel), CG_SMEM);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "shared-memory limit");
+    const size_t smem = 1024 + (size_t)EPI_WARPS * EPI_SLAB_BYTES + (size_t)(a.raw_stages + a.op_stages * halves) * raw_bytes;
+    if ((e = launch_k(kernel, dim3((unsigned)(units * slices)), dim3(CG_THREADS), smem, s, map_x, map_dy, map_out, a)) != cudaSuccess)
+        return cuda_fail(ctx, e, "conv2d_grad_filter launch");
+    ++ctx->launches;
+    if (slices > 1 && (e = launch_sum_rows(out, df, nullptr, slices, elems, 1, s, &ctx->launches)) != cudaSuccess)
+        return cuda_fail(ctx, e, "partial-sum launch");
+    return TFJSB_OK;
+}
+
+}  // namespace tfjsb

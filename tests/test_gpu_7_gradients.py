@@ -81,6 +81,52 @@ def test_depthwise_gradients(ctx, oracle, case, mult):
     assert rel_fro(df, oracle.depthwise_conv2d_backprop_filter(x, f.shape, g, (s, s), pad, (d, d))) <= 1e-5
 
 
+SPLIT_CASES = [
+    # N, H, W, Cin, Cout, fh, fw, stride, dilation, pad: fp32 gradients on the tensor cores in TF32 mode
+    (1, 5, 5, 4, 4, 3, 3, 1, 1, "same"),         # everything smaller than a tile
+    (2, 16, 16, 32, 32, 3, 3, 1, 1, "same"),
+    (3, 13, 17, 36, 68, 3, 3, 1, 1, "same"),     # ragged channel blocks, two 64-wide column tiles or one of 128
+    (2, 12, 12, 160, 40, 3, 3, 1, 1, "valid"),   # five 32-channel blocks: M tiles across taps
+    (2, 14, 15, 40, 132, 3, 3, 2, 1, "same"),    # four residue classes, two column tiles of dy
+    (2, 15, 14, 24, 20, 3, 3, 2, 1, "valid"),    # samples that no output reads
+    (1, 17, 19, 16, 16, 5, 4, 3, 1, "same"),     # nine classes, uneven numbers of taps
+    (2, 11, 13, 16, 8, 2, 2, 4, 1, "same"),      # classes without a tap: exact zeros
+    (2, 9, 9, 8, 8, 1, 1, 2, 1, "same"),         # strided 1x1
+    (1, 14, 18, 32, 24, 3, 3, 1, 2, "same"),     # dilated
+    (2, 8, 9, 3, 32, 3, 3, 2, 1, "same"),        # three input channels: input gradient with scalar stores
+    (2, 9, 11, 6, 12, 1, 1, 1, 1, "same"),       # pointwise, Cin no multiple of 4
+    (1, 7, 7, 128, 256, 3, 3, 1, 1, "same"),     # few tiles, long K: parts of the K loop
+    (24, 28, 28, 64, 64, 3, 3, 1, 1, "same"),    # several tiles per CTA, slices of 32 pixel blocks
+]
+
+
+@pytest.mark.parametrize("case", SPLIT_CASES)
+def test_conv2d_gradients_keep_fp32_accuracy_in_tf32_mode(ctx, oracle, case):
+    N, H, W, Cin, Cout, fh, fw, s, d, pad = case
+    Ho, Wo = geometry(oracle, H, W, fh, fw, s, d, pad)
+    args = ((s, s), pad, (d, d))
+    # small integers: hi parts and their products exact, lo parts zero
+    x = si.small_integers(93, 0, (N, H, W, Cin), -3, 3)
+    f = si.small_integers(93, 1, (fh, fw, Cin, Cout), -3, 3)
+    g = si.small_integers(93, 2, (N, Ho, Wo, Cout), -3, 3)
+    dx = host(ctx.conv2d_backprop_input(x.shape, dev(f), dev(g), *args))
+    df = host(ctx.conv2d_backprop_filter(dev(x), f.shape, dev(g), *args))
+    ctx.check_device_status()
+    assert same_bits(dx + 0.0, oracle.conv2d_backprop_input(x.shape, f, g, *args) + 0.0)
+    assert same_bits(df + 0.0, oracle.conv2d_backprop_filter(x, f.shape, g, *args) + 0.0)
+    # the bar of the CUDA-core kernels.  Operands are 2^-21 at worst; K <= 2304 makes 288 additions of eight products,
+    # each cut by at most 2^-23 of the sum (7e-9 seen on average)
+    x = si.uniform(94, 0, x.shape, -1, 1)
+    f = si.normal(94, 1, f.shape, 0, 0.3)
+    g = si.normal(94, 2, g.shape, 0, 1)
+    dx = host(ctx.conv2d_backprop_input(x.shape, dev(f), dev(g), *args))
+    df = host(ctx.conv2d_backprop_filter(dev(x), f.shape, dev(g), *args))
+    ctx.check_device_status()
+    assert rel_fro(dx, oracle.conv2d_backprop_input(x.shape, f, g, *args)) <= 1e-5
+    # a pointwise filter gradient with a multiple of 4 pixels is a TF32 product
+    assert rel_fro(df, oracle.conv2d_backprop_filter(x, f.shape, g, *args)) <= 1e-5
+
+
 DEPTHWISE_3X3_CASES = [
     # N, H, W, C, stride, dilation, pad: tile edges of the pipelined kernels and of the stride-2 column pairs
     (1, 1, 1, 4, 1, 1, "same"),
