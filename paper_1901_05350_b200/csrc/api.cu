@@ -306,6 +306,13 @@ static tfjsb_status matmul_2d(tfjsb_ctx* ctx, const float* pa, const float* pb, 
     }
     const int64_t a_rs = transpose_a ? 1 : K, a_cs = transpose_a ? M : 1;
     const int64_t b_rs = transpose_b ? 1 : N, b_cs = transpose_b ? K : 1;
+    if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(1, M, N, K)) {
+        // rows that are no multiples of 16 bytes: fp32 accuracy on the tensor cores
+        if ((e = launch_gemm_strided(pa, a_rs, a_cs, pb, b_rs, b_cs, nullptr, TFJSB_ACT_NONE, pc, 1, M, N, K, ctx->sm_count,
+                                     ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
+            return cuda_fail(ctx, e, "strided gemm launch");
+        return TFJSB_OK;
+    }
     if ((e = launch_gemm_fp32(pa, a_rs, a_cs, pb, b_rs, b_cs, nullptr, TFJSB_ACT_NONE, pc, N, M, N, K, s,
                               &ctx->launches)) != cudaSuccess)
         return cuda_fail(ctx, e, "fp32 gemm launch");
@@ -402,6 +409,12 @@ tfjsb_status tfjsb_batch_matmul(tfjsb_ctx* ctx, const tfjsb_tensor* a, const tfj
             return cuda_fail(ctx, e, "batched tf32 gemm launch");
         return TFJSB_OK;
     }
+    if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(B, M, N, K) && !gemm_tf32_supported(M, N, K)) {
+        cudaError_t e = launch_gemm_strided(pa, transpose_a ? 1 : K, transpose_a ? M : 1, pb, transpose_b ? 1 : N, transpose_b ? K : 1,
+                                            nullptr, TFJSB_ACT_NONE, pc, B, M, N, K, ctx->sm_count, ctx->dev_status, s, &ctx->launches);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "batched strided gemm launch");
+        return TFJSB_OK;
+    }
     for (int64_t i = 0; i < B; ++i) {
         st = matmul_2d(ctx, pa + i * M * K, pb + i * K * N, pc + i * M * N, M, K, N, transpose_a, transpose_b,
                        static_cast<cudaStream_t>(stream));
@@ -450,6 +463,12 @@ tfjsb_status tfjsb_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_ten
             if ((st = gemm_tf32_plan(ctx, px, ctx->scratch_b.ptr, py, M, N, K, &plan)) != TFJSB_OK) return st;
             if ((e = launch_gemm_tf32(plan, pbias, act, ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
                 return cuda_fail(ctx, e, "tf32 gemm launch");
+            return TFJSB_OK;
+        }
+        if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(1, M, N, K)) {
+            if ((e = launch_gemm_strided(px, K, 1, pf, N, 1, pbias, act, py, 1, M, N, K, ctx->sm_count, ctx->dev_status, s,
+                                         &ctx->launches)) != cudaSuccess)
+                return cuda_fail(ctx, e, "strided gemm launch");
             return TFJSB_OK;
         }
         if ((e = launch_gemm_fp32(px, K, 1, pf, N, 1, pbias, act, py, N, M, N, K, s, &ctx->launches)) != cudaSuccess)

@@ -188,6 +188,13 @@ cudaError_t launch_gemm_fp32(const float* a, int64_t a_rs, int64_t a_cs, const f
                              const float* bias, int act, float* c, int64_t ldc, int64_t M, int64_t N, int64_t K,
                              cudaStream_t s, int64_t* launches);
 
+// The same with fp32 accuracy on the tensor cores, for operands with either dimension contiguous and any alignment
+// (gemm_strided_tcgen05.cu); `batches` products stored one after the other.
+bool gemm_strided_supported(int64_t batches, int64_t M, int64_t N, int64_t K);
+cudaError_t launch_gemm_strided(const float* a, int64_t a_rs, int64_t a_ks, const float* b, int64_t b_ks, int64_t b_cs, const float* bias,
+                                int act, float* c, int64_t batches, int64_t M, int64_t N, int64_t K, int sm_count,
+                                unsigned int* dev_status, cudaStream_t s, int64_t* launches);
+
 // Direct convolution on CUDA cores (any window, stride, dilation).  filter [fh,fw,Cin,Cout].
 cudaError_t launch_conv2d_fp32(const float* x, const float* f, const float* bias, int act, float* y,
                                const ConvGeom& g, cudaStream_t s, int64_t* launches);

@@ -48,12 +48,6 @@ constexpr int CG_THREADS = (2 + EPI_WARPS + CVT_WARPS) * 32;
 constexpr int CG_MAX_STAGES = 4;
 constexpr int GROUP_BYTES = 4096;  // 32 pixels x 32 channels
 
-__device__ __forceinline__ float tf32_rest(float v) {
-    const float hi = __uint_as_float(__float_as_uint(v) & 0xffffe000u);
-    uint32_t lo;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(v - hi));
-    return __uint_as_float(lo);
-}
 __device__ __forceinline__ float4 lds4(uint32_t a) {
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");

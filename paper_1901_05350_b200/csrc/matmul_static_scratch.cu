@@ -121,9 +121,15 @@ extern "C" tfjsb_status tfjsb_matmul_static_scratch(tfjsb_ctx* ctx, const tfjsb_
             return cuda_fail(ctx, e, "tf32 gemm launch");
         return TFJSB_OK;
     }
-    // CUDA-core path: strided operand access, no scratch at all
+    // rows that are no multiples of 16 bytes, or FP32 mode: strided operand access, no scratch at all
     const int64_t a_rs = transpose_a ? 1 : K, a_cs = transpose_a ? M : 1;
     const int64_t b_rs = transpose_b ? 1 : N, b_cs = transpose_b ? K : 1;
+    if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(1, M, N, K)) {
+        if ((e = launch_gemm_strided(pa, a_rs, a_cs, pb, b_rs, b_cs, nullptr, TFJSB_ACT_NONE, pc, 1, M, N, K, ctx->sm_count,
+                                     ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
+            return cuda_fail(ctx, e, "strided gemm launch");
+        return TFJSB_OK;
+    }
     if ((e = launch_gemm_fp32(pa, a_rs, a_cs, pb, b_rs, b_cs, nullptr, TFJSB_ACT_NONE, pc, N, M, N, K, s,
                               &ctx->launches)) != cudaSuccess)
         return cuda_fail(ctx, e, "fp32 gemm launch");

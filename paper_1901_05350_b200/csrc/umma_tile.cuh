@@ -43,6 +43,14 @@ __device__ __forceinline__ void stage_chunk(const uint32_t (&r)[32], const float
     }
 }
 
+// What the tensor core drops of an fp32 operand it reads as TF32, rounded to TF32: v = tf32(v) + tf32_rest(v) to 2^-21.
+__device__ __forceinline__ float tf32_rest(float v) {
+    const float hi = __uint_as_float(__float_as_uint(v) & 0xffffe000u);
+    uint32_t lo;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(v - hi));
+    return __uint_as_float(lo);
+}
+
 // ---- bfloat16 storage ------------------------------------------------------------------------------
 // Instruction descriptor: fp32 accumulator, bfloat16 A and B (format 1), both K-major.
 __device__ __forceinline__ uint32_t make_idesc_bf16(int m, int n) {

@@ -211,6 +211,61 @@ def test_tf32_result_is_deterministic(ctx):
     ctx.check_device_status()
 
 
+STRIDED_CASES = [
+    # batch (0: rank 2), M, K, N: rows that are no multiples of 16 bytes, fp32 accuracy on the tensor cores
+    (0, 1, 1, 1),
+    (0, 128, 32, 33),       # one tile and one column more
+    (0, 31, 33, 129),       # the transposed tile is the smaller one
+    (0, 64, 1024, 101),     # few tiles, long K: a cluster of eight
+    (0, 5, 513, 7),         # a cluster, last k-block of one
+    (0, 200, 150, 257),     # K % 4 != 0
+    (0, 999, 66, 1001),     # more tiles than SMs
+    (0, 130, 4099, 61),     # three accumulators per slice
+    (7, 199, 64, 199),
+    (150, 17, 19, 23),      # more products than SMs
+    (3, 40, 700, 30),       # a cluster per product
+]
+
+
+@pytest.mark.parametrize("ta", [False, True])
+@pytest.mark.parametrize("tb", [False, True])
+@pytest.mark.parametrize("case", STRIDED_CASES)
+def test_matmul_of_unaligned_rows(ctx, oracle, case, ta, tb):
+    B, M, K, N = case
+    lead = (B,) if B else ()
+    sa, sb = lead + ((K, M) if ta else (M, K)), lead + ((N, K) if tb else (K, N))
+    call, want = (ctx.batch_matmul, oracle.batch_matmul) if B else (ctx.matmul, oracle.matmul)
+    a, b = si.small_integers(321, 0, sa, -8, 8), si.small_integers(321, 1, sb, -8, 8)
+    got = host(call(dev(a), dev(b), ta, tb))  # |sums| <= 64 K < 2^24: exact in any order
+    ctx.check_device_status()
+    assert same_bits(got + 0.0, want(a, b, ta, tb) + 0.0)
+    a, b = si.uniform(322, 0, sa, -1, 1), si.uniform(322, 1, sb, -1, 1)
+    # the bar of the CUDA-core kernel: operands to 2^-21, at most 4099 / 8 / 3 additions per accumulator
+    assert rel_fro(host(call(dev(a), dev(b), ta, tb)), want(a, b, ta, tb)) <= 1e-5
+
+
+@pytest.mark.parametrize("classes", [1, 33, 101, 1001])
+@pytest.mark.parametrize("batch", [1, 3, 130])
+def test_unaligned_epilogue_and_dense_layer(ctx, oracle, batch, classes):
+    """Bias and activation of the same kernel: a pointwise convolution and a model's dense layer."""
+    from seeded_inputs.workloads import Layer
+
+    x = si.uniform(323, 0, (batch, 5, 3, 70), -1, 1)
+    f, b = si.normal(323, 1, (1, 1, 70, classes), 0, 0.2), si.normal(323, 2, (classes,), 0, 0.5)
+    got = host(ctx.conv2d(dev(x), dev(f), bias=dev(b), act="relu6"))
+    assert rel_fro(got, oracle.conv2d(x, f, bias=b, act="relu6")) <= 1e-5
+    layer = Layer("dense", act="relu", out_channels=classes)
+    layer.filter, layer.bias = si.normal(323, 3, (5 * 3 * 70, classes), 0, 0.05), b
+    model = ctx.model([layer], x.shape)
+    xd = dev(x)
+    for graph in (False, True):
+        model.set_graph(graph)
+        assert rel_fro(host(model.run(xd)), oracle.run_model([layer], x)) <= 1e-5
+    assert model.layer_kernels() == ["gemm_strided_kernel"]
+    ctx.check_device_status()
+    model.close()
+
+
 IM2COL_CASES = [
     # N, H, W, Cin, fh, fw, Cout, strides, pad, dilations: A tiles fetched by im2col copies (Cin >= 16, Cin % 4 == 0)
     (1, 16, 16, 32, 3, 3, 64, (1, 1), "same", (1, 1)),
