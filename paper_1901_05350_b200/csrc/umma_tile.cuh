@@ -43,12 +43,12 @@ __device__ __forceinline__ void stage_chunk(const uint32_t (&r)[32], const float
     }
 }
 
-// What the tensor core drops of an fp32 operand it reads as TF32, rounded to TF32: v = tf32(v) + tf32_rest(v) to 2^-21.
+// What the tensor core drops of an fp32 operand it reads as TF32, rounded to TF32 (half away from zero; the bits below are
+// left in, the tensor core drops them): v = tf32(v) + tf32(tf32_rest(v)) to 2^-21.  With the conversion instruction
+// instead of the integer addition a 2001^3 product took 243 us instead of 220, a 3x3 convolution's gradients 6 us more.
 __device__ __forceinline__ float tf32_rest(float v) {
     const float hi = __uint_as_float(__float_as_uint(v) & 0xffffe000u);
-    uint32_t lo;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(v - hi));
-    return __uint_as_float(lo);
+    return __uint_as_float(__float_as_uint(v - hi) + 0x1000u);
 }
 
 // ---- bfloat16 storage ------------------------------------------------------------------------------
