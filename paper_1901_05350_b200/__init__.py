@@ -122,6 +122,23 @@ def _load_library() -> ctypes.CDLL:
 
 lib = _load_library()
 
+# The op calls marshalled in C++ (binding/fast_calls.cpp); loaded with the first Context, since it needs torch.  A call that
+# it does not take (it returns None) goes through ctypes below, which raises whatever there is to raise.
+_fast = None
+
+
+def _load_fast_calls():
+    global _fast
+    if _fast is None:
+        import importlib.machinery
+        import importlib.util
+
+        loader = importlib.machinery.ExtensionFileLoader("_fast_calls", _build.build_binding())
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fast_calls", loader))
+        loader.exec_module(module)
+        module.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in module.CALLS})
+        _fast = module
+
 
 def window_out_shape(size: int, k: int, stride: int, dilation: int, pad: str):
     """(out, pad_before, pad_after) of one spatial dimension (host arithmetic in the library)."""
@@ -168,10 +185,13 @@ class Context:
         torch.cuda.set_device(device)
         torch.cuda.init()
         self.device = device
+        _load_fast_calls()
+        self._fh = 0  # the handle as _fast takes it
         self._h = ctypes.c_void_p()
         rc = lib.tfjsb_init(device, ctypes.byref(self._h))
         if rc:
             raise TfjsbError(rc, "tfjsb_init failed (needs a compute-capability 10.x device)")
+        self._fh = self._h.value
         self.set_math(math)
 
     # -- plumbing
@@ -183,6 +203,7 @@ class Context:
         if self._h:
             self._check(lib.tfjsb_shutdown(self._h))
             self._h = ctypes.c_void_p()
+            self._fh = 0
 
     def set_math(self, math: str):
         self._check(lib.tfjsb_set_math(self._h, MATH[math]))
@@ -202,6 +223,9 @@ class Context:
 
     # -- ops
     def matmul(self, a, b, transpose_a: bool = False, transpose_b: bool = False, out=None):
+        done = _fast.matmul(self._fh, self.device, a, b, transpose_a, transpose_b, out)
+        if done is not None:
+            return done
         M = a.shape[1] if transpose_a else a.shape[0]
         N = b.shape[0] if transpose_b else b.shape[1]
         out = self._empty((M, N)) if out is None else out
@@ -248,6 +272,9 @@ class Context:
         return self._empty((x.shape[0], ho, wo, channels))
 
     def conv2d(self, x, filter, strides=(1, 1), pad="same", dilations=(1, 1), bias=None, act="none", out=None):
+        done = _fast.conv2d(self._fh, self.device, x, filter, strides, PAD[pad], dilations, bias, ACT[act], out)
+        if done is not None:
+            return done
         if out is None:
             out = self._conv_out(x, filter.shape[0], filter.shape[1], strides, pad, dilations, filter.shape[3])
         self._check(lib.tfjsb_conv2d(self._h, _desc(x), _desc(filter), _int2(strides), PAD[pad], _int2(dilations),
@@ -256,6 +283,9 @@ class Context:
 
     def depthwise_conv2d(self, x, filter, strides=(1, 1), pad="same", dilations=(1, 1), bias=None, act="none",
                          out=None):
+        done = _fast.depthwise_conv2d(self._fh, self.device, x, filter, strides, PAD[pad], dilations, bias, ACT[act], out)
+        if done is not None:
+            return done
         if out is None:
             out = self._conv_out(x, filter.shape[0], filter.shape[1], strides, pad, dilations,
                                  filter.shape[2] * filter.shape[3])
@@ -265,6 +295,9 @@ class Context:
         return out
 
     def avg_pool(self, x, filter_size, strides, pad="valid", out=None):
+        done = _fast.avg_pool(self._fh, self.device, x, filter_size, strides, PAD[pad], out)
+        if done is not None:
+            return done
         if out is None:
             out = self._conv_out(x, filter_size[0], filter_size[1], strides, pad, (1, 1), x.shape[3])
         self._check(lib.tfjsb_avg_pool(self._h, _desc(x), _int2(filter_size), _int2(strides), PAD[pad], _desc(out),
@@ -272,6 +305,9 @@ class Context:
         return out
 
     def max_pool(self, x, filter_size, strides, pad="valid", out=None):
+        done = _fast.max_pool(self._fh, self.device, x, filter_size, strides, PAD[pad], out)
+        if done is not None:
+            return done
         if out is None:
             out = self._conv_out(x, filter_size[0], filter_size[1], strides, pad, (1, 1), x.shape[3])
         self._check(lib.tfjsb_max_pool(self._h, _desc(x), _int2(filter_size), _int2(strides), PAD[pad], _desc(out),
@@ -280,11 +316,17 @@ class Context:
 
     def binary(self, op: str, a, b, out=None):
         """a op b elementwise, op in 'add' / 'sub' / 'mul'; b has a's shape or is a vector of a's last dimension."""
+        done = _fast.binary(self._fh, self.device, BINARY_OP[op], a, b, out)
+        if done is not None:
+            return done
         out = self._empty(a.shape) if out is None else out
         self._check(lib.tfjsb_binary(self._h, BINARY_OP[op], _desc(a), _desc(b), _desc(out), _stream()))
         return out
 
     def batch_matmul(self, a, b, transpose_a: bool = False, transpose_b: bool = False, out=None):
+        done = _fast.batch_matmul(self._fh, self.device, a, b, transpose_a, transpose_b, out)
+        if done is not None:
+            return done
         M = a.shape[2] if transpose_a else a.shape[1]
         N = b.shape[1] if transpose_b else b.shape[2]
         out = self._empty((a.shape[0], M, N)) if out is None else out
@@ -293,11 +335,17 @@ class Context:
         return out
 
     def softmax(self, logits, out=None):
+        done = _fast.softmax(self._fh, self.device, logits, out)
+        if done is not None:
+            return done
         out = self._empty(logits.shape) if out is None else out
         self._check(lib.tfjsb_softmax(self._h, _desc(logits), _desc(out), _stream()))
         return out
 
     def bias_act(self, x, bias=None, act="none", out=None):
+        done = _fast.bias_act(self._fh, self.device, x, bias, ACT[act], out)
+        if done is not None:
+            return done
         out = self._empty(x.shape) if out is None else out
         self._check(lib.tfjsb_bias_act(self._h, _desc(x), None if bias is None else _desc(bias), ACT[act],
                                        _desc(out), _stream()))
@@ -308,35 +356,53 @@ class Context:
 
     # -- gradients (geometry arguments are the forward call's)
     def conv2d_backprop_input(self, x_shape, filter, dy, strides=(1, 1), pad="same", dilations=(1, 1), out=None):
+        done = _fast.conv_grad(self._fh, self.device, 0, x_shape, dy, filter, strides, PAD[pad], dilations, out)
+        if done is not None:
+            return done
         out = self._empty(x_shape) if out is None else out
         self._check(lib.tfjsb_conv2d_backprop_input(self._h, _desc(dy), _desc(filter), _int2(strides), PAD[pad],
                                                     _int2(dilations), _desc(out), _stream()))
         return out
 
     def conv2d_backprop_filter(self, x, filter_shape, dy, strides=(1, 1), pad="same", dilations=(1, 1), out=None):
+        done = _fast.conv_grad(self._fh, self.device, 1, filter_shape, x, dy, strides, PAD[pad], dilations, out)
+        if done is not None:
+            return done
         out = self._empty(filter_shape) if out is None else out
         self._check(lib.tfjsb_conv2d_backprop_filter(self._h, _desc(x), _desc(dy), _int2(strides), PAD[pad],
                                                      _int2(dilations), _desc(out), _stream()))
         return out
 
     def depthwise_conv2d_backprop_input(self, x_shape, filter, dy, strides=(1, 1), pad="same", dilations=(1, 1), out=None):
+        done = _fast.conv_grad(self._fh, self.device, 2, x_shape, dy, filter, strides, PAD[pad], dilations, out)
+        if done is not None:
+            return done
         out = self._empty(x_shape) if out is None else out
         self._check(lib.tfjsb_depthwise_conv2d_backprop_input(self._h, _desc(dy), _desc(filter), _int2(strides), PAD[pad],
                                                               _int2(dilations), _desc(out), _stream()))
         return out
 
     def depthwise_conv2d_backprop_filter(self, x, filter_shape, dy, strides=(1, 1), pad="same", dilations=(1, 1), out=None):
+        done = _fast.conv_grad(self._fh, self.device, 3, filter_shape, x, dy, strides, PAD[pad], dilations, out)
+        if done is not None:
+            return done
         out = self._empty(filter_shape) if out is None else out
         self._check(lib.tfjsb_depthwise_conv2d_backprop_filter(self._h, _desc(x), _desc(dy), _int2(strides), PAD[pad],
                                                                _int2(dilations), _desc(out), _stream()))
         return out
 
     def act_backprop(self, y, dy, act="none", out=None):
+        done = _fast.act_backprop(self._fh, self.device, y, dy, ACT[act], out)
+        if done is not None:
+            return done
         out = self._empty(y.shape) if out is None else out
         self._check(lib.tfjsb_act_backprop(self._h, _desc(y), _desc(dy), ACT[act], _desc(out), _stream()))
         return out
 
     def bias_backprop(self, dz, out=None):
+        done = _fast.bias_backprop(self._fh, self.device, dz, out)
+        if done is not None:
+            return done
         out = self._empty((dz.shape[-1],)) if out is None else out
         self._check(lib.tfjsb_bias_backprop(self._h, _desc(dz), _desc(out), _stream()))
         return out
@@ -380,6 +446,7 @@ class Model:
         odims = (ctypes.c_int64 * 4)()
         ctx._check(lib.tfjsb_model_output_shape(self._h, ctypes.byref(rank), odims))
         self.output_shape = tuple(odims[i] for i in range(rank.value))
+        self._fh = self._h.value
 
     @property
     def launches_per_run(self) -> int:
@@ -390,9 +457,13 @@ class Model:
         if self._h:
             self.ctx._check(lib.tfjsb_model_destroy(self._h))
             self._h = ctypes.c_void_p()
+            self._fh = 0
 
     def run(self, x, out=None):
         """Enqueue one forward pass on the current stream; device tensors in and out."""
+        done = _fast.run_model(self._fh, self.ctx.device, x, self.output_shape, out)
+        if done is not None:
+            return done
         out = self.ctx._empty(self.output_shape) if out is None else out
         self.ctx._check(lib.tfjsb_run_model(self._h, _desc(x), _desc(out), _stream()))
         return out
@@ -449,6 +520,9 @@ class Model:
     def layer_output_f32(self, layer: int):
         """fp32 copy of the output of layer `layer` whatever its storage format (bfloat16 layers are
         widened on the device); use set_keep_all(True) before the run."""
+        done = _fast.layer_output_f32(self._fh, self.ctx.device, layer)
+        if done is not None:
+            return done
         rank = ctypes.c_int32()
         dims = (ctypes.c_int64 * 4)()
         self.ctx._check(lib.tfjsb_model_layer_shape(self._h, layer, ctypes.byref(rank), dims))

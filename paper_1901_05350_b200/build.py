@@ -87,6 +87,42 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+BINDING_SRC = os.path.join(PKG, "binding", "fast_calls.cpp")
+
+
+def binding_path() -> str:
+    """The C++ half of the Python binding is compiled against one version of torch, which its name carries."""
+    import torch
+
+    version = "".join(c if c.isalnum() else "_" for c in torch.__version__)
+    return os.path.join(PKG, f"_fast_calls_torch{version}.so")
+
+
+def build_binding(force: bool = False) -> str:
+    import sysconfig
+
+    import torch
+
+    path = binding_path()
+    newest = max(os.path.getmtime(p) for p in (BINDING_SRC, os.path.join(INCLUDE, "tfjsb.h"), __file__))
+    if not force and os.path.exists(path) and os.path.getmtime(path) >= newest:
+        return path
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    scratch = f"{path}.{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", INCLUDE, "-I", sysconfig.get_paths()["include"], "-I", os.path.join(root, "include"),
+           "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"), "-I", os.path.join(cuda, "include"),
+           BINDING_SRC, "-o", scratch, "-L", os.path.join(root, "lib"),
+           "-ltorch_python", "-ltorch", "-ltorch_cuda", "-lc10", "-lc10_cuda", f"-Wl,-rpath,{os.path.join(root, 'lib')}"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"g++ failed on {BINDING_SRC}:\n{res.stdout}\n{res.stderr}")
+    os.replace(scratch, path)
+    return path
+
+
 if __name__ == "__main__":
     path = build(force="--force" in sys.argv, verbose="--verbose" in sys.argv)
     print(path)
+    print(build_binding(force="--force" in sys.argv))

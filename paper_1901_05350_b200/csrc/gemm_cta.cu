@@ -734,15 +734,12 @@ cudaError_t launch_gemm_tf32(const GemmTf32Plan& plan, const float* bias, int ac
                              cudaStream_t s, int64_t* launches) {
     if (plan.pair) return launch_gemm_tf32_pair(plan, bias, act, dev_status, s, launches);
     if (plan.cluster_split) return launch_gemm_tf32_splitk(plan, bias, act, dev_status, s, launches);
-    {
-        cudaError_t ae = cudaSuccess;
-        if (ae == cudaSuccess) ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_tf32_kernel<false>), SMEM_LIMIT - 2048);
-        if (ae == cudaSuccess) ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_tf32_kernel<true>), SMEM_LIMIT - 2048);
-        if (ae == cudaSuccess) ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_tf32_batched_kernel), SMEM_LIMIT - 2048);
-        if (ae == cudaSuccess) ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_tf32_im2col_kernel), SMEM_LIMIT - 2048);
-        if (ae != cudaSuccess) return ae;
-    }
-    cudaError_t e;
+    const void* kernel = plan.gather ? reinterpret_cast<const void*>(&gemm_tf32_kernel<true>)
+                         : plan.im2col ? reinterpret_cast<const void*>(&gemm_tf32_im2col_kernel)
+                         : plan.batches > 1 ? reinterpret_cast<const void*>(&gemm_tf32_batched_kernel)
+                                            : reinterpret_cast<const void*>(&gemm_tf32_kernel<false>);
+    cudaError_t e = smem_attr_once(kernel, SMEM_LIMIT - 2048);
+    if (e != cudaSuccess) return e;
     KernelArgs args;
     args.M = (int)plan.M; args.N = (int)plan.N; args.K = (int)plan.K;
     args.block_n = plan.block_n;
