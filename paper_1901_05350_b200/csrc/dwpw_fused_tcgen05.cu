@@ -604,8 +604,15 @@ dwpw_fused_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
                         if (args.dw_bias) b = __ldg(reinterpret_cast<const float2*>(args.dw_bias + c));
                         loaded_kb = kb;
                     }
-                    bool got = bounded_wait(smem_u32(&bar_patch_full[ps]), pphase, abort_flag);
-                    got = got && bounded_wait(smem_u32(&bar_a_empty[as]), aphase ^ 1u, abort_flag);
+                    // The operand stage first.  With two groups and a patch ring of three, this group did not wait for the
+                    // stage's previous patch (the other group's k-block), and a wait for a phase whose predecessor has
+                    // not completed returns at once: were that patch late (copies land in any order), the group would
+                    // read the stage before its own patch is there and hand it back early, which lets the producer arm
+                    // a barrier twice in one phase (seen as rare launch failures).  A free operand stage means that
+                    // k-block kb - a_stages has been multiplied, so every patch up to there has landed, and
+                    // a_stages <= 3 covers the ring of three; rings of two and four give each group its own stages.
+                    bool got = bounded_wait(smem_u32(&bar_a_empty[as]), aphase ^ 1u, abort_flag);
+                    got = got && bounded_wait(smem_u32(&bar_patch_full[ps]), pphase, abort_flag);
                     if (!__all_sync(0xffffffffu, got)) {
                         if (lane == 0 && !*abort_flag) {
                             *abort_flag = 1;
@@ -713,6 +720,7 @@ tfjsb_status dwpw_fused_plan(tfjsb_ctx* ctx, const void* x, const float* bt, voi
     int ps = (SMEM_LIMIT - 2048 - fixed) / patch_stride;
     if (ps > 4) ps = 4;
     if (ps < 2) return fail(ctx, TFJSB_ERR_UNSUPPORTED, "no room for the input patch ring");
+    static_assert(F_DW_GROUPS == 2, "an odd patch ring must not be shorter than the operand ring (see the depthwise warps' waits)");
     plan->conv = false;
     plan->y_bf16 = narrow;
     plan->patch_stages = ps;
