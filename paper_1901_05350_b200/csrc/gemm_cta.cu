@@ -251,132 +251,119 @@ __device__ __forceinline__ void gemm_pipeline(const CUtensorMap& map_a, const CU
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int armed[MAX_STAGES];      // parity of the last phase armed on each stage, -1 = never
-#pragma unroll
-            for (int s = 0; s < MAX_STAGES; ++s) armed[s] = -1;
-            bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < args.num_tiles; tile += gridDim.x) {
-                const int batch = BATCHED ? tile / args.tiles_per_batch : 0;
-                const int in_batch = tile - batch * args.tiles_per_batch;
-                const int m0 = (in_batch / args.n_tiles) * BLOCK_M;
-                const int n0 = (in_batch % args.n_tiles) * block_n;
-                (void)m0;
-                // im2col: the tile's first output pixel, and the filter tap and channel of the next k-block
-                int img = 0, h0 = 0, w0 = 0, c0 = 0, off_h = 0, off_w = 0;
-                if (IM2COL) {
-                    const int row = m0 / args.g.Wo;
-                    img = row / args.g.Ho;
-                    h0 = (row - img * args.g.Ho) * args.g.sh - args.g.pt;
-                    w0 = (m0 - row * args.g.Wo) * args.g.sw - args.g.pl;
-                }
-                for (int kb = 0; kb < num_k_blocks; ++kb) {
-                    if (!bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag)) {
-                        if (!*abort_flag) {
-                            *abort_flag = 1;
-                            atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
-                        }
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t full = smem_u32(&bar_full[stage]);
-                    const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
+        int stage = 0, filled = 0;
+        uint32_t phase = 0;
+        const bool leader = elect_one();
+        bool ok = true;  // the leader's
+        for (int tile = blockIdx.x; tile < args.num_tiles; tile += gridDim.x) {
+            const int batch = BATCHED ? tile / args.tiles_per_batch : 0;
+            const int in_batch = tile - batch * args.tiles_per_batch;
+            const int m0 = (in_batch / args.n_tiles) * BLOCK_M;
+            const int n0 = (in_batch % args.n_tiles) * block_n;
+            (void)m0;
+            // im2col: the tile's first output pixel, and the filter tap and channel of the next k-block
+            int img = 0, h0 = 0, w0 = 0, c0 = 0, off_h = 0, off_w = 0;
+            if (IM2COL) {
+                const int row = m0 / args.g.Wo;
+                img = row / args.g.Ho;
+                h0 = (row - img * args.g.Ho) * args.g.sh - args.g.pt;
+                w0 = (m0 - row * args.g.Wo) * args.g.sw - args.g.pl;
+            }
+            for (int kb = 0; kb < num_k_blocks; ++kb) {
+                const uint32_t full = smem_u32(&bar_full[stage]);
+                const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
+                if (leader && ok && (ok = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag))) {
+                    ++filled;
                     if (GATHER) {
                         mbar_arrive_expect_tx(full, (uint32_t)(stage_bytes - A_STAGE_BYTES));
                     } else {
                         mbar_arrive_expect_tx(full, (uint32_t)stage_bytes);
-                        if (IM2COL) {
-                            tma_load_im2col(a_dst, &map_a, full, c0, w0, h0, img, off_w, off_h);
-                            if ((c0 += BK) >= args.g.C) {
-                                c0 = 0;
-                                if ((off_w += args.g.dw) == args.g.fw * args.g.dw) { off_w = 0; off_h += args.g.dh; }
-                            }
-                        } else if (BATCHED) tma_load_3d(a_dst, &map_a, full, kb * BK, m0, batch);
+                        if (IM2COL) tma_load_im2col(a_dst, &map_a, full, c0, w0, h0, img, off_w, off_h);
+                        else if (BATCHED) tma_load_3d(a_dst, &map_a, full, kb * BK, m0, batch);
                         else tma_load_2d(a_dst, &map_a, full, kb * BK, m0);
                     }
                     if (BATCHED) tma_load_3d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BK, n0, batch);
                     else tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BK, n0);
-#pragma unroll
-                    for (int s = 0; s < MAX_STAGES; ++s)
-                        if (s == stage) armed[s] = (int)phase;
-                    if (++stage == stages) { stage = 0; phase ^= 1u; }
                 }
+                if (IM2COL && (c0 += BK) >= args.g.C) {
+                    c0 = 0;
+                    if ((off_w += args.g.dw) == args.g.fw * args.g.dw) { off_w = 0; off_h += args.g.dh; }
+                }
+                if (++stage == stages) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) {
-                // Another role may never consume what was armed: wait (bounded) for the copies in
-                // flight so that nothing lands in shared memory after the CTA has gone.
-#pragma unroll
-                for (int s = 0; s < MAX_STAGES; ++s) {
-                    if (s < stages && armed[s] >= 0) {
-                        const unsigned long long t0 = global_ns();
-                        while (!mbar_try_wait(smem_u32(&bar_full[s]), (uint32_t)armed[s])) {
-                            if (global_ns() - t0 > WAIT_LIMIT_NS) {
-                                atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
-                                break;
-                            }
-                        }
+        }
+        if (!ok) {
+            if (!*abort_flag) {
+                *abort_flag = 1;
+                atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
+            }
+            // Another role may never consume what was armed: wait (bounded) for the copies in flight so that nothing
+            // lands in shared memory after the CTA has gone.
+            for (int k = filled > stages ? filled - stages : 0; k < filled; ++k) {
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(smem_u32(&bar_full[k % stages]), (uint32_t)((k / stages) & 1))) {
+                    if (global_ns() - t0 > WAIT_LIMIT_NS) {
+                        atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
+                        break;
                     }
                 }
             }
         }
+        __syncwarp();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = IN_BF16 ? make_idesc_bf16(BLOCK_M, block_n) : make_idesc_tf32(BLOCK_M, block_n);
-            int stage = 0;
-            uint32_t phase = 0;
-            int acc = 0;
-            uint32_t acc_phase = 0;
-            bool ok = true;
-            bool issued_any = false;
-            for (int tile = blockIdx.x; ok && tile < args.num_tiles; tile += gridDim.x) {
-                if (!bounded_wait(smem_u32(&bar_acc_empty[acc]), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * block_n);
-                for (int kb = 0; kb < num_k_blocks; ++kb) {
-                    if (!bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag)) { ok = false; break; }
+        const uint32_t idesc = IN_BF16 ? make_idesc_bf16(BLOCK_M, block_n) : make_idesc_tf32(BLOCK_M, block_n);
+        int stage = 0;
+        uint32_t phase = 0;
+        int acc = 0;
+        uint32_t acc_phase = 0;
+        const bool leader = elect_one();
+        bool ok = true;  // the leader's
+        bool issued_any = false;
+        for (int tile = blockIdx.x; tile < args.num_tiles; tile += gridDim.x) {
+            if (leader && ok) ok = bounded_wait(smem_u32(&bar_acc_empty[acc]), acc_phase ^ 1u, abort_flag);
+            const uint32_t d_tmem = tmem_base + (uint32_t)(acc * block_n);
+            for (int kb = 0; kb < num_k_blocks; ++kb) {
+                const uint32_t a_addr = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
+                const uint64_t a_desc = make_kmajor_sw128_desc(a_addr);
+                const uint64_t b_desc = make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
+                // steps along K inside the 128-byte swizzled row: 32 bytes = 2 descriptor units
+                uint64_t ak[MMAS_PER_KB], bk[MMAS_PER_KB];
+#pragma unroll
+                for (int k = 0; k < MMAS_PER_KB; ++k) { ak[k] = a_desc + (uint64_t)(2 * k); bk[k] = b_desc + (uint64_t)(2 * k); }
+                if (leader && ok && (ok = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag))) {
                     tc_fence_after();
-                    const uint32_t a_addr = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
-                    const uint64_t a_desc = make_kmajor_sw128_desc(a_addr);
-                    const uint64_t b_desc = make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
 #pragma unroll
                     for (int k = 0; k < MMAS_PER_KB; ++k) {
-                        // step along K inside the 128-byte swizzled row: 32 bytes = 2 descriptor units
-                        if (IN_BF16)
-                            tc_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                        (kb | k) != 0 ? 1u : 0u);
-                        else
-                            tc_mma_tf32(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                        (kb | k) != 0 ? 1u : 0u);
+                        if (IN_BF16) tc_mma_bf16(d_tmem, ak[k], bk[k], idesc, (kb | k) != 0 ? 1u : 0u);
+                        else tc_mma_tf32(d_tmem, ak[k], bk[k], idesc, (kb | k) != 0 ? 1u : 0u);
                     }
-                    issued_any = true;
                     tc_commit(smem_u32(&bar_empty[stage]));
-                    if (++stage == stages) { stage = 0; phase ^= 1u; }
+                    issued_any = true;
                 }
-                if (!ok) break;
-                tc_commit(smem_u32(&bar_acc_full[acc]));
-                if (++acc == acc_stages) { acc = 0; acc_phase ^= 1u; }
+                if (++stage == stages) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) {
-                if (!*abort_flag) {
-                    *abort_flag = 1;
-                    atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_MMA);
-                }
-                if (issued_any) {
-                    // let the MMAs already issued finish before tensor memory is released
-                    tc_commit(smem_u32(&bar_drain));
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(smem_u32(&bar_drain), 0u)) {
-                        if (global_ns() - t0 > WAIT_LIMIT_NS) {
-                            atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
-                            break;
-                        }
+            if (leader && ok) tc_commit(smem_u32(&bar_acc_full[acc]));
+            if (++acc == acc_stages) { acc = 0; acc_phase ^= 1u; }
+        }
+        if (!ok) {
+            if (!*abort_flag) {
+                *abort_flag = 1;
+                atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_MMA);
+            }
+            if (issued_any) {
+                // let the MMAs already issued finish before tensor memory is released
+                tc_commit(smem_u32(&bar_drain));
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(smem_u32(&bar_drain), 0u)) {
+                    if (global_ns() - t0 > WAIT_LIMIT_NS) {
+                        atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
+                        break;
                     }
                 }
             }
         }
+        __syncwarp();
     } else if (warp < 2 + epi_warps) {
         // ---------------------------------------------------------------- epilogue (warps 2..)
         // Two or four warps share each TMEM lane quadrant (a warp may only read lanes 32*(warp%4)..+31)

@@ -105,6 +105,19 @@ __device__ __forceinline__ void tc_mma_tf32(uint32_t d_tmem, uint64_t a_desc, ui
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// One thread of a converged warp.  A role that one thread plays (issuing copies or MMAs) runs its loops with the whole
+// warp and lets the elected thread alone wait and issue:
+//     const bool leader = elect_one();
+//     for (...) { <addresses, descriptors>;  if (leader && ok && (ok = bounded_wait(...))) { <issue> }  <stage, phase> }
+// The addresses and descriptors are then warp-uniform values in uniform registers, which is where the issuing
+// instructions want them.  In loops that one lane had entered on its own each operand was moved there one by one, and a
+// k-block took about 690 cycles whatever the size of its MMAs (now 400; 64 k-blocks of 128 x 128 x 32: 26.8 -> 18.6 us).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // 32 lanes x 32 columns of 32-bit accumulators: thread t of the warp gets lane (base lane + t).
 __device__ __forceinline__ void tc_ld_32x32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
