@@ -58,8 +58,10 @@ depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ f, co
     const int c = c4 * 4;
 
     float4 w[9];
+    const int f_step = g.reversed ? -g.C : g.C;
+    if (g.reversed) f += 8 * (int64_t)g.C;
 #pragma unroll
-    for (int t = 0; t < 9; ++t) w[t] = ld4(f + (int64_t)(g.reversed ? 8 - t : t) * g.C + c);
+    for (int t = 0; t < 9; ++t) w[t] = ld4(f + (int64_t)t * f_step + c);
 
     float4 acc[ROWS];
 #pragma unroll
@@ -189,6 +191,7 @@ constexpr int DW_MAX_STAGES = 4;
 struct DwTiling {
     int tiles_x, tiles_y, c_blocks, stages;
     long long num_tiles;
+    int f_step;  // from one tap of the filter to the next: C, or -C with f at the last tap (the taps reversed)
 };
 
 template <int S, int TW, int R, int D = 1, int CB = DW_CB, bool NARROW = false>
@@ -316,7 +319,7 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
             if (cb != loaded_cb) {
 #pragma unroll
                 for (int k = 0; k < 9; ++k)
-                    w[k] = __ldg(reinterpret_cast<const float4*>(f + (int64_t)(g.reversed ? 8 - k : k) * g.C + c));
+                    w[k] = __ldg(reinterpret_cast<const float4*>(f + (int64_t)k * t.f_step + c));
                 if (bias) b = __ldg(reinterpret_cast<const float4*>(bias + c));
                 loaded_cb = cb;
             }
@@ -398,7 +401,8 @@ cudaError_t launch_tma_instance(const DepthwisePlan& plan, const float* f, const
     auto kernel = depthwise3x3_tma_kernel<S, TW, R, D, CB, NARROW>;
     cudaError_t ae = smem_attr_once(reinterpret_cast<const void*>(kernel), DW_SMEM_BUDGET);
     if (ae != cudaSuccess) return ae;
-    DwTiling t{plan.tiles_x, plan.tiles_y, plan.c_blocks, plan.stages, (long long)plan.num_tiles};
+    DwTiling t{plan.tiles_x, plan.tiles_y, plan.c_blocks, plan.stages, (long long)plan.num_tiles, g.reversed ? -g.C : g.C};
+    if (g.reversed) f += 8 * (int64_t)g.C;
     return launch_k(kernel, dim3(plan.grid), dim3(DW_TMA_THREADS), plan.smem_bytes, s, plan.map_x, f, bias, act, y,
                     y_f32 ? 1 : 0, g, t, dev_status);
 }

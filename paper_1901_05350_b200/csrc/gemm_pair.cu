@@ -136,84 +136,85 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer (both CTAs)
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int issued = 0;
-            bool ok = true;
-            for (int tile = pair; ok && tile < args.num_tiles; tile += num_pairs) {
-                const int m0 = (tile / args.n_tiles) * P_TILE_M + (int)rank * BLOCK_M;
-                const int n0 = (tile % args.n_tiles) * block_n + (int)rank * half_n;
-                for (int kb = 0; kb < num_k_blocks; ++kb) {
-                    if (!bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag)) {
-                        if (!*abort_flag) {
-                            *abort_flag = 1;
-                            atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
-                        }
-                        ok = false;
-                        break;
-                    }
-                    // the bytes of both CTAs' copies of this stage are counted on the even CTA's barrier
-                    const uint32_t full = map_to_cta(smem_u32(&bar_full[stage]), 0u);
+        int stage = 0;
+        uint32_t phase = 0;
+        int issued = 0;
+        const bool elected = elect_one();
+        bool ok = true;  // the elected thread's
+        for (int tile = pair; tile < args.num_tiles; tile += num_pairs) {
+            const int m0 = (tile / args.n_tiles) * P_TILE_M + (int)rank * BLOCK_M;
+            const int n0 = (tile % args.n_tiles) * block_n + (int)rank * half_n;
+            for (int kb = 0; kb < num_k_blocks; ++kb) {
+                // the bytes of both CTAs' copies of this stage are counted on the even CTA's barrier
+                const uint32_t full = map_to_cta(smem_u32(&bar_full[stage]), 0u);
+                const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
+                if (elected && ok && (ok = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag))) {
                     if (leader) mbar_arrive_expect_tx(smem_u32(&bar_full[stage]), (uint32_t)(2 * stage_bytes));
-                    const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
                     tma_load_2d_pair(a_dst, &map_a, full, kb * BK, m0);
                     tma_load_2d_pair(a_dst + A_STAGE_BYTES, &map_b, full, kb * BK, n0);
                     ++issued;
-                    if (++stage == stages) { stage = 0; phase ^= 1u; }
                 }
-            }
-            if (!ok) {
-                // Copies in flight must land before this CTA's shared memory goes away.  The even CTA
-                // can watch its "full" barriers (a phase completes when both CTAs' bytes are in); the
-                // partner has no barrier of its own to watch and waits out the longest a copy can take.
-                const unsigned long long t0 = global_ns();
-                if (leader) {
-                    for (int k = (issued > stages ? issued - stages : 0); k < issued; ++k) {
-                        while (!mbar_try_wait(smem_u32(&bar_full[k % stages]), (uint32_t)((k / stages) & 1))) {
-                            if (global_ns() - t0 > WAIT_LIMIT_NS) {
-                                atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
-                                break;
-                            }
-                        }
-                    }
-                } else {
-                    while (global_ns() - t0 < 2000000ull) {}  // 2 ms
-                }
+                if (++stage == stages) { stage = 0; phase ^= 1u; }
             }
         }
+        if (!ok) {
+            if (!*abort_flag) {
+                *abort_flag = 1;
+                atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
+            }
+            // Copies in flight must land before this CTA's shared memory goes away.  The even CTA
+            // can watch its "full" barriers (a phase completes when both CTAs' bytes are in); the
+            // partner has no barrier of its own to watch and waits out the longest a copy can take.
+            const unsigned long long t0 = global_ns();
+            if (leader) {
+                for (int k = (issued > stages ? issued - stages : 0); k < issued; ++k) {
+                    while (!mbar_try_wait(smem_u32(&bar_full[k % stages]), (uint32_t)((k / stages) & 1))) {
+                        if (global_ns() - t0 > WAIT_LIMIT_NS) {
+                            atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
+                            break;
+                        }
+                    }
+                }
+            } else {
+                while (global_ns() - t0 < 2000000ull) {}  // 2 ms
+            }
+        }
+        __syncwarp();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer (even CTA only)
-        if (lane == 0 && leader) {
+        if (leader) {
             const uint32_t idesc = BF16 ? make_idesc_bf16(P_TILE_M, block_n) : make_idesc_tf32(P_TILE_M, block_n);
             const uint16_t both = 3;
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
             uint32_t acc_phase = 0;
-            bool ok = true;
+            const bool elected = elect_one();
+            bool ok = true;  // the elected thread's
             bool issued_any = false;
-            for (int tile = pair; ok && tile < args.num_tiles; tile += num_pairs) {
-                if (!bounded_wait(smem_u32(&bar_acc_empty[acc]), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
-                tc_fence_after();
+            for (int tile = pair; tile < args.num_tiles; tile += num_pairs) {
+                if (elected && ok) ok = bounded_wait(smem_u32(&bar_acc_empty[acc]), acc_phase ^ 1u, abort_flag);
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * block_n);
                 for (int kb = 0; kb < num_k_blocks; ++kb) {
-                    if (!bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag)) { ok = false; break; }
-                    tc_fence_after();
                     const uint32_t a_addr = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
                     const uint64_t a_desc = make_kmajor_sw128_desc(a_addr);
                     const uint64_t b_desc = make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
+                    uint64_t ak[BK / MMA_K], bk[BK / MMA_K];  // 32 bytes along K per MMA: 2 descriptor units
 #pragma unroll
-                    for (int k = 0; k < BK / MMA_K; ++k) {  // 32 bytes along K per MMA: 2 descriptor units
-                        if (BF16) tc_mma_bf16_pair(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
-                        else tc_mma_tf32_pair(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
+                    for (int k = 0; k < BK / MMA_K; ++k) { ak[k] = a_desc + (uint64_t)(2 * k); bk[k] = b_desc + (uint64_t)(2 * k); }
+                    if (elected && ok && (ok = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag))) {
+                        tc_fence_after();
+#pragma unroll
+                        for (int k = 0; k < BK / MMA_K; ++k) {
+                            if (BF16) tc_mma_bf16_pair(d_tmem, ak[k], bk[k], idesc, (kb | k) != 0 ? 1u : 0u);
+                            else tc_mma_tf32_pair(d_tmem, ak[k], bk[k], idesc, (kb | k) != 0 ? 1u : 0u);
+                        }
+                        tc_commit_pair(smem_u32(&bar_empty[stage]), both);
+                        issued_any = true;
                     }
-                    issued_any = true;
-                    tc_commit_pair(smem_u32(&bar_empty[stage]), both);
                     if (++stage == stages) { stage = 0; phase ^= 1u; }
                 }
-                if (!ok) break;
-                tc_commit_pair(smem_u32(&bar_acc_full[acc]), both);
+                if (elected && ok) tc_commit_pair(smem_u32(&bar_acc_full[acc]), both);
                 if (++acc == P_ACC_STAGES) { acc = 0; acc_phase ^= 1u; }
             }
             if (!ok) {
@@ -234,6 +235,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 }
             }
         }
+        __syncwarp();
     } else {
         // ---------------------------------------------------------------- epilogue (warps 2..9, both CTAs)
         // As in the single-CTA kernel: two warps per tensor-memory lane quadrant take alternate

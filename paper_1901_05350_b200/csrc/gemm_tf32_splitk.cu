@@ -128,84 +128,84 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int issued = 0;
-            bool ok = true;
-            for (int kb = kb_begin; kb < kb_end; ++kb) {
-                if (!bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag)) {
-                    if (!*abort_flag) {
-                        *abort_flag = 1;
-                        atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
-                    }
-                    ok = false;
-                    break;
-                }
-                const uint32_t full = smem_u32(&bar_full[stage]);
-                const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
+        int stage = 0;
+        uint32_t phase = 0;
+        int issued = 0;
+        const bool leader = elect_one();
+        bool ok = true;  // the leader's
+        for (int kb = kb_begin; kb < kb_end; ++kb) {
+            const uint32_t full = smem_u32(&bar_full[stage]);
+            const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
+            if (leader && ok && (ok = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag))) {
                 mbar_arrive_expect_tx(full, (uint32_t)stage_bytes);
                 tma_load_2d(a_dst, &map_a, full, kb * BLOCK_K, m0);
                 tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BLOCK_K, n0);
                 ++issued;
-                if (++stage == stages) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) {
-                // wait (bounded) for the copies in flight so that nothing lands after the CTA has gone
-                const unsigned long long t0 = global_ns();
-                for (int k = (issued > stages ? issued - stages : 0); k < issued; ++k) {
-                    while (!mbar_try_wait(smem_u32(&bar_full[k % stages]), (uint32_t)((k / stages) & 1))) {
-                        if (global_ns() - t0 > WAIT_LIMIT_NS) {
-                            atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
-                            break;
-                        }
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
+        }
+        if (!ok) {
+            if (!*abort_flag) {
+                *abort_flag = 1;
+                atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
+            }
+            // wait (bounded) for the copies in flight so that nothing lands after the CTA has gone
+            const unsigned long long t0 = global_ns();
+            for (int k = (issued > stages ? issued - stages : 0); k < issued; ++k) {
+                while (!mbar_try_wait(smem_u32(&bar_full[k % stages]), (uint32_t)((k / stages) & 1))) {
+                    if (global_ns() - t0 > WAIT_LIMIT_NS) {
+                        atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
+                        break;
                     }
                 }
             }
         }
+        __syncwarp();
         cluster_wait();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_tf32(BLOCK_M, block_n);
-            int stage = 0;
-            uint32_t phase = 0;
-            bool ok = true;
-            bool issued_any = false;
-            for (int kb = kb_begin; kb < kb_end; ++kb) {
-                if (!bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag)) { ok = false; break; }
+        const uint32_t idesc = make_idesc_tf32(BLOCK_M, block_n);
+        int stage = 0;
+        uint32_t phase = 0;
+        const bool leader = elect_one();
+        bool ok = true;  // the leader's
+        bool issued_any = false;
+        for (int kb = kb_begin; kb < kb_end; ++kb) {
+            const uint32_t a_addr = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
+            const uint64_t a_desc = make_kmajor_sw128_desc(a_addr);
+            const uint64_t b_desc = make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
+            uint64_t ak[BLOCK_K / UMMA_K], bk[BLOCK_K / UMMA_K];
+#pragma unroll
+            for (int k = 0; k < BLOCK_K / UMMA_K; ++k) { ak[k] = a_desc + (uint64_t)(2 * k); bk[k] = b_desc + (uint64_t)(2 * k); }
+            if (leader && ok && (ok = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag))) {
                 tc_fence_after();
-                const uint32_t a_addr = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
-                const uint64_t a_desc = make_kmajor_sw128_desc(a_addr);
-                const uint64_t b_desc = make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
 #pragma unroll
                 for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
-                    tc_mma_tf32(tmem_base, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                (kb != kb_begin || k != 0) ? 1u : 0u);
-                issued_any = true;
+                    tc_mma_tf32(tmem_base, ak[k], bk[k], idesc, (kb != kb_begin || k != 0) ? 1u : 0u);
                 tc_commit(smem_u32(&bar_empty[stage]));
-                if (++stage == stages) { stage = 0; phase ^= 1u; }
+                issued_any = true;
             }
-            if (ok) {
-                tc_commit(smem_u32(&bar_acc_full));
-            } else {
-                if (!*abort_flag) {
-                    *abort_flag = 1;
-                    atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_MMA);
-                }
-                if (issued_any) {
-                    // let the MMAs already issued finish before tensor memory is released
-                    tc_commit(smem_u32(&bar_drain));
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(smem_u32(&bar_drain), 0u)) {
-                        if (global_ns() - t0 > WAIT_LIMIT_NS) {
-                            atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
-                            break;
-                        }
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
+        }
+        if (leader && ok) tc_commit(smem_u32(&bar_acc_full));
+        if (!ok) {
+            if (!*abort_flag) {
+                *abort_flag = 1;
+                atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_MMA);
+            }
+            if (issued_any) {
+                // let the MMAs already issued finish before tensor memory is released
+                tc_commit(smem_u32(&bar_drain));
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(smem_u32(&bar_drain), 0u)) {
+                    if (global_ns() - t0 > WAIT_LIMIT_NS) {
+                        atomicOr(args.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
+                        break;
                     }
                 }
             }
         }
+        __syncwarp();
         cluster_wait();
     } else {
         // ---------------------------------------------------------------- accumulator -> the band owners' shared memory (warps 2..5)
