@@ -258,7 +258,7 @@ tfjsb_status gemm_tf32_pair_plan(tfjsb_ctx* ctx, const float* a, const float* bt
 cudaError_t launch_gemm_tf32_pair(const GemmTf32Plan& plan, const float* bias, int act, unsigned int* dev_status,
                                   cudaStream_t s, int64_t* launches);
 // Split K across the CTAs of a cluster, for GEMMs with too few tiles for the SMs (gemm_tf32_splitk.cu).
-bool gemm_tf32_splitk_choice(int64_t M, int64_t N, int64_t K, int sm_count, int* block_n, int* splits);
+bool gemm_tf32_splitk_choice(int64_t M, int64_t N, int64_t K, int sm_count, int64_t whole_ns, int* block_n, int* splits);
 tfjsb_status gemm_tf32_splitk_plan(tfjsb_ctx* ctx, const float* a, const float* bt, float* c, int64_t M, int64_t N,
                                    int64_t K, int block_n, int splits, GemmTf32Plan* plan);
 cudaError_t launch_gemm_tf32_splitk(const GemmTf32Plan& plan, const float* bias, int act, unsigned int* dev_status,

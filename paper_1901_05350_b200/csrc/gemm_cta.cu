@@ -173,6 +173,7 @@ struct KernelArgs {
     int num_tiles;  // total, over all products of the batch
     int acc_stages;  // accumulator stages in tensor memory: 2 (block_n 256) or 4
     int epi_warps;   // 8 or 16
+    int stage_tx;    // bytes that the copies of one stage deliver (fewer rows of A than a tile has when M is smaller)
     const float* bias;
     int act;
     unsigned int* dev_status;
@@ -277,7 +278,7 @@ __device__ __forceinline__ void gemm_pipeline(const CUtensorMap& map_a, const CU
                     if (GATHER) {
                         mbar_arrive_expect_tx(full, (uint32_t)(stage_bytes - A_STAGE_BYTES));
                     } else {
-                        mbar_arrive_expect_tx(full, (uint32_t)stage_bytes);
+                        mbar_arrive_expect_tx(full, (uint32_t)args.stage_tx);
                         if (IM2COL) tma_load_im2col(a_dst, &map_a, full, c0, w0, h0, img, off_w, off_h);
                         else if (BATCHED) tma_load_3d(a_dst, &map_a, full, kb * BK, m0, batch);
                         else tma_load_2d(a_dst, &map_a, full, kb * BK, m0);
@@ -562,19 +563,39 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     gemm_pipeline<A_TILED, OUT_BF16 ? IO_BF16 : IO_BF16_F32, false>(map_a, map_b, map_c, args);
 }
 
-int choose_block_n(int64_t M, int64_t N, int sm_count, int64_t batches) {
-    int bn = 32;
-    while (bn < 256 && bn < N) bn <<= 1;
-    const int64_t m_tiles = batches * ((M + BLOCK_M - 1) / BLOCK_M);  // row tiles of all products
-    while (bn > 32 && m_tiles * ((N + bn - 1) / bn) < sm_count) bn >>= 1;
-    if (bn == 256 && N > 256) {
-        // Wave quantisation: every tile of a launch costs the same, so the launch takes
-        // ceil(tiles / SMs) rounds of one tile each.  192-wide tiles (six 32-column chunks) sometimes
-        // fill the last round where 256-wide ones leave most SMs idle (196 tiles on 148 SMs).
-        auto rounds = [&](int w) { return (m_tiles * ((N + w - 1) / w) + sm_count - 1) / sm_count; };
-        if (rounds(192) * 192 < rounds(256) * 256) bn = 192;
+// What a launch of the single-CTA kernel takes, in nanoseconds, as measured on warm operands (512 x 512 x K, 1024^3 ...
+// 4096^3, the pointwise layers of the 224 x 224 model at batch 1 ... 128; K-contiguous operands, 148 SMs):
+//   start, one load, the last tile's epilogue   3.4 us for 32 columns to 5.9 us for 256
+//   a k-block                                   205 ... 220 ns up to 160 columns (the issuing loops), 265 at 192, 320 at 256
+//   every further round of tiles                its k-blocks, and 14 ns per column (its epilogue beside the next K loop)
+// The largest tile that still gives every SM one, the rule before, took 23.7 us for 1024^3 (10.7 now with 64 columns),
+// 48 us for 2048^3 (25.8, 256 columns) and 24.5 us for [2312,1024] . [1024,1024] (12.6, 160 columns).
+struct TileCost {
+    int width, start_ns, kb_ns;
+};
+constexpr TileCost kTileCosts[] = {{32, 3400, 205}, {64, 3700, 215}, {96, 4300, 220}, {128, 4500, 220}, {160, 4900, 220}, {192, 5200, 265}, {256, 5900, 320}};
+
+int64_t tile_ns(const TileCost& t, int64_t M, int64_t N, int64_t k_blocks, int sm_count, int64_t batches, int min_kb_ns) {
+    const int64_t tiles = batches * ((M + BLOCK_M - 1) / BLOCK_M) * ((N + t.width - 1) / t.width);
+    const int64_t rounds = (tiles + sm_count - 1) / sm_count;
+    const int64_t k_loop = k_blocks * (t.kb_ns > min_kb_ns ? t.kb_ns : min_kb_ns);
+    return t.start_ns + k_loop + (rounds - 1) * (k_loop + 14 * t.width);
+}
+
+// `min_kb_ns`: what fetching a k-block of A takes at least (im2col copies, gathering threads).
+int choose_block_n(int64_t M, int64_t N, int64_t k_blocks, int sm_count, int64_t batches, int min_kb_ns = 0, int64_t* ns = nullptr) {
+    int best = 0;
+    int64_t best_ns = 0;
+    for (const TileCost& t : kTileCosts) {
+        const int64_t cost = tile_ns(t, M, N, k_blocks, sm_count, batches, min_kb_ns);
+        if (best == 0 || cost < best_ns) {
+            best = t.width;
+            best_ns = cost;
+        }
+        if (t.width >= N) break;
     }
-    return bn;
+    if (ns) *ns = best_ns;
+    return best;
 }
 
 // A row-major matrix [outer, inner], or (batches > 1: a rank-3 map) that many of them stored one after the other;
@@ -609,9 +630,11 @@ namespace {
 
 // tile choice, pipeline depth and the B / C tensor maps shared by the GEMM and the convolution
 tfjsb_status plan_common(tfjsb_ctx* ctx, const float* bt, int64_t k_pitch, float* c, GemmTf32Plan* plan, int64_t batches = 1) {
+    // an im2col copy delivers a pixel's 128 bytes in about five cycles; the gathering threads need about twice as long
+    const int min_kb_ns = plan->im2col ? 330 : plan->gather ? 600 : 0;
     const int64_t M = plan->M, N = plan->N;
     plan->batches = batches;
-    plan->block_n = choose_block_n(M, N, ctx->sm_count, batches);
+    plan->block_n = choose_block_n(M, N, (k_pitch + BLOCK_K - 1) / BLOCK_K, ctx->sm_count, batches, min_kb_ns);
     plan->acc_stages = plan->block_n > 128 ? 2 : MAX_ACC_STAGES;
     const int stage_bytes = A_STAGE_BYTES + plan->block_n * BLOCK_K * 4;
     int stages = (SMEM_LIMIT - 1024 - EPI_BYTES - 512) / stage_bytes;
@@ -642,7 +665,9 @@ tfjsb_status gemm_tf32_plan(tfjsb_ctx* ctx, const float* a, const float* bt, flo
     if (batches == 1) {
         // few tiles and a long K loop: the K loop is cut across the CTAs of a cluster (gemm_tf32_splitk.cu)
         int split_bn = 0, split_s = 0;
-        if (!getenv("TFJSB_NO_SPLIT_K") && gemm_tf32_splitk_choice(M, N, K, ctx->sm_count, &split_bn, &split_s))
+        int64_t whole_ns = 0;
+        choose_block_n(M, N, (K + BLOCK_K - 1) / BLOCK_K, ctx->sm_count, 1, 0, &whole_ns);
+        if (!getenv("TFJSB_NO_SPLIT_K") && gemm_tf32_splitk_choice(M, N, K, ctx->sm_count, whole_ns, &split_bn, &split_s))
             return gemm_tf32_splitk_plan(ctx, a, bt, c, M, N, K, split_bn, split_s, plan);
     }
     plan->M = M; plan->N = N; plan->K = K;
@@ -653,7 +678,7 @@ tfjsb_status gemm_tf32_plan(tfjsb_ctx* ctx, const float* a, const float* bt, flo
     plan->x = nullptr;
     tfjsb_status st;
     if ((st = plan_common(ctx, bt, K, c, plan, batches)) != TFJSB_OK) return st;
-    return encode_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, BLOCK_M, "A", batches);
+    return encode_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, a_box_rows(M), "A", batches);
 }
 
 // im2col copies where the channels can be 128-byte rows at least half full (16-byte strides) and the window and padding
@@ -736,6 +761,7 @@ cudaError_t launch_gemm_tf32(const GemmTf32Plan& plan, const float* bias, int ac
     args.num_tiles = plan.num_tiles;
     args.acc_stages = plan.acc_stages;
     args.epi_warps = GATHER_EPI_WARPS;  // sixteen measured slower with fp32 tiles
+    args.stage_tx = (plan.im2col ? BLOCK_M : a_box_rows(plan.M)) * 128 + plan.block_n * 128;
     args.bias = bias;
     args.act = act;
     args.dev_status = dev_status;
@@ -777,7 +803,7 @@ tfjsb_status gemm_bf16_plan(tfjsb_ctx* ctx, const void* a, const void* bt, void*
     plan->M = M; plan->N = N; plan->K = K;
     plan->c_is_bf16 = c_is_bf16;
     plan->pair = false;
-    plan->block_n = choose_block_n(M, N, ctx->sm_count, 1);
+    plan->block_n = choose_block_n(M, N, (K + BK16 - 1) / BK16, ctx->sm_count, 1);
     plan->acc_stages = plan->block_n > 128 ? 2 : MAX_ACC_STAGES;
     const int stage_bytes = A_STAGE_BYTES + plan->block_n * 128;
     plan->epi_warps = (K + BK16 - 1) / BK16 <= 4 ? 16 : 8;
@@ -792,7 +818,7 @@ tfjsb_status gemm_bf16_plan(tfjsb_ctx* ctx, const void* a, const void* bt, void*
     plan->num_tiles = (int)tiles;
     plan->grid = (int)(tiles < ctx->sm_count ? tiles : ctx->sm_count);
     tfjsb_status st;
-    if ((st = encode_2d(ctx, &plan->map_a, a, K, M, BK16, BLOCK_M, "A", 1, true)) != TFJSB_OK) return st;
+    if ((st = encode_2d(ctx, &plan->map_a, a, K, M, BK16, a_box_rows(M), "A", 1, true)) != TFJSB_OK) return st;
     if ((st = encode_2d(ctx, &plan->map_b, bt, K, N, BK16, plan->block_n, "B", 1, true)) != TFJSB_OK) return st;
     if (c_is_bf16) return encode_2d(ctx, &plan->map_c, c, N, M, EPI_COLS, 32, "C", 1, true, CU_TENSOR_MAP_SWIZZLE_64B);
     return encode_2d(ctx, &plan->map_c, c, N, M, EPI_COLS, 32, "C");
@@ -816,6 +842,7 @@ cudaError_t launch_gemm_bf16(const GemmBf16Plan& plan, const float* bias, int ac
     args.num_tiles = plan.num_tiles;
     args.acc_stages = plan.acc_stages;
     args.epi_warps = plan.epi_warps;
+    args.stage_tx = a_box_rows(plan.M) * 128 + plan.block_n * 128;
     args.bias = bias;
     args.act = act;
     args.dev_status = dev_status;

@@ -50,6 +50,7 @@ struct SplitArgs {
     int n_tiles;       // tiles along N
     int splits;        // = cluster size
     int kb_per_split;
+    int stage_tx;      // bytes that the copies of one stage deliver
     const float* bias;
     int act;
     float* c;
@@ -137,7 +138,7 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
             const uint32_t full = smem_u32(&bar_full[stage]);
             const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
             if (leader && ok && (ok = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag))) {
-                mbar_arrive_expect_tx(full, (uint32_t)stage_bytes);
+                mbar_arrive_expect_tx(full, (uint32_t)args.stage_tx);
                 tma_load_2d(a_dst, &map_a, full, kb * BLOCK_K, m0);
                 tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BLOCK_K, n0);
                 ++issued;
@@ -294,39 +295,38 @@ size_t splitk_smem_bytes(int block_n, int stages) {
     return (size_t)1024 + (size_t)BLOCK_M * block_n * 4 + (size_t)stages * (A_STAGE_BYTES + block_n * BLOCK_K * 4);
 }
 
-// Tile width and number of slices for a GEMM whose tiles cannot occupy the SMs; false: do not split.
-// Slices come in powers of two up to the portable cluster size, at least four k-blocks each.  Each
-// CTA runs a single work item, so everything should be resident at once (a second, partly filled
-// wave would cost a whole kernel's fixed latency again): the choice is the (width, slices) pair that
-// puts the most CTAs on the chip within what fits (one or two CTAs per SM, by shared memory); among
-// equals the wider tile, whose MMAs are the more efficient.
-bool gemm_tf32_splitk_choice(int64_t M, int64_t N, int64_t K, int sm_count, int* block_n, int* splits) {
+// Tile width and number of slices for a GEMM; false: the single-CTA kernel, which takes `whole_ns`, is the faster one.
+// Slices come in powers of two up to the portable cluster size, at least four k-blocks each, and every CTA runs a
+// single work item, so everything has to be resident at once: clusters of 2, 4, 8 fill about 97 %, 87 %, 65 % of the SMs
+// (a GPC's last SMs do not make a cluster), twice that for 32 columns, where two CTAs share an SM.  Measured (warm
+// operands): 5.0 us and 210 ns per k-block of a slice at 32 columns, 6.0 us and 230 ns at 64, 8.3 us and 220 ns at 128;
+// 5.9 us and 360 ns where two CTAs share an SM.  [49,1024] . [1024,1024]: 6.6 us in four slices, 9.2 us whole.
+bool gemm_tf32_splitk_choice(int64_t M, int64_t N, int64_t K, int sm_count, int64_t whole_ns, int* block_n, int* splits) {
     if (!gemm_tf32_supported(M, N, K)) return false;
     const int64_t m_tiles = (M + BLOCK_M - 1) / BLOCK_M;
     const int64_t nkb = (K + BLOCK_K - 1) / BLOCK_K;
-    if (m_tiles * ((N + 31) / 32) >= sm_count) return false;  // enough 32-wide tiles without cutting K
-    int max_s = 1;
-    while (max_s * 2 <= S_MAX_SPLITS && nkb / (max_s * 2) >= S_MIN_KB) max_s *= 2;
-    if (max_s < 2) return false;
-    int64_t best = 0;
-    for (int bn = S_MAX_BLOCK_N; bn >= 32; bn >>= 1) {
-        if (bn >= 2 * N && bn > 32) continue;  // wider than the matrix
+    int64_t best = whole_ns;
+    bool found = false;
+    for (int bn = 32; bn <= S_MAX_BLOCK_N; bn <<= 1) {
         const int64_t tiles = m_tiles * ((N + bn - 1) / bn);
-        for (int s = max_s; s >= 2; s >>= 1) {
-            const int kbs = (int)((nkb + s - 1) / s);
+        for (int s = 2; s <= S_MAX_SPLITS && nkb / s >= S_MIN_KB; s <<= 1) {
+            const int64_t kbs = (nkb + s - 1) / s;
             if ((int64_t)(s - 1) * kbs >= nkb) continue;  // the last slice would be empty
-            const size_t smem = splitk_smem_bytes(bn, splitk_stages(kbs));
-            const int64_t capacity = (int64_t)sm_count * (2 * smem + 2048 <= (size_t)SMEM_LIMIT ? 2 : 1);
-            if (tiles * s > capacity) continue;
-            if (tiles * s > best) {
-                best = tiles * s;
+            const int64_t room = (int64_t)sm_count * (s == 2 ? 97 : s == 4 ? 87 : 65) / 100, ctas = tiles * s;
+            int64_t ns;
+            if (ctas <= room) ns = bn == 32 ? 5000 + 210 * kbs : bn == 64 ? 6000 + 230 * kbs : 8300 + 220 * kbs;
+            else if (bn == 32 && ctas <= 2 * room) ns = 5900 + 360 * kbs;
+            else break;
+            if (ns < best || (ns == best && !found)) {
+                best = ns;
+                found = true;
                 *block_n = bn;
                 *splits = s;
             }
-            break;  // fewer slices of the same width only lower the count
         }
+        if (bn >= N) break;
     }
-    return best > 0;
+    return found;
 }
 
 tfjsb_status gemm_tf32_splitk_plan(tfjsb_ctx* ctx, const float* a, const float* bt, float* c, int64_t M, int64_t N, int64_t K,
@@ -353,7 +353,7 @@ tfjsb_status gemm_tf32_splitk_plan(tfjsb_ctx* ctx, const float* a, const float* 
     plan->num_tiles = (int)tiles;
     plan->grid = (int)(tiles * splits);
     tfjsb_status st;
-    if ((st = encode_split_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, BLOCK_M, "A")) != TFJSB_OK) return st;
+    if ((st = encode_split_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, a_box_rows(M), "A")) != TFJSB_OK) return st;
     if ((st = encode_split_2d(ctx, &plan->map_b, bt, K, N, BLOCK_K, block_n, "B")) != TFJSB_OK) return st;
     plan->map_c = plan->map_b;  // unused: C is stored directly
     return TFJSB_OK;
@@ -373,6 +373,7 @@ cudaError_t launch_gemm_tf32_splitk(const GemmTf32Plan& plan, const float* bias,
     args.n_tiles = (int)((plan.N + plan.block_n - 1) / plan.block_n);
     args.splits = plan.splits;
     args.kb_per_split = plan.kb_per_split;
+    args.stage_tx = a_box_rows(plan.M) * 128 + plan.block_n * 128;
     args.bias = bias;
     args.act = act;
     args.c = plan.c;

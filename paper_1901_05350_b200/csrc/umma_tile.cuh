@@ -20,6 +20,11 @@ constexpr int EPI_SLAB_BYTES = 32 * EPI_COLS * 4;                // 4 KiB: 32 ro
 constexpr int EPI_BYTES = 8 /*epilogue warps*/ * EPI_SLAB_BYTES;      // 32 KiB
 constexpr int SMEM_LIMIT = 232448;                               // 227 KiB
 
+// Rows of the copy box of an A tile: those that exist, when the whole matrix is less than a tile (a multiple of 8, the
+// swizzle's period).  The other rows of the operand tile keep what was there; their results are never stored.  The copy
+// unit spends as long on rows outside the tensor as on rows inside ([1,1024] . [1024,1000]: 8.3 us with 128-row boxes).
+inline int a_box_rows(int64_t M) { return M >= BLOCK_M ? BLOCK_M : (int)((M + 7) / 8 * 8); }
+
 // Fused epilogue of one 32-row x 32-column accumulator block held one row per lane: bias add,
 // activation, and the swizzled store into the staging slab the bulk tensor store reads from
 // (16-byte chunk j of row `lane` lives at chunk j ^ (lane % 8): the 128-byte swizzle).
