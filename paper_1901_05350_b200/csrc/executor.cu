@@ -40,7 +40,6 @@ struct Step {
     bool conv_patch = false;  // STEP_CONV_TF32 through the patch kernel (whole im2col row in one k-block)
     bool fuse_next = false;
     bool fusable = false;     // the pair's shapes fit the fused kernel
-    bool fuse_pays = false;   // and there are enough tiles for it to be the faster choice
     DwPwPlan fused_plan{};
     // narrow-storage mode: which of the layer's tensors are bfloat16, and the GEMM's bfloat16 filter [N,K]
     bool is_dense = false;
@@ -93,6 +92,8 @@ struct tfjsb_model {
     std::vector<tfjsb_model*> slices;
     std::vector<cudaEvent_t> slice_copied;
     int n_slices = 0;
+    std::vector<int64_t> slice_images;  // images of each slice
+    int fusion_mode = 1;                // tfjsb_model_set_fusion
     cudaStream_t copy_stream = nullptr;
     bool is_view = false;
     // optional CUDA-graph replay of one run (tfjsb_model_set_graph): captured for the current binding
@@ -260,6 +261,19 @@ cudaError_t launch_step(tfjsb_model* m, const Step& st, cudaStream_t s) {
     return cudaErrorUnknown;
 }
 
+// A fused block has one unit of parallelism per 8 x 16 pixel tile: it pays off when there are several waves of tiles;
+// with few tiles (small batches, 14 x 14 images) the stand-alone kernels spread channel blocks and column tiles over more
+// SMs.  In the bfloat16 storage mode it is paced by its own pipeline, not by memory traffic, so halving the bytes does not
+// speed it up, while the separate narrow kernels do gain from it (batch 128: 118 / 106 / 66 us fused against 66+55 /
+// 63+37 / 35+26): never the default there.
+bool fusion_pays(const tfjsb_model* m, const Step& dw) {
+    const int64_t tiles = dw.g.N * ((dw.g.Ho + 7) / 8) * ((dw.g.Wo + 15) / 16);
+    return !m->narrow && tiles >= 4 * (int64_t)m->ctx->sm_count;
+}
+void choose_fusion(tfjsb_model* m) {
+    for (Step& st : m->steps) st.fuse_next = st.fusable && (m->fusion_mode == 2 || (m->fusion_mode == 1 && fusion_pays(m, st)));
+}
+
 // A view of `parent` for a batch of `n` images: steps copied with every batch-proportional size scaled.
 tfjsb_model* make_batch_view(tfjsb_model* parent, int64_t n) {
     const int64_t pn = parent->in_dims[0];
@@ -284,6 +298,8 @@ tfjsb_model* make_batch_view(tfjsb_model* parent, int64_t n) {
         st.in = nullptr;
         st.out = nullptr;
     }
+    v->fusion_mode = parent->fusion_mode;
+    choose_fusion(v);  // by the view's own batch
     return v;
 }
 
@@ -618,13 +634,7 @@ tfjsb_status tfjsb_model_create(tfjsb_ctx* ctx, const tfjsb_layer_desc* layers, 
             const Step& pw = m->steps[i + 1];
             if (dw.kind == STEP_DEPTHWISE && pw.kind == STEP_GEMM_TF32 && pw.K == dw.g.Co &&
                 pw.M == dw.g.N * dw.g.Ho * dw.g.Wo && dwpw_fused_supported(dw.g, pw.N)) {
-                // The fused kernel has one unit of parallelism per 8 x 16 pixel tile: it pays off when
-                // there are several waves of tiles; with few tiles (small batches, 14 x 14 images) the
-                // stand-alone kernels spread channel blocks and column tiles over more SMs.
-                const int64_t tiles = dw.g.N * ((dw.g.Ho + 7) / 8) * ((dw.g.Wo + 15) / 16);
                 dw.fusable = true;
-                dw.fuse_pays = tiles >= 4 * (int64_t)ctx->sm_count;
-                dw.fuse_next = dw.fuse_pays;
             }
         }
     }
@@ -636,17 +646,11 @@ tfjsb_status tfjsb_model_create(tfjsb_ctx* ctx, const tfjsb_layer_desc* layers, 
             const Step& pw = m->steps[i + 1];
             if (dw.kind == STEP_DEPTHWISE_NARROW && pw.kind == STEP_GEMM_NARROW && !pw.is_dense && pw.filter_km && pw.K == dw.g.Co &&
                 pw.M == dw.g.N * dw.g.Ho * dw.g.Wo && pw.N % 8 == 0 && dw.out_bf16 && pw.out_bf16 && dwpw_fused_supported(dw.g, pw.N)) {
-                const int64_t tiles = dw.g.N * ((dw.g.Ho + 7) / 8) * ((dw.g.Wo + 15) / 16);
-                // Available (tfjsb_model_set_fusion(model, 2)) but not chosen: the fused kernel is paced by its own
-                // pipeline, not by memory traffic, so halving the bytes does not speed it up, while the separate
-                // narrow kernels do gain from it (batch 128: 118 / 106 / 66 us fused against 66+55 / 63+37 / 35+26).
-                (void)tiles;
                 dw.fusable = true;
-                dw.fuse_pays = false;
-                dw.fuse_next = false;
             }
         }
     }
+    choose_fusion(m);
     if ((st = dev_alloc(m, 2 * m->region_elems, &m->arena)) != TFJSB_OK) return bail(st, ctx->last_error);
     cudaError_t e = cudaDeviceSynchronize();  // weight transposes done
     if (e != cudaSuccess) return bail(TFJSB_ERR_CUDA, std::string("model set-up: ") + cudaGetErrorString(e));
@@ -711,9 +715,11 @@ tfjsb_status tfjsb_run_model(tfjsb_model* m, const tfjsb_tensor* input, tfjsb_te
 tfjsb_status tfjsb_model_set_fusion(tfjsb_model* m, int mode) {
     if (!m) return TFJSB_ERR_INVALID_ARG;
     if (mode < 0 || mode > 2) return fail(m->ctx, TFJSB_ERR_INVALID_ARG, "fusion mode must be 0 (off), 1 (auto) or 2 (always)");
-    for (Step& st : m->steps) st.fuse_next = st.fusable && (mode == 2 || (mode == 1 && st.fuse_pays));
+    m->fusion_mode = mode;
+    choose_fusion(m);
     for (tfjsb_model* v : m->slices) {
-        for (Step& st : v->steps) st.fuse_next = st.fusable && (mode == 2 || (mode == 1 && st.fuse_pays));
+        v->fusion_mode = mode;
+        choose_fusion(v);
         v->bound_in = nullptr; v->bound_out = nullptr;
         drop_graph(v);
     }
@@ -746,11 +752,13 @@ tfjsb_status enqueue_host_run(tfjsb_model* m, const float* host_input, float* ho
         m->host_run_pending[b] = false;
     }
     if (!m->staged_in[b]) {
-        if ((st = dev_alloc(m, (size_t)m->in_elems, &m->staged_in[b])) != TFJSB_OK) return st;
-        if ((st = dev_alloc(m, (size_t)last.out_elems, &m->staged_out[b])) != TFJSB_OK) return st;
+        // a slice starts on 16 bytes: up to three values of padding after each image, at most
+        if ((st = dev_alloc(m, (size_t)(m->in_elems + 4 * m->in_dims[0]), &m->staged_in[b])) != TFJSB_OK) return st;
+        if ((st = dev_alloc(m, (size_t)(last.out_elems + 4 * m->in_dims[0]), &m->staged_out[b])) != TFJSB_OK) return st;
         if ((e = cudaEventCreateWithFlags(&m->host_run_done[b], cudaEventDisableTiming)) != cudaSuccess)
             return cuda_fail(ctx, e, "cudaEventCreate");
     }
+    const int64_t out_image = last.out_elems / m->in_dims[0];
     if (m->keep_all) {
         // debug mode: the whole batch through the model itself, so that every layer's output stays readable
         e = cudaMemcpyAsync(m->staged_in[b], host_input, (size_t)m->in_elems * 4, cudaMemcpyHostToDevice, s);
@@ -761,12 +769,16 @@ tfjsb_status enqueue_host_run(tfjsb_model* m, const float* host_input, float* ho
     } else {
         if (m->slices.empty()) {
             const int64_t n = m->in_dims[0];
-            // four slices: more of them lose more to per-launch fixed costs than the extra overlap returns
-            int n_slices = (n % 4 == 0 && n >= 32) ? 4 : 1;
+            // Slices of 24 images or so: an image's copy takes longer than its share of the computation (11 against
+            // 6 us for 224 x 224 x 3 and the full model), but a slice also costs about 115 us of fixed chain, so more
+            // slices make the computation the longer of the two.  50 images: 1000 us whole, 850 in two or three
+            // slices, 945 in four.
+            int n_slices = n < 24 ? 1 : n < 72 ? 2 : n < 96 ? 3 : 4;
             if (const char* env = getenv("TFJSB_HOST_SLICES")) {  // tuning knob: 1 disables the slicing
                 const int v = atoi(env);
-                if (v >= 1 && n % v == 0) n_slices = v;
+                if (v >= 1 && v <= n) n_slices = v;
             }
+            for (int c = 0; c < n_slices; ++c) m->slice_images.push_back(n / n_slices + (c < n % n_slices ? 1 : 0));
             if ((e = cudaStreamCreateWithFlags(&m->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
                 return cuda_fail(ctx, e, "cudaStreamCreate");
             for (int i = 0; i < 2 * n_slices; ++i) {
@@ -774,34 +786,50 @@ tfjsb_status enqueue_host_run(tfjsb_model* m, const float* host_input, float* ho
                 if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess)
                     return cuda_fail(ctx, e, "cudaEventCreate");
                 m->slice_copied.push_back(ev);
-                m->slices.push_back(make_batch_view(m, n / n_slices));
+                m->slices.push_back(make_batch_view(m, m->slice_images[i % n_slices]));
             }
             m->n_slices = n_slices;
         }
         const int n_slices = m->n_slices;
-        const int64_t in_slice = m->in_elems / n_slices, out_slice = last.out_elems / n_slices;
+        const int64_t in_image = m->in_elems / m->in_dims[0];
         // The copies wait for nothing on `stream`: the staging set is free (checked above), so they may
         // run while an earlier run is still computing.
+        auto padded = [](int64_t elems) { return (elems + 3) / 4 * 4; };
+        int64_t first = 0, at = 0;  // image, offset in the staging buffer
         for (int c = 0; c < n_slices; ++c) {
-            e = cudaMemcpyAsync(m->staged_in[b] + c * in_slice, host_input + c * in_slice, (size_t)in_slice * 4,
-                                cudaMemcpyHostToDevice, m->copy_stream);
+            const int64_t elems = m->slice_images[c] * in_image;
+            e = cudaMemcpyAsync(m->staged_in[b] + at, host_input + first * in_image, (size_t)elems * 4, cudaMemcpyHostToDevice, m->copy_stream);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "host-to-device copy of the input");
             if ((e = cudaEventRecord(m->slice_copied[b * n_slices + c], m->copy_stream)) != cudaSuccess)
                 return cuda_fail(ctx, e, "cudaEventRecord");
+            first += m->slice_images[c];
+            at += padded(elems);
         }
+        int64_t out_at = 0;
+        at = 0;
         for (int c = 0; c < n_slices; ++c) {
             tfjsb_model* v = m->slices[b * n_slices + c];
             if ((e = cudaStreamWaitEvent(s, m->slice_copied[b * n_slices + c], 0)) != cudaSuccess)
                 return cuda_fail(ctx, e, "cudaStreamWaitEvent");
-            tfjsb_tensor in{m->staged_in[b] + c * in_slice, 4, {v->in_dims[0], v->in_dims[1], v->in_dims[2], v->in_dims[3]}};
+            tfjsb_tensor in{m->staged_in[b] + at, 4, {v->in_dims[0], v->in_dims[1], v->in_dims[2], v->in_dims[3]}};
             const Step& vl = v->steps.back();
-            tfjsb_tensor out{m->staged_out[b] + c * out_slice, vl.out_rank, {vl.out_dims[0], vl.out_dims[1], vl.out_dims[2], vl.out_dims[3]}};
+            tfjsb_tensor out{m->staged_out[b] + out_at, vl.out_rank, {vl.out_dims[0], vl.out_dims[1], vl.out_dims[2], vl.out_dims[3]}};
+            at += padded(m->slice_images[c] * in_image);
+            out_at += padded(m->slice_images[c] * out_image);
             if ((st = tfjsb_run_model(v, &in, &out, s)) != TFJSB_OK) return st;
             v->use_graph = true;  // the first pass ran launch by launch; later passes replay a graph
         }
     }
-    e = cudaMemcpyAsync(host_output, m->staged_out[b], (size_t)last.out_elems * 4, cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "device-to-host copy of the output");
+    // one copy when the slices' results lie next to each other, else one per slice
+    bool gaps = false;
+    for (int c = 0; !m->keep_all && c + 1 < m->n_slices; ++c) gaps = gaps || (m->slice_images[c] * out_image) % 4 != 0;
+    for (int64_t c = 0, first = 0, at = 0; first < m->in_dims[0]; ++c) {
+        const int64_t images = gaps ? m->slice_images[c] : m->in_dims[0];
+        e = cudaMemcpyAsync(host_output + first * out_image, m->staged_out[b] + at, (size_t)(images * out_image) * 4, cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "device-to-host copy of the output");
+        first += images;
+        at += (images * out_image + 3) / 4 * 4;
+    }
     if ((e = cudaEventRecord(m->host_run_done[b], s)) != cudaSuccess) return cuda_fail(ctx, e, "cudaEventRecord");
     m->host_run_pending[b] = true;
     return TFJSB_OK;

@@ -195,3 +195,21 @@ def test_model_rejects_wrong_shapes(ctx, tfjsb):
         ctx.model(bad, x.shape)
     assert e.value.status_name == "UNSUPPORTED"
     model.close()
+
+
+@pytest.mark.parametrize("batch,hw,classes", [(23, 33, 10), (25, 33, 10), (37, 32, 101), (50, 33, 7), (75, 31, 6), (97, 32, 33)])
+def test_host_runs_in_uneven_slices(ctx, oracle, batch, hw, classes):
+    """Batches that do not divide evenly, images and results whose size is no multiple of 16 bytes."""
+    import torch
+
+    x, layers = si.config_mobilenet(0.25, hw, batch, seed=4243, classes=classes)
+    want = oracle.run_model(layers, x)
+    model = ctx.model(layers, x.shape)
+    hin = torch.from_numpy(x).pin_memory()
+    for _ in range(3):  # launch by launch, then as graph replays, on both sets of staging buffers
+        hout = torch.full(model.output_shape, -1.0).pin_memory()
+        model.run_host(hin, hout)
+        # probabilities in [0, 1] of a model whose logits are within 1e-2 of their range (the whole-model bar)
+        assert np.max(np.abs(hout.numpy() - want)) <= 2e-2 * want.max() and np.allclose(hout.numpy().sum(-1), 1, atol=1e-5)
+    ctx.check_device_status()
+    model.close()
