@@ -385,22 +385,20 @@ tfjsb_status tfjsb_batch_matmul(tfjsb_ctx* ctx, const tfjsb_tensor* a, const tfj
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (B > 1 && ctx->math == TFJSB_MATH_TF32 && gemm_tf32_supported(M, N, K) && ctx->encode_tiled) {
         // All products in one launch of the tensor-core kernel: their tiles share the SMs.  Operands
-        // that are not K-contiguous are transposed into scratch first, one product at a time.
+        // that are not K-contiguous are transposed into scratch first, all products of an operand in one launch.
         cudaError_t e;
         const float* a_km = pa;
         const float* b_km = pb;
         if (transpose_a) {
             if ((st = ensure_scratch(ctx, &ctx->scratch_a, (size_t)B * M * K * 4)) != TFJSB_OK) return st;
-            for (int64_t i = 0; i < B; ++i)
-                if ((e = launch_transpose(pa + i * M * K, ctx->scratch_a.ptr + i * M * K, K, M, s, &ctx->launches)) != cudaSuccess)
-                    return cuda_fail(ctx, e, "transpose(a)");
+            if ((e = launch_transpose_batched(pa, ctx->scratch_a.ptr, B, K, M, s, &ctx->launches)) != cudaSuccess)
+                return cuda_fail(ctx, e, "transpose(a)");
             a_km = ctx->scratch_a.ptr;
         }
         if (!transpose_b) {
             if ((st = ensure_scratch(ctx, &ctx->scratch_b, (size_t)B * N * K * 4)) != TFJSB_OK) return st;
-            for (int64_t i = 0; i < B; ++i)
-                if ((e = launch_transpose(pb + i * N * K, ctx->scratch_b.ptr + i * N * K, K, N, s, &ctx->launches)) != cudaSuccess)
-                    return cuda_fail(ctx, e, "transpose(b)");
+            if ((e = launch_transpose_batched(pb, ctx->scratch_b.ptr, B, K, N, s, &ctx->launches)) != cudaSuccess)
+                return cuda_fail(ctx, e, "transpose(b)");
             b_km = ctx->scratch_b.ptr;
         }
         GemmTf32Plan plan;

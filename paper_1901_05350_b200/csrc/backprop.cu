@@ -293,23 +293,6 @@ act_backprop_kernel(const float* __restrict__ y, const float* __restrict__ dy, f
     if (first < (n & 3)) dz[4 * n4 + first] = act_grad(y[4 * n4 + first], dy[4 * n4 + first], act);
 }
 
-// out[b, c, r] = in[b, r, c] for B matrices of shape [rows, cols] stored one after the other
-__global__ void transpose_batched_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t rows, int64_t cols) {
-    __shared__ float tile[32][33];
-    in += (int64_t)blockIdx.z * rows * cols;
-    out += (int64_t)blockIdx.z * rows * cols;
-    const int64_t c0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 32;
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int64_t r = r0 + j, c = c0 + threadIdx.x;
-        if (r < rows && c < cols) tile[j][threadIdx.x] = in[r * cols + c];
-    }
-    __syncthreads();
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int64_t c = c0 + j, r = r0 + threadIdx.x;
-        if (r < rows && c < cols) out[c * rows + r] = tile[threadIdx.x][j];
-    }
-}
-
 int blocks_for(int64_t items, int sm_count) {
     int64_t b = (items + BP_THREADS - 1) / BP_THREADS;
     const int64_t cap = (int64_t)sm_count * 16;
@@ -446,16 +429,6 @@ cudaError_t launch_depthwise_backprop_filter(const float* x, const float* dy, fl
 cudaError_t launch_act_backprop(const float* y, const float* dy, float* dz, int64_t n, int act, int sm_count, cudaStream_t s,
                                 int64_t* launches) {
     act_backprop_kernel<<<blocks_for((n + 3) / 4, sm_count), BP_THREADS, 0, s>>>(y, dy, dz, n, act);
-    ++*launches;
-    return cudaGetLastError();
-}
-
-cudaError_t launch_transpose_batched(const float* in, float* out, int64_t batches, int64_t rows, int64_t cols, cudaStream_t s,
-                                     int64_t* launches) {
-    if (rows == 0 || cols == 0 || batches == 0) return cudaSuccess;
-    dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32), (unsigned)batches);
-    if ((rows + 31) / 32 > 65535 || batches > 65535) return cudaErrorInvalidConfiguration;
-    transpose_batched_kernel<<<grid, dim3(32, 8), 0, s>>>(in, out, rows, cols);
     ++*launches;
     return cudaGetLastError();
 }

@@ -270,18 +270,26 @@ __global__ void softmax_rows_kernel(const float* __restrict__ x, float* __restri
 }
 
 // ---- transpose --------------------------------------------------------------------------------
-__global__ void transpose_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t rows,
-                                 int64_t cols) {
+// out[b, c, r] = in[b, r, c]: a 32 x 32 tile through shared memory per block.  The grid covers (columns, rows, matrices) and
+// walks on over rows and matrices beyond its limits.
+__global__ void transpose_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t batches, int64_t rows, int64_t cols) {
     __shared__ float tile[32][33];
-    const int64_t c0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 32;
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int64_t r = r0 + j, c = c0 + threadIdx.x;
-        if (r < rows && c < cols) tile[j][threadIdx.x] = in[r * cols + c];
-    }
-    __syncthreads();
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int64_t c = c0 + j, r = r0 + threadIdx.x;
-        if (r < rows && c < cols) out[c * rows + r] = tile[threadIdx.x][j];
+    const int64_t c0 = (int64_t)blockIdx.x * 32;
+    for (int64_t b = blockIdx.z; b < batches; b += gridDim.z) {
+        const float* from = in + b * rows * cols;
+        float* to = out + b * rows * cols;
+        for (int64_t r0 = (int64_t)blockIdx.y * 32; r0 < rows; r0 += (int64_t)gridDim.y * 32) {
+            for (int j = threadIdx.y; j < 32; j += 8) {
+                const int64_t r = r0 + j, c = c0 + threadIdx.x;
+                if (r < rows && c < cols) tile[j][threadIdx.x] = from[r * cols + c];
+            }
+            __syncthreads();
+            for (int j = threadIdx.y; j < 32; j += 8) {
+                const int64_t c = c0 + j, r = r0 + threadIdx.x;
+                if (r < rows && c < cols) to[c * rows + r] = tile[threadIdx.x][j];
+            }
+            __syncthreads();
+        }
     }
 }
 
@@ -391,14 +399,18 @@ cudaError_t launch_softmax(const float* x, float* y, int64_t rows, int64_t cols,
     return e;
 }
 
-cudaError_t launch_transpose(const float* in, float* out, int64_t rows, int64_t cols, cudaStream_t s,
-                             int64_t* launches) {
-    if (rows == 0 || cols == 0) return cudaSuccess;
-    dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
-    if (grid.y > 65535) return cudaErrorInvalidConfiguration;
-    transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(in, out, rows, cols);
+cudaError_t launch_transpose_batched(const float* in, float* out, int64_t batches, int64_t rows, int64_t cols, cudaStream_t s,
+                                     int64_t* launches) {
+    if (rows == 0 || cols == 0 || batches == 0) return cudaSuccess;
+    const int64_t gy = (rows + 31) / 32;
+    const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)(gy < 65535 ? gy : 65535), (unsigned)(batches < 65535 ? batches : 65535));
+    transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(in, out, batches, rows, cols);
     ++*launches;
     return cudaGetLastError();
+}
+
+cudaError_t launch_transpose(const float* in, float* out, int64_t rows, int64_t cols, cudaStream_t s, int64_t* launches) {
+    return launch_transpose_batched(in, out, 1, rows, cols, s, launches);
 }
 
 }  // namespace tfjsb

@@ -89,6 +89,7 @@ BATCH_MATMUL_CASES = [
     (2, 49, 1024, 256, True, False),     # few tiles, long K: each product is cut along K
     (5, 9, 13, 5, False, False),         # slices not 16-byte aligned: CUDA-core kernel
     (1, 512, 512, 512, True, True),
+    (70, 68, 36, 100, True, False),      # both operands transposed in one launch each, ragged 32 x 32 tiles
 ]
 
 
