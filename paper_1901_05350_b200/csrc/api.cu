@@ -753,6 +753,13 @@ tfjsb_status tfjsb_conv2d_backprop_filter(tfjsb_ctx* ctx, const tfjsb_tensor* x,
             return TFJSB_OK;
         }
     }
+    if (conv2d_small_filter_supported(g)) {
+        const int n = conv2d_small_filter_slices(g, ctx->sm_count);
+        if (n > 1 && (st = ensure_scratch(ctx, &ctx->scratch_c, (size_t)n * numel(dfilter) * 4)) != TFJSB_OK) return st;
+        if ((e = launch_conv2d_small_filter(px, pg, pdf, ctx->scratch_c.ptr, n, g, s, &ctx->launches)) != cudaSuccess)
+            return cuda_fail(ctx, e, "conv2d_backprop_filter launch");
+        return TFJSB_OK;
+    }
     int slices = backprop_slices(pixels, ctx->sm_count);
     const int64_t tile_blocks = (int64_t)g.fh * g.fw * ((g.C + 31) / 32) * ((g.Co + 31) / 32);
     while (slices > 1 && tile_blocks * slices > 16 * (int64_t)ctx->sm_count) slices >>= 1;

@@ -328,6 +328,11 @@ cudaError_t launch_conv2d_backprop_filter(const float* x, const float* dy, float
 // 3x3 kernels of depthwise.cu can run it for this forward geometry, and the geometry that they get.
 bool depthwise_backprop_is_forward(const ConvGeom& g);
 ConvGeom depthwise_backprop_geometry(const ConvGeom& g);
+// The same for fh*fw*Cin <= 32 and Cout % 4 == 0 (the first layer's filter); `partial` holds slices * fh*fw*C*Co floats.
+bool conv2d_small_filter_supported(const ConvGeom& g);
+int conv2d_small_filter_slices(const ConvGeom& g, int sm_count);
+cudaError_t launch_conv2d_small_filter(const float* x, const float* dy, float* df, float* partial, int slices, const ConvGeom& g,
+                                       cudaStream_t s, int64_t* launches);
 cudaError_t launch_depthwise_backprop_input(const float* dy, const float* f, float* dx, const ConvGeom& g, int sm_count,
                                             cudaStream_t s, int64_t* launches);
 // `partial` holds slices * fh*fw*Co floats (unused when slices == 1)

@@ -127,6 +127,38 @@ def test_conv2d_gradients_keep_fp32_accuracy_in_tf32_mode(ctx, oracle, case):
     assert rel_fro(df, oracle.conv2d_backprop_filter(x, f.shape, g, *args)) <= 1e-5
 
 
+SMALL_FILTER_CASES = [
+    # N, H, W, Cin, Cout, fh, fw, stride, dilation, pad: windows of up to 32 elements
+    (1, 3, 3, 3, 4, 3, 3, 1, 1, "same"),
+    (2, 31, 17, 3, 32, 3, 3, 2, 1, "same"),      # four pixel lanes per channel group
+    (3, 40, 33, 3, 64, 3, 3, 1, 1, "same"),      # two
+    (2, 29, 30, 3, 100, 3, 3, 2, 1, "valid"),    # one, ragged channels
+    (2, 20, 21, 3, 260, 3, 3, 1, 1, "same"),     # three channel tiles
+    (1, 1, 90, 1, 36, 1, 5, 1, 1, "same"),       # one row
+    (70, 9, 5, 2, 8, 4, 4, 1, 1, "same"),        # 32 elements; images smaller than a step of pixels
+    (2, 24, 18, 3, 16, 3, 3, 1, 3, "same"),      # dilated
+]
+
+
+@pytest.mark.parametrize("math", ["tf32", "fp32"])
+@pytest.mark.parametrize("case", SMALL_FILTER_CASES)
+def test_gradient_of_a_small_filter(ctx, oracle, case, math):
+    N, H, W, Cin, Cout, fh, fw, s, d, pad = case
+    Ho, Wo = geometry(oracle, H, W, fh, fw, s, d, pad)
+    ctx.set_math(math)
+    try:
+        x = si.small_integers(95, 0, (N, H, W, Cin), -3, 3)
+        g = si.small_integers(95, 1, (N, Ho, Wo, Cout), -3, 3)
+        df = host(ctx.conv2d_backprop_filter(dev(x), (fh, fw, Cin, Cout), dev(g), (s, s), pad, (d, d)))
+        assert same_bits(df + 0.0, oracle.conv2d_backprop_filter(x, (fh, fw, Cin, Cout), g, (s, s), pad, (d, d)) + 0.0)
+        x, g = si.uniform(96, 0, x.shape, -1, 1), si.normal(96, 1, g.shape, 0, 1)
+        df = host(ctx.conv2d_backprop_filter(dev(x), (fh, fw, Cin, Cout), dev(g), (s, s), pad, (d, d)))
+        assert rel_fro(df, oracle.conv2d_backprop_filter(x, (fh, fw, Cin, Cout), g, (s, s), pad, (d, d))) <= 1e-5
+    finally:
+        ctx.set_math("tf32")
+    ctx.check_device_status()
+
+
 DEPTHWISE_3X3_CASES = [
     # N, H, W, C, stride, dilation, pad: tile edges of the pipelined kernels and of the stride-2 column pairs
     (1, 1, 1, 4, 1, 1, "same"),
