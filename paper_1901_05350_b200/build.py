@@ -38,6 +38,7 @@ SOURCES = [
     "depthwise_grad.cu",
     "conv_grad_tcgen05.cu",
     "gemm_strided_tcgen05.cu",
+    "chain_cluster.cu",
 ]
 
 NVCC_FLAGS = [

@@ -396,4 +396,53 @@ cudaError_t launch_dwpw_fused(const DwPwPlan& plan, const float* dw_filter, cons
                               const float* pw_bias, int pw_act, unsigned int* dev_status, cudaStream_t s,
                               int64_t* launches);
 
+// ---- several layers as one kernel (chain_cluster.cu) ----------------------------------------------------
+enum ChainKind { CHAIN_STEM, CHAIN_BLOCK, CHAIN_POOL, CHAIN_DENSE, CHAIN_SOFTMAX };
+struct ChainOp {
+    int kind = CHAIN_SOFTMAX;
+    int H = 0, W = 0, C = 0, Ho = 0, Wo = 0, Co = 0;  // of one image; dense and softmax: C -> Co
+    int sh = 1, sw = 1, dh = 1, dw = 1, pt = 0, pl = 0;
+    int act1 = 0, act2 = 0;                 // after the depthwise part, after the step
+    int round1 = 0, round2 = 0, store_bf16 = 0;  // round to bfloat16 (stem: its input), and how the result is stored
+    // a block's tiles: `pixels` rows for one of `groups` groups of `group_cols` columns is a unit; columns are multiplied
+    // `tile_cols` at a time by warp tiles of `variant`'s shape, K divided among `k_splits` warps
+    int pixels = 0, groups = 1, group_cols = 0, tile_cols = 0, units = 0, variant = 0, k_splits = 1;
+    int w_stride = 0, chunk_rows = 0, n_chunks = 0, chunk_floats = 0, group_tiles = 0, tasks = 0, task_n = 0, task_rows = 0, task_cols = 0, lanes = 0, strip = 1;
+    // ceil(2^32 / d) for the divisors Wo, groups, tile_cols / 4 (stem: w_stride), C / 4 (stem: in_row), tasks, task_n (0 for
+    // d = 1)
+    unsigned int by_wo = 0, by_groups = 0, by_pieces = 0, by_quads = 0, by_tasks = 0, by_task_n = 0;
+    float lo1 = 0, hi1 = 0, lo2 = 0, hi2 = 0;       // the activations as bounds
+    int in_row = 0, out_row = 0, out_origin = 0;    // floats between rows of the input and of the output, and its first element
+    int64_t out_buffer = 0;                         // in the cluster's workspace
+    const float *f1 = nullptr, *b1 = nullptr, *f2 = nullptr, *b2 = nullptr;  // depthwise (stem, dense) and pointwise [C,Co]
+    // pool and dense: where the layer's own output tensor is, [images][Co], which a caller may read after the run
+    float* also = nullptr;
+    int also_bf16 = 0;
+};
+constexpr int CHAIN_MAX_OPS = 22;
+struct ChainArgs {
+    ChainOp ops[CHAIN_MAX_OPS];
+    int n_ops = 0, cluster_size = 1;
+    int64_t images = 0, in_elems = 0, out_elems = 0;  // elements per image
+    int64_t cluster_elems = 0;                        // of workspace
+    const float* input = nullptr;
+    float* output = nullptr;
+    float* workspace = nullptr;  // [clusters][cluster_elems], zero before the first launch
+    unsigned int* dev_status = nullptr;
+};
+struct ChainPlan {
+    ChainArgs args;
+    int blocks = 0;
+    double ns = 0;  // estimate
+};
+bool chain_stem_supported(const ConvGeom& g);
+bool chain_block_supported(const ConvGeom& dw, int64_t Cout);
+// Fills in everything but the pointers and the element counts; false where no cluster of this kernel fits.
+bool chain_plan(const ChainOp* ops, int n_ops, int64_t images, ChainPlan* plan);
+// The blocks' filters in the plan's layout, `dst` of chain_packed_floats; the plan then refers to them.
+int64_t chain_packed_floats(const ChainPlan& plan);
+cudaError_t chain_pack(ChainPlan* plan, float* dst, cudaStream_t s, int64_t* launches);
+cudaError_t launch_chain(const ChainPlan& plan, const float* input, float* output, unsigned int* dev_status, cudaStream_t s,
+                         int64_t* launches);
+
 }  // namespace tfjsb

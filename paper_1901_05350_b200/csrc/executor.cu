@@ -8,6 +8,7 @@
 // the paper's texture recycler, Sec. 4.1.2), tensor maps encoded once against those fixed
 // addresses.  Running (tfjsb_run_model) therefore does no allocation, no shape arithmetic and
 // no synchronisation: it enqueues the kernels and returns (Sec. 4.1.1).
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <vector>
@@ -94,6 +95,13 @@ struct tfjsb_model {
     int n_slices = 0;
     std::vector<int64_t> slice_images;  // images of each slice
     int fusion_mode = 1;                // tfjsb_model_set_fusion
+    int chain_len = 0;                  // the first layers that run as one kernel (0: none), outside keep-all mode
+    ChainPlan chain;
+    int chain_layer[CHAIN_MAX_OPS] = {};  // the layer whose output an operation makes
+    float* chain_workspace = nullptr;
+    int64_t chain_elems = 0;  // of workspace per cluster, for the longest chain
+    bool chain_allowed = false, chain_chosen = false;
+    int chain_best = 0;       // chain_len where the fusion mode lets it be chosen
     cudaStream_t copy_stream = nullptr;
     bool is_view = false;
     // optional CUDA-graph replay of one run (tfjsb_model_set_graph): captured for the current binding
@@ -195,11 +203,21 @@ tfjsb_status bind_all(tfjsb_model* m, const float* input, float* output) {
             // A fused pair is one kernel: it reads the first layer's input and writes the second
             // layer's output, so the pair takes one region (the first layer's own output buffer is
             // never written) and the region flips once per kernel, not once per layer.
-            if (!st.fuse_next) region ^= 1;
+            // A chain of layers likewise, but for the vectors at its end, which it writes as the layers do.
+            if (!st.fuse_next && (i >= m->chain_len || st.out_rank == 2)) region ^= 1;
         }
         tfjsb_status rc = bind_step(m, st, cur, dst);
         if (rc != TFJSB_OK) return rc;
         cur = dst;
+    }
+    if (!m->keep_all && m->chain_len) {
+        for (int k = 0; k + 1 < m->chain.args.n_ops; ++k) {
+            ChainOp& o = m->chain.args.ops[k];
+            const Step& st = m->steps[m->chain_layer[k]];
+            if (st.out_rank != 2) continue;
+            o.also = st.out;
+            o.also_bf16 = st.out_bf16;
+        }
     }
     if (!m->keep_all) {
         for (int i = 0; i + 1 < n; ++i) {
@@ -270,8 +288,129 @@ bool fusion_pays(const tfjsb_model* m, const Step& dw) {
     const int64_t tiles = dw.g.N * ((dw.g.Ho + 7) / 8) * ((dw.g.Wo + 15) / 16);
     return !m->narrow && tiles >= 4 * (int64_t)m->ctx->sm_count;
 }
-void choose_fusion(tfjsb_model* m) {
+
+// What a layer takes as a kernel of its own, in ns: about 4 us however small it is, and its bytes.  Within 10 % of the
+// measured sums of small models (30 layers: 102 to 112 us for one image, 132 for 32 and 205 for 128 images of 128 x 128
+// at a width of 0.25); too low for large layers, whose products take longer, which only keeps the chain away from them.
+double separate_ns(const tfjsb_model* m, const Step& st) {
+    const double width = m->narrow ? 2 : 4;
+    const double in = st.kind == STEP_SOFTMAX || st.K ? (double)st.M * (st.K ? st.K : st.N) : (double)st.g.N * st.g.H * st.g.W * st.g.C;
+    const double bytes = width * (in + (double)st.out_elems);
+    return 3800 + bytes / 4000;
+}
+
+// The leading layers as one kernel's operations: first convolution, depthwise + pointwise pairs, pool, dense, softmax.
+// `layers_of` gets the number of layers up to and with each.
+int chain_ops(const tfjsb_model* m, ChainOp* ops, int* layers_of) {
+    const int n = (int)m->steps.size();
+    int n_ops = 0, i = 0;
+    while (i < n && n_ops < CHAIN_MAX_OPS) {
+        const Step& st = m->steps[i];
+        const ConvGeom& g = st.g;
+        ChainOp o;
+        o.H = g.H; o.W = g.W; o.C = g.C; o.Ho = g.Ho; o.Wo = g.Wo; o.Co = g.Co;
+        o.sh = g.sh; o.sw = g.sw; o.dh = g.dh; o.dw = g.dw; o.pt = g.pt; o.pl = g.pl;
+        o.f1 = st.filter; o.b1 = st.bias;
+        o.act2 = st.act;
+        int used = 1;
+        if (i == 0) {
+            if ((st.kind != STEP_CONV_TF32 && st.kind != STEP_CONV_FP32 && st.kind != STEP_CONV_NARROW) || !chain_stem_supported(g)) break;
+            o.kind = CHAIN_STEM;
+            o.round1 = m->narrow;
+            o.round2 = st.out_bf16;
+        } else if (st.kind == STEP_DEPTHWISE || st.kind == STEP_DEPTHWISE_NARROW) {
+            if (i + 1 >= n) break;
+            const Step& pw = m->steps[i + 1];
+            const bool pointwise = pw.kind == STEP_GEMM_TF32 || pw.kind == STEP_GEMM_FP32 || pw.kind == STEP_GEMM_NARROW || pw.kind == STEP_CONV_NARROW;
+            if (!pointwise || pw.is_dense || pw.out_rank != 4 || pw.g.fh != 1 || pw.g.fw != 1 || pw.g.sh != 1 || pw.g.sw != 1 ||
+                pw.g.pt != 0 || pw.g.pl != 0 || !chain_block_supported(g, pw.g.Co))
+                break;
+            o.kind = CHAIN_BLOCK;
+            o.act1 = st.act;
+            o.round1 = st.out_bf16;
+            o.Co = pw.g.Co;
+            o.f2 = pw.filter; o.b2 = pw.bias;
+            o.act2 = pw.act;
+            o.round2 = pw.out_bf16;
+            used = 2;
+        } else if ((st.kind == STEP_POOL || st.kind == STEP_POOL_NARROW) && g.Ho == 1 && g.Wo == 1 && g.fh == g.H && g.fw == g.W && g.pt == 0 &&
+                   g.pl == 0 && g.C % 4 == 0) {
+            o.kind = CHAIN_POOL;
+            o.Co = g.C;
+            o.act2 = TFJSB_ACT_NONE;
+            o.round2 = st.out_bf16;
+            if (st.out_rank != 2) break;
+        } else if (n_ops && ops[n_ops - 1].kind == CHAIN_POOL && st.out_rank == 2 && st.K == m->steps[i - 1].g.C && st.N % 4 == 0 && st.N <= 0xffff) {
+            o.kind = CHAIN_DENSE;
+            o.C = (int)st.K; o.Co = (int)st.N;
+            o.H = o.W = o.Ho = o.Wo = 1;
+        } else if (n_ops && ops[n_ops - 1].kind == CHAIN_DENSE && st.kind == STEP_SOFTMAX) {
+            o.kind = CHAIN_SOFTMAX;
+            o.C = o.Co = (int)st.N;
+            o.H = o.W = o.Ho = o.Wo = 1;
+            o.act2 = TFJSB_ACT_NONE;
+        } else break;
+        i += used;
+        ops[n_ops] = o;
+        layers_of[n_ops++] = i;
+    }
+    return n_ops;
+}
+
+// The number of leading layers that run as one kernel, 0 where their own kernels are faster.  The choice, the filters in
+// the kernel's layout and the workspace are made once.  `owner` has the memory: the model itself, or the model that a view belongs to (its layers have the same layout in it).
+int plan_chain(tfjsb_model* m, tfjsb_model* owner) {
+    ChainOp ops[CHAIN_MAX_OPS];
+    int layers_of[CHAIN_MAX_OPS] = {}, len = 0;
+    const int n_ops = chain_ops(m, ops, layers_of);
+    const int64_t images = m->in_dims[0];
+    double separate = 0, done = 0;
+    for (const Step& st : m->steps) separate += separate_ns(m, st);
+    double best = separate;
+    for (int k = 0, i = 0; k < n_ops; ++k) {
+        for (; i < layers_of[k]; ++i) done += separate_ns(m, m->steps[i]);
+        if (ops[k].kind < CHAIN_POOL) continue;
+        const Step& last = m->steps[layers_of[k] - 1];
+        ChainPlan plan;
+        ops[k].store_bf16 = last.out_bf16;
+        if (!chain_plan(ops, k + 1, images, &plan)) break;
+        ops[k].store_bf16 = 0;
+        m->chain_elems = plan.args.cluster_elems;
+        if (plan.ns + separate - done < best) {
+            best = plan.ns + separate - done;
+            plan.args.in_elems = m->in_elems / images;
+            plan.args.out_elems = last.out_elems / images;
+            m->chain = plan;
+            len = layers_of[k];
+        }
+    }
+    if (!len) return 0;
+    for (int k = 0; k < n_ops; ++k) m->chain_layer[k] = layers_of[k] - 1;
+    float* packed = nullptr;
+    const size_t elems = (size_t)(std::min<int64_t>(owner->in_dims[0], m->ctx->sm_count) * m->chain_elems);
+    bool ok = dev_alloc(owner, (size_t)chain_packed_floats(m->chain), &packed) == TFJSB_OK &&
+              chain_pack(&m->chain, packed, 0, &m->ctx->launches) == cudaSuccess;
+    if (ok && !owner->chain_workspace)
+        ok = dev_alloc(owner, elems, &owner->chain_workspace) == TFJSB_OK && cudaMemsetAsync(owner->chain_workspace, 0, elems * 4, 0) == cudaSuccess;
+    if (!ok || cudaDeviceSynchronize() != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;  // the layers' own kernels need no memory
+    }
+    m->chain.args.workspace = owner->chain_workspace;
+    m->chain.args.cluster_elems = m->chain_elems;  // the same for every length: the borders of zeros stay where they are
+    return len;
+}
+
+void choose_fusion(tfjsb_model* m, tfjsb_model* owner) {
     for (Step& st : m->steps) st.fuse_next = st.fusable && (m->fusion_mode == 2 || (m->fusion_mode == 1 && fusion_pays(m, st)));
+    m->chain_len = 0;
+    if (m->fusion_mode != 1 || !m->chain_allowed) return;
+    if (!m->chain_chosen) {
+        m->chain_chosen = true;
+        m->chain_best = plan_chain(m, owner);
+    }
+    m->chain_len = m->chain_best;
+    for (int i = 0; i < m->chain_len; ++i) m->steps[i].fuse_next = false;
 }
 
 // A view of `parent` for a batch of `n` images: steps copied with every batch-proportional size scaled.
@@ -299,7 +438,8 @@ tfjsb_model* make_batch_view(tfjsb_model* parent, int64_t n) {
         st.out = nullptr;
     }
     v->fusion_mode = parent->fusion_mode;
-    choose_fusion(v);  // by the view's own batch
+    v->chain_allowed = parent->chain_allowed;
+    choose_fusion(v, parent);  // by the view's own batch
     return v;
 }
 
@@ -350,6 +490,10 @@ struct PdlScope {
 cudaError_t launch_layers(tfjsb_model* m, int i, cudaStream_t s, int* consumed) {
     const Step& st = m->steps[i];
     PdlScope pdl(m->use_pdl);
+    if (i == 0 && m->chain_len && !m->keep_all) {
+        *consumed = m->chain_len;
+        return launch_chain(m->chain, st.in, m->steps[m->chain_len - 1].out, m->ctx->dev_status, s, &m->ctx->launches);
+    }
     if (st.fuse_next && !m->keep_all) {
         const Step& pw = m->steps[i + 1];
         *consumed = 2;
@@ -364,6 +508,7 @@ int launches_per_run(const tfjsb_model* m) {
     int n = (int)m->steps.size();
     if (!m->keep_all)
         for (const Step& st : m->steps) n -= st.fuse_next ? 1 : 0;
+    if (!m->keep_all && m->chain_len) n -= m->chain_len - 1;
     return n;
 }
 
@@ -650,7 +795,8 @@ tfjsb_status tfjsb_model_create(tfjsb_ctx* ctx, const tfjsb_layer_desc* layers, 
             }
         }
     }
-    choose_fusion(m);
+    m->chain_allowed = (m->use_tf32 || m->narrow) && !getenv("TFJSB_NO_FUSION");
+    choose_fusion(m, m);
     if ((st = dev_alloc(m, 2 * m->region_elems, &m->arena)) != TFJSB_OK) return bail(st, ctx->last_error);
     cudaError_t e = cudaDeviceSynchronize();  // weight transposes done
     if (e != cudaSuccess) return bail(TFJSB_ERR_CUDA, std::string("model set-up: ") + cudaGetErrorString(e));
@@ -716,10 +862,10 @@ tfjsb_status tfjsb_model_set_fusion(tfjsb_model* m, int mode) {
     if (!m) return TFJSB_ERR_INVALID_ARG;
     if (mode < 0 || mode > 2) return fail(m->ctx, TFJSB_ERR_INVALID_ARG, "fusion mode must be 0 (off), 1 (auto) or 2 (always)");
     m->fusion_mode = mode;
-    choose_fusion(m);
+    choose_fusion(m, m);
     for (tfjsb_model* v : m->slices) {
         v->fusion_mode = mode;
-        choose_fusion(v);
+        choose_fusion(v, m);
         v->bound_in = nullptr; v->bound_out = nullptr;
         drop_graph(v);
     }
@@ -878,6 +1024,18 @@ tfjsb_status tfjsb_model_set_keep_all(tfjsb_model* m, int keep_all) {
         if (st != TFJSB_OK) return st;
     }
     m->keep_all = keep_all != 0;
+    if (keep_all) {
+        // From here on every layer has its own kernel in every run: what the debug mode shows is, bit for bit, what a run
+        // without it computes.  (A chain's products are added in another order.)
+        m->chain_allowed = false;
+        choose_fusion(m, m);
+        for (tfjsb_model* v : m->slices) {
+            v->chain_allowed = false;
+            choose_fusion(v, m);
+            v->bound_in = nullptr; v->bound_out = nullptr;
+            drop_graph(v);
+        }
+    }
     drop_graph(m);
     m->bound_in = nullptr;  // force a re-bind on the next run
     m->bound_out = nullptr;
@@ -904,7 +1062,8 @@ tfjsb_status tfjsb_model_layer_kernel(tfjsb_model* m, int layer, char* name, int
     if (!st.out) return fail(m->ctx, TFJSB_ERR_INVALID_ARG, "the model has not run yet");
     const bool fused_mode = !m->keep_all;
     const char* k = "?";
-    if (fused_mode && layer > 0 && m->steps[layer - 1].fuse_next) k = "(in the previous layer's kernel)";
+    if (fused_mode && layer < m->chain_len) k = layer ? "(in the previous layer's kernel)" : "chain_kernel";
+    else if (fused_mode && layer > 0 && m->steps[layer - 1].fuse_next) k = "(in the previous layer's kernel)";
     else if (fused_mode && st.fuse_next) k = "dwpw_fused_kernel<false>";
     else switch (st.kind) {
         case STEP_GEMM_TF32:

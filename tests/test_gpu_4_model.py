@@ -213,3 +213,73 @@ def test_host_runs_in_uneven_slices(ctx, oracle, batch, hw, classes):
         assert np.max(np.abs(hout.numpy() - want)) <= 2e-2 * want.max() and np.allclose(hout.numpy().sum(-1), 1, atol=1e-5)
     ctx.check_device_status()
     model.close()
+
+
+def _close_logits(got, want, rel=1e-2):
+    span = want.max(-1, keepdims=True) - want.min(-1, keepdims=True)
+    assert np.max(np.abs(got - want) / span) <= rel
+
+
+@pytest.mark.parametrize("math", ["tf32", "bf16"])
+@pytest.mark.parametrize("batch,hw,alpha,output_stride", [
+    (1, 64, 0.25, 32), (2, 65, 0.25, 32), (3, 33, 0.5, 32), (1, 96, 0.75, 32), (5, 47, 0.25, 32), (9, 64, 0.25, 32), (17, 32, 0.25, 32), (20, 50, 0.25, 32),
+    (38, 32, 0.25, 32), (60, 32, 0.25, 32), (100, 32, 0.25, 32), (2, 81, 0.25, 16), (1, 81, 0.25, 8), (40, 33, 0.25, 8)])
+def test_layers_of_a_small_model_in_one_kernel(ctx, oracle, batch, hw, alpha, output_stride, math):
+    """Clusters of 16 blocks down to a few, several images per cluster, odd widths, dilated layers: the layers in one
+    kernel against the layers' own kernels (both at the whole-model bar from the oracle; a bfloat16 value at a rounding
+    boundary may go either way, 2^-8 of it, in a layer of hundreds), and the first images against the oracle."""
+    if output_stride == 32:
+        x, layers = si.config_mobilenet(alpha, hw, batch, seed=4243, classes=100)
+    else:
+        if math == "bf16":
+            pytest.skip("no dilation in the bfloat16 storage mode")
+        x, layers = si.config_mobilenet_atrous(alpha, hw, batch, output_stride, seed=4243, classes=100)
+    ctx.set_math(math)
+    try:
+        model = ctx.model(layers, x.shape)
+    finally:
+        ctx.set_math("tf32")
+    xd, n = dev(x), len(layers)
+    probs = [host(model.run(xd)) for _ in range(2)]
+    one_kernel = model.layer_kernels()
+    logits, pooled = host(model.layer_output(n - 2)), host(model.layer_output_f32(n - 3))
+    model.set_graph(True)
+    probs.append(host(model.run(xd)))
+    model.set_graph(False)
+    ctx.check_device_status()
+    assert all(same_bits(p, probs[0]) for p in probs)
+    assert np.allclose(probs[0].sum(-1), 1, atol=1e-5)
+    if (alpha, hw) != (0.75, 96):
+        assert one_kernel[0] == "chain_kernel", one_kernel[0]
+    model.set_fusion("off")
+    model.run(xd)
+    assert "chain_kernel" not in model.layer_kernels()
+    _close_logits(logits, host(model.layer_output(n - 2)))
+    own = host(model.layer_output_f32(n - 3))
+    assert rel_fro(pooled, own) <= 1e-2
+    if math == "tf32":
+        few = min(batch, 3)
+        _close_logits(logits[:few], oracle.run_model(layers, x[:few], keep_all=True)[-2])
+    model.close()
+
+
+@pytest.mark.parametrize("batch", [1, 6])
+def test_layers_in_one_kernel_without_bias_or_padding(ctx, oracle, batch):
+    layers = si.mobilenet_v1_layers(0.25, 32)
+    si.make_model_weights(layers, 3, 77)
+    for i, layer in enumerate(layers):
+        if i < 12 and layer.kind in ("conv2d", "depthwise_conv2d"):
+            layer.pad = "valid"
+        if i % 3 == 0 and layer.kind in ("conv2d", "depthwise_conv2d", "dense"):
+            layer.bias = None
+        if i % 5 == 1 and layer.kind in ("conv2d", "depthwise_conv2d"):
+            layer.act = "none" if i % 2 else "relu"
+    x = si.uniform(78, 0, (batch, 101, 79, 3), -1, 1)
+    want = oracle.run_model(layers, x, keep_all=True)
+    model = ctx.model(layers, x.shape)
+    probs = host(model.run(dev(x)))
+    assert model.layer_kernels()[0] == "chain_kernel"
+    _close_logits(host(model.layer_output(len(layers) - 2)), want[-2])
+    assert np.max(np.abs(probs - want[-1])) <= 2e-2 * want[-1].max()
+    ctx.check_device_status()
+    model.close()
