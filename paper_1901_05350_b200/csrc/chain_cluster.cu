@@ -809,13 +809,12 @@ bool chain_block_supported(const ConvGeom& g, int64_t N) {
            (int64_t)g.H * g.W * g.C <= 0x3fffffff && (int64_t)g.Ho * g.Wo * N <= 0x3fffffff;
 }
 
-// The cluster size, the tiles of every step and an estimate of the time, for `images` images.
-bool chain_plan(const ChainOp* ops, int n_ops, int64_t images, ChainPlan* plan) {
-    if (n_ops < 1 || n_ops > CHAIN_MAX_OPS || images < 1) return false;
+int chain_plan(const ChainOp* ops, int n_ops, int64_t images, const double* rest, double separate, ChainPlan* plan) {
+    if (n_ops < 1 || n_ops > CHAIN_MAX_OPS || images < 1) return 0;
     if (smem_attr_once(reinterpret_cast<const void*>(chain_kernel), SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         (void)cudaGetLastError();
-        return false;
+        return 0;
     }
     // every layer's output has a buffer of its own, with the zeros around it that the next layer's windows reach into
     ChainOp laid[CHAIN_MAX_OPS];
@@ -833,37 +832,41 @@ bool chain_plan(const ChainOp* ops, int n_ops, int64_t images, ChainPlan* plan) 
             o.out_row = cols * o.Co;
             o.out_origin = next.pt * o.out_row + next.pl * o.Co;
             size = (int64_t)rows * o.out_row;
-            if (size > 0x7fffffff) return false;
+            if (size > 0x7fffffff) return 0;
         }
         if (i && o.kind == CHAIN_BLOCK) o.in_row = laid[i - 1].out_row;
         if (i + 1 < n_ops) elems += (size + 63) / 64 * 64;
     }
-    double best = 1e30;
+    double best = separate;
+    int used = 0;
     for (int cs = 16; cs >= 1; cs /= 2) {
         const int fit = max_clusters(cs);
         if (fit < 1) continue;
         // the clocks above are those of the arithmetic and the copies; measured, a step takes about twice as long (its
         // instructions are fetched and run once: 1.9 to 2.1 for clusters of 16 and 8, up to 2.4 for smaller ones)
         const double slower = cs >= 8 ? 2.1 : 2.4;
-        ChainArgs args{};
-        double clocks = 0;
-        for (int i = 0; i < n_ops; ++i) {
-            args.ops[i] = laid[i];
-            clocks += tune_op(args.ops[i], cs) + (cs > 1 ? 700 : 100);
-        }
         const int64_t clusters = std::min<int64_t>(fit, images), rounds = (images + clusters - 1) / clusters;
-        if (clocks * rounds * slower < best) {
-            best = clocks * rounds * slower;
-            args.n_ops = n_ops;
-            args.cluster_size = cs;
-            args.images = images;
-            args.cluster_elems = elems;
-            plan->args = args;
-            plan->blocks = (int)clusters * cs;
-            plan->ns = best / 1.9;
+        double ns = 0;
+        int ends = 0;
+        ChainOp tuned[CHAIN_MAX_OPS];
+        for (int i = 0; i < n_ops && ns < best; ++i) {
+            tuned[i] = laid[i];
+            ns += (tune_op(tuned[i], cs) + (cs > 1 ? 700 : 100)) * rounds * slower / 1.9;
+            if (rest[i] < 0 || ns + rest[i] >= best) continue;
+            best = ns + rest[i];
+            ends = i + 1;
         }
+        if (!ends) continue;
+        used = ends;
+        ChainArgs& args = plan->args;
+        std::copy(tuned, tuned + ends, args.ops);
+        args.n_ops = ends;
+        args.cluster_size = cs;
+        args.images = images;
+        args.cluster_elems = elems;  // the same for every length: the borders of zeros stay where they are
+        plan->blocks = (int)clusters * cs;
     }
-    return best < 1e30;
+    return used;
 }
 
 static int64_t packed_floats(const ChainOp& o) {

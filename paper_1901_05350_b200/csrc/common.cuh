@@ -433,12 +433,13 @@ struct ChainArgs {
 struct ChainPlan {
     ChainArgs args;
     int blocks = 0;
-    double ns = 0;  // estimate
 };
 bool chain_stem_supported(const ConvGeom& g);
 bool chain_block_supported(const ConvGeom& dw, int64_t Cout);
-// Fills in everything but the pointers and the element counts; false where no cluster of this kernel fits.
-bool chain_plan(const ChainOp* ops, int n_ops, int64_t images, ChainPlan* plan);
+// Plans the first operations as one kernel where that is estimated to be faster than `separate` ns: rest[k] is what the
+// layers after operation k take as their own kernels, negative where the kernel cannot end there.  Fills in everything but
+// the pointers and the element counts; returns the number of operations, 0 for none.
+int chain_plan(const ChainOp* ops, int n_ops, int64_t images, const double* rest, double separate, ChainPlan* plan);
 // The blocks' filters in the plan's layout, `dst` of chain_packed_floats; the plan then refers to them.
 int64_t chain_packed_floats(const ChainPlan& plan);
 cudaError_t chain_pack(ChainPlan* plan, float* dst, cudaStream_t s, int64_t* launches);

@@ -364,25 +364,28 @@ int plan_chain(tfjsb_model* m, tfjsb_model* owner) {
     int layers_of[CHAIN_MAX_OPS] = {}, len = 0;
     const int n_ops = chain_ops(m, ops, layers_of);
     const int64_t images = m->in_dims[0];
-    double separate = 0, done = 0;
+    if (!n_ops) return 0;
+    for (const tfjsb_model* v : owner->slices)
+        if (v->chain_chosen && v->in_dims[0] == images) {  // a slice of the same batch: the same plan, filters and workspace
+            m->chain = v->chain;
+            m->chain_elems = v->chain_elems;
+            std::copy(v->chain_layer, v->chain_layer + CHAIN_MAX_OPS, m->chain_layer);
+            return v->chain_best;
+        }
+    double separate = 0, done = 0, rest[CHAIN_MAX_OPS];
     for (const Step& st : m->steps) separate += separate_ns(m, st);
-    double best = separate;
     for (int k = 0, i = 0; k < n_ops; ++k) {
         for (; i < layers_of[k]; ++i) done += separate_ns(m, m->steps[i]);
-        if (ops[k].kind < CHAIN_POOL) continue;
-        const Step& last = m->steps[layers_of[k] - 1];
-        ChainPlan plan;
-        ops[k].store_bf16 = last.out_bf16;
-        if (!chain_plan(ops, k + 1, images, &plan)) break;
-        ops[k].store_bf16 = 0;
-        m->chain_elems = plan.args.cluster_elems;
-        if (plan.ns + separate - done < best) {
-            best = plan.ns + separate - done;
-            plan.args.in_elems = m->in_elems / images;
-            plan.args.out_elems = last.out_elems / images;
-            m->chain = plan;
-            len = layers_of[k];
-        }
+        rest[k] = ops[k].kind < CHAIN_POOL ? -1 : separate - done;
+    }
+    const int used = chain_plan(ops, n_ops, images, rest, separate, &m->chain);
+    if (used) {
+        len = layers_of[used - 1];
+        const Step& last = m->steps[len - 1];
+        m->chain.args.ops[used - 1].store_bf16 = last.out_bf16;
+        m->chain.args.in_elems = m->in_elems / images;
+        m->chain.args.out_elems = last.out_elems / images;
+        m->chain_elems = m->chain.args.cluster_elems;
     }
     if (!len) return 0;
     for (int k = 0; k < n_ops; ++k) m->chain_layer[k] = layers_of[k] - 1;
@@ -397,7 +400,6 @@ int plan_chain(tfjsb_model* m, tfjsb_model* owner) {
         return 0;  // the layers' own kernels need no memory
     }
     m->chain.args.workspace = owner->chain_workspace;
-    m->chain.args.cluster_elems = m->chain_elems;  // the same for every length: the borders of zeros stay where they are
     return len;
 }
 
