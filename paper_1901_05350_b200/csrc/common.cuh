@@ -55,6 +55,21 @@ __device__ __forceinline__ void fma2(float2& acc, const float2& a, const float2&
         : "+l"(d)
         : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
 }
+__device__ __forceinline__ float2 add2(const float2& a, const float2& b) {
+    float2 r;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long&>(r))
+        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+    return r;
+}
+// relu / relu6 of two bfloat16: their bounds are bfloat16 values and rounding is monotonic, so this after the rounding is the
+// rounded activation, in half the instructions.
+template <int ACT>
+__device__ __forceinline__ uint32_t apply_act_bf16x2(uint32_t v) {
+    if (ACT == TFJSB_ACT_RELU || ACT == TFJSB_ACT_RELU6) asm("max.NaN.bf16x2 %0, %0, %1;" : "+r"(v) : "r"(0u));
+    if (ACT == TFJSB_ACT_RELU6) asm("min.NaN.bf16x2 %0, %0, %1;" : "+r"(v) : "r"(0x40c040c0u));
+    return v;
+}
 __device__ __forceinline__ void fma4_packed(float4& acc, const float4& a, const float4& b) {
     fma2(reinterpret_cast<float2*>(&acc)[0], reinterpret_cast<const float2*>(&a)[0], reinterpret_cast<const float2*>(&b)[0]);
     fma2(reinterpret_cast<float2*>(&acc)[1], reinterpret_cast<const float2*>(&a)[1], reinterpret_cast<const float2*>(&b)[1]);

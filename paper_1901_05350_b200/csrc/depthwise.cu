@@ -147,15 +147,17 @@ __device__ __forceinline__ void store_rows(const float4 (&acc)[R], const float4 
     for (int r = 0; r < R; ++r) {
         if (r < rows) {
             float4 v = acc[r];
-            v.x = apply_act_t<ACT>(v.x + b.x); v.y = apply_act_t<ACT>(v.y + b.y);
-            v.z = apply_act_t<ACT>(v.z + b.z); v.w = apply_act_t<ACT>(v.w + b.w);
+            reinterpret_cast<float2*>(&v)[0] = add2(reinterpret_cast<const float2*>(&v)[0], reinterpret_cast<const float2*>(&b)[0]);
+            reinterpret_cast<float2*>(&v)[1] = add2(reinterpret_cast<const float2*>(&v)[1], reinterpret_cast<const float2*>(&b)[1]);
             if (OUT16) {
                 const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
                 uint2 o;
-                o.x = *reinterpret_cast<const uint32_t*>(&lo);
-                o.y = *reinterpret_cast<const uint32_t*>(&hi);
+                o.x = apply_act_bf16x2<ACT>(*reinterpret_cast<const uint32_t*>(&lo));
+                o.y = apply_act_bf16x2<ACT>(*reinterpret_cast<const uint32_t*>(&hi));
                 *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(y) + idx) = o;
             } else {
+                v.x = apply_act_t<ACT>(v.x); v.y = apply_act_t<ACT>(v.y);
+                v.z = apply_act_t<ACT>(v.z); v.w = apply_act_t<ACT>(v.w);
                 *reinterpret_cast<float4*>(static_cast<float*>(y) + idx) = v;
             }
         }
@@ -260,7 +262,8 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
                 const int tile = first + i * step;
                 const int cb = tile % t.c_blocks;
                 int q = tile / t.c_blocks;
-                const int tx = q % t.tiles_x; q /= t.tiles_x;
+                int tx = q % t.tiles_x; q /= t.tiles_x;
+                tx = (tx + q) % t.tiles_x;  // the grid is often a multiple of c_blocks x tiles_x: not always the narrow last column
                 const int ty = q % t.tiles_y;
                 const int n = q / t.tiles_y;
                 tile_info[slot] = make_int4(cb, tx, ty, n);
