@@ -55,6 +55,16 @@ __device__ __forceinline__ void fma2(float2& acc, const float2& a, const float2&
         : "+l"(d)
         : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
 }
+// acc.{x,y,z,w} += a * b of four bfloat16 each, as they lie in memory: exact products, one rounding, as fmaf of the widened
+// values, without widening them.
+__device__ __forceinline__ void fma4_bf16(float4& acc, const uint2& a, const uint2& b) {
+    asm("{\n\t.reg .b16 a0, a1, a2, a3, b0, b1, b2, b3;\n\t"
+        "mov.b32 {a0, a1}, %4;\n\tmov.b32 {a2, a3}, %5;\n\tmov.b32 {b0, b1}, %6;\n\tmov.b32 {b2, b3}, %7;\n\t"
+        "fma.rn.f32.bf16 %0, a0, b0, %0;\n\tfma.rn.f32.bf16 %1, a1, b1, %1;\n\t"
+        "fma.rn.f32.bf16 %2, a2, b2, %2;\n\tfma.rn.f32.bf16 %3, a3, b3, %3;\n\t}"
+        : "+f"(acc.x), "+f"(acc.y), "+f"(acc.z), "+f"(acc.w)
+        : "r"(a.x), "r"(a.y), "r"(b.x), "r"(b.y));
+}
 __device__ __forceinline__ float2 add2(const float2& a, const float2& b) {
     float2 r;
     asm("add.rn.f32x2 %0, %1, %2;"

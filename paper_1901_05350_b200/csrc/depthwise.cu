@@ -174,16 +174,16 @@ __device__ __forceinline__ void store_rows_act(int act, const float4 (&acc)[R], 
     else store_rows<TFJSB_ACT_NONE, R, OUT16>(acc, b, y, idx, row_pitch, rows);
 }
 
-// Four consecutive channels of one patch sample as fp32: one 16-byte load, or one 8-byte load of four
-// bfloat16 (each is the upper half of its fp32).
-template <bool NARROW>
-__device__ __forceinline__ float4 ld_quad(const uint8_t* p) {
-    if (NARROW) {
-        const uint2 raw = *reinterpret_cast<const uint2*>(p);
-        return make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
-                           __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
-    }
-    return *reinterpret_cast<const float4*>(p);
+// Four consecutive channels of one patch sample, or of a filter tap: as stored, fp32 or (narrow) bfloat16.
+template <bool NARROW> struct DwQuad { typedef float4 type; };
+template <> struct DwQuad<true> { typedef uint2 type; };
+__device__ __forceinline__ void dw_fma(float4& acc, const float4& x, const float4& w) { fma4_packed(acc, x, w); }
+__device__ __forceinline__ void dw_fma(float4& acc, const uint2& x, const uint2& w) { fma4_bf16(acc, x, w); }
+__device__ __forceinline__ void dw_tap(float4& w, const float4& v) { w = v; }
+__device__ __forceinline__ void dw_tap(uint2& w, const float4& v) {  // exact: a narrow model's filter holds bfloat16 values
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+    w.x = *reinterpret_cast<const uint32_t*>(&lo);
+    w.y = *reinterpret_cast<const uint32_t*>(&hi);
 }
 
 // ---- pipelined kernel ---------------------------------------------------------------------------
@@ -210,8 +210,8 @@ struct DwTile {
 
 constexpr int DW_TMA_THREADS = DW_THREADS + 32;  // eight compute warps and the warp that issues the copies
 
-// NARROW: the input is bfloat16 (the patch is copied as such and widened by the compute threads; filter and bias
-// stay fp32, the sums are fp32 in the same order) and the output is bfloat16 or, with y_f32, fp32.
+// NARROW: the input is bfloat16 (the patch is copied as such and multiplied as such, with the filter, whose
+// values a narrow model has rounded to bfloat16; bias and sums are fp32, in the same order) and the output is bfloat16 or, with y_f32, fp32.
 template <int S, int TW, int R, int D = 1, int CB = DW_CB, bool NARROW = false>
 __global__ void __launch_bounds__(DW_TMA_THREADS, 2)
 depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* __restrict__ f,
@@ -300,7 +300,8 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
     const int rg = tid / (T::QUADS * TW);
     const int64_t row_pitch = (int64_t)g.Wo * g.Co;
 
-    float4 w[9];
+    typedef typename DwQuad<NARROW>::type Quad;
+    Quad w[9];
     float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
     int loaded_cb = -1;
     int slot = 0;
@@ -322,7 +323,7 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
             if (cb != loaded_cb) {
 #pragma unroll
                 for (int k = 0; k < 9; ++k)
-                    w[k] = __ldg(reinterpret_cast<const float4*>(f + (int64_t)k * t.f_step + c));
+                    dw_tap(w[k], __ldg(reinterpret_cast<const float4*>(f + (int64_t)k * t.f_step + c)));
                 if (bias) b = __ldg(reinterpret_cast<const float4*>(bias + c));
                 loaded_cb = cb;
             }
@@ -336,15 +337,15 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
 #pragma unroll
             for (int j = 0; j < IN_ROWS; ++j) {
                 const uint8_t* row = patch + j * T::TWIN * CB * T::EB;
-                const float4 v0 = ld_quad<NARROW>(row), v1 = ld_quad<NARROW>(row + D * CB * T::EB),
-                             v2 = ld_quad<NARROW>(row + 2 * D * CB * T::EB);
+                const Quad v0 = *reinterpret_cast<const Quad*>(row), v1 = *reinterpret_cast<const Quad*>(row + D * CB * T::EB),
+                           v2 = *reinterpret_cast<const Quad*>(row + 2 * D * CB * T::EB);
 #pragma unroll
                 for (int ky = 0; ky < 3; ++ky) {
                     const int d = j - ky * D;
                     if (d >= 0 && d % S == 0 && d / S < R) {
-                        fma4_packed(acc[d / S], v0, w[ky * 3 + 0]);
-                        fma4_packed(acc[d / S], v1, w[ky * 3 + 1]);
-                        fma4_packed(acc[d / S], v2, w[ky * 3 + 2]);
+                        dw_fma(acc[d / S], v0, w[ky * 3 + 0]);
+                        dw_fma(acc[d / S], v1, w[ky * 3 + 1]);
+                        dw_fma(acc[d / S], v2, w[ky * 3 + 2]);
                     }
                 }
             }
