@@ -779,7 +779,13 @@ double tune_op(ChainOp& o, int cs) {
     }
 }
 
+// How many clusters of `cs` blocks run at once; 0 where none can.
 int max_clusters(int cs) {
+    if (smem_attr_once(reinterpret_cast<const void*>(chain_kernel), SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cs);
     cfg.blockDim = dim3(THREADS + 32);
@@ -811,11 +817,6 @@ bool chain_block_supported(const ConvGeom& g, int64_t N) {
 
 int chain_plan(const ChainOp* ops, int n_ops, int64_t images, const double* rest, double separate, ChainPlan* plan) {
     if (n_ops < 1 || n_ops > CHAIN_MAX_OPS || images < 1) return 0;
-    if (smem_attr_once(reinterpret_cast<const void*>(chain_kernel), SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return 0;
-    }
     // every layer's output has a buffer of its own, with the zeros around it that the next layer's windows reach into
     ChainOp laid[CHAIN_MAX_OPS];
     int64_t elems = 0;
@@ -840,31 +841,36 @@ int chain_plan(const ChainOp* ops, int n_ops, int64_t images, const double* rest
     double best = separate;
     int used = 0;
     for (int cs = 16; cs >= 1; cs /= 2) {
-        const int fit = max_clusters(cs);
-        if (fit < 1) continue;
         // the clocks above are those of the arithmetic and the copies; measured, a step takes about twice as long (its
         // instructions are fetched and run once: 1.9 to 2.1 for clusters of 16 and 8, up to 2.4 for smaller ones)
         const double slower = cs >= 8 ? 2.1 : 2.4;
-        const int64_t clusters = std::min<int64_t>(fit, images), rounds = (images + clusters - 1) / clusters;
-        double ns = 0;
-        int ends = 0;
         ChainOp tuned[CHAIN_MAX_OPS];
-        for (int i = 0; i < n_ops && ns < best; ++i) {
-            tuned[i] = laid[i];
-            ns += (tune_op(tuned[i], cs) + (cs > 1 ? 700 : 100)) * rounds * slower / 1.9;
-            if (rest[i] < 0 || ns + rest[i] >= best) continue;
-            best = ns + rest[i];
-            ends = i + 1;
+        // first as if every SM were in a cluster, then, if that would win, with the clusters that there is room for
+        int fit = current_sm_count() / cs;
+        for (int pass = 0; pass < 2; ++pass) {
+            if (pass && (fit = max_clusters(cs)) < 1) break;
+            const int64_t clusters = std::min<int64_t>(fit, images), rounds = (images + clusters - 1) / clusters;
+            double ns = 0, least = best;
+            int ends = 0;
+            for (int i = 0; i < n_ops && ns < least; ++i) {
+                tuned[i] = laid[i];
+                ns += (tune_op(tuned[i], cs) + (cs > 1 ? 700 : 100)) * rounds * slower / 1.9;
+                if (rest[i] < 0 || ns + rest[i] >= least) continue;
+                least = ns + rest[i];
+                ends = i + 1;
+            }
+            if (!ends) break;
+            if (!pass) continue;
+            best = least;
+            used = ends;
+            ChainArgs& args = plan->args;
+            std::copy(tuned, tuned + ends, args.ops);
+            args.n_ops = ends;
+            args.cluster_size = cs;
+            args.images = images;
+            args.cluster_elems = elems;  // the same for every length: the borders of zeros stay where they are
+            plan->blocks = (int)clusters * cs;
         }
-        if (!ends) continue;
-        used = ends;
-        ChainArgs& args = plan->args;
-        std::copy(tuned, tuned + ends, args.ops);
-        args.n_ops = ends;
-        args.cluster_size = cs;
-        args.images = images;
-        args.cluster_elems = elems;  // the same for every length: the borders of zeros stay where they are
-        plan->blocks = (int)clusters * cs;
     }
     return used;
 }
