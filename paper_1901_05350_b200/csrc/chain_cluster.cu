@@ -31,6 +31,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "chain_copy.cuh"
 #include "common.cuh"
 #include "ptx_sm100.cuh"
 
@@ -86,7 +87,7 @@ __device__ __forceinline__ float bounded(float v, float lo, float hi) {
 // n / d from ceil(2^32 / d): exact while n d < 2^32
 __device__ __forceinline__ int div_by(int n, unsigned int magic) { return magic ? (int)__umulhi((unsigned)n, magic) : n; }
 
-// Waits of the pipeline; after the limit the kernel notes it, goes on without waiting and ends.
+// Waits of the computing warps; after the limit the kernel notes it, goes on without waiting and ends.
 struct Waiter {
     unsigned int* dev_status;
     bool off;
@@ -102,68 +103,42 @@ struct Waiter {
     }
 };
 
-__device__ __forceinline__ int column_tiles(const ChainOp& o, int group) {
-    int cols = min(o.group_cols, o.Co - group * o.group_cols), n = 0;
-    for (; cols > 0; cols -= o.tile_cols) ++n;
-    return n;
-}
-
-// The copying warp: every chunk of pointwise filter this block will need, in order, two ahead.  It takes part in the
-// cluster's barriers, but no later than its next wait needs: a chunk of the next layer is on its way before the barrier.
-__device__ __forceinline__ void copy_filters(const ChainOp* ops, int n_ops, int rank, int cs, int images, uint32_t w_sm, uint32_t f_sm,
-                                             uint32_t bars, Waiter& waiter) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t full = bars, empty = bars + 16, f_full = bars + 32, f_empty = bars + 40;
-    int chunk = 0, met = 0, before = 0, last = 0;  // chunks so far, barriers taken part in, layers of the two chunks before
-    int blocks = 0, f_before = 0;                  // depthwise filters so far, layer of the last
-    for (int img = 0; img < images; ++img)
-        for (int i = 0; i < n_ops; ++i) {
-            const ChainOp& o = ops[i];
-            if (o.kind != CHAIN_BLOCK || rank >= o.units) continue;
-            if (blocks) {
-                if (cs > 1)
-                    for (; met < f_before; ++met) cluster_sync();
-                waiter.wait(f_empty, (blocks - 1) & 1);
-            }
-            f_before = img * n_ops + i;
-            ++blocks;
-            if (lane == 0) {
-                ptx::mbar_arrive_expect_tx(f_full, 10 * o.C * 4);
-                bulk_copy(f_sm, o.f1, 10 * o.C * 4, f_full);
-            }
-            const int tile_floats = o.n_chunks * o.chunk_floats;
-            for (int u = rank; u < o.units; u += cs) {
-                const int group = u - div_by(u, o.by_groups) * o.groups;
-                const int chunks = o.n_chunks * column_tiles(o, group);
-                const float* src = o.f2 + (int64_t)group * o.group_tiles * tile_floats;
-                for (int k = 0; k < chunks; ++k, ++chunk, src += o.chunk_floats) {
-                    const int buf = chunk & 1;
-                    if (chunk >= 2) {
-                        // the buffer's last chunk is of layer `before`: its readers need the barriers up to that layer
-                        if (cs > 1)
-                            for (; met < before; ++met) cluster_sync();
-                        waiter.wait(empty + 8 * buf, ((chunk >> 1) - 1) & 1);
-                    }
-                    before = last;
-                    last = img * n_ops + i;
-                    if (lane == 0) {
-                        ptx::mbar_arrive_expect_tx(full + 8 * buf, o.chunk_floats * 4);
-                        bulk_copy(w_sm + (uint32_t)buf * W_FLOATS * 4, src, o.chunk_floats * 4, full + 8 * buf);
-                    }
-                }
-            }
+// The copying warp's side of chain_copy_filters.
+struct CopyPort {
+    unsigned int* dev_status;
+    uint32_t bars, w_sm, f_sm;
+    int rank;
+    __device__ __forceinline__ bool wants(const ChainOp& o) const { return o.kind == CHAIN_BLOCK && rank < o.units; }
+    __device__ __forceinline__ int group(const ChainOp& o, int u) const { return u - div_by(u, o.by_groups) * o.groups; }
+    __device__ __forceinline__ bool wait(int bar, uint32_t parity) const {
+        Waiter w{dev_status, false};  // of this one wait: one that gave up says nothing about the next
+        w.wait(bars + 8 * bar, parity);
+        return __all_sync(0xffffffffu, !w.off);
+    }
+    __device__ __forceinline__ void copy_filter(const ChainOp& o) const {
+        if ((threadIdx.x & 31) == 0) {
+            ptx::mbar_arrive_expect_tx(bars + 8 * CHAIN_F_FULL, 10 * o.C * 4);
+            bulk_copy(f_sm, o.f1, 10 * o.C * 4, bars + 8 * CHAIN_F_FULL);
         }
-    // none of the copies is in flight when the block ends
-    for (int c = max(0, chunk - 2); c < chunk; ++c) waiter.wait(full + 8 * (c & 1), (c >> 1) & 1);
-    if (blocks) waiter.wait(f_full, (blocks - 1) & 1);
-    if (cs > 1)
-        for (; met < images * n_ops; ++met) cluster_sync();
-}
+    }
+    __device__ __forceinline__ void copy_chunk(const ChainOp& o, int64_t from, int buf) const {
+        if ((threadIdx.x & 31) == 0) {
+            ptx::mbar_arrive_expect_tx(bars + 8 * (CHAIN_FULL0 + buf), o.chunk_floats * 4);
+            bulk_copy(w_sm + (uint32_t)buf * W_FLOATS * 4, o.f2 + from, o.chunk_floats * 4, bars + 8 * (CHAIN_FULL0 + buf));
+        }
+    }
+    __device__ __forceinline__ void meet() const { cluster_sync(); }
+};
 
 struct Pipeline {
     Waiter waiter;
     int chunk;  // the chunk that is waited for next
     uint32_t full, empty;
+    // This warp has read a buffer (or the depthwise filter).  A warp that gave up waiting hands nothing back: its buffer may
+    // have a copy in flight, and the copying warp, whose wait then gives up too, must not arm that barrier again.
+    __device__ __forceinline__ void hand_back(uint32_t bar) const {
+        if ((threadIdx.x & 31) == 0 && !waiter.off) ptx::mbar_arrive(bar);
+    }
 };
 
 __device__ __forceinline__ void store2(const ChainOp& o, int bf16, float* out, int at, float x, float y) {
@@ -255,7 +230,7 @@ __device__ __forceinline__ void block_columns(const ChainOp& o, const BlockWork&
             }
             if (kc + 1 < n_chunks) {
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(pipe.empty + 8 * buf);
+                pipe.hand_back(pipe.empty + 8 * buf);
             }
         }
         const int buf = (pipe.chunk & 1) ^ 1;  // of the last chunk: handed back when its bias has been read
@@ -309,7 +284,7 @@ __device__ __forceinline__ void block_columns(const ChainOp& o, const BlockWork&
             }
         }
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(pipe.empty + 8 * buf);
+        pipe.hand_back(pipe.empty + 8 * buf);
     }
 }
 
@@ -570,7 +545,7 @@ __device__ __forceinline__ void meet(int cs, bool met) {
 
 __global__ void __launch_bounds__(THREADS + 32, 1) chain_kernel(const __grid_constant__ ChainArgs a) {
     extern __shared__ __align__(16) float sm[];
-    __shared__ __align__(8) unsigned long long bars[6];  // full, empty of the chunks; of the depthwise filter
+    __shared__ __align__(8) unsigned long long bars[CHAIN_BARS];
     float* d_sm = sm;
     float* f_sm = sm + D_FLOATS;
     float* w_sm = f_sm + F_FLOATS;
@@ -578,14 +553,15 @@ __global__ void __launch_bounds__(THREADS + 32, 1) chain_kernel(const __grid_con
     ChainOp* ops = reinterpret_cast<ChainOp*>(red + RED_FLOATS);  // dynamically indexed constants are slower to reach
     for (int j = threadIdx.x; j < (int)(a.n_ops * sizeof(ChainOp) / 4); j += THREADS + 32)
         reinterpret_cast<uint32_t*>(ops)[j] = reinterpret_cast<const uint32_t*>(a.ops)[j];
-    const uint32_t full = ptx::smem_u32(bars), empty = full + 16;
+    const uint32_t bar0 = ptx::smem_u32(bars), full = bar0 + 8 * CHAIN_FULL0, empty = bar0 + 8 * CHAIN_EMPTY0;
+    const uint32_t f_full = bar0 + 8 * CHAIN_F_FULL, f_empty = bar0 + 8 * CHAIN_F_EMPTY;
     if (threadIdx.x == 0) {
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(full + 8 * b, 1);
             ptx::mbar_init(empty + 8 * b, WARPS);
         }
-        ptx::mbar_init(full + 32, 1);
-        ptx::mbar_init(full + 40, WARPS);
+        ptx::mbar_init(f_full, 1);
+        ptx::mbar_init(f_empty, WARPS);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -594,8 +570,8 @@ __global__ void __launch_bounds__(THREADS + 32, 1) chain_kernel(const __grid_con
     const int images = (int)((a.images - cluster + clusters - 1) / clusters);
     ptx::pdl_launch_dependents();
     if (threadIdx.x >= THREADS) {
-        Waiter waiter{a.dev_status, false};
-        copy_filters(ops, n_ops, rank, cs, images, ptx::smem_u32(w_sm), ptx::smem_u32(f_sm), full, waiter);
+        CopyPort port{a.dev_status, bar0, ptx::smem_u32(w_sm), ptx::smem_u32(f_sm), rank};
+        chain_copy_filters(ops, n_ops, rank, cs, images, port);
         return;
     }
     Pipeline pipe{Waiter{a.dev_status, false}, 0, full, empty};
@@ -614,7 +590,7 @@ __global__ void __launch_bounds__(THREADS + 32, 1) chain_kernel(const __grid_con
             // input and shared memory are free
             if (o.kind == CHAIN_BLOCK) {
                 const BlockWork work = block_work(o, rank);
-                if (rank < o.units) pipe.waiter.wait(full + 32, blocks++ & 1);
+                if (rank < o.units) pipe.waiter.wait(f_full, blocks++ & 1);
                 meet(cs, met);
                 for (int u = rank; u < o.units; u += cs) {
                     const int p0 = div_by(u, o.by_groups) * o.pixels;
@@ -623,7 +599,7 @@ __global__ void __launch_bounds__(THREADS + 32, 1) chain_kernel(const __grid_con
                     else if (o.strip == 2) block_depthwise<2>(o, work, u == rank, f_sm, in, p0, d_sm);
                     else block_depthwise<1>(o, work, u == rank, f_sm, in, p0, d_sm);
                     block_sync();
-                    if (u + cs >= o.units && (threadIdx.x & 31) == 0) ptx::mbar_arrive(full + 40);
+                    if (u + cs >= o.units) pipe.hand_back(f_empty);
                     const int v = o.variant;  // tests, not a jump table in constant memory
                     if (v == 0) block_columns<1, 1>(o, work, u, p0, out, d_sm, w_sm, red, pipe);
                     else if (v == 1) block_columns<1, 2>(o, work, u, p0, out, d_sm, w_sm, red, pipe);
