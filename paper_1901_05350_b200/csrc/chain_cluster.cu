@@ -48,7 +48,8 @@ constexpr int SMEM_BYTES = (D_FLOATS + F_FLOATS + 2 * W_FLOATS + RED_FLOATS) * 4
 
 // The computing threads of the block.
 __device__ __forceinline__ void block_sync() { asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory"); }
-// Every thread of the cluster, the copying warps included.
+// Every thread of the cluster, the copying warps included.  The aligned forms want the warp's threads together: a warp that
+// comes out of a wait or of one thread's work executes __syncwarp() first.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
@@ -87,16 +88,18 @@ __device__ __forceinline__ float bounded(float v, float lo, float hi) {
 // n / d from ceil(2^32 / d): exact while n d < 2^32
 __device__ __forceinline__ int div_by(int n, unsigned int magic) { return magic ? (int)__umulhi((unsigned)n, magic) : n; }
 
-// Waits of the computing warps; after the limit the kernel notes it, goes on without waiting and ends.
+// Waits of a converged warp, which comes out of them converged (mma.sync, bar.sync and barrier.cluster follow); after the
+// limit the kernel notes it and the warp goes on without waiting, to the kernel's end.  Threads that spin and leave on their
+// own would leave at different times, and only some of them on giving up.
 struct Waiter {
     unsigned int* dev_status;
-    bool off;
+    bool off;  // the same in all threads of the warp
     __device__ __forceinline__ void wait(uint32_t bar, uint32_t parity) {
-        if (off || ptx::mbar_try_wait(bar, parity)) return;
+        if (off || __all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity))) return;
         const unsigned long long t0 = ptx::global_ns();
-        while (!ptx::mbar_try_wait(bar, parity))
-            if (ptx::global_ns() - t0 > ptx::WAIT_LIMIT_NS) {
-                atomicOr(dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
+        while (!__all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity)))
+            if (__any_sync(0xffffffffu, ptx::global_ns() - t0 > ptx::WAIT_LIMIT_NS)) {
+                if ((threadIdx.x & 31) == 0) atomicOr(dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
                 off = true;
                 return;
             }
@@ -113,7 +116,7 @@ struct CopyPort {
     __device__ __forceinline__ bool wait(int bar, uint32_t parity) const {
         Waiter w{dev_status, false};  // of this one wait: one that gave up says nothing about the next
         w.wait(bars + 8 * bar, parity);
-        return __all_sync(0xffffffffu, !w.off);
+        return !w.off;
     }
     __device__ __forceinline__ void copy_filter(const ChainOp& o) const {
         if ((threadIdx.x & 31) == 0) {
@@ -127,6 +130,7 @@ struct CopyPort {
             bulk_copy(w_sm + (uint32_t)buf * W_FLOATS * 4, o.f2 + from, o.chunk_floats * 4, bars + 8 * (CHAIN_FULL0 + buf));
         }
     }
+    __device__ __forceinline__ void converge() const { __syncwarp(); }
     __device__ __forceinline__ void meet() const { cluster_sync(); }
 };
 

@@ -21,13 +21,22 @@ TFJSB_CHAIN_FN int chain_chunks(const Op& o, int group) {
     return n * o.n_chunks;
 }
 
+// The cluster's barriers up to the one that ends layer `upto` - 1.
+template <class Port>
+TFJSB_CHAIN_FN void chain_meet(Port& port, int cs, int& met, int upto) {
+    if (cs == 1 || met >= upto) return;
+    port.converge();
+    for (; met < upto; ++met) port.meet();
+}
+
 // Every chunk this block will need, in order, two ahead.  The warp takes part in the cluster's barriers, but no later than
 // its next wait needs: a chunk of the next layer is on its way before the barrier.
 //   port.wants(op)            whether this block has a unit of the operation
 //   port.group(op, u)         the column group of unit u
 //   port.wait(bar, parity)    false when the wait gave up
 //   port.copy_filter(op), port.copy_chunk(op, first float of its filter, buffer)    arm the barrier and copy
-//   port.meet()               one cluster barrier
+//   port.converge()           the warp's threads together again, after a wait or a copy
+//   port.meet()               one cluster barrier, by a converged warp
 // After a wait that gave up nothing more is copied: the buffer was not handed back, and its barrier may be armed already.
 // What is in flight is waited for, once more bounded, and the barriers that the cluster counts on are still taken part in.
 template <class Op, class Port>
@@ -40,8 +49,7 @@ TFJSB_CHAIN_FN void chain_copy_filters(const Op* ops, int n_ops, int rank, int c
             const Op& o = ops[i];
             if (!port.wants(o)) continue;
             if (filters) {
-                if (cs > 1)
-                    for (; met < f_before; ++met) port.meet();
+                chain_meet(port, cs, met, f_before);
                 if (!(going = port.wait(CHAIN_F_EMPTY, (filters - 1) & 1))) break;
             }
             f_before = img * n_ops + i;
@@ -54,8 +62,7 @@ TFJSB_CHAIN_FN void chain_copy_filters(const Op* ops, int n_ops, int rank, int c
                     const int buf = chunk & 1;
                     if (chunk >= 2) {
                         // the buffer's last chunk is of layer `before`: its readers need the barriers up to that layer
-                        if (cs > 1)
-                            for (; met < before; ++met) port.meet();
+                        chain_meet(port, cs, met, before);
                         if (!(going = port.wait(CHAIN_EMPTY0 + buf, ((chunk >> 1) - 1) & 1))) break;
                     }
                     before = last;
@@ -67,8 +74,7 @@ TFJSB_CHAIN_FN void chain_copy_filters(const Op* ops, int n_ops, int rank, int c
     // none of the copies is in flight when the block ends
     for (int c = chunk > 2 ? chunk - 2 : 0; c < chunk; ++c) port.wait(CHAIN_FULL0 + (c & 1), (c >> 1) & 1);
     if (filters) port.wait(CHAIN_F_FULL, (filters - 1) & 1);
-    if (cs > 1)
-        for (; met < images * n_ops; ++met) port.meet();
+    chain_meet(port, cs, met, images * n_ops);
 }
 
 }  // namespace tfjsb

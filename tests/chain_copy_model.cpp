@@ -27,9 +27,12 @@ struct Port {
     int back[CHAIN_BARS] = {};      // phases of an "empty" barrier that a wait has seen complete
     std::vector<long long> chunks;  // first float of every chunk, in order
 
+    bool converged = true;  // a wait and a copy by one thread leave the warp's threads apart
+
     bool wants(const Op& o) const { return o.block && rank < o.units; }
     int group(const Op& o, int u) const { return u % o.groups; }
     bool wait(int bar, unsigned parity) {
+        converged = false;
         if (waits++ == fail_at) {
             gave_up = 1;
             return false;
@@ -45,6 +48,7 @@ struct Port {
         if (gave_up) wrong("a copy after a wait that gave up");
         // one phase at a time: before phase n is armed, phase n - 1 has been handed back
         if (armed[full] != back[empty]) wrong("a buffer that was not handed back");
+        converged = false;
         ++armed[full];
         ++copies;
     }
@@ -53,7 +57,11 @@ struct Port {
         arm(CHAIN_FULL0 + buf, CHAIN_EMPTY0 + buf);
         chunks.push_back(from);
     }
-    void meet() { ++meets; }
+    void converge() { converged = true; }
+    void meet() {
+        if (!converged) wrong("a cluster barrier by a warp that has not converged");
+        ++meets;
+    }
 };
 
 int main(int argc, char** argv) {
