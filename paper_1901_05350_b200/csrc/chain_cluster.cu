@@ -145,17 +145,25 @@ struct Pipeline {
     }
 };
 
+__device__ __forceinline__ void store_pair(int bf16, float* out, int at, float x, float y) {
+    if (bf16) *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(out) + at) = __floats2bfloat162_rn(x, y);
+    else *reinterpret_cast<float2*>(out + at) = make_float2(x, y);
+}
 __device__ __forceinline__ void store2(const ChainOp& o, int bf16, float* out, int at, float x, float y) {
     x = bounded(x, o.lo2, o.hi2);
     y = bounded(y, o.lo2, o.hi2);
     if (o.round2) { x = round_bf16(x); y = round_bf16(y); }
-    if (bf16) *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(out) + at) = __floats2bfloat162_rn(x, y);
-    else *reinterpret_cast<float2*>(out + at) = make_float2(x, y);
+    store_pair(bf16, out, at, x, y);
 }
 // Where pixel p of a layer's output is: rows of out_row floats, the origin inside the next layer's padding.
 __device__ __forceinline__ int out_at(const ChainOp& o, int p) {
     const int oy = div_by(p, o.by_wo);
     return o.out_origin + oy * o.out_row + (p - oy * o.Wo) * o.Co;
+}
+
+// Element `at` of a tensor that is read after the run.
+__device__ __forceinline__ float* also_at(float* base, int bf16, int64_t at) {
+    return bf16 ? reinterpret_cast<float*>(reinterpret_cast<__nv_bfloat16*>(base) + at) : base + at;
 }
 
 // What a thread does in a block's units, worked out while the cluster meets.
@@ -182,8 +190,8 @@ __device__ __forceinline__ BlockWork block_work(const ChainOp& o, int rank) {
 }
 
 // The product of a unit: D [P][C] times this unit's columns of the filter.
-template <int MT, int NT>
-__device__ __forceinline__ void block_columns(const ChainOp& o, const BlockWork& work, int u, int p0, float* out, const float* d_sm,
+template <int MT, int NT, bool KEEP>
+__device__ __forceinline__ void block_columns(const ChainOp& o, const BlockWork& work, int u, int p0, int64_t image, float* out, const float* d_sm,
                                               const float* w_sm, float* red, Pipeline& pipe) {
     const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int ldd = o.C + 4, ldw = o.w_stride, splits = o.k_splits, tile_cols = o.tile_cols, Co = o.Co;
@@ -191,6 +199,7 @@ __device__ __forceinline__ void block_columns(const ChainOp& o, const BlockWork&
     const bool active = work.active;
     const int col0 = (u - div_by(u, o.by_groups) * o.groups) * o.group_cols, col_end = min(Co, col0 + o.group_cols);
     const int M = o.Ho * o.Wo;
+    float* also = KEEP && o.also ? also_at(o.also, o.also_bf16, image * M * Co) : nullptr;
     for (int n0 = col0; n0 < col_end; n0 += tile_cols) {
         float acc[MT][NT][4];
 #pragma unroll
@@ -258,7 +267,12 @@ __device__ __forceinline__ void block_columns(const ChainOp& o, const BlockWork&
                     for (int i = 0; i < MT; ++i)
 #pragma unroll
                         for (int h = 0; h < 2; ++h)
-                            if (at[i][h] >= 0) store2(o, 0, out, at[i][h] + n0 + c, acc[i][j][2 * h] + b.x, acc[i][j][2 * h + 1] + b.y);
+                            if (at[i][h] >= 0) {
+                                store2(o, 0, out, at[i][h] + n0 + c, acc[i][j][2 * h] + b.x, acc[i][j][2 * h + 1] + b.y);
+                                if (KEEP && also)
+                                    store2(o, o.also_bf16, also, (p0 + m_base + 16 * i + 8 * h + g) * Co + n0 + c, acc[i][j][2 * h] + b.x,
+                                           acc[i][j][2 * h + 1] + b.y);
+                            }
                 }
             }
         } else {
@@ -284,7 +298,10 @@ __device__ __forceinline__ void block_columns(const ChainOp& o, const BlockWork&
                     const float2 v = *reinterpret_cast<const float2*>(red + k * plane + 2 * j);
                     s.x += v.x; s.y += v.y;
                 }
-                if (p0 + p < M && n0 + c < Co) store2(o, 0, out, out_at(o, p0 + p) + n0 + c, s.x, s.y);
+                if (p0 + p < M && n0 + c < Co) {
+                    store2(o, 0, out, out_at(o, p0 + p) + n0 + c, s.x, s.y);
+                    if (KEEP && also) store2(o, o.also_bf16, also, (p0 + p) * Co + n0 + c, s.x, s.y);
+                }
             }
         }
         __syncwarp();
@@ -294,9 +311,9 @@ __device__ __forceinline__ void block_columns(const ChainOp& o, const BlockWork&
 
 // Depthwise 3x3 of a unit's pixels, all channels, into shared memory.  The input has its padding around it, so no tap is
 // tested.  R > 1 (stride 1, no dilation, Wo a multiple of R): R neighbouring pixels share their 3 (R + 2) loads.
-template <int R>
-__device__ __forceinline__ void block_depthwise(const ChainOp& o, const BlockWork& work, bool first_unit, const float* f_sm, const float* in, int p0,
-                                                float* d_sm) {
+template <int R, bool KEEP>
+__device__ __forceinline__ void block_depthwise(const ChainOp& o, const BlockWork& work, bool first_unit, int64_t image, const float* f_sm, const float* in,
+                                                int p0, float* d_sm) {
     const int C = o.C, quads = C >> 2, q = work.q, step = o.lanes * R;
     const int M = o.Ho * o.Wo, n = o.pixels, round = o.round1;
     const int in_row = o.in_row, tap_row = o.dh * in_row, tap_col = o.dw * C;
@@ -342,6 +359,11 @@ __device__ __forceinline__ void block_depthwise(const ChainOp& o, const BlockWor
                 if (round) {
                     v[r].x = round_bf16(v[r].x); v[r].y = round_bf16(v[r].y);
                     v[r].z = round_bf16(v[r].z); v[r].w = round_bf16(v[r].w);
+                }
+                if (KEEP && o.also_dw) {  // (by every group of columns: the same values)
+                    float* to = also_at(o.also_dw, o.also_dw_bf16, image * M * C);
+                    store_pair(o.also_dw_bf16, to, (p0 + i + r) * C + 4 * q, v[r].x, v[r].y);
+                    store_pair(o.also_dw_bf16, to, (p0 + i + r) * C + 4 * q + 2, v[r].z, v[r].w);
                 }
             }
         } else {
@@ -446,7 +468,7 @@ __device__ __forceinline__ void pool(const ChainOp& o, int64_t image, const floa
             store2(o, o.store_bf16, out, 4 * q, s.x * k, s.y * k);
             store2(o, o.store_bf16, out, 4 * q + 2, s.z * k, s.w * k);
             if (o.also) {
-                float* row = o.also_bf16 ? reinterpret_cast<float*>(reinterpret_cast<__nv_bfloat16*>(o.also) + image * o.Co) : o.also + image * o.Co;
+                float* row = also_at(o.also, o.also_bf16, image * o.Co);
                 store2(o, o.also_bf16, row, 4 * q, s.x * k, s.y * k);
                 store2(o, o.also_bf16, row, 4 * q + 2, s.z * k, s.w * k);
             }
@@ -547,6 +569,10 @@ __device__ __forceinline__ void meet(int cs, bool met) {
     else block_sync();
 }
 
+// KEEP: a block's own outputs are wanted as well (the model ends soon after it).  An instance of its own: every block's code
+// would be longer for it, and a step is bound by the fetch of instructions that run once (57.3 us instead of 55.3 for the
+// model of width 0.25 on one 128 x 128 image).
+template <bool KEEP>
 __global__ void __launch_bounds__(THREADS + 32, 1) chain_kernel(const __grid_constant__ ChainArgs a) {
     extern __shared__ __align__(16) float sm[];
     __shared__ __align__(8) unsigned long long bars[CHAIN_BARS];
@@ -599,17 +625,17 @@ __global__ void __launch_bounds__(THREADS + 32, 1) chain_kernel(const __grid_con
                 for (int u = rank; u < o.units; u += cs) {
                     const int p0 = div_by(u, o.by_groups) * o.pixels;
                     if (u != rank) block_sync();  // the unit before is done with D and red
-                    if (o.strip == 4) block_depthwise<4>(o, work, u == rank, f_sm, in, p0, d_sm);
-                    else if (o.strip == 2) block_depthwise<2>(o, work, u == rank, f_sm, in, p0, d_sm);
-                    else block_depthwise<1>(o, work, u == rank, f_sm, in, p0, d_sm);
+                    if (o.strip == 4) block_depthwise<4, KEEP>(o, work, u == rank, n, f_sm, in, p0, d_sm);
+                    else if (o.strip == 2) block_depthwise<2, KEEP>(o, work, u == rank, n, f_sm, in, p0, d_sm);
+                    else block_depthwise<1, KEEP>(o, work, u == rank, n, f_sm, in, p0, d_sm);
                     block_sync();
                     if (u + cs >= o.units) pipe.hand_back(f_empty);
                     const int v = o.variant;  // tests, not a jump table in constant memory
-                    if (v == 0) block_columns<1, 1>(o, work, u, p0, out, d_sm, w_sm, red, pipe);
-                    else if (v == 1) block_columns<1, 2>(o, work, u, p0, out, d_sm, w_sm, red, pipe);
-                    else if (v == 2) block_columns<1, 4>(o, work, u, p0, out, d_sm, w_sm, red, pipe);
-                    else if (v == 3) block_columns<2, 2>(o, work, u, p0, out, d_sm, w_sm, red, pipe);
-                    else block_columns<2, 4>(o, work, u, p0, out, d_sm, w_sm, red, pipe);
+                    if (v == 0) block_columns<1, 1, KEEP>(o, work, u, p0, n, out, d_sm, w_sm, red, pipe);
+                    else if (v == 1) block_columns<1, 2, KEEP>(o, work, u, p0, n, out, d_sm, w_sm, red, pipe);
+                    else if (v == 2) block_columns<1, 4, KEEP>(o, work, u, p0, n, out, d_sm, w_sm, red, pipe);
+                    else if (v == 3) block_columns<2, 2, KEEP>(o, work, u, p0, n, out, d_sm, w_sm, red, pipe);
+                    else block_columns<2, 4, KEEP>(o, work, u, p0, n, out, d_sm, w_sm, red, pipe);
                 }
             } else if (o.kind == CHAIN_STEM) {
                 meet(cs, met);
@@ -759,10 +785,15 @@ double tune_op(ChainOp& o, int cs) {
     }
 }
 
+template <bool KEEP>
+bool prepare_kernel() {
+    return smem_attr_once(reinterpret_cast<const void*>(chain_kernel<KEEP>), SMEM_BYTES) == cudaSuccess &&
+           cudaFuncSetAttribute(chain_kernel<KEEP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+}
+
 // How many clusters of `cs` blocks run at once; 0 where none can.
 int max_clusters(int cs) {
-    if (smem_attr_once(reinterpret_cast<const void*>(chain_kernel), SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    if (!prepare_kernel<false>() || !prepare_kernel<true>()) {
         (void)cudaGetLastError();
         return 0;
     }
@@ -777,7 +808,7 @@ int max_clusters(int cs) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, chain_kernel, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, chain_kernel<false>, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
         return 0;
     }
@@ -899,7 +930,9 @@ cudaError_t launch_chain(const ChainPlan& plan, const float* input, float* outpu
     cfg.attrs = attr;
     cfg.numAttrs = g_launch_pdl ? 2 : 1;
     ++*launches;
-    return cudaLaunchKernelEx(&cfg, chain_kernel, args);
+    bool keep = false;
+    for (int i = 0; i < args.n_ops; ++i) keep = keep || (args.ops[i].kind == CHAIN_BLOCK && (args.ops[i].also || args.ops[i].also_dw));
+    return cudaLaunchKernelEx(&cfg, keep ? chain_kernel<true> : chain_kernel<false>, args);
 }
 
 }  // namespace tfjsb

@@ -440,9 +440,10 @@ struct ChainOp {
     int in_row = 0, out_row = 0, out_origin = 0;    // floats between rows of the input and of the output, and its first element
     int64_t out_buffer = 0;                         // in the cluster's workspace
     const float *f1 = nullptr, *b1 = nullptr, *f2 = nullptr, *b2 = nullptr;  // depthwise (stem, dense) and pointwise [C,Co]
-    // pool and dense: where the layer's own output tensor is, [images][Co], which a caller may read after the run
-    float* also = nullptr;
-    int also_bf16 = 0;
+    // Layers' own output tensors that a caller may read after the run: of the operation, [images][Ho Wo][Co], and of a
+    // block's depthwise part, [images][Ho Wo][C]
+    float *also = nullptr, *also_dw = nullptr;
+    int also_bf16 = 0, also_dw_bf16 = 0;
 };
 constexpr int CHAIN_MAX_OPS = 22;
 struct ChainArgs {

@@ -203,20 +203,24 @@ tfjsb_status bind_all(tfjsb_model* m, const float* input, float* output) {
             // A fused pair is one kernel: it reads the first layer's input and writes the second
             // layer's output, so the pair takes one region (the first layer's own output buffer is
             // never written) and the region flips once per kernel, not once per layer.
-            // A chain of layers likewise, but for the vectors at its end, which it writes as the layers do.
-            if (!st.fuse_next && (i >= m->chain_len || st.out_rank == 2)) region ^= 1;
+            // A chain of layers likewise, but for its end and for the outputs that are there after any run (the
+            // last in each region: those of the two layers before the last), which it writes as the layers do.
+            if (!st.fuse_next && (i + 1 >= m->chain_len || i + 3 >= n)) region ^= 1;
         }
         tfjsb_status rc = bind_step(m, st, cur, dst);
         if (rc != TFJSB_OK) return rc;
         cur = dst;
     }
     if (!m->keep_all && m->chain_len) {
-        for (int k = 0; k + 1 < m->chain.args.n_ops; ++k) {
+        for (int k = 0; k < m->chain.args.n_ops; ++k) {
             ChainOp& o = m->chain.args.ops[k];
-            const Step& st = m->steps[m->chain_layer[k]];
-            if (st.out_rank != 2) continue;
-            o.also = st.out;
-            o.also_bf16 = st.out_bf16;
+            const int i = m->chain_layer[k];
+            const bool end = k + 1 == m->chain.args.n_ops;  // the chain's own result
+            o.also = !end && i + 3 >= n ? m->steps[i].out : nullptr;
+            o.also_bf16 = m->steps[i].out_bf16;
+            const bool dw = o.kind == CHAIN_BLOCK && i + 2 >= n;  // then layer i - 1 is among them too
+            o.also_dw = dw ? m->steps[i - 1].out : nullptr;
+            o.also_dw_bf16 = dw && m->steps[i - 1].out_bf16;
         }
     }
     if (!m->keep_all) {

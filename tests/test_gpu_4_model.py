@@ -283,3 +283,49 @@ def test_layers_in_one_kernel_without_bias_or_padding(ctx, oracle, batch):
     assert np.max(np.abs(probs - want[-1])) <= 2e-2 * want[-1].max()
     ctx.check_device_status()
     model.close()
+
+
+def _integer_mobilenet(alpha, hw, batch, classes, tail, seed):
+    """Small integers everywhere, the last layers left out: every product and sum is exact, and 2 x 2 or 4 x 4 positions
+    average to quarters or sixteenths, so two orders of summation give the same bits."""
+    layers = si.mobilenet_v1_layers(alpha, classes)[:tail]
+    chans = si.layer_channels(layers, 3)
+    for i, (layer, (cin, cout)) in enumerate(zip(layers, chans)):
+        fh, fw = layer.filter_hw
+        if layer.kind == "depthwise_conv2d":
+            layer.filter = si.small_integers(seed, 2 * i + 1, (fh, fw, cin, 1), -1, 1)
+        elif layer.kind == "conv2d":
+            layer.filter = si.small_integers(seed, 2 * i + 1, (fh, fw, cin, cout), -1, 1)
+        elif layer.kind == "dense":
+            layer.filter = si.small_integers(seed, 2 * i + 1, (cin, cout), -2, 2)
+        else:
+            continue
+        layer.bias = si.small_integers(seed, 2 * i + 2, (cout,), -2, 2)
+    return si.small_integers(seed, 0, (batch, hw, hw, 3), -3, 3), layers
+
+
+@pytest.mark.parametrize("math", ["tf32", "bf16"])
+@pytest.mark.parametrize("tail", [28, 29, 30])
+@pytest.mark.parametrize("batch,hw,alpha", [(1, 64, 0.25), (3, 128, 0.25), (40, 64, 0.25), (2, 64, 0.5)])
+def test_outputs_that_survive_a_run_in_one_kernel(ctx, batch, hw, alpha, tail, math):
+    """A model that ends in its pooled features, its logits or its probabilities: the outputs of the two layers before the
+    last can be read after a run, whether the layers ran as one kernel or each as its own; both with the same bits."""
+    x, layers = _integer_mobilenet(alpha, hw, batch, 12, tail, 4250)
+    ctx.set_math(math)
+    try:
+        model = ctx.model(layers, x.shape)
+    finally:
+        ctx.set_math("tf32")
+    xd, n = dev(x), len(layers)
+    out = host(model.run(xd))
+    assert model.layer_kernels()[0] == "chain_kernel"
+    survivors = [host(model.layer_output_f32(i)) for i in (n - 2, n - 3)]
+    ctx.check_device_status()
+    model.set_fusion("off")
+    want = host(model.run(xd))
+    assert "chain_kernel" not in model.layer_kernels()
+    for got, i in zip(survivors, (n - 2, n - 3)):
+        own = host(model.layer_output_f32(i))
+        assert len(np.unique(own)) > 4 and same_bits(got, own), layers[i].name
+    assert np.max(np.abs(out - want)) <= 1e-6 if tail == 30 else same_bits(out, want)  # exp() is not exact
+    model.close()
