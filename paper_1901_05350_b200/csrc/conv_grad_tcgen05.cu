@@ -1,12 +1,9 @@
 // Gradients of conv2d on the tensor cores (tcgen05), for any window, stride and dilation with channel counts that are
 // multiples of 4.
 //
-// Precision.  These gradients are fp32 results: every fp32 operand v is used as two TF32 values, hi = v as the tensor
-// core reads it (it drops the low 13 bits) and lo = v - hi rounded to TF32, and a product is hi*hi + hi*lo + lo*hi.
-// What is dropped, lo*lo, is at most 2^-20 of the product and 1e-7 of it on average.  The large products and the two
-// small ones are summed in separate fp32 accumulators in tensor memory and added at the end, so the accumulator that
-// matters sees one addition per eight products.  (Infinite operands give NaN: inf - inf in lo.)  Against the CUDA-core kernels: 2.7e-6 relative for
-// K = 1152 and for 1024-pixel slices.
+// Precision.  These gradients are fp32 results: every fp32 operand is used as two TF32 values and the large products are
+// summed in segments (umma_tile.cuh).  Against 64 bits, and fp32 multiply-adds on the same data: input gradient 1.5e-7 and
+// 1.4e-7 at K = 72, 2.4e-7 and 6.0e-7 at 1152, 3.9e-7 and 1.2e-6 at 4608; filter gradient of 12544 pixels 2.1e-7 and 5.6e-7.
 // (The filter gradient of a pointwise convolution whose operands are read as plain TF32 runs on the same kernel
 // without the lo half.)
 //
@@ -17,12 +14,14 @@
 //   warp 0      producer: A tile = im2col copy of 128 pixels x 32 channels of dy for one tap, B tile = block_n x 32
 //               box of f[tap]; both swizzled K-major operand tiles as they land.
 //   warp 1      MMA issuer: three products per 8 of K.
-//   warps 2-5   epilogue: both accumulators added, staged, and stored row by row to the class's pixels.
+//   warps 2-5   epilogue: segments added up, the sum staged and stored row by row to the class's pixels.
 //   warps 6-13  split: lo tile = elementwise function of the landed tile in the same layout (no index arithmetic).
 // All classes are tiles of one launch; with too few tiles for the SMs the K loop is cut and the parts are added
 // by a column sum.  Bound by shared memory: per k-block at block_n 128, 32 KB landed, 64 KB split and 96 KB read by the
 // MMAs are 1500 cycles (768 of MMAs, about 600 of im2col copy); measured 1900.
-// [16,28,28,128], 3x3, 128 channels: 6600 us with one CUDA-core thread per sample, 38 us here.
+// [16,28,28,128], 3x3, 128 channels: 6600 us with one CUDA-core thread per sample, 39 us here (35.6 with one accumulator for
+// the whole sum, which 2.7e-6 of it is then missing); [4,14,14,512], 512 channels: 92 us (104 with one accumulator, when one
+// lane and not an elected thread of a converged warp issued the MMAs).
 //
 // Filter gradient, conv2d_grad_filter_kernel.  df[(tap, ci), co] = sum over pixels: the summed index is the row of
 // both x and dy, so both landed tiles ([32 pixels][32 channels] groups: im2col or matrix boxes) are transposed into
@@ -30,8 +29,8 @@
 // 16-byte reads and writes are both free of bank conflicts under the 128-byte swizzle.  M = four (tap, 32-channel)
 // groups, N = 32..128 channels of dy, one (M tile, N tile, slice of the pixels) per CTA, partial sums added in slice
 // order.  Bound by shared-memory bandwidth (about 1800 cycles per k-block with the lo half, 1000 without, against 768 /
-// 256 of MMAs).  [16,28,28,128], 3x3: 811 us with 32 x 32 tiles on CUDA cores, 36 us here.  Pointwise, plain TF32,
-// [32,56,56] 128 x 128: 36 + 36 us of transposes and 23 + 8 us of batched products, 25 + 6 us here.
+// 256 of MMAs).  [16,28,28,128], 3x3: 811 us with 32 x 32 tiles on CUDA cores, 40 us here (38 with one accumulator).
+// Pointwise, plain TF32, [32,56,56] 128 x 128: 36 + 36 us of transposes and 23 + 8 us of batched products, 25 + 6 us here.
 #include "common.cuh"
 #include "ptx_sm100.cuh"
 #include "umma_tile.cuh"
@@ -89,6 +88,7 @@ struct GradInputArgs {
     int reach_h, reach_w;    // (taps of the largest class - 1) * dilation
     long long M;             // N * Qh * Qw
     int m_tiles, n_tiles, block_n, stages, splits, num_tiles;
+    int segment;             // k-blocks per accumulator of the large products
     float* out;              // dx, or `splits` of them one after the other
     long long out_elems;
     unsigned int* dev_status;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1)
 conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_f, const GradInputArgs g) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[CG_MAX_STAGES], bar_split[CG_MAX_STAGES], bar_empty[CG_MAX_STAGES];
-    __shared__ __align__(8) uint64_t bar_acc_full[2], bar_acc_empty[2], bar_drain;
+    __shared__ __align__(8) uint64_t bar_acc_full[2], bar_acc_empty[2], bar_small_empty, bar_drain;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag_s;
     volatile int* abort_flag = &abort_flag_s;
@@ -140,11 +140,12 @@ conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __gri
             mbar_init(smem_u32(&bar_acc_full[s]), 1);
             mbar_init(smem_u32(&bar_acc_empty[s]), EPI_WARPS);
         }
+        mbar_init(smem_u32(&bar_small_empty), EPI_WARPS);
         mbar_init(smem_u32(&bar_drain), 1);
         abort_flag_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    const uint32_t tmem_cols = (uint32_t)(4 * g.block_n);  // two stages of (large, small) accumulators; block_n 32, 64, 128
+    const uint32_t tmem_cols = (uint32_t)(4 * g.block_n);  // [large 0 | large 1 | small | sum]; block_n 32, 64, 128
     if (warp == 1) tmem_alloc(smem_u32(&tmem_slot), tmem_cols);
     tc_fence_before();
     __syncthreads();
@@ -180,51 +181,58 @@ conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __gri
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_tf32(BLOCK_M, g.block_n);
-            int stage = 0, acc = 0;
-            uint32_t phase = 0, acc_phase = 0;
-            bool ok = true, issued = false;
-            for (int t = blockIdx.x; ok && t < g.num_tiles; t += gridDim.x) {
-                const GradInputTile r = grad_input_tile(g, t);
-                if (r.kb_begin == r.kb_end) continue;  // no tap reaches these samples
-                if (!bounded_wait(smem_u32(&bar_acc_empty[acc]), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t large = tmem + (uint32_t)(acc * 2 * g.block_n), small = large + (uint32_t)g.block_n;
-                for (int kb = r.kb_begin; kb < r.kb_end; ++kb) {
-                    if (!bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag) ||
-                        !bounded_wait(smem_u32(&bar_split[stage]), phase, abort_flag)) { ok = false; break; }
+        const uint32_t idesc = make_idesc_tf32(BLOCK_M, g.block_n);
+        const uint32_t small = tmem + (uint32_t)(2 * g.block_n);
+        int stage = 0, acc = 0;
+        uint32_t phase = 0, acc_phase = 0, small_phase = 0;
+        const bool leader = elect_one();
+        bool ok = true, issued = false;  // the leader's
+        for (int t = blockIdx.x; t < g.num_tiles; t += gridDim.x) {
+            const GradInputTile r = grad_input_tile(g, t);
+            if (r.kb_begin == r.kb_end) continue;  // no tap reaches these samples
+            // the tile before has been added up
+            if (leader && ok) ok = bounded_wait(smem_u32(&bar_small_empty), small_phase ^ 1u, abort_flag);
+            small_phase ^= 1u;
+            int in_seg = 0;
+            for (int kb = r.kb_begin; kb < r.kb_end; ++kb) {
+                if (in_seg == 0 && leader && ok) ok = bounded_wait(smem_u32(&bar_acc_empty[acc]), acc_phase ^ 1u, abort_flag);
+                const uint32_t large = tmem + (uint32_t)(acc * g.block_n);
+                const uint32_t hi = stage_addr(stage), lo = hi + (uint32_t)raw_bytes;
+                const uint64_t ah = make_kmajor_sw128_desc(hi), bh = make_kmajor_sw128_desc(hi + A_STAGE_BYTES);
+                const uint64_t al = make_kmajor_sw128_desc(lo), bl = make_kmajor_sw128_desc(lo + A_STAGE_BYTES);
+                if (leader && ok && (ok = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag) &&
+                                          bounded_wait(smem_u32(&bar_split[stage]), phase, abort_flag))) {
                     tc_fence_after();
-                    const uint32_t hi = stage_addr(stage), lo = hi + (uint32_t)raw_bytes;
-                    const uint64_t ah = make_kmajor_sw128_desc(hi), bh = make_kmajor_sw128_desc(hi + A_STAGE_BYTES);
-                    const uint64_t al = make_kmajor_sw128_desc(lo), bl = make_kmajor_sw128_desc(lo + A_STAGE_BYTES);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const uint64_t o = (uint64_t)(2 * k);
-                        const uint32_t more = (kb != r.kb_begin || k != 0) ? 1u : 0u;
-                        tc_mma_tf32(large, ah + o, bh + o, idesc, more);
-                        tc_mma_tf32(small, ah + o, bl + o, idesc, more);
+                        tc_mma_tf32(large, ah + o, bh + o, idesc, (in_seg | k) != 0 ? 1u : 0u);
+                        tc_mma_tf32(small, ah + o, bl + o, idesc, (kb != r.kb_begin || k != 0) ? 1u : 0u);
                         tc_mma_tf32(small, al + o, bh + o, idesc, 1u);
                     }
                     issued = true;
                     tc_commit(smem_u32(&bar_empty[stage]));
-                    if (++stage == g.stages) { stage = 0; phase ^= 1u; }
                 }
-                if (!ok) break;
-                tc_commit(smem_u32(&bar_acc_full[acc]));
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
-            }
-            if (!ok) {
-                give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_MMA);
-                if (issued) {
-                    tc_commit(smem_u32(&bar_drain));
-                    drain(smem_u32(&bar_drain), 0u, g.dev_status);
+                if (++stage == g.stages) { stage = 0; phase ^= 1u; }
+                if (++in_seg == g.segment || kb + 1 == r.kb_end) {
+                    if (leader && ok) tc_commit(smem_u32(&bar_acc_full[acc]));
+                    in_seg = 0;
+                    if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
                 }
             }
         }
+        if (!ok) {
+            give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_MMA);
+            if (issued) {
+                tc_commit(smem_u32(&bar_drain));
+                drain(smem_u32(&bar_drain), 0u, g.dev_status);
+            }
+        }
+        __syncwarp();
     } else if (warp < 2 + EPI_WARPS) {
         const int quad = warp & 3;
         const uint32_t slab = epi_base + (uint32_t)(warp - 2) * EPI_SLAB_BYTES;
+        const uint32_t lanes = tmem + ((uint32_t)(quad * 32) << 16);
         const bool vec = (g.Cin & 3) == 0;
         int acc = 0;
         uint32_t acc_phase = 0;
@@ -242,33 +250,40 @@ conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __gri
                 const int iy = (g.q0h + qy) * g.sh + r.a - g.pt, ix = (g.q0w + qx) * g.sw + r.b - g.pl;
                 if (iy >= 0 && iy < g.H && ix >= 0 && ix < g.W) at = ((n * g.H + iy) * (long long)g.W + ix) * g.Cin;
             }
-            if (any) {
-                const bool got = bounded_wait(smem_u32(&bar_acc_full[acc]), acc_phase, abort_flag);
-                if (!__all_sync(0xffffffffu, got)) {
-                    if (lane == 0) give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_EPILOGUE);
-                    break;
-                }
-                tc_fence_after();
-            }
             float* out = g.out + (long long)r.split * g.out_elems;
             const int live = min(g.block_n, g.Cin - r.n0);
+            bool ok = true;
+            for (int kb = r.kb_begin; kb < r.kb_end; kb += g.segment) {
+                const bool got = bounded_wait(smem_u32(&bar_acc_full[acc]), acc_phase, abort_flag), last = kb + g.segment >= r.kb_end;
+                if (!(ok = __all_sync(0xffffffffu, got))) break;
+                tc_fence_after();
+                add_segment<16>(lanes + (uint32_t)(acc * g.block_n), lanes + (uint32_t)(2 * g.block_n), lanes + (uint32_t)(3 * g.block_n), (live + 15) & ~15,
+                            kb == r.kb_begin, last);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(smem_u32(&bar_acc_empty[acc]));
+                    if (last) mbar_arrive(smem_u32(&bar_small_empty));
+                }
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            }
+            if (!ok) {
+                if (lane == 0) give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_EPILOGUE);
+                break;
+            }
             for (int c0 = 0; c0 < live; c0 += 32) {
-                uint32_t u[32], v[32];
+                uint32_t u[32];
                 if (any) {
-                    const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 2 * g.block_n + c0);
-                    tc_ld_32x32(ta, u);
-                    tc_ld_32x32(ta + (uint32_t)g.block_n, v);
+                    tc_ld_32x32(lanes + (uint32_t)(3 * g.block_n + c0), u);
                     tc_ld_wait();
                 } else {
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) u[e] = v[e] = 0u;
+                    for (int e = 0; e < 32; ++e) u[e] = 0u;
                 }
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
-                    sts4(slab + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4),
-                         __uint_as_float(u[4 * j]) + __uint_as_float(v[4 * j]), __uint_as_float(u[4 * j + 1]) + __uint_as_float(v[4 * j + 1]),
-                         __uint_as_float(u[4 * j + 2]) + __uint_as_float(v[4 * j + 2]),
-                         __uint_as_float(u[4 * j + 3]) + __uint_as_float(v[4 * j + 3]));
+                    sts4(slab + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4), __uint_as_float(u[4 * j]), __uint_as_float(u[4 * j + 1]),
+                         __uint_as_float(u[4 * j + 2]), __uint_as_float(u[4 * j + 3]));
                 __syncwarp();
                 const int col0 = r.n0 + c0;
                 if (vec) {
@@ -290,12 +305,6 @@ conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __gri
                 }
                 __syncwarp();
             }
-            if (any) {
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[acc]));
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
-            }
         }
     } else {
         const uint32_t mine = (uint32_t)(threadIdx.x - (2 + EPI_WARPS) * 32) * 16u;
@@ -316,7 +325,8 @@ conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __gri
 #pragma unroll 4
                 for (int o = 0; o < raw_bytes; o += CVT_WARPS * 512) {
                     const float4 v = lds4(src + (uint32_t)o);
-                    sts4(dst + (uint32_t)o, tf32_rest(v.x), tf32_rest(v.y), tf32_rest(v.z), tf32_rest(v.w));
+                    const uint32_t round = o < A_STAGE_BYTES ? SPLIT_UP : SPLIT_NEAREST;
+                    sts4(dst + (uint32_t)o, tf32_rest(v.x, round), tf32_rest(v.y, round), tf32_rest(v.z, round), tf32_rest(v.w, round));
                 }
                 fence_async_smem();
                 __syncwarp();
@@ -341,6 +351,7 @@ struct GradFilterArgs {
     int n_tiles, block_n, raw_stages, op_stages;
     int pixel_blocks, blocks_per_slice;  // blocks of 32 pixels
     int m_tiles;
+    int segment;    // k-blocks per accumulator of the large products
     int tiled;      // x as a matrix [pixels, Cin] (1x1, stride 1) instead of im2col copies
     unsigned int* dev_status;
 };
@@ -352,7 +363,7 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_raw_full[CG_MAX_STAGES], bar_raw_empty[CG_MAX_STAGES];
     __shared__ __align__(8) uint64_t bar_op_full[CG_MAX_STAGES], bar_op_empty[CG_MAX_STAGES];
-    __shared__ __align__(8) uint64_t bar_acc, bar_drain;
+    __shared__ __align__(8) uint64_t bar_acc_full[2], bar_acc_empty[2], bar_drain;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag_s;
     volatile int* abort_flag = &abort_flag_s;
@@ -381,12 +392,15 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
             mbar_init(smem_u32(&bar_op_full[s]), CVT_WARPS);
             mbar_init(smem_u32(&bar_op_empty[s]), 1);
         }
-        mbar_init(smem_u32(&bar_acc), 1);
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(smem_u32(&bar_acc_full[s]), 1);
+            mbar_init(smem_u32(&bar_acc_empty[s]), EPI_WARPS);
+        }
         mbar_init(smem_u32(&bar_drain), 1);
         abort_flag_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    const uint32_t tmem_cols = (uint32_t)(HALVES * g.block_n);
+    const uint32_t tmem_cols = (uint32_t)((SPLIT ? 4 : 1) * g.block_n);  // [large 0 | large 1 | small | sum], or one accumulator
     if (warp == 1) tmem_alloc(smem_u32(&tmem_slot), tmem_cols);
     tc_fence_before();
     __syncthreads();
@@ -431,68 +445,81 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_tf32(BLOCK_M, g.block_n);
-            const uint32_t large = tmem, small = tmem + (uint32_t)g.block_n;
-            int stage = 0;
-            uint32_t phase = 0;
-            bool ok = true, issued = false;
-            for (int kb = 0; kb < kbs; ++kb) {
-                if (!bounded_wait(smem_u32(&bar_op_full[stage]), phase, abort_flag)) { ok = false; break; }
+        const uint32_t idesc = make_idesc_tf32(BLOCK_M, g.block_n);
+        const uint32_t small = tmem + (uint32_t)(2 * g.block_n);
+        int stage = 0, acc = 0, in_seg = 0;
+        uint32_t phase = 0, acc_phase = 0;
+        const bool leader = elect_one();
+        bool ok = true, issued = false;  // the leader's
+        for (int kb = 0; kb < kbs; ++kb) {
+            if (SPLIT && in_seg == 0 && leader && ok) ok = bounded_wait(smem_u32(&bar_acc_empty[acc]), acc_phase ^ 1u, abort_flag);
+            const uint32_t large = tmem + (uint32_t)(acc * g.block_n);
+            const uint32_t hi = op_base + (uint32_t)(stage * HALVES * raw_bytes), lo = hi + (uint32_t)raw_bytes;
+            const uint64_t ah = make_kmajor_sw128_desc(hi), bh = make_kmajor_sw128_desc(hi + A_STAGE_BYTES);
+            const uint64_t al = make_kmajor_sw128_desc(lo), bl = make_kmajor_sw128_desc(lo + A_STAGE_BYTES);
+            if (leader && ok && (ok = bounded_wait(smem_u32(&bar_op_full[stage]), phase, abort_flag))) {
                 tc_fence_after();
-                const uint32_t hi = op_base + (uint32_t)(stage * HALVES * raw_bytes), lo = hi + (uint32_t)raw_bytes;
-                const uint64_t ah = make_kmajor_sw128_desc(hi), bh = make_kmajor_sw128_desc(hi + A_STAGE_BYTES);
-                const uint64_t al = make_kmajor_sw128_desc(lo), bl = make_kmajor_sw128_desc(lo + A_STAGE_BYTES);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const uint64_t o = (uint64_t)(2 * k);
-                    const uint32_t more = (kb | k) != 0 ? 1u : 0u;
-                    tc_mma_tf32(large, ah + o, bh + o, idesc, more);
+                    tc_mma_tf32(large, ah + o, bh + o, idesc, ((SPLIT ? in_seg : kb) | k) != 0 ? 1u : 0u);
                     if (SPLIT) {
-                        tc_mma_tf32(small, ah + o, bl + o, idesc, more);
+                        tc_mma_tf32(small, ah + o, bl + o, idesc, (kb | k) != 0 ? 1u : 0u);
                         tc_mma_tf32(small, al + o, bh + o, idesc, 1u);
                     }
                 }
                 issued = true;
                 tc_commit(smem_u32(&bar_op_empty[stage]));
-                if (++stage == g.op_stages) { stage = 0; phase ^= 1u; }
             }
-            if (ok) tc_commit(smem_u32(&bar_acc));
-            else {
-                give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_MMA);
-                if (issued) {
-                    tc_commit(smem_u32(&bar_drain));
-                    drain(smem_u32(&bar_drain), 0u, g.dev_status);
-                }
+            if (++stage == g.op_stages) { stage = 0; phase ^= 1u; }
+            if (kb + 1 == kbs || (SPLIT && ++in_seg == g.segment)) {
+                if (leader && ok) tc_commit(smem_u32(&bar_acc_full[acc]));
+                in_seg = 0;
+                if (SPLIT && ++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
         }
+        if (!ok) {
+            give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_MMA);
+            if (issued) {
+                tc_commit(smem_u32(&bar_drain));
+                drain(smem_u32(&bar_drain), 0u, g.dev_status);
+            }
+        }
+        __syncwarp();
     } else if (warp < 2 + EPI_WARPS) {
         const int quad = warp & 3;  // the M tile's group whose 32 rows this warp may read
         const uint32_t slab = epi_base + (uint32_t)(warp - 2) * EPI_SLAB_BYTES;
-        const bool got = bounded_wait(smem_u32(&bar_acc), 0u, abort_flag);
-        if (!__all_sync(0xffffffffu, got)) {
+        const uint32_t lanes = tmem + ((uint32_t)(quad * 32) << 16);
+        bool ok = true;
+        int acc = 0;
+        uint32_t acc_phase = 0;
+        for (int kb = 0; kb < kbs; kb += SPLIT ? g.segment : kbs) {
+            const bool got = bounded_wait(smem_u32(&bar_acc_full[acc]), acc_phase, abort_flag);
+            if (!(ok = __all_sync(0xffffffffu, got))) break;
+            tc_fence_after();
+            if (SPLIT) {
+                add_segment<16>(lanes + (uint32_t)(acc * g.block_n), lanes + (uint32_t)(2 * g.block_n), lanes + (uint32_t)(3 * g.block_n), g.block_n, kb == 0,
+                            kb + g.segment >= kbs);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[acc]));
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            }
+        }
+        if (!ok) {
             if (lane == 0) give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_EPILOGUE);
         } else if (quad < live_groups) {
-            tc_fence_after();
             const int gi = g0 + quad, tap = gi / g.c_blocks, ci0 = (gi - tap * g.c_blocks) * 32;
             for (int c0 = 0; c0 < g.block_n; c0 += 32) {
-                uint32_t u[32], v[32];
-                const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
-                tc_ld_32x32(ta, u);
-                if (SPLIT) tc_ld_32x32(ta + (uint32_t)g.block_n, v);
+                uint32_t u[32];
+                tc_ld_32x32(lanes + (uint32_t)((SPLIT ? 3 * g.block_n : 0) + c0), u);
                 tc_ld_wait();
                 if (lane == 0) tma_store_wait_read<0>();
                 __syncwarp();
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    float w[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        w[e] = __uint_as_float(u[4 * j + e]);
-                        if (SPLIT) w[e] += __uint_as_float(v[4 * j + e]);
-                    }
-                    sts4(slab + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4), w[0], w[1], w[2], w[3]);
-                }
+                for (int j = 0; j < 8; ++j)
+                    sts4(slab + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4), __uint_as_float(u[4 * j]), __uint_as_float(u[4 * j + 1]),
+                         __uint_as_float(u[4 * j + 2]), __uint_as_float(u[4 * j + 3]));
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
@@ -533,9 +560,15 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
                 for (int e = 0; e < 4; ++e) {
                     const int row = 4 * q + e;
                     const uint32_t at = (uint32_t)(grp * GROUP_BYTES + row * 128 + ((l ^ (row & 7)) << 4));
-                    sts4(hi + at, f[e], f[4 + e], f[8 + e], f[12 + e]);
-                    if (SPLIT)
-                        sts4(hi + (uint32_t)raw_bytes + at, tf32_rest(f[e]), tf32_rest(f[4 + e]), tf32_rest(f[8 + e]), tf32_rest(f[12 + e]));
+                    if (SPLIT) {
+                        float large[4], small[4];
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) tf32_split(f[4 * p + e], large[p], small[p]);
+                        sts4(hi + at, large[0], large[1], large[2], large[3]);
+                        sts4(hi + (uint32_t)raw_bytes + at, small[0], small[1], small[2], small[3]);
+                    } else {
+                        sts4(hi + at, f[e], f[4 + e], f[8 + e], f[12 + e]);
+                    }
                 }
             }
             fence_async_smem();
@@ -606,7 +639,7 @@ bool conv2d_grad_input_supported(const ConvGeom& g) {
     return g.Co % 4 == 0 && reach_h <= 127 && reach_w <= 127 && corner_ok(q0h - reach_h) && corner_ok(q0w - reach_w) &&
            corner_ok(q0h - reach_h + Qh - g.Ho) && corner_ok(q0w - reach_w + Qw - g.Wo) && g.Ho > 0 && g.Wo > 0 &&
            g.N * Qh * Qw < (1LL << 31) - 256 && m_tiles * g.sh * g.sw * ((g.C + 31) / 32) * 16 < (1LL << 31) &&
-           (int64_t)g.fh * g.fw * ((g.Co + 31) / 32) < (1LL << 24);
+           (int64_t)g.fh * g.fw * ((g.Co + 31) / 32) * 32 <= SPLIT_MAX_K;
 }
 
 tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float* f, float* dx, const ConvGeom& g, cudaStream_t s) {
@@ -642,6 +675,7 @@ tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float*
         if (a.splits < 1) a.splits = 1;
     }
     a.num_tiles = (int)(tiles * a.splits);
+    a.segment = split_segment((int64_t)kbs * BLOCK_K);
     const int stage_bytes = 2 * (A_STAGE_BYTES + a.block_n * 128);
     a.stages = (CG_SMEM - 1024 - EPI_WARPS * EPI_SLAB_BYTES) / stage_bytes;
     if (a.stages > CG_MAX_STAGES) a.stages = CG_MAX_STAGES;
@@ -709,6 +743,7 @@ tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float*
     if (slices < 1) slices = 1;
     a.blocks_per_slice = (int)((a.pixel_blocks + slices - 1) / slices);
     slices = (a.pixel_blocks + a.blocks_per_slice - 1) / a.blocks_per_slice;
+    a.segment = split_segment((int64_t)a.blocks_per_slice * 32);
     const int raw_bytes = (4 + a.block_n / 32) * GROUP_BYTES, halves = split ? 2 : 1;
     a.op_stages = split ? 2 : 3;
     a.raw_stages = (CG_SMEM - 1024 - EPI_WARPS * EPI_SLAB_BYTES - a.op_stages * halves * raw_bytes) / raw_bytes;

@@ -3,14 +3,13 @@
 //
 // The bulk copy unit wants rows that start on 16 bytes and delivers K-contiguous tiles only from K-contiguous memory.
 // Here eight loader warps fetch the tiles instead: they read global memory in runs of 32 floats along whichever dimension
-// is contiguous, the next k-block's values while this one's are stored, and write the K-major, 128-byte-swizzled operand
+// is contiguous, the next k-block's values as soon as this one's are stored, and write the K-major, 128-byte-swizzled operand
 // tiles that tcgen05.mma reads (K-contiguous: a warp's 32 floats are one row; otherwise a lane collects four k of its own
 // row and stores 16 bytes; both are free of bank conflicts).
 //
-// An operand value v is stored twice, as hi = v (the tensor core drops the low 13 bits) and as lo = v - hi rounded to
-// TF32; a product is hi*hi + hi*lo + lo*hi.  The two small products have an accumulator of their own and the large one
-// three, one per third of the K loop, so that an accumulator sees a few hundred additions at most; all are added in fp32
-// registers.  (Infinite operands give NaN: inf - inf in lo.)
+// An operand value is stored as two TF32 values, and the large products are summed in segments (umma_tile.cuh), which the
+// loader warps add up between two k-blocks.  Error against 64 bits, and of fp32 multiply-adds: 1.2e-7 and 1.4e-7 at K = 64,
+// 2.7e-7 and 8.0e-7 at 2001; sums of one sign 4.2e-7 and 6.6e-7 at 2001, 1.9e-6 and 2.2e-6 at 20001.
 //
 // A tile is 128 x BN (BN 32, 64) of C or of its transpose, whichever wastes fewer rows.  Small products are a chain of one
 // load, a few MMAs and the store, so two CTAs share an SM and cover each other's latency.  With fewer tiles than CTAs fit
@@ -18,8 +17,9 @@
 // barrier every CTA adds one band of rows from all of them, in rank order, and stores it.
 //
 // Bound by the loaders: a k-block costs a CTA about 2500 cycles (address arithmetic, 4-byte loads and stores) against 400
-// of MMAs; sixteen loader warps per CTA were slower (2001^3: 297 us against 220).  64 products [199,64] . [64,199]: 1179 us
-// as 64 launches of the CUDA-core kernel, 18.6 us here; [64,1024] . [1024,101]: 201 us and 10.5 us.
+// of MMAs; sixteen loader warps per CTA were slower (2001^3: 297 us against 220), and so was fetching the next values before
+// this k-block's are stored, which takes twice the registers (2001^3: 275 us against 205).  64 products [199,64] . [64,199]:
+// 1179 us as 64 launches of the CUDA-core kernel, 18.6 us here; [64,1024] . [1024,101]: 201 us and 10.5 us.
 #include "common.cuh"
 #include "ptx_sm100.cuh"
 #include "umma_tile.cuh"
@@ -33,7 +33,7 @@ namespace {
 
 constexpr int LOADERS = 8;
 constexpr int GS_THREADS = 32 + LOADERS * 32;
-constexpr int GS_MAX_STAGES = 4;
+constexpr int GS_MAX_STAGES = 2;  // what fits beside a second CTA, for tiles of 64 and of 32 columns
 constexpr int GS_MAX_CLUSTER = 8;
 
 // One operand: element (row, k) of product b at ptr[b * batch_stride + row * row_stride + k * k_stride].
@@ -47,6 +47,7 @@ struct Side {
 struct StridedArgs {
     Side p, q;          // p: the 128 rows of a tile, q: its BN columns
     int K, num_kb, stages, splits;
+    int segment;        // k-blocks per accumulator of the large products
     int p_tiles, q_tiles;
     float* c;           // element (row of p, row of q) of product b
     long long c_p, c_q, c_batch;
@@ -83,17 +84,20 @@ struct Fetch {
             const uint32_t at = tile + (uint32_t)(w * 128 + (((lane >> 2) ^ w) << 4) + (lane & 3) * 4);
 #pragma unroll
             for (int i = 0; i < ROWS / 8; ++i) {
-                asm volatile("st.shared.f32 [%0], %1;" ::"r"(at + (uint32_t)i * 1024u), "f"(v[i]) : "memory");
-                asm volatile("st.shared.f32 [%0], %1;" ::"r"(at + lo_offset + (uint32_t)i * 1024u), "f"(tf32_rest(v[i])) : "memory");
+                float hi, lo;
+                tf32_split(v[i], hi, lo);
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(at + (uint32_t)i * 1024u), "f"(hi) : "memory");
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(at + lo_offset + (uint32_t)i * 1024u), "f"(lo) : "memory");
             }
         } else {
             const uint32_t at = tile + (uint32_t)(lane * 128 + ((w ^ (lane & 7)) << 4));
 #pragma unroll
             for (int i = 0; i < ROWS / 32; ++i) {
-                const float* u = v + 4 * i;
-                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + (uint32_t)i * 4096u), "f"(u[0]), "f"(u[1]), "f"(u[2]), "f"(u[3]) : "memory");
-                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + lo_offset + (uint32_t)i * 4096u), "f"(tf32_rest(u[0])),
-                             "f"(tf32_rest(u[1])), "f"(tf32_rest(u[2])), "f"(tf32_rest(u[3])) : "memory");
+                float hi[4], lo[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) tf32_split(v[4 * i + e], hi[e], lo[e]);
+                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + (uint32_t)i * 4096u), "f"(hi[0]), "f"(hi[1]), "f"(hi[2]), "f"(hi[3]) : "memory");
+                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + lo_offset + (uint32_t)i * 4096u), "f"(lo[0]), "f"(lo[1]), "f"(lo[2]), "f"(lo[3]) : "memory");
             }
         }
     }
@@ -104,8 +108,10 @@ __global__ void __launch_bounds__(GS_THREADS, 2)
 gemm_strided_kernel(const StridedArgs g) {
     constexpr int OPERANDS = A_STAGE_BYTES + BN * 128;  // hi (or lo) of one stage
     constexpr int STAGE_BYTES = OPERANDS * 2;
-    constexpr int SEGMENTS = 3;                         // accumulators of the large products
-    constexpr uint32_t TMEM_COLS = (SEGMENTS + 1) * BN;
+    constexpr uint32_t TMEM_COLS = 4 * BN;              // [large 0 | large 1 | small | sum]
+    // Segment j has been multiplied when its last stage comes free, `stages` k-blocks later, and the loaders add it to the
+    // sum before they hand over the first k-block of segment j + 2, which takes its accumulator: no barriers of its own.
+    static_assert(GS_MAX_STAGES <= 2, "a segment of one k-block is added up before its accumulator is used again");
     constexpr int PITCH = BN + 1;                       // words per row of the partial tile in shared memory
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[GS_MAX_STAGES], bar_empty[GS_MAX_STAGES], bar_acc, bar_drain;
@@ -142,21 +148,21 @@ gemm_strided_kernel(const StridedArgs g) {
     const int pt = t % g.p_tiles, batch = t / g.p_tiles;
     const int p0 = pt * BLOCK_M, q0 = qt * BN;
     const int kb0 = (int)((long long)g.num_kb * rank / g.splits), kb1 = (int)((long long)g.num_kb * (rank + 1) / g.splits);
-    const int seg_len = (kb1 - kb0 + SEGMENTS - 1) / SEGMENTS;  // k-blocks per accumulator; never zero (splits <= num_kb)
+    const int segments = (kb1 - kb0 + g.segment - 1) / g.segment;  // never zero (splits <= num_kb)
 
     if (warp == 0) {
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_tf32(BLOCK_M, BN);
-            const uint32_t small = tmem + SEGMENTS * BN;
-            int stage = 0, in_seg = 0;
-            uint32_t phase = 0, large = tmem;
-            bool ok = true, issued = false;
-            for (int kb = kb0; kb < kb1; ++kb) {
-                if (!bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag)) { ok = false; break; }
+        const uint32_t idesc = make_idesc_tf32(BLOCK_M, BN);
+        const uint32_t small = tmem + 2 * BN;
+        int stage = 0, in_seg = 0;
+        uint32_t phase = 0, large = tmem;
+        const bool leader = elect_one();
+        bool ok = true, issued = false;  // the leader's
+        for (int kb = kb0; kb < kb1; ++kb) {
+            const uint32_t hi = base + (uint32_t)(stage * STAGE_BYTES), lo = hi + OPERANDS;
+            const uint64_t ah = make_kmajor_sw128_desc(hi), bh = make_kmajor_sw128_desc(hi + A_STAGE_BYTES);
+            const uint64_t al = make_kmajor_sw128_desc(lo), bl = make_kmajor_sw128_desc(lo + A_STAGE_BYTES);
+            if (leader && ok && (ok = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag))) {
                 tc_fence_after();
-                const uint32_t hi = base + (uint32_t)(stage * STAGE_BYTES), lo = hi + OPERANDS;
-                const uint64_t ah = make_kmajor_sw128_desc(hi), bh = make_kmajor_sw128_desc(hi + A_STAGE_BYTES);
-                const uint64_t al = make_kmajor_sw128_desc(lo), bl = make_kmajor_sw128_desc(lo + A_STAGE_BYTES);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const uint64_t o = (uint64_t)(2 * k);
@@ -166,24 +172,24 @@ gemm_strided_kernel(const StridedArgs g) {
                 }
                 issued = true;
                 tc_commit(smem_u32(&bar_empty[stage]));
-                if (++stage == g.stages) { stage = 0; phase ^= 1u; }
-                if (++in_seg == seg_len) { in_seg = 0; large += BN; }
             }
-            if (ok) tc_commit(smem_u32(&bar_acc));
-            else {
-                if (!*abort_flag) {
-                    *abort_flag = 1;
-                    atomicOr(g.dev_status, DEV_STATUS_TIMEOUT_MMA);
-                }
-                if (issued) {
-                    tc_commit(smem_u32(&bar_drain));
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(smem_u32(&bar_drain), 0u))
-                        if (global_ns() - t0 > WAIT_LIMIT_NS) {
-                            atomicOr(g.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
-                            break;
-                        }
-                }
+            if (++stage == g.stages) { stage = 0; phase ^= 1u; }
+            if (++in_seg == g.segment) { in_seg = 0; large = tmem + (large == tmem ? BN : 0); }
+        }
+        if (leader && ok) tc_commit(smem_u32(&bar_acc));
+        if (!ok) {
+            if (!*abort_flag) {
+                *abort_flag = 1;
+                atomicOr(g.dev_status, DEV_STATUS_TIMEOUT_MMA);
+            }
+            if (issued) {
+                tc_commit(smem_u32(&bar_drain));
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(smem_u32(&bar_drain), 0u))
+                    if (global_ns() - t0 > WAIT_LIMIT_NS) {
+                        atomicOr(g.dev_status, DEV_STATUS_TIMEOUT_DRAIN);
+                        break;
+                    }
             }
         }
         __syncwarp();
@@ -193,30 +199,41 @@ gemm_strided_kernel(const StridedArgs g) {
         const float* qb = g.q.ptr + batch * g.q.batch_stride;
         const bool p_k = g.p.k_stride == 1, q_k = g.q.k_stride == 1;
         bool ok = true;
-        Fetch<BLOCK_M> fp[2];
-        Fetch<BN> fq[2];
-        fp[0].load(g.p, pb, p0, kb0 * BLOCK_K, g.K, w, lane);
-        fq[0].load(g.q, qb, q0, kb0 * BLOCK_K, g.K, w, lane);
+        Fetch<BLOCK_M> fp;
+        Fetch<BN> fq;
+        fp.load(g.p, pb, p0, kb0 * BLOCK_K, g.K, w, lane);
+        fq.load(g.q, qb, q0, kb0 * BLOCK_K, g.K, w, lane);
+        // the sum: the two warps of a lane quadrant take 32 columns each
+        const int quad = warp & 3, c0 = (w >> 2) * 32;
+        const uint32_t lanes = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
+        int added = 0;                                        // segments that are in the sum
+        int add_at = kb0 + g.segment - 1 + g.stages;          // the k-block before which the next is added
+        auto add = [&](bool last) {
+            tc_fence_after();
+            if (c0 < BN) add_segment<16>(lanes + (uint32_t)((added & 1) * BN), lanes + 2 * BN, lanes + 3 * BN, 32, added == 0, last);
+            tc_fence_before();
+            ++added;
+        };
         int stage = 0;
         uint32_t phase = 0;
-        for (int kb = kb0; ok && kb < kb1; kb += 2) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (kb + h >= kb1) break;
-                if (kb + h + 1 < kb1) {
-                    fp[h ^ 1].load(g.p, pb, p0, (kb + h + 1) * BLOCK_K, g.K, w, lane);
-                    fq[h ^ 1].load(g.q, qb, q0, (kb + h + 1) * BLOCK_K, g.K, w, lane);
-                }
-                const bool got = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag);
-                if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-                const uint32_t hi = base + (uint32_t)(stage * STAGE_BYTES);
-                fp[h].store(p_k, hi, OPERANDS, w, lane);
-                fq[h].store(q_k, hi + A_STAGE_BYTES, OPERANDS, w, lane);
-                fence_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bar_full[stage]));
-                if (++stage == g.stages) { stage = 0; phase ^= 1u; }
+        for (int kb = kb0; kb < kb1; ++kb) {
+            const bool got = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag);
+            if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+            const uint32_t hi = base + (uint32_t)(stage * STAGE_BYTES);
+            fp.store(p_k, hi, OPERANDS, w, lane);
+            fq.store(q_k, hi + A_STAGE_BYTES, OPERANDS, w, lane);
+            if (kb == add_at) {  // before the next values are fetched: it wants their registers
+                add(false);
+                add_at += g.segment;
             }
+            if (kb + 1 < kb1) {
+                fp.load(g.p, pb, p0, (kb + 1) * BLOCK_K, g.K, w, lane);
+                fq.load(g.q, qb, q0, (kb + 1) * BLOCK_K, g.K, w, lane);
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bar_full[stage]));
+            if (++stage == g.stages) { stage = 0; phase ^= 1u; }
         }
         ok = ok && bounded_wait(smem_u32(&bar_acc), 0u, abort_flag);
         if (!__all_sync(0xffffffffu, ok)) {
@@ -225,24 +242,13 @@ gemm_strided_kernel(const StridedArgs g) {
                 atomicOr(g.dev_status, DEV_STATUS_TIMEOUT_EPILOGUE);
             }
         } else {
-            // accumulators -> partial tile in shared memory (all operand reads are done: bar_acc); the two warps of a
-            // lane quadrant take 32 columns each
-            tc_fence_after();
-            const int quad = warp & 3;
-            const int segments = (kb1 - kb0 + seg_len - 1) / seg_len;
-            for (int c0 = (w >> 2) * 32; c0 < BN; c0 += 64) {
-                const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
+            // the rest of the sum (one segment or two), and the sum -> partial tile in shared memory (all operand reads are
+            // done: bar_acc)
+            while (added < segments) add(added + 1 == segments);
+            if (c0 < BN) {
                 uint32_t u[32];
-                tc_ld_32x32(ta, u);
+                tc_ld_32x32(lanes + 3 * BN, u);
                 tc_ld_wait();
-                for (int s = 1; s <= SEGMENTS; ++s) {
-                    if (s < SEGMENTS && s >= segments) continue;
-                    uint32_t v[32];
-                    tc_ld_32x32(ta + (uint32_t)(s * BN), v);
-                    tc_ld_wait();
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) u[e] = __float_as_uint(__uint_as_float(u[e]) + __uint_as_float(v[e]));
-                }
                 const uint32_t row = base + (uint32_t)(((quad * 32 + lane) * PITCH + c0) * 4);
 #pragma unroll
                 for (int e = 0; e < 32; ++e) asm volatile("st.shared.b32 [%0], %1;" ::"r"(row + 4u * e), "r"(u[e]) : "memory");
@@ -382,7 +388,7 @@ Choice choose(int64_t batches, int64_t M, int64_t N, int64_t K, int sm_count) {
 
 bool gemm_strided_supported(int64_t batches, int64_t M, int64_t N, int64_t K) {
     constexpr int64_t LIM = (1LL << 31) - 256;
-    return batches >= 1 && M >= 1 && N >= 1 && K >= 1 && M < LIM && N < LIM && K < LIM && batches < LIM &&
+    return batches >= 1 && M >= 1 && N >= 1 && K >= 1 && M < LIM && N < LIM && K <= SPLIT_MAX_K && batches < LIM &&
            (double)batches * (double)((M + 31) / 32) * (double)((N + 31) / 32) < 1e9;
 }
 
@@ -398,6 +404,7 @@ cudaError_t launch_gemm_strided(const float* a, int64_t a_rs, int64_t a_ks, cons
     g.K = (int)K;
     g.num_kb = (int)((K + BLOCK_K - 1) / BLOCK_K);
     g.splits = ch.splits;
+    g.segment = split_segment(K);
     g.p_tiles = (g.p.rows + BLOCK_M - 1) / BLOCK_M;
     g.q_tiles = (g.q.rows + ch.bn - 1) / ch.bn;
     g.c = c;

@@ -48,12 +48,66 @@ __device__ __forceinline__ void stage_chunk(const uint32_t (&r)[32], const float
     }
 }
 
-// What the tensor core drops of an fp32 operand it reads as TF32, rounded to TF32 (half away from zero; the bits below are
-// left in, the tensor core drops them): v = tf32(v) + tf32(tf32_rest(v)) to 2^-21.  With the conversion instruction
-// instead of the integer addition a 2001^3 product took 243 us instead of 220, a 3x3 convolution's gradients 6 us more.
-__device__ __forceinline__ float tf32_rest(float v) {
+// ---- fp32 accuracy from TF32 products ----------------------------------------------------------------
+// An fp32 operand v is used as two TF32 values (the tensor core drops the low 13 bits of what it reads), hi + lo, and a
+// product as hi * hi + hi * lo + lo * hi.
+//
+// Where threads write the operand tiles themselves, hi is v rounded to nearest and lo the rest, exact in fp32 and cut to
+// TF32 after the addition of half a unit (7e-8 of v on average; values that lo represents exactly stay as they are).  The
+// rounding of hi carries a NaN of all ones over to -0, but lo is then a NaN.
+__device__ __forceinline__ void tf32_split(float v, float& hi, float& lo) {
+    const uint32_t up = __float_as_uint(v) + 0x1000u;
+    hi = __uint_as_float(up);
+    const float rest = v - __uint_as_float(up & 0xffffe000u);
+    lo = fmaf(rest, 0.00048828125f, rest);
+}
+// Where the tile is left as it was copied, hi is v cut to TF32, and lo the rest, rounded by an integer addition.  The
+// product lo * lo that is left out then has the sign of the whole: on average 2^-23 of it, a bias.  The lo half of one
+// operand is therefore rounded away from zero (SPLIT_UP), which adds as much on average, that of the other to nearest.
+constexpr uint32_t SPLIT_UP = 0x1fffu, SPLIT_NEAREST = 0x1000u;
+__device__ __forceinline__ float tf32_rest(float v, uint32_t round) {
     const float hi = __uint_as_float(__float_as_uint(v) & 0xffffe000u);
-    return __uint_as_float(__float_as_uint(v - hi) + 0x1000u);
+    return __uint_as_float(__float_as_uint(v - hi) + round);
+}
+
+// The tensor core cuts every sum it makes towards zero, so an accumulator's error grows with the number of additions,
+// where the errors of fp32 fused multiply-adds, which round to nearest, mostly cancel.  The large products (hi * hi)
+// therefore go to an accumulator for a segment of a few k-blocks only (4 additions of 8 products each), and these parts are
+// added by threads, in tensor memory: two accumulators in turn, one for the small products, which are 2^-11 of the large
+// ones, and the sum:  columns [large 0 | large 1 | small | sum].
+//
+// Length of a segment, in k-blocks, for sums of K products.  Measured against 64 bits: 7e-8 of the result per k-block of a
+// segment, 1.5e-7 if all products have one sign, beside 1.2e-7 from the operands; sums by fp32 multiply-adds 1.8e-8 sqrt(K).
+// Without segments a 3x3 convolution's input gradient over 512 channels was 1.0e-5 off (multiply-adds: 1.2e-6).
+inline int split_segment(int64_t K) {
+    int n = 1;
+    while ((int64_t)(n + 1) * (n + 1) * 196 <= K) ++n;  // sqrt(K) / 14
+    return n;
+}
+// Of longer sums the small products' accumulator would be the less exact part.
+constexpr int64_t SPLIT_MAX_K = 1LL << 22;
+
+// One 32-lane x `cols`-column part of  sum = (first ? 0 : sum) + large, and + small after the last segment; both addresses
+// and `cols` (a multiple of STEP, 8 or 16) are of the caller's lanes and columns.
+template <int STEP>
+__device__ __forceinline__ void add_segment(uint32_t large, uint32_t small, uint32_t sum, int cols, bool first, bool last) {
+#pragma unroll 1
+    for (int c = 0; c < cols; c += STEP) {
+        uint32_t u[STEP], v[STEP], w[STEP];
+        ptx::tc_ld_cols(large + (uint32_t)c, u);
+        if (!first) ptx::tc_ld_cols(sum + (uint32_t)c, v);
+        if (last) ptx::tc_ld_cols(small + (uint32_t)c, w);
+        ptx::tc_ld_wait();
+#pragma unroll
+        for (int e = 0; e < STEP; ++e) {
+            float s = __uint_as_float(u[e]);
+            if (!first) s = __uint_as_float(v[e]) + s;
+            if (last) s += __uint_as_float(w[e]);
+            u[e] = __float_as_uint(s);
+        }
+        ptx::tc_st_cols(sum + (uint32_t)c, u);
+    }
+    ptx::tc_st_wait();
 }
 
 // ---- bfloat16 storage ------------------------------------------------------------------------------

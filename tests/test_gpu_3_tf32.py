@@ -220,7 +220,7 @@ STRIDED_CASES = [
     (0, 5, 513, 7),         # a cluster, last k-block of one
     (0, 200, 150, 257),     # K % 4 != 0
     (0, 999, 66, 1001),     # more tiles than SMs
-    (0, 130, 4099, 61),     # three accumulators per slice
+    (0, 130, 4099, 61),     # segments of the sum in each slice of K
     (7, 199, 64, 199),
     (150, 17, 19, 23),      # more products than SMs
     (3, 40, 700, 30),       # a cluster per product
@@ -240,8 +240,21 @@ def test_matmul_of_unaligned_rows(ctx, oracle, case, ta, tb):
     ctx.check_device_status()
     assert same_bits(got + 0.0, want(a, b, ta, tb) + 0.0)
     a, b = si.uniform(322, 0, sa, -1, 1), si.uniform(322, 1, sb, -1, 1)
-    # the bar of the CUDA-core kernel: operands to 2^-21, at most 4099 / 8 / 3 additions per accumulator
+    # the bar of the CUDA-core kernel
     assert rel_fro(host(call(dev(a), dev(b), ta, tb)), want(a, b, ta, tb)) <= 1e-5
+
+
+@pytest.mark.parametrize("M,K,N,ta,tb", [(199, 64, 199, False, True), (301, 513, 303, True, True), (1301, 2001, 1303, False, False),
+                                         (1301, 8191, 1303, False, True), (257, 20001, 255, True, False)])
+@pytest.mark.parametrize("positive", [False, True])
+def test_unaligned_products_are_as_exact_as_fp32_multiply_adds(ctx, M, K, N, ta, tb, positive):
+    """Sums from 64 to 20001 products, whole and cut over clusters, of both signs and of one: the kernel that they ran on
+    before, fp32 multiply-adds in order, is 1.8e-8 sqrt(K) of the result off (2^-25 per addition, errors cancelling)."""
+    a, b = (si.uniform(324, i, s, 0.0 if positive else -1.0, 1.0) for i, s in ((0, (K, M) if ta else (M, K)), (1, (N, K) if tb else (K, N))))
+    want = (a.T if ta else a).astype(np.float64) @ (b.T if tb else b).astype(np.float64)
+    got = host(ctx.matmul(dev(a), dev(b), ta, tb))
+    ctx.check_device_status()
+    assert rel_fro(got, want) <= 1.8e-8 * K ** 0.5
 
 
 @pytest.mark.parametrize("classes", [1, 33, 101, 1001])

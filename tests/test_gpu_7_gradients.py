@@ -127,6 +127,25 @@ def test_conv2d_gradients_keep_fp32_accuracy_in_tf32_mode(ctx, oracle, case):
     assert rel_fro(df, oracle.conv2d_backprop_filter(x, f.shape, g, *args)) <= 1e-5
 
 
+@pytest.mark.parametrize("case", [(2, 14, 14, 16, 32, 3, 3, 1), (24, 28, 28, 64, 64, 3, 3, 1), (4, 14, 14, 512, 512, 3, 3, 1), (1, 20, 20, 256, 512, 5, 5, 1),
+                                  (2, 56, 56, 32, 64, 3, 3, 2)])
+def test_conv2d_gradients_are_as_exact_as_fp32_multiply_adds(ctx, oracle, case):
+    """Long sums too: the input gradient's are over taps and output channels, 288 to 12800 products, the filter gradient's
+    over pixels, of which a partial sum takes 1024 at least.  fp32 multiply-adds in order, the kernels before, are
+    1.8e-8 sqrt(K) off (2^-25 per addition, errors cancelling); the oracle's result is rounded to fp32 (2.5e-8)."""
+    N, H, W, Cin, Cout, fh, fw, s = case
+    Ho, Wo = geometry(oracle, H, W, fh, fw, s, 1, "same")
+    x = si.uniform(97, 0, (N, H, W, Cin), 0, 6)
+    f = si.normal(97, 1, (fh, fw, Cin, Cout), 0, float(np.sqrt(2.0 / (fh * fw * Cin))))
+    g = si.normal(97, 2, (N, Ho, Wo, Cout), 0, 1)
+    dx = host(ctx.conv2d_backprop_input(x.shape, dev(f), dev(g), (s, s), "same"))
+    df = host(ctx.conv2d_backprop_filter(dev(x), f.shape, dev(g), (s, s), "same"))
+    ctx.check_device_status()
+    products = fh * fw * Cout / (s * s)  # of the average residue class
+    assert rel_fro(dx, oracle.conv2d_backprop_input(x.shape, f, g, (s, s), "same")) <= 1.8e-8 * products ** 0.5 + 2.5e-8
+    assert rel_fro(df, oracle.conv2d_backprop_filter(x, f.shape, g, (s, s), "same")) <= 1.8e-8 * min(N * Ho * Wo, 1024) ** 0.5 + 2.5e-8
+
+
 SMALL_FILTER_CASES = [
     # N, H, W, Cin, Cout, fh, fw, stride, dilation, pad: windows of up to 32 elements
     (1, 3, 3, 3, 4, 3, 3, 1, 1, "same"),
