@@ -123,7 +123,9 @@ tfjsb_status tfjsb_window_out_shape(int64_t in, int k, int stride, int dilation,
  * TF32 mode uses the tensor-core kernel when K % 4 == 0 and N % 4 == 0 (row pitches must be
  * multiples of 16 bytes for the bulk tensor copies); operands that are not already K-contiguous
  * are transposed into context-owned scratch first (grown on demand without synchronising, see
- * tfjsb_reserve_scratch).  Other shapes, and FP32 mode, run on CUDA cores. */
+ * tfjsb_reserve_scratch).  Other shapes are fp32 products, on the tensor cores too (each operand as two TF32
+ * values: as exact as fp32 multiply-adds, with the same infinities and NaNs) up to K = 2^22, else, and in FP32
+ * mode, on CUDA cores. */
 tfjsb_status tfjsb_matmul(tfjsb_ctx* ctx, const tfjsb_tensor* a, const tfjsb_tensor* b, int transpose_a,
                           int transpose_b, tfjsb_tensor* out, void* stream);
 
@@ -228,8 +230,8 @@ tfjsb_status tfjsb_bias_act(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_t
  * not depend on scheduling.  1x1 / stride-1 convolutions run their two gradients as matrix products on
  * the tensor cores in TF32 mode (channel counts multiples of 4; for the filter gradient the pixel count
  * a multiple of 4).  Every other case is fp32 arithmetic: in TF32 mode on the tensor cores too where the
- * channel counts are multiples of 4 (each operand as two TF32 values, which keeps fp32 accuracy), on CUDA
- * cores otherwise and in FP32 mode.  All enqueue on `stream` and return;
+ * channel counts are multiples of 4 (each operand as two TF32 values and long sums in parts, which is as exact as
+ * fp32 multiply-adds, with the same infinities and NaNs), on CUDA cores otherwise and in FP32 mode.  All enqueue on `stream` and return;
  * the gradients use context-owned scratch (see tfjsb_reserve_scratch). */
 
 /* dx[n,iy,ix,ci] = sum over (oy,ky), (ox,kx) with oy*sh - pt + ky*dh = iy and ox*sw - pl + kx*dw = ix, and co,

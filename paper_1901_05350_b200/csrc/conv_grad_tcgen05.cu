@@ -81,6 +81,25 @@ __device__ __forceinline__ void tmem_free(uint32_t base, uint32_t cols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
 }
 
+// A row of 32 results, and where it lies in the slab: the ones that are not finite among the first `live` are asked for again.
+__device__ __forceinline__ bool row_not_finite(const uint32_t (&u)[32]) {
+    bool odd = false;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) odd = odd || not_finite(u[e]);
+    return odd;
+}
+template <typename F>
+__device__ __forceinline__ void mend_row(uint32_t slab, int lane, int live, F again) {
+    for (int e = 0; e < min(32, live); ++e) {
+        const uint32_t at = slab + (uint32_t)lane * 128u + (uint32_t)((((e >> 2) ^ (lane & 7)) << 4) + (e & 3) * 4);
+        uint32_t bits;
+        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(bits) : "r"(at) : "memory");
+        if (!not_finite(bits)) continue;
+        const float v = again(e);
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(at), "f"(v) : "memory");
+    }
+}
+
 // ---- input gradient --------------------------------------------------------------------------------------
 struct GradInputArgs {
     int H, W, Cin, Cout, fh, fw, sh, sw, dh, dw, pt, pl;  // the forward convolution's
@@ -89,6 +108,8 @@ struct GradInputArgs {
     long long M;             // N * Qh * Qw
     int m_tiles, n_tiles, block_n, stages, splits, num_tiles;
     int segment;             // k-blocks per accumulator of the large products
+    int Ho, Wo;
+    const float *dy, *f;     // for results that are not finite
     float* out;              // dx, or `splits` of them one after the other
     long long out_elems;
     unsigned int* dev_status;
@@ -116,8 +137,26 @@ __device__ __forceinline__ GradInputTile grad_input_tile(const GradInputArgs& g,
     return r;
 }
 
+// A result that is not finite once more: the tile's k-blocks of sample (n, qy, qx) of its class, channel ci, by fp32
+// multiply-adds.  Taps whose output pixel does not exist take no part (in the copied tiles they are zeros, which an
+// infinite filter value turns into NaN).
+__device__ __noinline__ float grad_input_in_fp32(const GradInputArgs& g, const GradInputTile& r, long long n, int qy, int qx, int ci) {
+    float acc = 0.f;
+    for (int kb = r.kb_begin; kb < r.kb_end; ++kb) {
+        const int tap = kb / r.c_blocks, co0 = (kb - tap * r.c_blocks) * BLOCK_K, jy = tap / r.taps_x, jx = tap - jy * r.taps_x;
+        const int oy = g.q0h + qy - jy * g.dh, ox = g.q0w + qx - jx * g.dw;
+        if (oy < 0 || oy >= g.Ho || ox < 0 || ox >= g.Wo) continue;
+        const float* dy = g.dy + ((n * g.Ho + oy) * (long long)g.Wo + ox) * g.Cout;
+        const float* f = g.f + ((long long)((r.a + jy * g.sh) * g.fw + r.b + jx * g.sw) * g.Cin + ci) * g.Cout;
+        for (int co = co0; co < min(co0 + BLOCK_K, g.Cout); ++co) acc = fmaf(__ldg(dy + co), __ldg(f + co), acc);
+        if (acc != acc) break;
+    }
+    return acc;
+}
+
 __global__ void __launch_bounds__(CG_THREADS, 1)
-conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_f, const GradInputArgs g) {
+conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_f,
+                         const __grid_constant__ GradInputArgs g) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[CG_MAX_STAGES], bar_split[CG_MAX_STAGES], bar_empty[CG_MAX_STAGES];
     __shared__ __align__(8) uint64_t bar_acc_full[2], bar_acc_empty[2], bar_small_empty, bar_drain;
@@ -240,13 +279,14 @@ conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __gri
             const GradInputTile r = grad_input_tile(g, t);
             const bool any = r.kb_begin != r.kb_end;
             // lane = one sample of dx: where its row of channels goes, or -1
-            long long at = -1;
+            long long at = -1, n = 0;
+            int qx = 0, qy = 0;
             const long long p = (long long)r.m0 + quad * 32 + lane;
             if (p < g.M) {
                 const long long row = p / g.Qw;
-                const int qx = (int)(p - row * g.Qw);
-                const long long n = row / g.Qh;
-                const int qy = (int)(row - n * g.Qh);
+                qx = (int)(p - row * g.Qw);
+                n = row / g.Qh;
+                qy = (int)(row - n * g.Qh);
                 const int iy = (g.q0h + qy) * g.sh + r.a - g.pt, ix = (g.q0w + qx) * g.sw + r.b - g.pl;
                 if (iy >= 0 && iy < g.H && ix >= 0 && ix < g.W) at = ((n * g.H + iy) * (long long)g.W + ix) * g.Cin;
             }
@@ -284,8 +324,10 @@ conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __gri
                 for (int j = 0; j < 8; ++j)
                     sts4(slab + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4), __uint_as_float(u[4 * j]), __uint_as_float(u[4 * j + 1]),
                          __uint_as_float(u[4 * j + 2]), __uint_as_float(u[4 * j + 3]));
-                __syncwarp();
                 const int col0 = r.n0 + c0;
+                if (any && at >= 0 && row_not_finite(u))
+                    mend_row(slab, lane, g.Cin - col0, [&](int e) { return grad_input_in_fp32(g, r, n, qy, qx, col0 + e); });
+                __syncwarp();
                 if (vec) {
                     // four rows per step, eight lanes to a row's 128 bytes
 #pragma unroll
@@ -353,13 +395,29 @@ struct GradFilterArgs {
     int m_tiles;
     int segment;    // k-blocks per accumulator of the large products
     int tiled;      // x as a matrix [pixels, Cin] (1x1, stride 1) instead of im2col copies
+    int H, W, Cin, Cout;
+    long long pixels;
+    const float *x, *dy;  // for results that are not finite
     unsigned int* dev_status;
 };
+
+// A result that is not finite once more: output pixels p0 .. p1 by fp32 multiply-adds, samples outside the image as zeros.
+__device__ __noinline__ float grad_filter_in_fp32(const GradFilterArgs& g, long long p0, long long p1, int tap, int ci, int co) {
+    const int ky = tap / g.fw, off_h = ky * g.dh - g.pt, off_w = (tap - ky * g.fw) * g.dw - g.pl;
+    float acc = 0.f;
+    for (long long p = p0; p < p1 && acc == acc; ++p) {
+        const long long row = p / g.Wo, n = row / g.Ho;
+        const int iy = (int)(row - n * g.Ho) * g.sh + off_h, ix = (int)(p - row * g.Wo) * g.sw + off_w;
+        const bool inside = iy >= 0 && iy < g.H && ix >= 0 && ix < g.W;
+        acc = fmaf(inside ? __ldg(g.x + ((n * g.H + iy) * (long long)g.W + ix) * g.Cin + ci) : 0.f, __ldg(g.dy + p * g.Cout + co), acc);
+    }
+    return acc;
+}
 
 template <bool SPLIT>
 __global__ void __launch_bounds__(CG_THREADS, 1)
 conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_dy,
-                          const __grid_constant__ CUtensorMap map_out, const GradFilterArgs g) {
+                          const __grid_constant__ CUtensorMap map_out, const __grid_constant__ GradFilterArgs g) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_raw_full[CG_MAX_STAGES], bar_raw_empty[CG_MAX_STAGES];
     __shared__ __align__(8) uint64_t bar_op_full[CG_MAX_STAGES], bar_op_empty[CG_MAX_STAGES];
@@ -520,6 +578,10 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
                 for (int j = 0; j < 8; ++j)
                     sts4(slab + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) << 4), __uint_as_float(u[4 * j]), __uint_as_float(u[4 * j + 1]),
                          __uint_as_float(u[4 * j + 2]), __uint_as_float(u[4 * j + 3]));
+                if (SPLIT && ci0 + lane < g.Cin && row_not_finite(u)) {
+                    const long long p0 = (long long)pb0 * 32, p1 = min(g.pixels, p0 + kbs * 32LL);
+                    mend_row(slab, lane, g.Cout - n0 - c0, [&](int e) { return grad_filter_in_fp32(g, p0, p1, tap, ci0 + lane, n0 + c0 + e); });
+                }
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
@@ -680,6 +742,8 @@ tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float*
     a.stages = (CG_SMEM - 1024 - EPI_WARPS * EPI_SLAB_BYTES) / stage_bytes;
     if (a.stages > CG_MAX_STAGES) a.stages = CG_MAX_STAGES;
     a.out_elems = (long long)g.N * g.H * g.W * g.C;
+    a.Ho = g.Ho; a.Wo = g.Wo;
+    a.dy = dy; a.f = f;
     a.dev_status = ctx->dev_status;
     tfjsb_status st;
     a.out = dx;
@@ -721,6 +785,9 @@ tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float*
     const int64_t pixels = g.N * g.Ho * g.Wo;
     a.taps = g.fh * g.fw; a.fw = g.fw; a.sh = g.sh; a.sw = g.sw; a.dh = g.dh; a.dw = g.dw; a.pt = g.pt; a.pl = g.pl;
     a.Ho = g.Ho; a.Wo = g.Wo;
+    a.H = g.H; a.W = g.W; a.Cin = g.C; a.Cout = g.Co;
+    a.pixels = pixels;
+    a.x = x; a.dy = dy;
     a.c_blocks = (g.C + 31) / 32;
     a.groups = a.taps * a.c_blocks;
     a.m_tiles = (a.groups + 3) / 4;

@@ -103,6 +103,13 @@ struct Fetch {
     }
 };
 
+// One element over k0 .. k1 by fp32 multiply-adds.
+__device__ __noinline__ float sum_in_fp32(const float* p, const float* q, int p_step, int q_step, int k0, int k1) {
+    float acc = 0.f;
+    for (int k = k0; k < k1 && acc == acc; ++k) acc = fmaf(__ldg(p + (long long)k * p_step), __ldg(q + (long long)k * q_step), acc);
+    return acc;
+}
+
 template <int BN>
 __global__ void __launch_bounds__(GS_THREADS, 2)
 gemm_strided_kernel(const StridedArgs g) {
@@ -250,8 +257,21 @@ gemm_strided_kernel(const StridedArgs g) {
                 tc_ld_32x32(lanes + 3 * BN, u);
                 tc_ld_wait();
                 const uint32_t row = base + (uint32_t)(((quad * 32 + lane) * PITCH + c0) * 4);
+                bool odd = false;
 #pragma unroll
-                for (int e = 0; e < 32; ++e) asm volatile("st.shared.b32 [%0], %1;" ::"r"(row + 4u * e), "r"(u[e]) : "memory");
+                for (int e = 0; e < 32; ++e) {
+                    odd = odd || not_finite(u[e]);
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(row + 4u * e), "r"(u[e]) : "memory");
+                }
+                const int pr = p0 + quad * 32 + lane;
+                for (int e = 0; odd && pr < g.p.rows && e < min(32, g.q.rows - q0 - c0); ++e) {
+                    uint32_t bits;
+                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(bits) : "r"(row + 4u * e) : "memory");
+                    if (!not_finite(bits)) continue;
+                    const float again = sum_in_fp32(pb + (long long)pr * g.p.row_stride, qb + (long long)(q0 + c0 + e) * g.q.row_stride, g.p.k_stride,
+                                                    g.q.k_stride, kb0 * BLOCK_K, min(g.K, kb1 * BLOCK_K));
+                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(row + 4u * e), "f"(again) : "memory");
+                }
             }
             tc_fence_before();
         }

@@ -87,6 +87,12 @@ inline int split_segment(int64_t K) {
 // Of longer sums the small products' accumulator would be the less exact part.
 constexpr int64_t SPLIT_MAX_K = 1LL << 22;
 
+// What is not finite may be a result of the split: with an infinite operand lo is NaN or the opposite infinity, a value
+// above the largest TF32 number is rounded to infinity, and a NaN with low bits only is cut to infinity.  Such a result is
+// summed again in fp32 by the thread that has it, as the CUDA-core kernels do.  (A result that is finite had none of these
+// among its operands: every one of them leaves an infinity or a NaN in hi or in lo.)
+__device__ __forceinline__ bool not_finite(uint32_t bits) { return (bits & 0x7f800000u) == 0x7f800000u; }
+
 // One 32-lane x `cols`-column part of  sum = (first ? 0 : sum) + large, and + small after the last segment; both addresses
 // and `cols` (a multiple of STEP, 8 or 16) are of the caller's lanes and columns.
 template <int STEP>

@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 
 import seeded_inputs as si
-from helpers import dev, host, rel_fro, same_bits
+from helpers import dev, host, plant_specials, rel_fro, same_bits, same_classes
 
 pytestmark = pytest.mark.gpu
 
@@ -255,6 +255,28 @@ def test_unaligned_products_are_as_exact_as_fp32_multiply_adds(ctx, M, K, N, ta,
     got = host(ctx.matmul(dev(a), dev(b), ta, tb))
     ctx.check_device_status()
     assert rel_fro(got, want) <= 1.8e-8 * K ** 0.5
+
+
+@pytest.mark.parametrize("case", [(0, 5, 3, 7), (0, 64, 70, 101), (0, 200, 150, 257), (0, 40, 1030, 33), (7, 50, 64, 51)])
+@pytest.mark.parametrize("ta,tb", [(False, False), (True, True)])
+def test_unaligned_products_of_values_that_are_not_finite(ctx, case, ta, tb):
+    """The same infinities and NaNs as fp32 multiply-adds give, and finite results beside them (the largest number is above
+    the largest TF32 number, a NaN with low bits only below the smallest TF32 NaN)."""
+    B, M, K, N = case
+    lead = (B,) if B else ()
+    a = si.uniform(325, 0, lead + ((K, M) if ta else (M, K)), -0.5, 0.5)
+    b = si.uniform(325, 1, lead + ((N, K) if tb else (K, N)), -0.5, 0.5)
+    call = ctx.batch_matmul if B else ctx.matmul
+    for x, y in ((plant_specials(a, 1), b), (a, plant_specials(b, 2)), (plant_specials(a, 3), plant_specials(b, 4, largest=False)),
+                 (np.full_like(a, np.inf), b), (np.full_like(a, np.nan), b)):
+        got = host(call(dev(x), dev(y), ta, tb))
+        ctx.set_math("fp32")
+        try:
+            want = host(call(dev(x), dev(y), ta, tb))
+        finally:
+            ctx.set_math("tf32")
+        assert same_classes(got, want)
+    ctx.check_device_status()
 
 
 @pytest.mark.parametrize("classes", [1, 33, 101, 1001])

@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 import seeded_inputs as si
-from helpers import dev, host, rel_fro, same_bits
+from helpers import dev, host, plant_specials, rel_fro, same_bits, same_classes
 
 pytestmark = pytest.mark.gpu
 
@@ -144,6 +144,35 @@ def test_conv2d_gradients_are_as_exact_as_fp32_multiply_adds(ctx, oracle, case):
     products = fh * fw * Cout / (s * s)  # of the average residue class
     assert rel_fro(dx, oracle.conv2d_backprop_input(x.shape, f, g, (s, s), "same")) <= 1.8e-8 * products ** 0.5 + 2.5e-8
     assert rel_fro(df, oracle.conv2d_backprop_filter(x, f.shape, g, (s, s), "same")) <= 1.8e-8 * min(N * Ho * Wo, 1024) ** 0.5 + 2.5e-8
+
+
+@pytest.mark.parametrize("case", [SPLIT_CASES[i] for i in (0, 2, 4, 5, 7, 9, 11, 12)])
+@pytest.mark.parametrize("planted", ["x", "f", "g", "all"])
+def test_conv2d_gradients_of_values_that_are_not_finite(ctx, oracle, case, planted):
+    """The same infinities and NaNs as the CUDA-core kernels give, also at the border, where the copied tiles hold zeros for
+    what does not exist: an infinite filter value reaches no sample through a tap that it does not meet."""
+    N, H, W, Cin, Cout, fh, fw, s, d, pad = case
+    Ho, Wo = geometry(oracle, H, W, fh, fw, s, d, pad)
+    args = ((s, s), pad, (d, d))
+    x, f, g = si.uniform(98, 0, (N, H, W, Cin), -1, 1), si.normal(98, 1, (fh, fw, Cin, Cout), 0, 0.2), si.normal(98, 2, (N, Ho, Wo, Cout), 0, 0.5)
+    if planted in ("x", "all"):
+        x = plant_specials(x, 5, (0, x.size - 1), planted != "all")
+    if planted in ("f", "all"):
+        f = plant_specials(f, 6, (0, f.size - 1), planted != "all")
+    if planted in ("g", "all"):
+        g = plant_specials(g, 7, (0, g.size - 1), planted != "all")
+
+    def both():
+        return (host(ctx.conv2d_backprop_input(x.shape, dev(f), dev(g), *args)), host(ctx.conv2d_backprop_filter(dev(x), f.shape, dev(g), *args)))
+
+    got = both()
+    ctx.check_device_status()
+    ctx.set_math("fp32")
+    try:
+        want = both()
+    finally:
+        ctx.set_math("tf32")
+    assert same_classes(got[0], want[0]) and same_classes(got[1], want[1])
 
 
 SMALL_FILTER_CASES = [
