@@ -318,6 +318,23 @@ depthwise3x3_s2_backprop_input_kernel(const float* __restrict__ dy, const float*
         b[j] = row && r < g.Wo ? __ldg(reinterpret_cast<const float4*>(p)) : zero;
     }
     float* out = dx + n * (int64_t)g.H * g.W * g.C + c;
+    // a filter that is not finite: only taps that meet an output pixel take part, where the zeros make NaNs of the others
+    bool odd = false;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) odd = odd || !finite4(w[t]);
+    for (int e = 0; odd && e < 4 * ROWS; ++e) {
+        const int iy = 2 * (q0 + (e >> 2)) - g.pt + ((e >> 1) & 1), jx = ix + (e & 1);
+        if (iy < 0 || iy >= g.H || jx < 0 || jx >= g.W) continue;
+        float4 v = zero;
+        for (int t = 0; t < 9; ++t) {
+            const int oy = source_of(iy, g.pt, t / 3, 1, 2, g.Ho), ox = source_of(jx, g.pl, t % 3, 1, 2, g.Wo);
+            if (oy < 0 || ox < 0) continue;
+            fma4_packed(v, __ldg(reinterpret_cast<const float4*>(gy + ((int64_t)oy * g.Wo + ox) * g.C)),
+                        __ldg(reinterpret_cast<const float4*>(f + (int64_t)t * g.C + c)));
+        }
+        *reinterpret_cast<float4*>(out + ((int64_t)iy * g.W + jx) * g.C) = v;
+    }
+    if (odd) return;
 #pragma unroll
     for (int j = 1; j <= ROWS; ++j) {
         const int iy = 2 * (q0 + j - 1) - g.pt;

@@ -92,6 +92,10 @@ __device__ __forceinline__ float apply_act_t(float v) {
     return relu_nan(v);
 }
 
+__device__ __forceinline__ bool finite4(const float4& v) {
+    return isfinite(v.x) && isfinite(v.y) && isfinite(v.z) && isfinite(v.w);
+}
+
 // ---- context --------------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -373,6 +377,7 @@ tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float*
 // shape is one of its own.  `partial` holds slices * 9 * C floats (unused when slices == 1).
 struct DepthwiseGradPlan {
     CUtensorMap map_x, map_dy;
+    const float *x = nullptr, *dy = nullptr;
     ConvGeom g{};
     int variant = 0, th = 0, tw = 0, thin = 0, twin = 0, stage_bytes = 0, stages = 0;
     int tiles_x = 0, tiles_y = 0, c_blocks = 0, num_tiles = 0, slices = 0;

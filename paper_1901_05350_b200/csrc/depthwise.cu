@@ -43,10 +43,26 @@ __device__ __forceinline__ void fma4(float4& acc, const float4& a, const float4&
     acc.z = fmaf(a.z, b.z, acc.z); acc.w = fmaf(a.w, b.w, acc.w);
 }
 
+// Four channels of one result of the input gradient (the taps reversed: f at the last, f_step to the one before), for a
+// filter that is not finite: taps that meet no output pixel take no part, where a zero sample would make a NaN of them.
+__device__ __noinline__ float4 gradient_of_existing(const float* x, const float* f, int f_step, const ConvGeom& g, int64_t n, int oy, int ox, int c) {
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int ky = 0; ky < 3; ++ky) {
+        const int iy = oy - g.pt + ky * g.dh;
+        if (iy < 0 || iy >= g.H) continue;
+        for (int kx = 0; kx < 3; ++kx) {
+            const int ix = ox - g.pl + kx * g.dw;
+            if (ix < 0 || ix >= g.W) continue;
+            fma4(acc, ld4(x + ((n * g.H + iy) * (int64_t)g.W + ix) * g.C + c), ld4(f + (int64_t)(3 * ky + kx) * f_step + c));
+        }
+    }
+    return acc;
+}
+
 template <int S, int ROWS, int D = 1>
 __global__ void __launch_bounds__(DW_THREADS)
 depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ f, const float* __restrict__ bias,
-                    int act, float* __restrict__ y, ConvGeom g, int tc, int c4_tiles) {
+                    int act, float* __restrict__ y, const __grid_constant__ ConvGeom g, int tc, int c4_tiles) {
     // block = tx_count output columns x tc channel quads
     const int C4 = g.C >> 2;
     const int tx_count = DW_THREADS / tc;
@@ -110,6 +126,11 @@ depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ f, co
             *reinterpret_cast<float4*>(y + ((n * g.Ho + oy) * (int64_t)g.Wo + ox) * g.Co + c) = v;
         }
     }
+    if (!g.reversed) return;
+    bool odd = false;  // (a gradient has neither bias nor activation)
+    for (int t = 0; t < 9; ++t) odd = odd || !finite4(ld4(f + (int64_t)t * f_step + c));
+    for (int oy = oy0; odd && oy < min(g.Ho, oy0 + ROWS); ++oy)
+        *reinterpret_cast<float4*>(y + ((n * g.Ho + oy) * (int64_t)g.Wo + ox) * g.Co + c) = gradient_of_existing(x, f, f_step, g, n, oy, ox, c);
 }
 
 __global__ void depthwise_generic_kernel(const float* __restrict__ x, const float* __restrict__ f,
@@ -212,11 +233,12 @@ constexpr int DW_TMA_THREADS = DW_THREADS + 32;  // eight compute warps and the 
 
 // NARROW: the input is bfloat16 (the patch is copied as such and multiplied as such, with the filter, whose
 // values a narrow model has rounded to bfloat16; bias and sums are fp32, in the same order) and the output is bfloat16 or, with y_f32, fp32.
-template <int S, int TW, int R, int D = 1, int CB = DW_CB, bool NARROW = false>
+// GRADIENT: the forward pass over dy that is the input gradient; `x` is the tensor itself, for filters that are not finite.
+template <int S, int TW, int R, int D = 1, int CB = DW_CB, bool NARROW = false, bool GRADIENT = false>
 __global__ void __launch_bounds__(DW_TMA_THREADS, 2)
-depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* __restrict__ f,
-                        const float* __restrict__ bias, int act, void* __restrict__ y, int y_f32, ConvGeom g, DwTiling t,
-                        unsigned int* dev_status) {
+depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* __restrict__ x, const float* __restrict__ f,
+                        const float* __restrict__ bias, int act, void* __restrict__ y, int y_f32, const __grid_constant__ ConvGeom g,
+                        const __grid_constant__ DwTiling t, unsigned int* dev_status) {
     using T = DwTile<S, TW, R, D, CB, NARROW>;
     extern __shared__ uint8_t dw_smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[DW_MAX_STAGES];   // copy landed (1 arrival + bytes)
@@ -303,6 +325,7 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
     typedef typename DwQuad<NARROW>::type Quad;
     Quad w[9];
     float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool odd = false;  // a filter that is not finite
     int loaded_cb = -1;
     int slot = 0;
     uint32_t parity = 0;
@@ -325,6 +348,10 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
                 for (int k = 0; k < 9; ++k)
                     dw_tap(w[k], __ldg(reinterpret_cast<const float4*>(f + (int64_t)k * t.f_step + c)));
                 if (bias) b = __ldg(reinterpret_cast<const float4*>(bias + c));
+                if constexpr (GRADIENT) {
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) odd = odd || !finite4(w[k]);
+                }
                 loaded_cb = cb;
             }
             float4 acc[R];
@@ -361,6 +388,19 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
             if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&bar_empty[slot]));
         }
         if (++slot == t.stages) { slot = 0; parity ^= 1u; }
+    }
+    if (GRADIENT && odd) {
+        // This thread's results once more, apart from the loop above, whose registers a call would take.  (A gradient has
+        // neither bias nor activation.)
+        for (int i = 0; i < my_tiles; ++i) {
+            const int tile = first + i * step, c = (tile % t.c_blocks) * CB + c4 * 4;
+            int q = tile / t.c_blocks, tx = q % t.tiles_x;
+            q /= t.tiles_x;
+            const int ox = (tx + q) % t.tiles_x * TW + col, n = q / t.tiles_y, oy0 = q % t.tiles_y * T::TH + rg * R;
+            for (int oy = oy0; c < g.C && ox < g.Wo && oy < min(g.Ho, oy0 + R); ++oy)
+                *reinterpret_cast<float4*>(static_cast<float*>(y) + (((int64_t)n * g.Ho + oy) * g.Wo + ox) * g.Co + c) =
+                    gradient_of_existing(x, f, t.f_step, g, n, oy, ox, c);
+        }
     }
 }
 
@@ -400,20 +440,23 @@ constexpr int DW_FIRST_NARROW = 9;
 constexpr int DW_SMEM_BUDGET = 113 * 1024;  // two CTAs per SM
 
 template <int S, int TW, int R, int D = 1, int CB = DW_CB, bool NARROW = false>
-cudaError_t launch_tma_instance(const DepthwisePlan& plan, const float* f, const float* bias, int act, void* y, bool y_f32,
+cudaError_t launch_tma_instance(const DepthwisePlan& plan, const float* x, const float* f, const float* bias, int act, void* y, bool y_f32,
                                 const ConvGeom& g, unsigned int* dev_status, cudaStream_t s) {
     auto kernel = depthwise3x3_tma_kernel<S, TW, R, D, CB, NARROW>;
+    if constexpr (S == 1 && !NARROW) {
+        if (g.reversed) kernel = depthwise3x3_tma_kernel<S, TW, R, D, CB, NARROW, true>;
+    }
     cudaError_t ae = smem_attr_once(reinterpret_cast<const void*>(kernel), DW_SMEM_BUDGET);
     if (ae != cudaSuccess) return ae;
     DwTiling t{plan.tiles_x, plan.tiles_y, plan.c_blocks, plan.stages, (long long)plan.num_tiles, g.reversed ? -g.C : g.C};
     if (g.reversed) f += 8 * (int64_t)g.C;
-    return launch_k(kernel, dim3(plan.grid), dim3(DW_TMA_THREADS), plan.smem_bytes, s, plan.map_x, f, bias, act, y,
+    return launch_k(kernel, dim3(plan.grid), dim3(DW_TMA_THREADS), plan.smem_bytes, s, plan.map_x, x, f, bias, act, y,
                     y_f32 ? 1 : 0, g, t, dev_status);
 }
 
-cudaError_t launch_tma_variant(const DepthwisePlan& plan, const float* f, const float* bias, int act, void* y, bool y_f32,
+cudaError_t launch_tma_variant(const DepthwisePlan& plan, const float* x, const float* f, const float* bias, int act, void* y, bool y_f32,
                                const ConvGeom& g, unsigned int* dev_status, cudaStream_t s) {
-#define DW_CASE(V, ...) case V: return launch_tma_instance<__VA_ARGS__>(plan, f, bias, act, y, y_f32, g, dev_status, s)
+#define DW_CASE(V, ...) case V: return launch_tma_instance<__VA_ARGS__>(plan, x, f, bias, act, y, y_f32, g, dev_status, s)
     switch (plan.variant) {
         DW_CASE(0, 1, 16, 7, 1, 32, false);
         DW_CASE(1, 1, 8, 2, 1, 32, false);
@@ -516,7 +559,7 @@ cudaError_t launch_depthwise(const DepthwisePlan& plan, const float* x, const fl
     if (n_out == 0) return cudaSuccess;
     if (plan.variant >= 0) {
         if (plan.narrow) return cudaErrorInvalidValue;  // a plan made for bfloat16 storage: launch_depthwise_tma_narrow
-        cudaError_t e = launch_tma_variant(plan, f, bias, act, y, true, g, dev_status, s);
+        cudaError_t e = launch_tma_variant(plan, x, f, bias, act, y, true, g, dev_status, s);
         ++*launches;
         return e;
     }
@@ -558,7 +601,7 @@ cudaError_t launch_depthwise_tma_narrow(const DepthwisePlan& plan, const float* 
                                         int64_t* launches) {
     if (g.N * g.Ho * g.Wo * g.Co == 0) return cudaSuccess;
     if (plan.variant < DW_FIRST_NARROW || !plan.narrow) return cudaErrorInvalidValue;
-    cudaError_t e = launch_tma_variant(plan, f, bias, act, y, !y_is_bf16, g, dev_status, s);
+    cudaError_t e = launch_tma_variant(plan, nullptr, f, bias, act, y, !y_is_bf16, g, dev_status, s);
     ++*launches;
     return e;
 }

@@ -37,10 +37,39 @@ struct DgTiling {
     int tiles_x, tiles_y, c_blocks, stages, num_tiles;
 };
 
+// The tensors themselves, for sums that are not finite.
+struct DgTensors {
+    const float *x, *dy;
+    int H, W, Ho, Wo;
+};
+
+// A sum that is not finite once more, over the CTA's tiles: products with samples that do not exist take no part, where
+// the zeros that were copied for them make NaNs of infinite values of dy.
+__device__ __noinline__ float sum_of_existing(const DgTensors& d, const DgTiling& t, int S, int TH, int TW, int C, int pt, int pl, int c, int tap,
+                                              int first, int step) {
+    const int off_y = tap / 3 - pt, off_x = tap % 3 - pl;
+    float acc = 0.f;
+    for (int tile = first; tile < t.num_tiles; tile += step) {
+        int q = tile / t.c_blocks;
+        const int tx = q % t.tiles_x; q /= t.tiles_x;
+        const int ty = q % t.tiles_y;
+        const int64_t n = q / t.tiles_y;
+        for (int oy = ty * TH; oy < min(d.Ho, (ty + 1) * TH); ++oy)
+            for (int ox = tx * TW; ox < min(d.Wo, (tx + 1) * TW); ++ox) {
+                const int iy = oy * S + off_y, ix = ox * S + off_x;
+                if (iy < 0 || iy >= d.H || ix < 0 || ix >= d.W) continue;
+                acc = fmaf(__ldg(d.x + ((n * d.H + iy) * d.W + ix) * C + c), __ldg(d.dy + ((n * d.Ho + oy) * d.Wo + ox) * C + c), acc);
+            }
+        if (acc != acc) break;
+    }
+    return acc;
+}
+
 template <int S, int TW, int R>
 __global__ void __launch_bounds__(DG_ALL_THREADS, 2)
 depthwise3x3_backprop_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_dy,
-                                    float* __restrict__ partial, int C, int pt, int pl, DgTiling t, unsigned int* dev_status) {
+                                    float* __restrict__ partial, int C, int pt, int pl, const __grid_constant__ DgTiling t,
+                                    const __grid_constant__ DgTensors d, unsigned int* dev_status) {
     using T = DgTile<S, TW, R>;
     extern __shared__ uint8_t dg_smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[DG_MAX_STAGES], bar_empty[DG_MAX_STAGES];
@@ -158,6 +187,11 @@ depthwise3x3_backprop_filter_kernel(const __grid_constant__ CUtensorMap map_x, c
             const float4 v = red[w][k][tid % DG_QUADS];
             s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
         }
+        if (!finite4(s)) {
+            float* v = &s.x;
+            for (int e = 0; e < 4; ++e)
+                if (!isfinite(v[e])) v[e] = sum_of_existing(d, t, S, T::TH, TW, C, pt, pl, c + e, k, first, step);
+        }
         *reinterpret_cast<float4*>(partial + ((int64_t)(first / t.c_blocks) * 9 + k) * C + c) = s;
     }
 }
@@ -174,8 +208,9 @@ cudaError_t launch_instance(const DepthwiseGradPlan& p, float* out, unsigned int
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kernel), DG_SMEM_BUDGET);
     if (e != cudaSuccess) return e;
     const DgTiling t{p.tiles_x, p.tiles_y, p.c_blocks, p.stages, p.num_tiles};
+    const DgTensors d{p.x, p.dy, p.g.H, p.g.W, p.g.Ho, p.g.Wo};
     kernel<<<p.slices * p.c_blocks, DG_ALL_THREADS, (size_t)p.stages * p.stage_bytes + 128, s>>>(p.map_x, p.map_dy, out, p.g.C, p.g.pt,
-                                                                                                p.g.pl, t, dev_status);
+                                                                                                p.g.pl, t, d, dev_status);
     return cudaGetLastError();
 }
 
@@ -195,6 +230,7 @@ bool depthwise_grad_plan(tfjsb_ctx* ctx, const float* x, const float* dy, const 
     if (g.fh != 3 || g.fw != 3 || g.mult != 1 || g.sh != g.sw || g.sh > 2 || g.dh != 1 || g.dw != 1 || g.C % 4 != 0 || !ctx->encode_tiled)
         return false;
     p->g = g;
+    p->x = x; p->dy = dy;
     // eight columns per tile where that wastes fewer of them
     const bool narrow = (g.Wo + 7) / 8 * 8 < (g.Wo + 15) / 16 * 16;
     p->variant = (g.sh == 1 ? 0 : 2) + (narrow ? 1 : 0);

@@ -239,6 +239,28 @@ def test_depthwise_3x3_gradients_at_tile_edges(ctx, oracle, case):
     assert same_bits(df + 0.0, oracle.depthwise_conv2d_backprop_filter(x, f.shape, g, (s, s), pad, (d, d)) + 0.0)
 
 
+@pytest.mark.parametrize("case", [DEPTHWISE_3X3_CASES[i] for i in (0, 1, 2, 3, 4, 5, 7, 8, 9, 10)])
+@pytest.mark.parametrize("planted", ["x", "f", "g", "all"])
+def test_depthwise_3x3_gradients_of_values_that_are_not_finite(ctx, oracle, case, planted):
+    """A sample that does not exist takes part in no sum: an infinite dy at the border, or an infinite filter value, makes no
+    NaN of it."""
+    N, H, W, C, s, d, pad = case
+    Ho, Wo = geometry(oracle, H, W, 3, 3, s, d, pad)
+    args = ((s, s), pad, (d, d))
+    x, f, g = si.uniform(99, 0, (N, H, W, C), -1, 1), si.normal(99, 1, (3, 3, C, 1), 0, 0.3), si.normal(99, 2, (N, Ho, Wo, C), 0, 0.5)
+    if planted in ("x", "all"):
+        x = plant_specials(x, 5, (0, x.size - 1), planted != "all")
+    if planted in ("f", "all"):
+        f = plant_specials(f, 6, (0, f.size - 1), planted != "all")
+    if planted in ("g", "all"):
+        g = plant_specials(g, 7, (0, g.size - 1), planted != "all")
+    dx = host(ctx.depthwise_conv2d_backprop_input(x.shape, dev(f), dev(g), *args))
+    df = host(ctx.depthwise_conv2d_backprop_filter(dev(x), f.shape, dev(g), *args))
+    ctx.check_device_status()
+    assert same_classes(dx, oracle.depthwise_conv2d_backprop_input(x.shape, f, g, *args))
+    assert same_classes(df, oracle.depthwise_conv2d_backprop_filter(x, f.shape, g, *args))
+
+
 @pytest.mark.parametrize("shape", [(1, 1), (1024, 3), (1025, 32), (5000, 101), (3000, 8192), (40, 3, 7, 4), (1 << 17, 4), (70001, 36)])
 def test_bias_gradient_slices(ctx, oracle, shape):
     dz = si.small_integers(92, 0, shape, -8, 8)  # |sums| <= 8 * 2^17: exact in any order
