@@ -338,7 +338,7 @@ tfjsb_status tfjsb_model_set_fusion(tfjsb_model* model, int mode);
  * program is what the paper's async design hides, Sec. 4.1.1; a graph removes it from the host).
  * The graph is captured on a private stream at the next tfjsb_run_model, for the input / output
  * buffers of that call, and re-captured when they change.  Run the model once without the graph
- * first.  Off by default. */
+ * first.  Off by default.  A run of at most three kernels is launched as it is in this mode too. */
 tfjsb_status tfjsb_model_set_graph(tfjsb_model* model, int use_graph);
 
 /* Debug aid (the paper's debug mode downloads every intermediate, Sec. 3.8): a view of the

@@ -452,6 +452,11 @@ tfjsb_model* make_batch_view(tfjsb_model* parent, int64_t n) {
 cudaError_t launch_layers(tfjsb_model* m, int i, cudaStream_t s, int* consumed);
 int launches_per_run(const tfjsb_model* m);
 
+// Runs of up to this many kernels are launched as they are in graph mode too: a graph saves a launch's 2 us on the host per
+// kernel, but its replay starts later, and every new buffer costs an instantiation.  Small models as one kernel, with pool,
+// dense or softmax after it (width 0.25, 32 images of 128 x 128, three kernels: 94.2 us launched, 96.3 replayed).
+constexpr int GRAPH_MIN_LAUNCHES = 3;
+
 void drop_graph(tfjsb_model* m) {
     if (m->graph_exec) {
         cudaGraphExecDestroy(m->graph_exec);
@@ -850,7 +855,7 @@ tfjsb_status tfjsb_run_model(tfjsb_model* m, const tfjsb_tensor* input, tfjsb_te
         drop_graph(m);  // the captured launches point at the old buffers
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (m->use_graph) {
+    if (m->use_graph && launches_per_run(m) > GRAPH_MIN_LAUNCHES) {
         if (!m->graph_exec && (st = capture_graph(m)) != TFJSB_OK) return st;
         cudaError_t e = cudaGraphLaunch(m->graph_exec, s);
         if (e != cudaSuccess) return cuda_fail(m->ctx, e, "cudaGraphLaunch");

@@ -329,3 +329,29 @@ def test_outputs_that_survive_a_run_in_one_kernel(ctx, batch, hw, alpha, tail, m
         assert len(np.unique(own)) > 4 and same_bits(got, own), layers[i].name
     assert np.max(np.abs(out - want)) <= 1e-6 if tail == 30 else same_bits(out, want)  # exp() is not exact
     model.close()
+
+
+def test_one_kernel_models_launch_their_kernel_in_graph_mode_too(ctx):
+    """A run of one kernel leaves a graph nothing to save, and costs its instantiation for every new buffer: in graph mode it
+    is launched as it is.  Seen from outside: it can be recorded into a graph of the caller's, which a replay cannot."""
+    import torch
+
+    x, layers = si.config_mobilenet(0.25, 64, 2, seed=4243, classes=20)
+    model = ctx.model(layers, x.shape)
+    xd, out = dev(x), torch.empty(model.output_shape, device="cuda")
+    model.run(xd, out=out)
+    assert model.launches_per_run == 1
+    plain = host(out).copy()
+    model.set_graph(True)
+    model.run(xd, out=out)
+    assert same_bits(host(out), plain)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        model.run(xd, out=out)
+    out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert same_bits(host(out), plain)
+    ctx.check_device_status()
+    del graph
+    model.close()
