@@ -304,10 +304,10 @@ tfjsb_status tfjsb_run_model(tfjsb_model* model, const tfjsb_tensor* input, tfjs
 
 /* The same run from HOST memory: copies `host_input` (input-shape fp32, ideally pinned) to the
  * device, runs the model, copies the output to `host_output`, and synchronises `stream` before
- * returning (the blocking dataSync() of Sec. 3.6).  Batches of 24 images or more are pipelined in two
- * to four slices: slice c+1 is copied on an internal stream while slice c is computed
- * on `stream` as a graph replay (images are independent, so the result is that of the whole-batch
- * run). */
+ * returning (the blocking dataSync() of Sec. 3.6).  A batch whose copy and computation are both long is
+ * pipelined in two to four slices: slice c+1 is copied on an internal stream while slice c is computed on
+ * `stream` as a graph replay.  Images are independent, so the result is that of the whole-batch run, up to
+ * the order of fp32 sums: kernels are chosen by the slice's batch. */
 tfjsb_status tfjsb_run_model_host(tfjsb_model* model, const float* host_input, float* host_output, void* stream);
 
 /* The asynchronous form of the same run (the data() promise of Sec. 3.6 beside the blocking

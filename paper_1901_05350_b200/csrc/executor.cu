@@ -89,11 +89,14 @@ struct tfjsb_model {
     // Host-buffer runs pipeline the batch in slices: slice c+1 is copied to the device on a stream
     // of its own while slice c is computed.  Each slice has a view of this model with a smaller
     // batch: the same weights and arena, its own shapes, plans and fixed staging addresses.  There is
-    // one set of views and events per staging buffer: entry b * n_slices + c.
-    std::vector<tfjsb_model*> slices;
-    std::vector<cudaEvent_t> slice_copied;
-    int n_slices = 0;
-    std::vector<int64_t> slice_images;  // images of each slice
+    // one set of views and events per staging buffer: entry b * count + c.
+    struct HostSlices {
+        std::vector<tfjsb_model*> views;
+        std::vector<cudaEvent_t> copied;
+        std::vector<int64_t> images;  // of each slice
+        int count = 0;
+    };
+    HostSlices host_slices[2];          // for the blocking call and for the asynchronous one
     int fusion_mode = 1;                // tfjsb_model_set_fusion
     int chain_len = 0;                  // the first layers that run as one kernel (0: none), outside keep-all mode
     ChainPlan chain;
@@ -296,11 +299,11 @@ bool fusion_pays(const tfjsb_model* m, const Step& dw) {
 // What a layer takes as a kernel of its own, in ns: about 4 us however small it is, and its bytes.  Within 10 % of the
 // measured sums of small models (30 layers: 102 to 112 us for one image, 132 for 32 and 205 for 128 images of 128 x 128
 // at a width of 0.25); too low for large layers, whose products take longer, which only keeps the chain away from them.
+constexpr double LAYER_FIXED_NS = 3800, LAYER_BYTES_PER_NS = 4000;
+double layer_bytes(const tfjsb_model* m, double values) { return (m->narrow ? 2 : 4) * values; }
 double separate_ns(const tfjsb_model* m, const Step& st) {
-    const double width = m->narrow ? 2 : 4;
     const double in = st.kind == STEP_SOFTMAX || st.K ? (double)st.M * (st.K ? st.K : st.N) : (double)st.g.N * st.g.H * st.g.W * st.g.C;
-    const double bytes = width * (in + (double)st.out_elems);
-    return 3800 + bytes / 4000;
+    return LAYER_FIXED_NS + layer_bytes(m, in + (double)st.out_elems) / LAYER_BYTES_PER_NS;
 }
 
 // The leading layers as one kernel's operations: first convolution, depthwise + pointwise pairs, pool, dense, softmax.
@@ -369,13 +372,14 @@ int plan_chain(tfjsb_model* m, tfjsb_model* owner) {
     const int n_ops = chain_ops(m, ops, layers_of);
     const int64_t images = m->in_dims[0];
     if (!n_ops) return 0;
-    for (const tfjsb_model* v : owner->slices)
-        if (v->chain_chosen && v->in_dims[0] == images) {  // a slice of the same batch: the same plan, filters and workspace
-            m->chain = v->chain;
-            m->chain_elems = v->chain_elems;
-            std::copy(v->chain_layer, v->chain_layer + CHAIN_MAX_OPS, m->chain_layer);
-            return v->chain_best;
-        }
+    for (const auto& set : owner->host_slices)
+        for (const tfjsb_model* v : set.views)
+            if (v->chain_chosen && v->in_dims[0] == images) {  // a slice of the same batch: the same plan, filters and workspace
+                m->chain = v->chain;
+                m->chain_elems = v->chain_elems;
+                std::copy(v->chain_layer, v->chain_layer + CHAIN_MAX_OPS, m->chain_layer);
+                return v->chain_best;
+            }
     double separate = 0, done = 0, rest[CHAIN_MAX_OPS];
     for (const Step& st : m->steps) separate += separate_ns(m, st);
     for (int k = 0, i = 0; k < n_ops; ++k) {
@@ -821,12 +825,14 @@ tfjsb_status tfjsb_model_destroy(tfjsb_model* m) {
     cudaDeviceSynchronize();
     drop_graph(m);
     if (m->capture_stream) cudaStreamDestroy(m->capture_stream);
-    for (tfjsb_model* v : m->slices) {
-        drop_graph(v);
-        if (v->capture_stream) cudaStreamDestroy(v->capture_stream);
-        delete v;
+    for (auto& set : m->host_slices) {
+        for (tfjsb_model* v : set.views) {
+            drop_graph(v);
+            if (v->capture_stream) cudaStreamDestroy(v->capture_stream);
+            delete v;
+        }
+        for (cudaEvent_t e : set.copied) cudaEventDestroy(e);
     }
-    for (cudaEvent_t e : m->slice_copied) cudaEventDestroy(e);
     for (cudaEvent_t e : m->host_run_done)
         if (e) cudaEventDestroy(e);
     if (m->copy_stream) cudaStreamDestroy(m->copy_stream);
@@ -874,12 +880,13 @@ tfjsb_status tfjsb_model_set_fusion(tfjsb_model* m, int mode) {
     if (mode < 0 || mode > 2) return fail(m->ctx, TFJSB_ERR_INVALID_ARG, "fusion mode must be 0 (off), 1 (auto) or 2 (always)");
     m->fusion_mode = mode;
     choose_fusion(m, m);
-    for (tfjsb_model* v : m->slices) {
-        v->fusion_mode = mode;
-        choose_fusion(v, m);
-        v->bound_in = nullptr; v->bound_out = nullptr;
-        drop_graph(v);
-    }
+    for (auto& set : m->host_slices)
+        for (tfjsb_model* v : set.views) {
+            v->fusion_mode = mode;
+            choose_fusion(v, m);
+            v->bound_in = nullptr; v->bound_out = nullptr;
+            drop_graph(v);
+        }
     m->bound_in = nullptr;  // buffers and plans are re-assigned on the next run
     m->bound_out = nullptr;
     drop_graph(m);
@@ -897,9 +904,43 @@ tfjsb_status tfjsb_model_set_graph(tfjsb_model* m, int use_graph) {
 
 namespace {
 
+// How many slices a run from host memory is cut into.  A batch's input copy takes n c, its computation F + n k (F: the
+// kernels' fixed times, which every slice pays), and a slice is copied while the one before it is computed.
+//   blocking   n c + F + n k / S where the copies are the longer part, n c / S + S F + n k where the kernels are: the S that
+//              takes the least.  Full model, 224 x 224: 50 images 1005 us whole, 854 in two slices, 958 in four; 128 images
+//              2296, 1931 and 1744; width 0.25, 128 x 128, 24 images: 241 us whole, 343 in two slices; 127 images 696 and,
+//              in three, 639.
+//   async      the copies of one run overlap the kernels of the run before it, sliced or not, so slices only add F as long
+//              as the kernels are the longer part (full model, 96 x 96, 127 images: 362 us whole, 636 in four slices); where
+//              the copies are, they start the kernels sooner (224 x 224, 128 images: 1515 and 1443 us).
+int host_slice_count(const tfjsb_model* m, bool async) {
+    const int64_t n = m->in_dims[0];
+    const double nc = 4.0 * (double)m->in_elems / 55.0;  // ns: pinned memory over PCIe, 55 GB/s
+    double fixed = 0, nk = 0;
+    for (size_t i = 0; i < m->steps.size(); ++i) {
+        const Step& st = m->steps[i];
+        double own = separate_ns(m, st) - LAYER_FIXED_NS;
+        // a fused pair's tensor between its layers is neither written nor read
+        if (st.fuse_next) own -= layer_bytes(m, (double)st.out_elems) / LAYER_BYTES_PER_NS;
+        else fixed += LAYER_FIXED_NS;
+        if (i && m->steps[i - 1].fuse_next) own -= layer_bytes(m, (double)m->steps[i - 1].out_elems) / LAYER_BYTES_PER_NS;
+        nk += own;
+    }
+    int best = 1;
+    double best_ns = nc + fixed + nk;
+    for (int s = 2; s <= 4 && s <= n; ++s) {
+        const double ns = std::max(nc + fixed + nk / s, nc / s + s * fixed + nk);
+        if (async ? s * fixed + nk <= nc : ns < 0.98 * best_ns) {
+            best = s;
+            best_ns = ns;
+        }
+    }
+    return best;
+}
+
 // Enqueues one run from / to host memory on staging set `b` and records host_run_done[b]; no waiting
 // except for the run that last used the same staging set.
-tfjsb_status enqueue_host_run(tfjsb_model* m, const float* host_input, float* host_output, cudaStream_t s, int b) {
+tfjsb_status enqueue_host_run(tfjsb_model* m, const float* host_input, float* host_output, cudaStream_t s, int b, bool async) {
     tfjsb_ctx* ctx = m->ctx;
     tfjsb_status st;
     cudaError_t e;
@@ -916,6 +957,7 @@ tfjsb_status enqueue_host_run(tfjsb_model* m, const float* host_input, float* ho
             return cuda_fail(ctx, e, "cudaEventCreate");
     }
     const int64_t out_image = last.out_elems / m->in_dims[0];
+    tfjsb_model::HostSlices& set = m->host_slices[async ? 1 : 0];
     if (m->keep_all) {
         // debug mode: the whole batch through the model itself, so that every layer's output stays readable
         e = cudaMemcpyAsync(m->staged_in[b], host_input, (size_t)m->in_elems * 4, cudaMemcpyHostToDevice, s);
@@ -924,64 +966,60 @@ tfjsb_status enqueue_host_run(tfjsb_model* m, const float* host_input, float* ho
         tfjsb_tensor out{m->staged_out[b], last.out_rank, {last.out_dims[0], last.out_dims[1], last.out_dims[2], last.out_dims[3]}};
         if ((st = tfjsb_run_model(m, &in, &out, s)) != TFJSB_OK) return st;
     } else {
-        if (m->slices.empty()) {
+        if (set.count == 0) {
             const int64_t n = m->in_dims[0];
-            // Slices of 24 images or so: an image's copy takes longer than its share of the computation (11 against
-            // 6 us for 224 x 224 x 3 and the full model), but a slice also costs about 115 us of fixed chain, so more
-            // slices make the computation the longer of the two.  50 images: 1000 us whole, 850 in two or three
-            // slices, 945 in four.
-            int n_slices = n < 24 ? 1 : n < 72 ? 2 : n < 96 ? 3 : 4;
+            int count = host_slice_count(m, async);
             if (const char* env = getenv("TFJSB_HOST_SLICES")) {  // tuning knob: 1 disables the slicing
                 const int v = atoi(env);
-                if (v >= 1 && v <= n) n_slices = v;
+                if (v >= 1 && v <= n) count = v;
             }
-            for (int c = 0; c < n_slices; ++c) m->slice_images.push_back(n / n_slices + (c < n % n_slices ? 1 : 0));
-            if ((e = cudaStreamCreateWithFlags(&m->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
+            if (!m->copy_stream && (e = cudaStreamCreateWithFlags(&m->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
                 return cuda_fail(ctx, e, "cudaStreamCreate");
-            for (int i = 0; i < 2 * n_slices; ++i) {
+            while ((int)set.copied.size() < 2 * count) {
                 cudaEvent_t ev;
                 if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess)
                     return cuda_fail(ctx, e, "cudaEventCreate");
-                m->slice_copied.push_back(ev);
-                m->slices.push_back(make_batch_view(m, m->slice_images[i % n_slices]));
+                set.copied.push_back(ev);
             }
-            m->n_slices = n_slices;
+            for (int c = 0; c < count; ++c) set.images.push_back(n / count + (c < n % count ? 1 : 0));
+            for (int i = 0; i < 2 * count; ++i) set.views.push_back(make_batch_view(m, set.images[i % count]));
+            set.count = count;
         }
-        const int n_slices = m->n_slices;
+        const int n_slices = set.count;
         const int64_t in_image = m->in_elems / m->in_dims[0];
         // The copies wait for nothing on `stream`: the staging set is free (checked above), so they may
         // run while an earlier run is still computing.
         auto padded = [](int64_t elems) { return (elems + 3) / 4 * 4; };
         int64_t first = 0, at = 0;  // image, offset in the staging buffer
         for (int c = 0; c < n_slices; ++c) {
-            const int64_t elems = m->slice_images[c] * in_image;
+            const int64_t elems = set.images[c] * in_image;
             e = cudaMemcpyAsync(m->staged_in[b] + at, host_input + first * in_image, (size_t)elems * 4, cudaMemcpyHostToDevice, m->copy_stream);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "host-to-device copy of the input");
-            if ((e = cudaEventRecord(m->slice_copied[b * n_slices + c], m->copy_stream)) != cudaSuccess)
+            if ((e = cudaEventRecord(set.copied[b * n_slices + c], m->copy_stream)) != cudaSuccess)
                 return cuda_fail(ctx, e, "cudaEventRecord");
-            first += m->slice_images[c];
+            first += set.images[c];
             at += padded(elems);
         }
         int64_t out_at = 0;
         at = 0;
         for (int c = 0; c < n_slices; ++c) {
-            tfjsb_model* v = m->slices[b * n_slices + c];
-            if ((e = cudaStreamWaitEvent(s, m->slice_copied[b * n_slices + c], 0)) != cudaSuccess)
+            tfjsb_model* v = set.views[b * n_slices + c];
+            if ((e = cudaStreamWaitEvent(s, set.copied[b * n_slices + c], 0)) != cudaSuccess)
                 return cuda_fail(ctx, e, "cudaStreamWaitEvent");
             tfjsb_tensor in{m->staged_in[b] + at, 4, {v->in_dims[0], v->in_dims[1], v->in_dims[2], v->in_dims[3]}};
             const Step& vl = v->steps.back();
             tfjsb_tensor out{m->staged_out[b] + out_at, vl.out_rank, {vl.out_dims[0], vl.out_dims[1], vl.out_dims[2], vl.out_dims[3]}};
-            at += padded(m->slice_images[c] * in_image);
-            out_at += padded(m->slice_images[c] * out_image);
+            at += padded(set.images[c] * in_image);
+            out_at += padded(set.images[c] * out_image);
             if ((st = tfjsb_run_model(v, &in, &out, s)) != TFJSB_OK) return st;
             v->use_graph = true;  // the first pass ran launch by launch; later passes replay a graph
         }
     }
     // one copy when the slices' results lie next to each other, else one per slice
     bool gaps = false;
-    for (int c = 0; !m->keep_all && c + 1 < m->n_slices; ++c) gaps = gaps || (m->slice_images[c] * out_image) % 4 != 0;
+    for (int c = 0; !m->keep_all && c + 1 < set.count; ++c) gaps = gaps || (set.images[c] * out_image) % 4 != 0;
     for (int64_t c = 0, first = 0, at = 0; first < m->in_dims[0]; ++c) {
-        const int64_t images = gaps ? m->slice_images[c] : m->in_dims[0];
+        const int64_t images = gaps ? set.images[c] : m->in_dims[0];
         e = cudaMemcpyAsync(host_output + first * out_image, m->staged_out[b] + at, (size_t)(images * out_image) * 4, cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "device-to-host copy of the output");
         first += images;
@@ -992,17 +1030,21 @@ tfjsb_status enqueue_host_run(tfjsb_model* m, const float* host_input, float* ho
     return TFJSB_OK;
 }
 
+tfjsb_status start_host_run(tfjsb_model* m, const float* host_input, float* host_output, cudaStream_t s, bool async) {
+    if (!host_input || !host_output) return fail(m->ctx, TFJSB_ERR_INVALID_ARG, "host_input / host_output is null");
+    const int b = m->next_staging;
+    tfjsb_status st = enqueue_host_run(m, host_input, host_output, s, b, async);
+    if (st == TFJSB_OK) m->next_staging = b ^ 1;
+    return st;
+}
+
 }  // namespace
 
 extern "C" {
 
 tfjsb_status tfjsb_run_model_host_async(tfjsb_model* m, const float* host_input, float* host_output, void* stream) {
     if (!m) return TFJSB_ERR_INVALID_ARG;
-    if (!host_input || !host_output) return fail(m->ctx, TFJSB_ERR_INVALID_ARG, "host_input / host_output is null");
-    const int b = m->next_staging;
-    tfjsb_status st = enqueue_host_run(m, host_input, host_output, static_cast<cudaStream_t>(stream), b);
-    if (st == TFJSB_OK) m->next_staging = b ^ 1;
-    return st;
+    return start_host_run(m, host_input, host_output, static_cast<cudaStream_t>(stream), true);
 }
 
 tfjsb_status tfjsb_model_host_wait(tfjsb_model* m) {
@@ -1018,7 +1060,8 @@ tfjsb_status tfjsb_model_host_wait(tfjsb_model* m) {
 }
 
 tfjsb_status tfjsb_run_model_host(tfjsb_model* m, const float* host_input, float* host_output, void* stream) {
-    tfjsb_status st = tfjsb_run_model_host_async(m, host_input, host_output, stream);
+    if (!m) return TFJSB_ERR_INVALID_ARG;
+    tfjsb_status st = start_host_run(m, host_input, host_output, static_cast<cudaStream_t>(stream), false);
     if (st != TFJSB_OK) return st;
     if ((st = tfjsb_model_host_wait(m)) != TFJSB_OK) return st;
     cudaError_t e = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
@@ -1040,12 +1083,13 @@ tfjsb_status tfjsb_model_set_keep_all(tfjsb_model* m, int keep_all) {
         // without it computes.  (A chain's products are added in another order.)
         m->chain_allowed = false;
         choose_fusion(m, m);
-        for (tfjsb_model* v : m->slices) {
-            v->chain_allowed = false;
-            choose_fusion(v, m);
-            v->bound_in = nullptr; v->bound_out = nullptr;
-            drop_graph(v);
-        }
+        for (auto& set : m->host_slices)
+            for (tfjsb_model* v : set.views) {
+                v->chain_allowed = false;
+                choose_fusion(v, m);
+                v->bound_in = nullptr; v->bound_out = nullptr;
+                drop_graph(v);
+            }
     }
     drop_graph(m);
     m->bound_in = nullptr;  // force a re-bind on the next run

@@ -355,3 +355,30 @@ def test_one_kernel_models_launch_their_kernel_in_graph_mode_too(ctx):
     ctx.check_device_status()
     del graph
     model.close()
+
+
+@pytest.mark.parametrize("alpha,hw,batch,sliced", [(0.25, 96, 25, False), (0.25, 64, 127, False), (0.5, 64, 101, False), (0.5, 160, 127, True)])
+def test_host_runs_are_sliced_only_where_copies_are_long(ctx, alpha, hw, batch, sliced):
+    """Small images through small models: a slice would add its kernels' fixed times and hide next to no copying, in the
+    blocking call and more so in the asynchronous one, whose copies overlap the run before.  Seen in the kernels launched."""
+    import torch
+
+    x, layers = si.config_mobilenet(alpha, hw, batch, seed=4243, classes=12)
+    model = ctx.model(layers, x.shape)
+    hin, hout = torch.from_numpy(x).pin_memory(), torch.zeros(model.output_shape).pin_memory()
+    model.run_host(hin, hout)
+    first = hout.clone()
+
+    def launched(call):
+        before = ctx.launch_count
+        call(hin, hout.zero_())
+        model.host_wait()
+        return ctx.launch_count - before
+
+    whole = model.launches_per_run
+    blocking, asynchronous = launched(model.run_host), launched(model.run_host_async)
+    assert (blocking > whole) if sliced else (blocking == asynchronous == whole)
+    # the two calls may cut the batch differently: the same results up to the order of sums
+    assert np.max(np.abs(hout.numpy() - first.numpy())) <= 2e-2 * float(first.max())
+    ctx.check_device_status()
+    model.close()
