@@ -122,8 +122,8 @@ def _load_library() -> ctypes.CDLL:
 
 lib = _load_library()
 
-# The op calls marshalled in C++ (binding/fast_calls.cpp); loaded with the first Context, since it needs torch.  A call that
-# it does not take (it returns None) goes through ctypes below, which raises whatever there is to raise.
+# The op calls marshalled in C++ (binding/fast_calls.cpp); loaded with the first Context, since it needs torch.  A call whose
+# arguments it does not take (it returns None) goes through ctypes below, which raises whatever there is to raise.
 _fast = None
 
 
@@ -136,7 +136,7 @@ def _load_fast_calls():
         loader = importlib.machinery.ExtensionFileLoader("_fast_calls", _build.build_binding())
         module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fast_calls", loader))
         loader.exec_module(module)
-        module.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in module.CALLS})
+        module.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in module.CALLS}, TfjsbError)
         _fast = module
 
 
@@ -461,7 +461,7 @@ class Model:
 
     def run(self, x, out=None):
         """Enqueue one forward pass on the current stream; device tensors in and out."""
-        done = _fast.run_model(self._fh, self.ctx.device, x, self.output_shape, out)
+        done = _fast.run_model(self.ctx._fh, self.ctx.device, self._fh, x, self.output_shape, out)
         if done is not None:
             return done
         out = self.ctx._empty(self.output_shape) if out is None else out
@@ -520,7 +520,7 @@ class Model:
     def layer_output_f32(self, layer: int):
         """fp32 copy of the output of layer `layer` whatever its storage format (bfloat16 layers are
         widened on the device); use set_keep_all(True) before the run."""
-        done = _fast.layer_output_f32(self._fh, self.ctx.device, layer)
+        done = _fast.layer_output_f32(self.ctx._fh, self.ctx.device, self._fh, layer)
         if done is not None:
             return done
         rank = ctypes.c_int32()

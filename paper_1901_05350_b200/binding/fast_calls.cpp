@@ -2,10 +2,11 @@
 //
 // A ctypes call with its argument structs, torch.empty and the stream lookup cost 12-16 us of host time, several times
 // what the launch itself takes and more than most small ops run on the GPU; the same steps on the C++ side of torch take
-// about 2 us.  Every function takes the library handle as an integer and returns the output tensor, or None whenever an
-// argument is not the plain case (contiguous fp32 CUDA tensors of rank 1..4, whole-number options) or the library reports
-// an error: the caller then takes the ctypes path, which raises what it always raised (a call that fails has enqueued
-// nothing).  The library is called through addresses that the caller hands over once, so both paths use one copy of it.
+// about 2 us.  Every function takes the context's handle as an integer and returns the output tensor, or None whenever an
+// argument is not the plain case (contiguous fp32 CUDA tensors of rank 1..4, whole-number options): the caller then takes
+// the ctypes path, which raises what there is to raise.  An error that the library reports is raised from here and the
+// call is not repeated: a model run, or a call that packs or transposes an operand first, may have enqueued a part of it.
+// The library is called through addresses that the caller hands over once, so both paths use one copy of it.
 #include <Python.h>
 
 #include <ATen/core/Tensor.h>
@@ -23,10 +24,12 @@ namespace {
     X(tfjsb_matmul) X(tfjsb_batch_matmul) X(tfjsb_conv2d) X(tfjsb_depthwise_conv2d) X(tfjsb_avg_pool) X(tfjsb_max_pool)       \
     X(tfjsb_binary) X(tfjsb_softmax) X(tfjsb_bias_act) X(tfjsb_conv2d_backprop_input) X(tfjsb_conv2d_backprop_filter)         \
     X(tfjsb_depthwise_conv2d_backprop_input) X(tfjsb_depthwise_conv2d_backprop_filter) X(tfjsb_act_backprop)                  \
-    X(tfjsb_bias_backprop) X(tfjsb_run_model) X(tfjsb_model_layer_output_f32) X(tfjsb_model_layer_shape) X(tfjsb_window_out_shape)
+    X(tfjsb_bias_backprop) X(tfjsb_run_model) X(tfjsb_model_layer_output_f32) X(tfjsb_model_layer_shape) X(tfjsb_window_out_shape)       \
+    X(tfjsb_last_error)
 #define DECLARE(name) decltype(&::name) p_##name = nullptr;
 FAST_CALLS(DECLARE)
 #undef DECLARE
+PyObject* error_type = nullptr;  // called with (status, message)
 
 // An argument list read from left to right; `ok` turns false at the first argument that is not the plain case.
 struct Args {
@@ -116,8 +119,13 @@ struct Out {
         desc.rank = rank;
         for (int i = 0; i < rank; ++i) desc.dims[i] = dims[i];
     }
-    PyObject* done(tfjsb_status st) {
-        if (st != TFJSB_OK) Py_RETURN_NONE;
+    PyObject* done(tfjsb_ctx* ctx, tfjsb_status st) {
+        if (st != TFJSB_OK) {
+            PyObject* error = PyObject_CallFunction(error_type, "is", (int)st, p_tfjsb_last_error(ctx));
+            if (error) PyErr_SetObject(error_type, error);
+            Py_XDECREF(error);
+            return nullptr;
+        }
         if (given) { Py_INCREF(given); return given; }
         return THPVariable_Wrap(std::move(made));
     }
@@ -133,8 +141,8 @@ tfjsb_status unlocked(F f) {
     Py_END_ALLOW_THREADS return st;
 }
 
-// The Python entry point of an op with N arguments.  Whatever goes wrong in it (an allocation that throws, say) goes wrong
-// again on the ctypes path, which reports it.
+// The Python entry point of an op with N arguments.  What is thrown in it (by an allocation, say), before the library is
+// called, goes wrong again on the ctypes path, which reports it.
 template <PyObject* (*OP)(Args&), int N>
 PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n) {
     try {
@@ -147,7 +155,11 @@ PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n) {
     }
 }
 
-PyObject* bind(PyObject*, PyObject* addresses) {  // {name: address}
+PyObject* bind(PyObject*, PyObject* args) {  // {name: address}, the type of the errors
+    PyObject *addresses, *type;
+    if (!PyArg_ParseTuple(args, "O!O", &PyDict_Type, &addresses, &type)) return nullptr;
+    Py_INCREF(type);
+    Py_XSETREF(error_type, type);
 #define TAKE(name)                                                                         \
     {                                                                                      \
         PyObject* o = PyDict_GetItemString(addresses, #name);                              \
@@ -185,7 +197,7 @@ PyObject* matmul(Args& a) {
     }
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] { return (BATCH ? p_tfjsb_batch_matmul : p_tfjsb_matmul)(h.ctx, &ta, &tb, x, y, &out.desc, s); }));
+    return out.done(h.ctx, unlocked([&] { return (BATCH ? p_tfjsb_batch_matmul : p_tfjsb_matmul)(h.ctx, &ta, &tb, x, y, &out.desc, s); }));
 }
 
 bool window_shape(const tfjsb_tensor& x, const int64_t size[2], const int strides[2], int pad, const int dilations[2], int64_t channels,
@@ -222,7 +234,7 @@ PyObject* conv2d(Args& a) {
     }
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] {
+    return out.done(h.ctx, unlocked([&] {
         return (DEPTHWISE ? p_tfjsb_depthwise_conv2d : p_tfjsb_conv2d)(h.ctx, &x, &f, st, (tfjsb_pad)pad, dl, bias, (tfjsb_act)act, &out.desc, s);
     }));
 }
@@ -249,7 +261,7 @@ PyObject* pool(Args& a) {
     }
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] { return (MAX ? p_tfjsb_max_pool : p_tfjsb_avg_pool)(h.ctx, &x, size, st, (tfjsb_pad)pad, &out.desc, s); }));
+    return out.done(h.ctx, unlocked([&] { return (MAX ? p_tfjsb_max_pool : p_tfjsb_avg_pool)(h.ctx, &x, size, st, (tfjsb_pad)pad, &out.desc, s); }));
 }
 
 // binary(ctx, device, op, a, b, out)
@@ -263,7 +275,7 @@ PyObject* binary(Args& a) {
     if (!out.take(a) && a.ok) out.make(a, h.device, u.dims, u.rank);
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] { return p_tfjsb_binary(h.ctx, (tfjsb_binary_op)op, &u, &v, &out.desc, s); }));
+    return out.done(h.ctx, unlocked([&] { return p_tfjsb_binary(h.ctx, (tfjsb_binary_op)op, &u, &v, &out.desc, s); }));
 }
 
 // softmax(ctx, device, logits, out)
@@ -275,7 +287,7 @@ PyObject* softmax(Args& a) {
     if (!out.take(a) && a.ok) out.make(a, h.device, x.dims, x.rank);
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] { return p_tfjsb_softmax(h.ctx, &x, &out.desc, s); }));
+    return out.done(h.ctx, unlocked([&] { return p_tfjsb_softmax(h.ctx, &x, &out.desc, s); }));
 }
 
 // bias_act(ctx, device, x, bias, act, out)
@@ -289,7 +301,7 @@ PyObject* bias_act(Args& a) {
     if (!out.take(a) && a.ok) out.make(a, h.device, x.dims, x.rank);
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] { return p_tfjsb_bias_act(h.ctx, &x, bias, (tfjsb_act)act, &out.desc, s); }));
+    return out.done(h.ctx, unlocked([&] { return p_tfjsb_bias_act(h.ctx, &x, bias, (tfjsb_act)act, &out.desc, s); }));
 }
 
 // conv_grad(ctx, device, which, shape of the result, first, second, strides, pad, dilations, out): which = 0 conv2d input
@@ -314,7 +326,7 @@ PyObject* conv_grad(Args& a) {
                       : which == 2 ? p_tfjsb_depthwise_conv2d_backprop_input
                                    : p_tfjsb_depthwise_conv2d_backprop_filter;
     void* s = stream();
-    return out.done(unlocked([&] { return call(h.ctx, &u, &v, st, (tfjsb_pad)pad, dl, &out.desc, s); }));
+    return out.done(h.ctx, unlocked([&] { return call(h.ctx, &u, &v, st, (tfjsb_pad)pad, dl, &out.desc, s); }));
 }
 
 // act_backprop(ctx, device, y, dy, act, out)
@@ -328,7 +340,7 @@ PyObject* act_backprop(Args& a) {
     if (!out.take(a) && a.ok) out.make(a, h.device, y.dims, y.rank);
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] { return p_tfjsb_act_backprop(h.ctx, &y, &g, (tfjsb_act)act, &out.desc, s); }));
+    return out.done(h.ctx, unlocked([&] { return p_tfjsb_act_backprop(h.ctx, &y, &g, (tfjsb_act)act, &out.desc, s); }));
 }
 
 // bias_backprop(ctx, device, dz, out)
@@ -340,41 +352,42 @@ PyObject* bias_backprop(Args& a) {
     if (!out.take(a) && a.ok) out.make(a, h.device, &g.dims[g.rank - 1], 1);
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] { return p_tfjsb_bias_backprop(h.ctx, &g, &out.desc, s); }));
+    return out.done(h.ctx, unlocked([&] { return p_tfjsb_bias_backprop(h.ctx, &g, &out.desc, s); }));
 }
 
-// run_model(model, device, x, output shape, out)
+// run_model(ctx, device, model, x, output shape, out)
 PyObject* run_model(Args& a) {
+    const Head h(a);
     auto* m = static_cast<tfjsb_model*>(a.handle());
-    const int device = (int)a.integer();
     tfjsb_tensor x;
     Out out;
     int64_t d[4];
     a.tensor(&x);
     const int rank = a.integers(d, 0);
-    if (!out.take(a) && a.ok) out.make(a, device, d, rank);
+    if (!out.take(a) && a.ok) out.make(a, h.device, d, rank);
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] { return p_tfjsb_run_model(m, &x, &out.desc, s); }));
+    return out.done(h.ctx, unlocked([&] { return p_tfjsb_run_model(m, &x, &out.desc, s); }));
 }
 
-// layer_output_f32(model, device, layer)
+// layer_output_f32(ctx, device, model, layer)
 PyObject* layer_output_f32(Args& a) {
+    const Head h(a);
     auto* m = static_cast<tfjsb_model*>(a.handle());
-    const int device = (int)a.integer(), layer = (int)a.integer();
+    const int layer = (int)a.integer();
     Out out;
     int32_t rank = 0;
     int64_t d[4];
     if (!a.ok || p_tfjsb_model_layer_shape(m, layer, &rank, d) != TFJSB_OK) Py_RETURN_NONE;
-    out.make(a, device, d, rank);
+    out.make(a, h.device, d, rank);
     if (!a.ok) Py_RETURN_NONE;
     void* s = stream();
-    return out.done(unlocked([&] { return p_tfjsb_model_layer_output_f32(m, layer, static_cast<float*>(out.desc.data), s); }));
+    return out.done(h.ctx, unlocked([&] { return p_tfjsb_model_layer_output_f32(m, layer, static_cast<float*>(out.desc.data), s); }));
 }
 
 #define METHOD(name, op, n) {name, (PyCFunction)(void (*)(void))(&entry<op, n>), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
-    {"bind", bind, METH_O, nullptr},
+    {"bind", bind, METH_VARARGS, nullptr},
     METHOD("matmul", matmul<false>, 7),
     METHOD("batch_matmul", matmul<true>, 7),
     METHOD("conv2d", conv2d<false>, 10),
@@ -387,8 +400,8 @@ PyMethodDef methods[] = {
     METHOD("conv_grad", conv_grad, 10),
     METHOD("act_backprop", act_backprop, 6),
     METHOD("bias_backprop", bias_backprop, 4),
-    METHOD("run_model", run_model, 5),
-    METHOD("layer_output_f32", layer_output_f32, 3),
+    METHOD("run_model", run_model, 6),
+    METHOD("layer_output_f32", layer_output_f32, 4),
     {nullptr, nullptr, 0, nullptr},
 };
 #undef METHOD

@@ -172,3 +172,29 @@ def test_atrous_mobilenet_every_layer(ctx, oracle, output_stride):
     model.set_keep_all(False)
     assert same_bits(host(model.run(dev(x))), probs)          # the ping-pong run gives the same bits
     model.close()
+
+
+@pytest.mark.parametrize("call", ["tfjsb_matmul", "tfjsb_conv2d", "tfjsb_bias_backprop", "tfjsb_run_model"])
+def test_a_call_that_fails_is_not_made_twice(ctx, tfjsb, monkeypatch, call):
+    """A failing call may have enqueued a part of its work (a model its first layers, a convolution the packing of its
+    filter): the error that the library reports is raised, and the call is not repeated through ctypes."""
+    import torch
+
+    def repeated(*args):
+        raise AssertionError("the call was made a second time")
+
+    monkeypatch.setattr(tfjsb.lib, call, repeated)
+    wrong = torch.zeros(3, 3, device="cuda")
+    x, layers = si.config_mobilenet(0.25, 32, 1, seed=5, classes=10)
+    model = ctx.model(layers, x.shape)
+    with pytest.raises(tfjsb.TfjsbError) as e:
+        if call == "tfjsb_matmul":
+            ctx.matmul(torch.zeros(8, 8, device="cuda"), torch.zeros(8, 12, device="cuda"), out=wrong)
+        elif call == "tfjsb_conv2d":
+            ctx.conv2d(torch.zeros(1, 8, 8, 16, device="cuda"), torch.zeros(3, 3, 16, 8, device="cuda"), out=torch.zeros(1, 8, 8, 9, device="cuda"))
+        elif call == "tfjsb_bias_backprop":
+            ctx.bias_backprop(torch.zeros(4, 8, device="cuda"), out=torch.zeros(7, device="cuda"))
+        else:
+            model.run(dev(x), out=wrong)
+    assert e.value.status_name == "SHAPE" and str(e.value)
+    model.close()
