@@ -92,11 +92,13 @@ BINDING_SRC = os.path.join(PKG, "binding", "fast_calls.cpp")
 
 
 def binding_path() -> str:
-    """The C++ half of the Python binding is compiled against one version of torch, which its name carries."""
+    """The C++ half of the Python binding is compiled against one version of torch and one ABI of Python: its name carries both."""
+    import sysconfig
+
     import torch
 
     version = "".join(c if c.isalnum() else "_" for c in torch.__version__)
-    return os.path.join(PKG, f"_fast_calls_torch{version}.so")
+    return os.path.join(PKG, f"_fast_calls_torch{version}{sysconfig.get_config_var('EXT_SUFFIX')}")
 
 
 def build_binding(force: bool = False) -> str:

@@ -84,3 +84,14 @@ def test_product_path_never_imports_the_oracle():
     orc = open(os.path.join(ROOT, "oracle", "__init__.py")).read() + open(
         os.path.join(ROOT, "oracle", "tfjs_ops_oracle.cpp")).read()
     assert "paper_1901_05350_b200" not in orc and "tfjsb" not in orc
+
+
+def test_the_binding_is_named_after_the_torch_and_the_python_it_is_built_for(pkg, monkeypatch):
+    import sysconfig
+
+    import torch
+
+    path = pkg._build.binding_path()
+    assert "torch" + torch.__version__.split(".")[0] in path and path.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    monkeypatch.setattr(sysconfig, "get_config_var", lambda name: ".cpython-399-x86_64-linux-gnu.so")
+    assert pkg._build.binding_path() != path
