@@ -127,16 +127,28 @@ lib = _load_library()
 _fast = None
 
 
+class _NoFastCalls:
+    """Stands in where the C++ half cannot be built or loaded: takes no call, so each goes through ctypes."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _load_fast_calls():
     global _fast
     if _fast is None:
         import importlib.machinery
         import importlib.util
+        import warnings
 
-        loader = importlib.machinery.ExtensionFileLoader("_fast_calls", _build.build_binding())
-        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fast_calls", loader))
-        loader.exec_module(module)
-        module.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in module.CALLS}, TfjsbError)
+        try:
+            loader = importlib.machinery.ExtensionFileLoader("_fast_calls", _build.build_binding())
+            module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fast_calls", loader))
+            loader.exec_module(module)
+            module.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in module.CALLS}, TfjsbError)
+        except (ImportError, OSError, RuntimeError) as e:  # no compiler, no headers, another torch
+            warnings.warn(f"op calls are marshalled in Python, about 10 us each slower: {e}", RuntimeWarning, stacklevel=3)
+            module = _NoFastCalls()
         _fast = module
 
 

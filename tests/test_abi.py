@@ -95,3 +95,15 @@ def test_the_binding_is_named_after_the_torch_and_the_python_it_is_built_for(pkg
     assert "torch" + torch.__version__.split(".")[0] in path and path.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
     monkeypatch.setattr(sysconfig, "get_config_var", lambda name: ".cpython-399-x86_64-linux-gnu.so")
     assert pkg._build.binding_path() != path
+
+
+@pytest.mark.parametrize("failure", [RuntimeError("g++ failed"), FileNotFoundError("g++"), ImportError("undefined symbol")])
+def test_a_binding_that_cannot_be_built_leaves_the_calls_to_ctypes(pkg, monkeypatch, failure):
+    def build_binding():
+        raise failure
+
+    monkeypatch.setattr(pkg, "_fast", None)
+    monkeypatch.setattr(pkg._build, "build_binding", build_binding)
+    with pytest.warns(RuntimeWarning, match="marshalled in Python"):
+        pkg._load_fast_calls()
+    assert pkg._fast.matmul(1, 0, None, None, False, False, None) is None  # "not taken": the ctypes path follows
