@@ -345,7 +345,8 @@ tfjsb_status tfjsb_model_set_graph(tfjsb_model* model, int use_graph);
  * output of layer `layer` as left by the last run.  With the ping-pong arena only the most
  * recent layers survive a full run, so call tfjsb_model_set_keep_all(model, 1) before the run
  * to give every layer its own buffer.  That also ends the running of a small model's layers as one
- * kernel for this model, so that later runs without keep_all give the same bits. */
+ * kernel for this model, so that later runs without keep_all give the same bits; the next call of
+ * tfjsb_model_set_fusion, with mode 1, lets them run as one kernel again. */
 tfjsb_status tfjsb_model_set_keep_all(tfjsb_model* model, int keep_all);
 tfjsb_status tfjsb_model_layer_output(tfjsb_model* model, int layer, tfjsb_tensor* view);
 /* The same read as fp32 values whatever the layer's storage format: writes the layer's output

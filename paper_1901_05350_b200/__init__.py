@@ -504,6 +504,8 @@ class Model:
         self.ctx._check(lib.tfjsb_model_host_wait(self._h))
 
     def set_keep_all(self, keep_all: bool):
+        """Every layer's output in a buffer of its own, for layer_output().  Also ends the running of a small model as one
+        kernel, so that runs without keep_all give the same bits, until set_fusion('auto') is called."""
         self.ctx._check(lib.tfjsb_model_set_keep_all(self._h, int(keep_all)))
 
     def set_fusion(self, mode: str):

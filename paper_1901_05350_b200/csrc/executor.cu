@@ -103,6 +103,7 @@ struct tfjsb_model {
     int chain_layer[CHAIN_MAX_OPS] = {};  // the layer whose output an operation makes
     float* chain_workspace = nullptr;
     int64_t chain_elems = 0;  // of workspace per cluster, for the longest chain
+    bool chain_possible = false;  // by the mode of arithmetic and the environment
     bool chain_allowed = false, chain_chosen = false;
     int chain_best = 0;       // chain_len where the fusion mode lets it be chosen
     cudaStream_t copy_stream = nullptr;
@@ -448,6 +449,7 @@ tfjsb_model* make_batch_view(tfjsb_model* parent, int64_t n) {
         st.out = nullptr;
     }
     v->fusion_mode = parent->fusion_mode;
+    v->chain_possible = parent->chain_possible;
     v->chain_allowed = parent->chain_allowed;
     choose_fusion(v, parent);  // by the view's own batch
     return v;
@@ -810,7 +812,7 @@ tfjsb_status tfjsb_model_create(tfjsb_ctx* ctx, const tfjsb_layer_desc* layers, 
             }
         }
     }
-    m->chain_allowed = (m->use_tf32 || m->narrow) && !getenv("TFJSB_NO_FUSION");
+    m->chain_allowed = m->chain_possible = (m->use_tf32 || m->narrow) && !getenv("TFJSB_NO_FUSION");
     choose_fusion(m, m);
     if ((st = dev_alloc(m, 2 * m->region_elems, &m->arena)) != TFJSB_OK) return bail(st, ctx->last_error);
     cudaError_t e = cudaDeviceSynchronize();  // weight transposes done
@@ -879,10 +881,12 @@ tfjsb_status tfjsb_model_set_fusion(tfjsb_model* m, int mode) {
     if (!m) return TFJSB_ERR_INVALID_ARG;
     if (mode < 0 || mode > 2) return fail(m->ctx, TFJSB_ERR_INVALID_ARG, "fusion mode must be 0 (off), 1 (auto) or 2 (always)");
     m->fusion_mode = mode;
+    m->chain_allowed = m->chain_possible;  // also where the keep-all mode has ended it
     choose_fusion(m, m);
     for (auto& set : m->host_slices)
         for (tfjsb_model* v : set.views) {
             v->fusion_mode = mode;
+            v->chain_allowed = v->chain_possible;
             choose_fusion(v, m);
             v->bound_in = nullptr; v->bound_out = nullptr;
             drop_graph(v);
@@ -1080,7 +1084,7 @@ tfjsb_status tfjsb_model_set_keep_all(tfjsb_model* m, int keep_all) {
     m->keep_all = keep_all != 0;
     if (keep_all) {
         // From here on every layer has its own kernel in every run: what the debug mode shows is, bit for bit, what a run
-        // without it computes.  (A chain's products are added in another order.)
+        // without it computes.  (A chain's products are added in another order.)  tfjsb_model_set_fusion ends that.
         m->chain_allowed = false;
         choose_fusion(m, m);
         for (auto& set : m->host_slices)

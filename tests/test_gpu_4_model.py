@@ -382,3 +382,21 @@ def test_host_runs_are_sliced_only_where_copies_are_long(ctx, alpha, hw, batch, 
     assert np.max(np.abs(hout.numpy() - first.numpy())) <= 2e-2 * float(first.max())
     ctx.check_device_status()
     model.close()
+
+
+def test_a_look_at_the_layers_does_not_end_the_one_kernel_for_good(ctx):
+    x, layers = si.config_mobilenet(0.25, 64, 1, seed=4243, classes=20)
+    model = ctx.model(layers, x.shape)
+    xd = dev(x)
+    first = host(model.run(xd))
+    assert model.launches_per_run == 1
+    model.set_keep_all(True)
+    every_layer = host(model.run(xd))
+    model.set_keep_all(False)
+    assert same_bits(host(model.run(xd)), every_layer) and model.launches_per_run == len(layers)
+    model.set_fusion("auto")
+    assert same_bits(host(model.run(xd)), first) and model.launches_per_run == 1
+    model.set_keep_all(True)
+    assert same_bits(host(model.run(xd)), every_layer)
+    ctx.check_device_status()
+    model.close()
