@@ -298,15 +298,18 @@ __global__ void transpose_kernel(const float* __restrict__ in, float* __restrict
 // sides are read and written in 128-byte runs.
 __global__ void pack_filter_kernel(const float* __restrict__ f, float* __restrict__ out, int64_t C, int64_t N, int64_t c_pad) {
     __shared__ float tile[32][33];
-    const int64_t n0 = (int64_t)blockIdx.x * 32, c0 = (int64_t)blockIdx.y * 32, t = blockIdx.z;
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int64_t c = c0 + j, n = n0 + threadIdx.x;
-        tile[j][threadIdx.x] = c < C && n < N ? f[(t * C + c) * N + n] : 0.0f;
-    }
-    __syncthreads();
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int64_t n = n0 + j, c = c0 + threadIdx.x;
-        if (n < N && c < c_pad) out[(n * gridDim.z + t) * c_pad + c] = tile[threadIdx.x][j];
+    const int64_t n0 = (int64_t)blockIdx.x * 32, t = blockIdx.z;
+    for (int64_t c0 = (int64_t)blockIdx.y * 32; c0 < c_pad; c0 += (int64_t)gridDim.y * 32) {
+        for (int j = threadIdx.y; j < 32; j += 8) {
+            const int64_t c = c0 + j, n = n0 + threadIdx.x;
+            tile[j][threadIdx.x] = c < C && n < N ? f[(t * C + c) * N + n] : 0.0f;
+        }
+        __syncthreads();
+        for (int j = threadIdx.y; j < 32; j += 8) {
+            const int64_t n = n0 + j, c = c0 + threadIdx.x;
+            if (n < N && c < c_pad) out[(n * gridDim.z + t) * c_pad + c] = tile[threadIdx.x][j];
+        }
+        __syncthreads();
     }
 }
 
@@ -315,9 +318,9 @@ __global__ void pack_filter_kernel(const float* __restrict__ f, float* __restric
 cudaError_t launch_pack_filter(const float* f, float* out, int64_t taps, int64_t C, int64_t N, int64_t c_pad, cudaStream_t s,
                                int64_t* launches) {
     if (taps * N * c_pad == 0) return cudaSuccess;
-    const int64_t gy = (c_pad + 31) / 32;
-    if (gy > 65535 || taps > 65535) return cudaErrorInvalidConfiguration;
-    pack_filter_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)gy, (unsigned)taps), dim3(32, 8), 0, s>>>(f, out, C, N, c_pad);
+    if (taps > 65535) return cudaErrorInvalidConfiguration;  // im2col copies have 128 x 128 at most
+    const int64_t gy = (c_pad + 31) / 32;                    // the grid walks on where there are more
+    pack_filter_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)(gy < 65535 ? gy : 65535), (unsigned)taps), dim3(32, 8), 0, s>>>(f, out, C, N, c_pad);
     ++*launches;
     return cudaGetLastError();
 }

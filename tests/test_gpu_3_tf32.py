@@ -337,6 +337,14 @@ def test_conv2d_im2col_copies(ctx, oracle, case):
     assert rel_fro(got, oracle.conv2d(x, f, strides, pad, dil, b, "relu", operand="tf32_rz")) <= MATCHED_TOL
 
 
+def test_conv2d_of_a_window_of_two_million_elements(ctx, oracle):
+    """More elements than 32 rows for each block of the largest grid."""
+    x, f = si.small_integers(317, 0, (1, 1025, 1026, 2), -1, 1), si.small_integers(317, 1, (1025, 1024, 2, 4), -1, 1)
+    got = host(ctx.conv2d(dev(x), dev(f), (1, 1), "valid"))  # |sums| <= 2.1e6 < 2^24: exact in any order
+    ctx.check_device_status()
+    assert got.shape == (1, 1, 3, 4) and same_bits(got, oracle.conv2d(x, f, (1, 1), "valid"))
+
+
 FUSED_BLOCK_CASES = [
     # N, H, W, C, Cout, pad: depthwise 3x3 stride 1 + pointwise, run by the executor as one fused kernel
     (1, 112, 112, 32, 64, "same"),     # config 2
