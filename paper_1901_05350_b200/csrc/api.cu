@@ -45,6 +45,22 @@ tfjsb_status ensure_scratch(tfjsb_ctx* ctx, Scratch* s, size_t bytes) {
     return TFJSB_OK;
 }
 
+bool scratch_is_short(const Scratch& s, size_t bytes, cudaStream_t stream) {
+    if (s.bytes >= bytes || !stream) return false;
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &status) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return status != cudaStreamCaptureStatusNone;
+}
+
+int64_t scratch_parts(const Scratch& s, int64_t wanted, size_t each, cudaStream_t stream) {
+    if (wanted <= 1 || !scratch_is_short(s, (size_t)wanted * each, stream)) return wanted;
+    const int64_t room = (int64_t)(s.bytes / each);
+    return room > 1 ? room : 1;
+}
+
 cudaError_t smem_attr_once(const void* kernel, int bytes) {
     static std::mutex mu;
     static std::map<std::pair<const void*, int>, int> done;  // (kernel, device) -> bytes set
@@ -475,6 +491,7 @@ tfjsb_status tfjsb_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_ten
     }
     if (ctx->math == TFJSB_MATH_TF32 && conv_igemm_supported(g) && ctx->encode_tiled) {
         // implicit GEMM on the tensor cores: the filter is packed [Cout, k_pad] into scratch first
+        g.gather_only = scratch_is_short(ctx->scratch_b, (size_t)Cout * conv_igemm_k_pad(g) * 4, s);
         const int64_t k_pad = conv_igemm_k_pad(g);
         if ((st = ensure_scratch(ctx, &ctx->scratch_b, (size_t)Cout * k_pad * 4)) != TFJSB_OK) return st;
         if ((e = launch_pack_conv_filter(pf, ctx->scratch_b.ptr, g, s, &ctx->launches)) != cudaSuccess)
@@ -754,7 +771,7 @@ tfjsb_status tfjsb_conv2d_backprop_filter(tfjsb_ctx* ctx, const tfjsb_tensor* x,
         }
     }
     if (conv2d_small_filter_supported(g)) {
-        const int n = conv2d_small_filter_slices(g, ctx->sm_count);
+        const int n = (int)scratch_parts(ctx->scratch_c, conv2d_small_filter_slices(g, ctx->sm_count), (size_t)numel(dfilter) * 4, s);
         if (n > 1 && (st = ensure_scratch(ctx, &ctx->scratch_c, (size_t)n * numel(dfilter) * 4)) != TFJSB_OK) return st;
         if ((e = launch_conv2d_small_filter(px, pg, pdf, ctx->scratch_c.ptr, n, g, s, &ctx->launches)) != cudaSuccess)
             return cuda_fail(ctx, e, "conv2d_backprop_filter launch");
@@ -820,6 +837,7 @@ tfjsb_status tfjsb_depthwise_conv2d_backprop_filter(tfjsb_ctx* ctx, const tfjsb_
     }
     DepthwiseGradPlan plan;
     if (depthwise_grad_plan(ctx, static_cast<const float*>(x->data), static_cast<const float*>(dy->data), g, &plan)) {
+        plan.slices = (int)scratch_parts(ctx->scratch_c, plan.slices, (size_t)numel(dfilter) * 4, s);
         if (plan.slices > 1 && (st = ensure_scratch(ctx, &ctx->scratch_c, (size_t)plan.slices * numel(dfilter) * 4)) != TFJSB_OK) return st;
         cudaError_t e = launch_depthwise_grad(plan, static_cast<float*>(dfilter->data), ctx->scratch_c.ptr, ctx->dev_status, s, &ctx->launches);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "depthwise_backprop_filter launch");
@@ -869,7 +887,7 @@ tfjsb_status tfjsb_bias_backprop(tfjsb_ctx* ctx, const tfjsb_tensor* dz, tfjsb_t
         cudaError_t e = cudaMemsetAsync(dbias->data, 0, (size_t)C * 4, s);
         return e == cudaSuccess ? TFJSB_OK : cuda_fail(ctx, e, "cudaMemsetAsync");
     }
-    const int slices = sum_rows_slices(rows, C, ctx->sm_count);
+    const int slices = (int)scratch_parts(ctx->scratch_c, sum_rows_slices(rows, C, ctx->sm_count), (size_t)C * 4, s);
     if (slices > 1 && (st = ensure_scratch(ctx, &ctx->scratch_c, (size_t)slices * C * 4)) != TFJSB_OK) return st;
     cudaError_t e = launch_sum_rows(static_cast<const float*>(dz->data), static_cast<float*>(dbias->data), ctx->scratch_c.ptr, rows, C,
                                     slices, s, &ctx->launches);

@@ -135,6 +135,11 @@ tfjsb_status cuda_fail(tfjsb_ctx* ctx, cudaError_t err, const char* what);
 // flight on any stream, so it is kept until tfjsb_shutdown; growth is geometric, so all outgrown blocks
 // together are smaller than the live one.  tfjsb_reserve_scratch sizes the blocks up front.
 tfjsb_status ensure_scratch(tfjsb_ctx* ctx, Scratch* s, size_t bytes);
+// Whether `s` has less than `bytes` and cannot grow, because `stream` is being captured (an allocation would end the
+// capture): a call that can do with less scratch then does.
+bool scratch_is_short(const Scratch& s, size_t bytes, cudaStream_t stream);
+// How many of `wanted` partial results of `each` bytes there is room for, 1 at least (one needs no scratch).
+int64_t scratch_parts(const Scratch& s, int64_t wanted, size_t each, cudaStream_t stream);
 
 // Raises a kernel's dynamic shared-memory limit once per (kernel, device): function attributes belong to
 // a device's copy of the function, and contexts on several devices or host threads may launch the same kernel.
@@ -196,6 +201,7 @@ struct ConvGeom {
     // 3x3 depthwise kernels: taps read last to first, which turns the forward pass over dy into the gradient with
     // respect to the input (stride 1)
     int reversed = 0;
+    int gather_only = 0;  // conv2d: no im2col copies, whose packed filter is the larger one
 };
 
 // ---- launchers (each returns the CUDA launch error; `launches` is incremented per kernel) -----

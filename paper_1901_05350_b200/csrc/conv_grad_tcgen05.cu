@@ -735,6 +735,7 @@ tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float*
         if (a.splits > kbs / 8) a.splits = kbs / 8;
         if (a.splits > 16) a.splits = 16;
         if (a.splits < 1) a.splits = 1;
+        a.splits = (int)scratch_parts(ctx->scratch_c, a.splits, (size_t)g.N * g.H * g.W * g.C * 4, s);
     }
     a.num_tiles = (int)(tiles * a.splits);
     a.segment = split_segment((int64_t)kbs * BLOCK_K);
@@ -808,6 +809,7 @@ tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float*
     }
     if (slices > (a.pixel_blocks + 3) / 4) slices = (a.pixel_blocks + 3) / 4;
     if (slices < 1) slices = 1;
+    slices = scratch_parts(ctx->scratch_c, slices, (size_t)elems * 4, s);
     a.blocks_per_slice = (int)((a.pixel_blocks + slices - 1) / slices);
     slices = (a.pixel_blocks + a.blocks_per_slice - 1) / a.blocks_per_slice;
     a.segment = split_segment((int64_t)a.blocks_per_slice * 32);

@@ -686,7 +686,7 @@ tfjsb_status gemm_tf32_plan(tfjsb_ctx* ctx, const float* a, const float* bt, flo
 // packs the taps, is the faster one.
 bool conv_igemm_uses_im2col(const ConvGeom& g) {
     const int64_t upper_w = (int64_t)(g.Wo - 1) * g.sw - g.pl - (g.W - 1), upper_h = (int64_t)(g.Ho - 1) * g.sh - g.pt - (g.H - 1);
-    return !conv_patch_supported(g) && g.C % 4 == 0 && g.C >= 16 && g.sh <= 8 && g.sw <= 8 && (int64_t)(g.fh - 1) * g.dh <= 127 && (int64_t)(g.fw - 1) * g.dw <= 127 &&
+    return !g.gather_only && !conv_patch_supported(g) && g.C % 4 == 0 && g.C >= 16 && g.sh <= 8 && g.sw <= 8 && (int64_t)(g.fh - 1) * g.dh <= 127 && (int64_t)(g.fw - 1) * g.dw <= 127 &&
            g.pl <= 127 && g.pt <= 127 && upper_w >= -128 && upper_w <= 127 && upper_h >= -128 && upper_h <= 127;
 }
 

@@ -359,3 +359,33 @@ def test_gradients_reject_bad_arguments(ctx, tfjsb):
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] == free0
     assert torch.equal(out, torch.full_like(out, 512.0))
+
+
+def test_gradients_in_a_capture_without_scratch(tfjsb, oracle):
+    """A context that has allocated nothing yet, first used inside a stream capture, where it must not allocate: the gradients
+    do without partial results, and a convolution whose reserved scratch holds the plainly packed filter only uses that."""
+    import torch
+
+    own = tfjsb.Context(0)
+    own.reserve_scratch(5120)  # 8 output channels x 160 (3 x 3 x 16 window elements, padded to whole k-blocks) x 4 bytes
+    x, f, g = si.small_integers(101, 0, (1, 7, 7, 128), -3, 3), si.small_integers(101, 1, (3, 3, 128, 256), -3, 3), si.small_integers(101, 2, (1, 7, 7, 256), -3, 3)
+    fd, gd = si.small_integers(101, 3, (3, 3, 128, 1), -3, 3), si.small_integers(101, 4, (1, 7, 7, 128), -3, 3)
+    x3, g3 = si.small_integers(101, 5, (2, 20, 20, 3), -3, 3), si.small_integers(101, 6, (2, 20, 20, 32), -3, 3)
+    x16, f16 = si.small_integers(101, 7, (1, 9, 9, 16), -3, 3), si.small_integers(101, 8, (3, 3, 16, 8), -3, 3)
+    rows = si.small_integers(101, 9, (5000, 40), -8, 8)
+    d = {k: dev(v) for k, v in dict(x=x, f=f, g=g, fd=fd, gd=gd, x3=x3, g3=g3, x16=x16, f16=f16, rows=rows).items()}
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = [own.conv2d_backprop_input(x.shape, d["f"], d["g"]), own.conv2d_backprop_filter(d["x"], f.shape, d["g"]),
+               own.conv2d_backprop_filter(d["x3"], (3, 3, 3, 32), d["g3"]), own.depthwise_conv2d_backprop_filter(d["x"], fd.shape, d["gd"]),
+               own.bias_backprop(d["rows"]), own.conv2d(d["x16"], d["f16"])]
+    graph.replay()
+    torch.cuda.synchronize()
+    want = [oracle.conv2d_backprop_input(x.shape, f, g), oracle.conv2d_backprop_filter(x, f.shape, g),
+            oracle.conv2d_backprop_filter(x3, (3, 3, 3, 32), g3), oracle.depthwise_conv2d_backprop_filter(x, fd.shape, gd),
+            oracle.bias_backprop(rows), oracle.conv2d(x16, f16)]
+    own.check_device_status()
+    for a, b in zip(got, want):
+        assert same_bits(host(a) + 0.0, b + 0.0)
+    del graph, got
+    own.close()
