@@ -366,7 +366,8 @@ tfjsb_status tfjsb_model_layer_kernel(tfjsb_model* model, int layer, char* name,
 
 /* Per-layer device timing (the paper's per-kernel profile, Sec. 3.8): runs the model `reps`
  * times with a CUDA event pair around every layer, synchronises, and writes the mean
- * milliseconds per layer into ms_per_layer[0..n_layers-1] (host). */
+ * milliseconds per layer into ms_per_layer[0..n_layers-1] (host).  The time of a fused pair is its first layer's; the
+ * layers of a small model that runs as one kernel are timed as kernels of their own. */
 tfjsb_status tfjsb_model_profile(tfjsb_model* model, const tfjsb_tensor* input, tfjsb_tensor* output, int reps,
                                  float* ms_per_layer, void* stream);
 

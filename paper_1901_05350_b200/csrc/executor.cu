@@ -1172,8 +1172,22 @@ tfjsb_status tfjsb_model_profile(tfjsb_model* m, const tfjsb_tensor* input, tfjs
     if (!ms_per_layer || reps < 1) return fail(ctx, TFJSB_ERR_INVALID_ARG, "ms_per_layer is null or reps < 1");
     tfjsb_status st = check_io(m, input, output);
     if (st != TFJSB_OK) return st;
+    // Layers that run as one kernel are timed as kernels of their own; the next run binds its buffers anew.
+    struct OwnKernels {
+        tfjsb_model* m;
+        const int chain_len;
+        explicit OwnKernels(tfjsb_model* model) : m(model), chain_len(model->chain_len) { set(0); }
+        ~OwnKernels() { set(chain_len); }
+        void set(int n) {
+            if (!chain_len) return;
+            m->chain_len = n;
+            m->bound_in = nullptr;
+            m->bound_out = nullptr;
+        }
+    } own_kernels(m);
     if (m->bound_in != input->data || m->bound_out != output->data) {
         if ((st = bind_all(m, static_cast<const float*>(input->data), static_cast<float*>(output->data))) != TFJSB_OK) return st;
+        drop_graph(m);  // the captured launches point at the old buffers
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int n = (int)m->steps.size();

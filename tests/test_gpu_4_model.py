@@ -400,3 +400,16 @@ def test_a_look_at_the_layers_does_not_end_the_one_kernel_for_good(ctx):
     assert same_bits(host(model.run(xd)), every_layer)
     ctx.check_device_status()
     model.close()
+
+
+def test_profile_of_a_model_that_runs_as_one_kernel(ctx):
+    x, layers = si.config_mobilenet(0.25, 64, 1, seed=4243, classes=20)
+    model = ctx.model(layers, x.shape)
+    xd = dev(x)
+    first = host(model.run(xd))
+    ms = model.profile(xd, reps=3)
+    # every layer has its time, none of them most of it
+    assert len(ms) == len(layers) and min(ms) > 0 and max(ms) < 0.5 * sum(ms)
+    assert same_bits(host(model.run(xd)), first) and model.layer_kernels()[0] == "chain_kernel"
+    ctx.check_device_status()
+    model.close()
