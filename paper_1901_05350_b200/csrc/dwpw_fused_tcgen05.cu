@@ -47,6 +47,16 @@ constexpr int F_THREADS = 832;        // 26 warps: producer, MMA, 8 epilogue, 16
 constexpr int F_DW_WARPS = 16;
 constexpr int F_DW_GROUPS = 2;        // groups of depthwise warps that take alternate k-blocks
 constexpr int F_DW_GROUP_WARPS = F_DW_WARPS / F_DW_GROUPS;
+// The block's rings of input patches and of A operand tiles.  A group that takes every F_DW_GROUPS-th k-block has stages of
+// its own in a patch ring of a multiple of that; in any other ring it must not be ahead of a patch that it does not wait
+// for itself, which a free operand stage says as long as that ring is no longer (see the depthwise warps' waits).
+constexpr int F_MAX_PATCHES = 4, F_MAX_A_STAGES = 3;
+constexpr bool patch_rings_are_safe() {
+    for (int patches = 2; patches <= F_MAX_PATCHES; ++patches)
+        if (patches % F_DW_GROUPS != 0 && patches < F_MAX_A_STAGES) return false;
+    return true;
+}
+static_assert(patch_rings_are_safe(), "an odd patch ring must not be shorter than the operand ring");
 constexpr int F_CONV_THREADS = 448;   // 14 warps: producer, MMA, 8 epilogue, 4 im2col; two CTAs per SM
 constexpr int F_CONV_CMP_WARPS = 4;
 constexpr int F_CONV_SMEM = 112 * 1024;  // per-CTA dynamic budget that lets two CTAs share an SM's 228 KiB
@@ -609,8 +619,8 @@ dwpw_fused_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
                     // not completed returns at once: were that patch late (copies land in any order), the group would
                     // read the stage before its own patch is there and hand it back early, which lets the producer arm
                     // a barrier twice in one phase (seen as rare launch failures).  A free operand stage means that
-                    // k-block kb - a_stages has been multiplied, so every patch up to there has landed, and
-                    // a_stages <= 3 covers the ring of three; rings of two and four give each group its own stages.
+                    // k-block kb - a_stages has been multiplied, so every patch up to there has landed, which covers the
+                    // ring of three; rings of two and four give each group its own stages (patch_rings_are_safe).
                     bool got = bounded_wait(smem_u32(&bar_a_empty[as]), aphase ^ 1u, abort_flag);
                     got = got && bounded_wait(smem_u32(&bar_patch_full[ps]), pphase, abort_flag);
                     if (!__all_sync(0xffffffffu, got)) {
@@ -704,7 +714,7 @@ tfjsb_status dwpw_fused_plan(tfjsb_ctx* ctx, const void* x, const float* bt, voi
     plan->n_sub = Cout > 256 ? 2 : 1;
     // tensor memory has 512 columns: two 256-wide halves leave room for one accumulator stage only
     plan->acc_stages = plan->n_sub == 2 ? 1 : (bn == 256 ? 2 : MAX_ACC_STAGES);
-    plan->a_stages = plan->n_sub == 2 ? 2 : 3;
+    plan->a_stages = plan->n_sub == 2 ? 2 : F_MAX_A_STAGES;
     plan->b_stages = plan->n_sub == 2 ? 3 : (bn == 256 ? 2 : 3);
     // all of Bt resident when its k-blocks fit the B ring's four barriers and leave room for three patches
     const int k_blocks = dw.C / BLOCK_K;
@@ -718,9 +728,8 @@ tfjsb_status dwpw_fused_plan(tfjsb_ctx* ctx, const void* x, const float* bt, voi
     if (plan->b_resident) plan->b_stages = k_blocks;
     const int fixed = epi_bytes + plan->a_stages * A_STAGE_BYTES + plan->b_stages * bn * BLOCK_K * 4;
     int ps = (SMEM_LIMIT - 2048 - fixed) / patch_stride;
-    if (ps > 4) ps = 4;
+    if (ps > F_MAX_PATCHES) ps = F_MAX_PATCHES;
     if (ps < 2) return fail(ctx, TFJSB_ERR_UNSUPPORTED, "no room for the input patch ring");
-    static_assert(F_DW_GROUPS == 2, "an odd patch ring must not be shorter than the operand ring (see the depthwise warps' waits)");
     plan->conv = false;
     plan->y_bf16 = narrow;
     plan->patch_stages = ps;
