@@ -326,9 +326,12 @@ tfjsb_status tfjsb_model_host_wait(tfjsb_model* model);
  * channels a multiple of 32) can run as ONE kernel that keeps the depthwise output in shared
  * memory as the tensor-core operand, so the intermediate tensor is neither written nor read back.
  * mode 0: never; 1 (default): where the pair has enough 8x16-pixel tiles for the fused kernel to be
- * the faster choice; 2: wherever the shapes allow.  In the fp32 storage modes results are bit-identical
- * in every mode.  Models in the BF16 storage mode have the same kernel in that format (bfloat16 in and
- * out, the depthwise result rounded to bfloat16 on its way into the operand tile); there it is never
+ * the faster choice; 2: wherever the shapes allow.  In mode 1 a small model's layers (a first 3x3 convolution of three
+ * channels, depthwise + pointwise pairs, then a global pool, dense and softmax) run as ONE kernel, all of them or up to
+ * the pool or the dense layer, where that is estimated to be faster than a kernel for each.  In the fp32 storage modes
+ * results of the pairs are bit-identical in every mode; those of the one kernel differ in the order of their fp32 sums
+ * (and its dense layer multiplies fp32 values).  Models in the BF16 storage mode have the fused pair in that format
+ * (bfloat16 in and out, the depthwise result rounded to bfloat16 on its way into the operand tile); there it is never
  * the default (the separate narrow kernels are faster) and agrees with the separate kernels to the
  * rounding of a stored value, not bit for bit.  The keep-all debug mode always runs the layers
  * separately. */

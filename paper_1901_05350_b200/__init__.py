@@ -509,7 +509,8 @@ class Model:
         self.ctx._check(lib.tfjsb_model_set_keep_all(self._h, int(keep_all)))
 
     def set_fusion(self, mode: str):
-        """'off', 'auto' (default) or 'always': run depthwise + pointwise pairs as one fused kernel."""
+        """'off', 'auto' (default) or 'always': run depthwise + pointwise pairs as one fused kernel.  'auto' also runs all
+        layers of a small model as one kernel where that is faster; its fp32 sums are in another order."""
         self.ctx._check(lib.tfjsb_model_set_fusion(self._h, {"off": 0, "auto": 1, "always": 2}[mode]))
 
     def set_graph(self, use_graph: bool):
