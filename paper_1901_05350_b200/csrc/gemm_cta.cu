@@ -570,23 +570,30 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 //   every further round of tiles                its k-blocks, and 14 ns per column (its epilogue beside the next K loop)
 // The largest tile that still gives every SM one, the rule before, took 23.7 us for 1024^3 (10.7 now with 64 columns),
 // 48 us for 2048^3 (25.8, 256 columns) and 24.5 us for [2312,1024] . [1024,1024] (12.6, 160 columns).
+// bfloat16 operands and results (k-blocks of 64, sixteen epilogue warps, half the bytes): the same measurements on the
+// pointwise layers at batch 1 ... 128.  With the fp32 figures [100352,128] . [128,256] took 15.8 us in 128 columns (14.8 in
+// 256) and [19600,512] . [512,512] 16.3 (15.8 in 256).
 struct TileCost {
-    int width, start_ns, kb_ns;
+    int width, start_ns, kb_ns, epilogue_ns;  // epilogue of a further round
 };
-constexpr TileCost kTileCosts[] = {{32, 3400, 205}, {64, 3700, 215}, {96, 4300, 220}, {128, 4500, 220}, {160, 4900, 220}, {192, 5200, 265}, {256, 5900, 320}};
+constexpr TileCost kTileCosts[] = {{32, 3400, 205, 450},   {64, 3700, 215, 900},   {96, 4300, 220, 1340}, {128, 4500, 220, 1790},
+                                   {160, 4900, 220, 2240}, {192, 5200, 265, 2690}, {256, 5900, 320, 3580}};
+constexpr TileCost kTileCosts16[] = {{32, 3600, 210, 200},  {64, 3800, 205, 340},   {96, 4000, 205, 510}, {128, 4100, 205, 680},
+                                     {160, 4400, 210, 850}, {192, 4500, 245, 1130}, {256, 4750, 310, 1150}};
 
 int64_t tile_ns(const TileCost& t, int64_t M, int64_t N, int64_t k_blocks, int sm_count, int64_t batches, int min_kb_ns) {
     const int64_t tiles = batches * ((M + BLOCK_M - 1) / BLOCK_M) * ((N + t.width - 1) / t.width);
     const int64_t rounds = (tiles + sm_count - 1) / sm_count;
     const int64_t k_loop = k_blocks * (t.kb_ns > min_kb_ns ? t.kb_ns : min_kb_ns);
-    return t.start_ns + k_loop + (rounds - 1) * (k_loop + 14 * t.width);
+    return t.start_ns + k_loop + (rounds - 1) * (k_loop + t.epilogue_ns);
 }
 
 // `min_kb_ns`: what fetching a k-block of A takes at least (im2col copies, gathering threads).
-int choose_block_n(int64_t M, int64_t N, int64_t k_blocks, int sm_count, int64_t batches, int min_kb_ns = 0, int64_t* ns = nullptr) {
+int choose_block_n(int64_t M, int64_t N, int64_t k_blocks, int sm_count, int64_t batches, int min_kb_ns = 0, int64_t* ns = nullptr,
+                   const TileCost (&costs)[7] = kTileCosts) {
     int best = 0;
     int64_t best_ns = 0;
-    for (const TileCost& t : kTileCosts) {
+    for (const TileCost& t : costs) {
         const int64_t cost = tile_ns(t, M, N, k_blocks, sm_count, batches, min_kb_ns);
         if (best == 0 || cost < best_ns) {
             best = t.width;
@@ -803,7 +810,7 @@ tfjsb_status gemm_bf16_plan(tfjsb_ctx* ctx, const void* a, const void* bt, void*
     plan->M = M; plan->N = N; plan->K = K;
     plan->c_is_bf16 = c_is_bf16;
     plan->pair = false;
-    plan->block_n = choose_block_n(M, N, (K + BK16 - 1) / BK16, ctx->sm_count, 1);
+    plan->block_n = choose_block_n(M, N, (K + BK16 - 1) / BK16, ctx->sm_count, 1, 0, nullptr, c_is_bf16 ? kTileCosts16 : kTileCosts);
     plan->acc_stages = plan->block_n > 128 ? 2 : MAX_ACC_STAGES;
     const int stage_bytes = A_STAGE_BYTES + plan->block_n * 128;
     // sixteen epilogue warps where the K loop is short: up to eight k-blocks ([25088,512] . [512,512]: 17.6 us with eight
