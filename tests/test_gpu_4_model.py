@@ -413,3 +413,26 @@ def test_profile_of_a_model_that_runs_as_one_kernel(ctx):
     assert same_bits(host(model.run(xd)), first) and model.layer_kernels()[0] == "chain_kernel"
     ctx.check_device_status()
     model.close()
+
+
+@pytest.mark.parametrize("batch,hw,alpha", [(1, 96, 0.25), (5, 64, 0.25), (40, 64, 0.25), (2, 96, 0.5)])
+def test_products_of_the_one_kernel_are_tf32_products_with_fp32_sums(ctx, oracle, batch, hw, alpha):
+    """The layers that can be read after a run as one kernel, each against the oracle on the input that it had: the last
+    pointwise layer at the operand-matched bar of the tensor-core kernels (operands cut to TF32, sums in another order),
+    the pool and the dense layer, which are fp32 arithmetic, at the bar of the CUDA-core kernels."""
+    x, layers = si.config_mobilenet(alpha, hw, batch, seed=4251, classes=52)
+    features, logits = ctx.model(layers[:28], x.shape), ctx.model(layers[:29], x.shape)
+    xd = dev(x)
+    pooled = host(features.run(xd))
+    dw, pw = (host(features.layer_output_f32(i)) for i in (25, 26))
+    out = host(logits.run(xd))
+    assert features.layer_kernels()[0] == logits.layer_kernels()[0] == "chain_kernel"
+    seen = host(logits.layer_output_f32(27))
+    ctx.check_device_status()
+    own = oracle.conv2d(dw, layers[26].filter, bias=layers[26].bias, act="relu6", operand="tf32_rz")
+    assert rel_fro(pw, own) <= 2e-5
+    assert rel_fro(pooled, pw.astype(np.float64).mean((1, 2))) <= 1e-6
+    assert rel_fro(seen, pooled) <= 1e-6  # (the two models' plans may differ)
+    assert rel_fro(out, seen.astype(np.float64) @ layers[28].filter.astype(np.float64) + layers[28].bias) <= 1e-6
+    features.close()
+    logits.close()
