@@ -702,7 +702,7 @@ tfjsb_status tfjsb_conv2d_backprop_input(tfjsb_ctx* ctx, const tfjsb_tensor* dy,
     }
     const bool pointwise = g.fh == 1 && g.fw == 1 && g.sh == 1 && g.sw == 1;
     if (ctx->math == TFJSB_MATH_TF32 && ctx->encode_tiled && conv2d_grad_input_supported(g) &&
-        !(pointwise && gemm_tf32_supported(g.N * g.H * g.W, g.C, g.Co)))
+        (pointwise ? !gemm_tf32_supported(g.N * g.H * g.W, g.C, g.Co) : conv2d_grad_input_preferred(g, ctx->sm_count)))
         return run_conv2d_grad_input(ctx, pg, pf, pdx, g, s);
     if (pointwise)
         // dx [M, Cin] = dy [M, Cout] . f [Cin, Cout]^T: both operands already have the summed index contiguous

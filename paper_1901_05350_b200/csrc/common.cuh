@@ -376,6 +376,7 @@ cudaError_t launch_depthwise_backprop_filter(const float* x, const float* dy, fl
 // Gradients of conv2d on the tensor cores (conv_grad_tcgen05.cu).  fp32 results: operands as two TF32 values each, except
 // the filter gradient with `split` false, which reads them as TF32.  Scratch for partial sums is the context's.
 bool conv2d_grad_input_supported(const ConvGeom& g);
+bool conv2d_grad_input_preferred(const ConvGeom& g, int sm_count);  // to the CUDA-core kernel (TFJSB_GRAD_INPUT=1: always)
 tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float* f, float* dx, const ConvGeom& g, cudaStream_t s);
 bool conv2d_grad_filter_supported(const ConvGeom& g);
 tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float* dy, float* df, const ConvGeom& g, bool split, cudaStream_t s);

@@ -31,6 +31,8 @@
 // order.  Bound by shared-memory bandwidth (about 1800 cycles per k-block with the lo half, 1000 without, against 768 /
 // 256 of MMAs).  [16,28,28,128], 3x3: 811 us with 32 x 32 tiles on CUDA cores, 40 us here (38 with one accumulator).
 // Pointwise, plain TF32, [32,56,56] 128 x 128: 36 + 36 us of transposes and 23 + 8 us of batched products, 25 + 6 us here.
+#include <cstdlib>
+
 #include "common.cuh"
 #include "ptx_sm100.cuh"
 #include "umma_tile.cuh"
@@ -692,6 +694,56 @@ static void grad_rows(int size, int pad, int s, int* q0, int* count) {
     *count = (size - 1 + pad) / s - *q0 + 1;
 }
 
+struct GradInputTiling {
+    int block_n = 32, kbs = 0, splits = 1;  // kbs: k-blocks of the largest class
+    int64_t tiles = 0;
+};
+static GradInputTiling grad_input_tiling(const ConvGeom& g, int64_t m_tiles, int sms) {
+    GradInputTiling t;
+    // Tile width: the fewest rounds, each as long as the slower of the MMAs (6 cycles per column and k-block) and the
+    // im2col copy (about 600 cycles per k-block).
+    int64_t best = INT64_MAX;
+    for (int bn = 32; bn <= 128; bn <<= 1) {
+        const int64_t tiles = m_tiles * ((g.C + bn - 1) / bn) * g.sh * g.sw;
+        const int64_t cost = (tiles + sms - 1) / sms * (6 * bn > 600 ? 6 * bn : 600);
+        if (cost < best) { best = cost; t.block_n = bn; t.tiles = tiles; }
+        if (bn >= g.C) break;
+    }
+    t.kbs = ((g.fh + g.sh - 1) / g.sh) * ((g.fw + g.sw - 1) / g.sw) * ((g.Co + 31) / 32);
+    // fewer tiles than half the SMs: the K loop in parts of at least eight k-blocks
+    if (2 * t.tiles <= sms) {
+        t.splits = (int)(sms / t.tiles);
+        if (t.splits > t.kbs / 8) t.splits = t.kbs / 8;
+        if (t.splits > 16) t.splits = 16;
+        if (t.splits < 1) t.splits = 1;
+    }
+    return t;
+}
+
+// Where a sample's sum is short, one CUDA-core thread per sample is the faster kernel.  In microseconds, fitted to both on
+// 110 shapes (4 to 64 output channels, windows up to 7 x 7, strides 1 to 3; 6 % of them still go to the slower one):
+//   here         3, and for each round of tiles 1.4 and 0.72 per k-block, of which a tap makes at least one however few its
+//                channels; parts of the K loop 2.5 more, several residue classes 1
+//   CUDA cores   2.5 and 0.42 per tap of a class, the chain of one thread; its samples x products at 0.2 to 1.7 per ps, the
+//                fewer the longer the filter rows that threads read apart
+// [15,8,8,20], 3x3, 8 channels: 11.3 us here and 7.6; [5,27,27,256]: 13.6 and 70; [35,108,108,4]: 174 and 75.
+bool conv2d_grad_input_preferred(const ConvGeom& g, int sm_count) {
+    if (const char* env = getenv("TFJSB_GRAD_INPUT")) return atoi(env) != 0;  // for tests: 1 = this kernel wherever it can
+    int q0h, q0w, Qh, Qw;
+    grad_rows(g.H, g.pt, g.sh, &q0h, &Qh);
+    grad_rows(g.W, g.pl, g.sw, &q0w, &Qw);
+    const GradInputTiling t = grad_input_tiling(g, (g.N * Qh * Qw + BLOCK_M - 1) / BLOCK_M, sm_count);
+    const bool strided = g.sh * g.sw > 1;
+    const double rounds = (double)((t.tiles * t.splits + sm_count - 1) / sm_count), taps = (double)g.fh * g.fw;
+    const double here = 3 + rounds * (0.72 * t.kbs / t.splits + 1.4) + (t.splits > 1 ? 2.5 : 0) + (strided ? 1 : 0);
+    const double samples = (double)g.N * g.H * g.W * g.C, products = taps * g.Co / (g.sh * g.sw);
+    const double per_us = g.C <= 8 && g.Co <= 16 ? 1.7e6 : g.Co <= 12 ? 1.0e6 : g.Co <= 16 || g.C <= 8 ? 0.52e6 : 0.22e6;
+    const double class_taps = (double)((g.fh + g.sh - 1) / g.sh) * ((g.fw + g.sw - 1) / g.sw);
+    // the threads of a warp are neighbouring channels: fewer than 32 of them and a strided window's taps diverge
+    const double chain = !strided ? 0.02 * products : (taps > 1 ? 0.08 * g.Co : 0) + (g.C < 32 ? 0.2 : 0.02) * taps;
+    return here <= 2.5 + 0.42 * class_taps + chain + samples * products * (strided ? 2 : 1) / per_us;
+}
+
 bool conv2d_grad_input_supported(const ConvGeom& g) {
     int q0h, q0w, Qh, Qw;
     grad_rows(g.H, g.pt, g.sh, &q0h, &Qh);
@@ -714,29 +766,13 @@ tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float*
     a.reach_w = (g.fw - 1) / g.sw * g.dw;
     a.M = g.N * a.Qh * a.Qw;
     a.m_tiles = (int)((a.M + BLOCK_M - 1) / BLOCK_M);
-    // Tile width: the fewest rounds, each as long as the slower of the MMAs (6 cycles per column and k-block) and the
-    // im2col copy (about 600 cycles per k-block).
     const int sms = ctx->sm_count;
-    const int classes = g.sh * g.sw;
-    int64_t best = INT64_MAX;
-    for (int bn = 32; bn <= 128; bn <<= 1) {
-        const int64_t tiles = (int64_t)a.m_tiles * ((g.C + bn - 1) / bn) * classes;
-        const int64_t cost = (tiles + sms - 1) / sms * (6 * bn > 600 ? 6 * bn : 600);
-        if (cost < best) { best = cost; a.block_n = bn; }
-        if (bn >= g.C) break;
-    }
+    const GradInputTiling tl = grad_input_tiling(g, a.m_tiles, sms);
+    a.block_n = tl.block_n;
     a.n_tiles = (g.C + a.block_n - 1) / a.block_n;
-    const int64_t tiles = (int64_t)a.m_tiles * a.n_tiles * classes;
-    const int kbs = ((g.fh + g.sh - 1) / g.sh) * ((g.fw + g.sw - 1) / g.sw) * ((g.Co + 31) / 32);  // of the largest class
-    // fewer tiles than half the SMs: the K loop in parts of at least eight k-blocks
-    a.splits = 1;
-    if (2 * tiles <= sms) {
-        a.splits = (int)(sms / tiles);
-        if (a.splits > kbs / 8) a.splits = kbs / 8;
-        if (a.splits > 16) a.splits = 16;
-        if (a.splits < 1) a.splits = 1;
-        a.splits = (int)scratch_parts(ctx->scratch_c, a.splits, (size_t)g.N * g.H * g.W * g.C * 4, s);
-    }
+    const int64_t tiles = tl.tiles;
+    const int kbs = tl.kbs;
+    a.splits = (int)scratch_parts(ctx->scratch_c, tl.splits, (size_t)g.N * g.H * g.W * g.C * 4, s);
     a.num_tiles = (int)(tiles * a.splits);
     a.segment = split_segment((int64_t)kbs * BLOCK_K);
     const int stage_bytes = 2 * (A_STAGE_BYTES + a.block_n * 128);

@@ -127,6 +127,28 @@ def test_conv2d_gradients_keep_fp32_accuracy_in_tf32_mode(ctx, oracle, case):
     assert rel_fro(df, oracle.conv2d_backprop_filter(x, f.shape, g, *args)) <= 1e-5
 
 
+@pytest.fixture
+def tensor_core_input_gradient(monkeypatch):
+    """Short sums run on the CUDA cores by default: the tensor-core kernel wherever it can, for its small cases."""
+    monkeypatch.setenv("TFJSB_GRAD_INPUT", "1")
+
+
+@pytest.mark.parametrize("case", SPLIT_CASES)
+def test_both_input_gradients_of_short_sums(ctx, oracle, case, tensor_core_input_gradient, monkeypatch):
+    N, H, W, Cin, Cout, fh, fw, s, d, pad = case
+    Ho, Wo = geometry(oracle, H, W, fh, fw, s, d, pad)
+    f, g = si.small_integers(93, 1, (fh, fw, Cin, Cout), -3, 3), si.small_integers(93, 2, (N, Ho, Wo, Cout), -3, 3)
+    want = oracle.conv2d_backprop_input((N, H, W, Cin), f, g, (s, s), pad, (d, d)) + 0.0
+    for cores in ("1", "0"):
+        monkeypatch.setenv("TFJSB_GRAD_INPUT", cores)
+        assert same_bits(host(ctx.conv2d_backprop_input((N, H, W, Cin), dev(f), dev(g), (s, s), pad, (d, d))) + 0.0, want)
+    monkeypatch.setenv("TFJSB_GRAD_INPUT", "1")
+    f, g = si.normal(94, 1, f.shape, 0, 0.3), si.normal(94, 2, g.shape, 0, 1)
+    dx = host(ctx.conv2d_backprop_input((N, H, W, Cin), dev(f), dev(g), (s, s), pad, (d, d)))
+    ctx.check_device_status()
+    assert rel_fro(dx, oracle.conv2d_backprop_input((N, H, W, Cin), f, g, (s, s), pad, (d, d))) <= 1e-5
+
+
 @pytest.mark.parametrize("case", [(2, 14, 14, 16, 32, 3, 3, 1), (24, 28, 28, 64, 64, 3, 3, 1), (4, 14, 14, 512, 512, 3, 3, 1), (1, 20, 20, 256, 512, 5, 5, 1),
                                   (2, 56, 56, 32, 64, 3, 3, 2)])
 def test_conv2d_gradients_are_as_exact_as_fp32_multiply_adds(ctx, oracle, case):
@@ -148,7 +170,7 @@ def test_conv2d_gradients_are_as_exact_as_fp32_multiply_adds(ctx, oracle, case):
 
 @pytest.mark.parametrize("case", [SPLIT_CASES[i] for i in (0, 2, 4, 5, 7, 9, 11, 12)])
 @pytest.mark.parametrize("planted", ["x", "f", "g", "all"])
-def test_conv2d_gradients_of_values_that_are_not_finite(ctx, oracle, case, planted):
+def test_conv2d_gradients_of_values_that_are_not_finite(ctx, oracle, case, planted, tensor_core_input_gradient):
     """The same infinities and NaNs as the CUDA-core kernels give, also at the border, where the copied tiles hold zeros for
     what does not exist: an infinite filter value reaches no sample through a tap that it does not meet."""
     N, H, W, Cin, Cout, fh, fw, s, d, pad = case
