@@ -319,9 +319,10 @@ depthwise3x3_s2_backprop_input_kernel(const float* __restrict__ dy, const float*
     }
     float* out = dx + n * (int64_t)g.H * g.W * g.C + c;
     // a filter that is not finite: only taps that meet an output pixel take part, where the zeros make NaNs of the others
-    bool odd = false;
+    float4 nil = zero;
 #pragma unroll
-    for (int t = 0; t < 9; ++t) odd = odd || !finite4(w[t]);
+    for (int t = 0; t < 9; ++t) fma4_packed(nil, w[t], zero);
+    const bool odd = !all_zero(nil);
     for (int e = 0; odd && e < 4 * ROWS; ++e) {
         const int iy = 2 * (q0 + (e >> 2)) - g.pt + ((e >> 1) & 1), jx = ix + (e & 1);
         if (iy < 0 || iy >= g.H || jx < 0 || jx >= g.W) continue;

@@ -96,6 +96,9 @@ __device__ __forceinline__ bool finite4(const float4& v) {
     return isfinite(v.x) && isfinite(v.y) && isfinite(v.z) && isfinite(v.w);
 }
 
+// Of sums of values times zero: false when one of the values was not finite.
+__device__ __forceinline__ bool all_zero(const float4& v) { return v.x + v.y + (v.z + v.w) == 0.f; }
+
 // ---- context --------------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,

@@ -59,7 +59,7 @@ __device__ __noinline__ float4 gradient_of_existing(const float* x, const float*
     return acc;
 }
 
-template <int S, int ROWS, int D = 1>
+template <int S, int ROWS, int D = 1, bool GRADIENT = false>
 __global__ void __launch_bounds__(DW_THREADS)
 depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ f, const float* __restrict__ bias,
                     int act, float* __restrict__ y, const __grid_constant__ ConvGeom g, int tc, int c4_tiles) {
@@ -74,8 +74,8 @@ depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ f, co
     const int c = c4 * 4;
 
     float4 w[9];
-    const int f_step = g.reversed ? -g.C : g.C;
-    if (g.reversed) f += 8 * (int64_t)g.C;
+    const int f_step = GRADIENT ? -g.C : g.C;
+    if (GRADIENT) f += 8 * (int64_t)g.C;
 #pragma unroll
     for (int t = 0; t < 9; ++t) w[t] = ld4(f + (int64_t)t * f_step + c);
 
@@ -126,9 +126,11 @@ depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ f, co
             *reinterpret_cast<float4*>(y + ((n * g.Ho + oy) * (int64_t)g.Wo + ox) * g.Co + c) = v;
         }
     }
-    if (!g.reversed) return;
-    bool odd = false;  // (a gradient has neither bias nor activation)
-    for (int t = 0; t < 9; ++t) odd = odd || !finite4(ld4(f + (int64_t)t * f_step + c));
+    if (!GRADIENT) return;
+    float4 nil = zero;  // (a gradient has neither bias nor activation)
+#pragma unroll
+    for (int t = 0; t < 9; ++t) fma4_packed(nil, w[t], zero);
+    const bool odd = !all_zero(nil);
     for (int oy = oy0; odd && oy < min(g.Ho, oy0 + ROWS); ++oy)
         *reinterpret_cast<float4*>(y + ((n * g.Ho + oy) * (int64_t)g.Wo + ox) * g.Co + c) = gradient_of_existing(x, f, f_step, g, n, oy, ox, c);
 }
@@ -349,8 +351,11 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
                     dw_tap(w[k], __ldg(reinterpret_cast<const float4*>(f + (int64_t)k * t.f_step + c)));
                 if (bias) b = __ldg(reinterpret_cast<const float4*>(bias + c));
                 if constexpr (GRADIENT) {
+                    float4 nil = make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float4 zero = nil;
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) odd = odd || !finite4(w[k]);
+                    for (int k = 0; k < 9; ++k) fma4_packed(nil, w[k], zero);
+                    odd = odd || !all_zero(nil);
                 }
                 loaded_cb = cb;
             }
@@ -577,14 +582,11 @@ cudaError_t launch_depthwise(const DepthwisePlan& plan, const float* x, const fl
         const int gy = (g.Ho + ROWS - 1) / ROWS;
         if (gx <= 2147483647LL && gy <= 65535) {
             dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)g.N);
-            if (g.dh == 2)
-                depthwise3x3_kernel<1, ROWS, 2><<<grid, DW_THREADS, 0, s>>>(x, f, bias, act, y, g, tc, c4_tiles);
-            else if (g.dh == 4)
-                depthwise3x3_kernel<1, ROWS, 4><<<grid, DW_THREADS, 0, s>>>(x, f, bias, act, y, g, tc, c4_tiles);
-            else if (g.sh == 1)
-                depthwise3x3_kernel<1, ROWS><<<grid, DW_THREADS, 0, s>>>(x, f, bias, act, y, g, tc, c4_tiles);
-            else
-                depthwise3x3_kernel<2, ROWS><<<grid, DW_THREADS, 0, s>>>(x, f, bias, act, y, g, tc, c4_tiles);
+            auto kernel = depthwise3x3_kernel<2, ROWS>;
+            if (g.dh == 2) kernel = g.reversed ? depthwise3x3_kernel<1, ROWS, 2, true> : depthwise3x3_kernel<1, ROWS, 2>;
+            else if (g.dh == 4) kernel = g.reversed ? depthwise3x3_kernel<1, ROWS, 4, true> : depthwise3x3_kernel<1, ROWS, 4>;
+            else if (g.sh == 1) kernel = g.reversed ? depthwise3x3_kernel<1, ROWS, 1, true> : depthwise3x3_kernel<1, ROWS>;
+            kernel<<<grid, DW_THREADS, 0, s>>>(x, f, bias, act, y, g, tc, c4_tiles);
             ++*launches;
             return cudaGetLastError();
         }
