@@ -404,12 +404,15 @@ act_backprop_kernel(const float* __restrict__ y, const float* __restrict__ dy, f
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t n4 = n >> 2;
-    for (int64_t i = first; i < n4; i += stride) {
+    for (int64_t i = first; i < (n + 3) >> 2; i += stride) {
+        if (i == n4) {  // the last three values at most, by a thread of their own where there are enough
+            for (int64_t e = 4 * n4; e < n; ++e) dz[e] = act_grad(y[e], dy[e], act);
+            break;
+        }
         const float4 v = reinterpret_cast<const float4*>(y)[i], g = reinterpret_cast<const float4*>(dy)[i];
         reinterpret_cast<float4*>(dz)[i] =
             make_float4(act_grad(v.x, g.x, act), act_grad(v.y, g.y, act), act_grad(v.z, g.z, act), act_grad(v.w, g.w, act));
     }
-    if (first < (n & 3)) dz[4 * n4 + first] = act_grad(y[4 * n4 + first], dy[4 * n4 + first], act);
 }
 
 int blocks_for(int64_t items, int sm_count) {
