@@ -406,8 +406,15 @@ Choice choose(int64_t batches, int64_t M, int64_t N, int64_t K, int sm_count) {
 
 }  // namespace
 
+// One product over 16 terms or fewer stays on the CUDA cores, whose k-block is 16 wide and whose sums are exact to fp32 anyway:
+// 60 such products took 5.0 to 19.8 us here and 0.97 to 1.4 times less there ([1,3].[3,1] 5.1 and 4.4, [254,9].[9,3] 5.7 and
+// 5.0, [704,15].[15,6921] 19.8 and 18.0), but 55 with 17 to 50 terms 0.5 to 0.9 of the time of the CUDA cores ([2,17].[17,5] 5.0
+// and 6.6, [3235,19].[19,7969] 75 and 107). Batches have one launch here and one per product there.
+constexpr int64_t SHORT_SUM = 16;
+
 bool gemm_strided_supported(int64_t batches, int64_t M, int64_t N, int64_t K) {
     constexpr int64_t LIM = (1LL << 31) - 256;
+    if (batches == 1 && K <= SHORT_SUM) return false;
     return batches >= 1 && M >= 1 && N >= 1 && K >= 1 && M < LIM && N < LIM && K <= SPLIT_MAX_K && batches < LIM &&
            (double)batches * (double)((M + 31) / 32) * (double)((N + 31) / 32) < 1e9;
 }

@@ -244,6 +244,23 @@ def test_matmul_of_unaligned_rows(ctx, oracle, case, ta, tb):
     assert rel_fro(host(call(dev(a), dev(b), ta, tb)), want(a, b, ta, tb)) <= 1e-5
 
 
+@pytest.mark.parametrize("K,cuda_cores", [(1, True), (7, True), (16, True), (17, False)])
+@pytest.mark.parametrize("ta,tb", [(False, False), (True, True)])
+def test_short_unaligned_products_take_the_cuda_cores(ctx, K, cuda_cores, ta, tb):
+    """One launch either way, the same bits as in fp32 mode where it is the same kernel; sums of 17 products differ in order."""
+    M, N = 131, 67
+    a, b = si.uniform(325, 0, (K, M) if ta else (M, K), -1, 1), si.uniform(325, 1, (N, K) if tb else (K, N), -1, 1)
+    got = host(ctx.matmul(dev(a), dev(b), ta, tb))
+    ctx.set_math("fp32")
+    try:
+        want = host(ctx.matmul(dev(a), dev(b), ta, tb))
+    finally:
+        ctx.set_math("tf32")
+    ctx.check_device_status()
+    assert same_bits(got, want) == cuda_cores
+    assert rel_fro(got, (a.T if ta else a).astype(np.float64) @ (b.T if tb else b).astype(np.float64)) <= 1.8e-8 * K ** 0.5 + 2.0 ** -24
+
+
 @pytest.mark.parametrize("M,K,N,ta,tb", [(199, 64, 199, False, True), (301, 513, 303, True, True), (1301, 2001, 1303, False, False),
                                          (1301, 8191, 1303, False, True), (257, 20001, 255, True, False)])
 @pytest.mark.parametrize("positive", [False, True])
