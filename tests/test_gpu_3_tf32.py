@@ -332,8 +332,8 @@ IM2COL_CASES = [
     (2, 12, 10, 132, 2, 4, 260, (1, 1), "same", (1, 1)),   # even windows: padding after one more than before
     (4, 9, 7, 64, 1, 1, 40, (2, 2), "same", (1, 1)),       # strided 1x1
     (9, 30, 30, 64, 3, 3, 64, (1, 1), "same", (1, 1)),     # several tiles per CTA
-    # a large window.  The tensor core cuts its fp32 sums (2^-24 of the sum at most per MMA, 7e-9 seen on average): with
-    # 33 x 33 taps, 4356 MMAs long, that alone is 3e-5; 13 x 13 taps stay below the bar of 2e-5
+    # a large window.  The tensor core cuts its fp32 sums at every MMA, by 7e-9 of the result on average with these operands
+    # (1.8e-8 seen with others): with 33 x 33 taps, 4356 MMAs long, that alone is 3e-5; 13 x 13 taps stay below 2e-5
     (1, 40, 40, 16, 13, 13, 4, (1, 1), "valid", (1, 1)),
 ]
 

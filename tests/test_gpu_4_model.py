@@ -220,10 +220,14 @@ def _close_logits(got, want, rel=1e-2):
     assert np.max(np.abs(got - want) / span) <= rel
 
 
-@pytest.mark.parametrize("math", ["tf32", "bf16"])
-@pytest.mark.parametrize("batch,hw,alpha,output_stride", [
+SMALL_MODELS = [
     (1, 64, 0.25, 32), (2, 65, 0.25, 32), (3, 33, 0.5, 32), (1, 96, 0.75, 32), (5, 47, 0.25, 32), (9, 64, 0.25, 32), (17, 32, 0.25, 32), (20, 50, 0.25, 32),
-    (38, 32, 0.25, 32), (60, 32, 0.25, 32), (100, 32, 0.25, 32), (2, 81, 0.25, 16), (1, 81, 0.25, 8), (40, 33, 0.25, 8)])
+    (38, 32, 0.25, 32), (60, 32, 0.25, 32), (100, 32, 0.25, 32), (2, 81, 0.25, 16), (1, 81, 0.25, 8), (40, 33, 0.25, 8)]
+
+
+# (no dilation in the bfloat16 storage mode)
+@pytest.mark.parametrize("batch,hw,alpha,output_stride,math",
+                         [(*m, math) for math in ("tf32", "bf16") for m in SMALL_MODELS if math == "tf32" or m[3] == 32])
 def test_layers_of_a_small_model_in_one_kernel(ctx, oracle, batch, hw, alpha, output_stride, math):
     """Clusters of 16 blocks down to a few, several images per cluster, odd widths, dilated layers: the layers in one
     kernel against the layers' own kernels (both at the whole-model bar from the oracle; a bfloat16 value at a rounding
@@ -231,8 +235,6 @@ def test_layers_of_a_small_model_in_one_kernel(ctx, oracle, batch, hw, alpha, ou
     if output_stride == 32:
         x, layers = si.config_mobilenet(alpha, hw, batch, seed=4243, classes=100)
     else:
-        if math == "bf16":
-            pytest.skip("no dilation in the bfloat16 storage mode")
         x, layers = si.config_mobilenet_atrous(alpha, hw, batch, output_stride, seed=4243, classes=100)
     ctx.set_math(math)
     try:
