@@ -322,7 +322,7 @@ static tfjsb_status matmul_2d(tfjsb_ctx* ctx, const float* pa, const float* pb, 
     }
     const int64_t a_rs = transpose_a ? 1 : K, a_cs = transpose_a ? M : 1;
     const int64_t b_rs = transpose_b ? 1 : N, b_cs = transpose_b ? K : 1;
-    if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(1, M, N, K)) {
+    if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(1, M, N, K, ctx->sm_count)) {
         // rows that are no multiples of 16 bytes: fp32 accuracy on the tensor cores
         if ((e = launch_gemm_strided(pa, a_rs, a_cs, pb, b_rs, b_cs, nullptr, TFJSB_ACT_NONE, pc, 1, M, N, K, ctx->sm_count,
                                      ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
@@ -423,7 +423,7 @@ tfjsb_status tfjsb_batch_matmul(tfjsb_ctx* ctx, const tfjsb_tensor* a, const tfj
             return cuda_fail(ctx, e, "batched tf32 gemm launch");
         return TFJSB_OK;
     }
-    if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(B, M, N, K) && !gemm_tf32_supported(M, N, K)) {
+    if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(B, M, N, K, ctx->sm_count) && !gemm_tf32_supported(M, N, K)) {
         cudaError_t e = launch_gemm_strided(pa, transpose_a ? 1 : K, transpose_a ? M : 1, pb, transpose_b ? 1 : N, transpose_b ? K : 1,
                                             nullptr, TFJSB_ACT_NONE, pc, B, M, N, K, ctx->sm_count, ctx->dev_status, s, &ctx->launches);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "batched strided gemm launch");
@@ -479,7 +479,7 @@ tfjsb_status tfjsb_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_ten
                 return cuda_fail(ctx, e, "tf32 gemm launch");
             return TFJSB_OK;
         }
-        if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(1, M, N, K)) {
+        if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(1, M, N, K, ctx->sm_count)) {
             if ((e = launch_gemm_strided(px, K, 1, pf, N, 1, pbias, act, py, 1, M, N, K, ctx->sm_count, ctx->dev_status, s,
                                          &ctx->launches)) != cudaSuccess)
                 return cuda_fail(ctx, e, "strided gemm launch");

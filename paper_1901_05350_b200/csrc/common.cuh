@@ -228,7 +228,7 @@ cudaError_t launch_gemm_fp32(const float* a, int64_t a_rs, int64_t a_cs, const f
 
 // The same with fp32 accuracy on the tensor cores, for operands with either dimension contiguous and any alignment
 // (gemm_strided_tcgen05.cu); `batches` products stored one after the other.
-bool gemm_strided_supported(int64_t batches, int64_t M, int64_t N, int64_t K);
+bool gemm_strided_supported(int64_t batches, int64_t M, int64_t N, int64_t K, int sm_count);
 cudaError_t launch_gemm_strided(const float* a, int64_t a_rs, int64_t a_ks, const float* b, int64_t b_ks, int64_t b_cs, const float* bias,
                                 int act, float* c, int64_t batches, int64_t M, int64_t N, int64_t K, int sm_count,
                                 unsigned int* dev_status, cudaStream_t s, int64_t* launches);

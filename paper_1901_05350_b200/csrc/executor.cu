@@ -252,7 +252,7 @@ cudaError_t launch_step(tfjsb_model* m, const Step& st, cudaStream_t s) {
         case STEP_GEMM_TF32:
             return launch_gemm_tf32(st.plan, st.bias, st.act, ctx->dev_status, s, &ctx->launches);
         case STEP_GEMM_FP32:
-            if (m->use_tf32 && gemm_strided_supported(1, st.M, st.N, st.K))
+            if (m->use_tf32 && gemm_strided_supported(1, st.M, st.N, st.K, m->ctx->sm_count))
                 return launch_gemm_strided(st.in, st.K, 1, st.filter, st.N, 1, st.bias, st.act, st.out, 1, st.M, st.N, st.K,
                                            ctx->sm_count, ctx->dev_status, s, &ctx->launches);
             return launch_gemm_fp32(st.in, st.K, 1, st.filter, st.N, 1, st.bias, st.act, st.out, st.N, st.M, st.N, st.K,
@@ -1129,7 +1129,7 @@ tfjsb_status tfjsb_model_layer_kernel(tfjsb_model* m, int layer, char* name, int
             k = st.plan.pair ? "gemm_pair_kernel<false>" : st.plan.cluster_split ? "gemm_tf32_splitk_kernel" : "gemm_tf32_kernel<false>";
             break;
         case STEP_CONV_TF32: k = st.conv_patch ? "dwpw_fused_kernel<true>" : st.plan.im2col ? "gemm_tf32_im2col_kernel" : "gemm_tf32_kernel<true>"; break;
-        case STEP_GEMM_FP32: k = m->use_tf32 && gemm_strided_supported(1, st.M, st.N, st.K) ? "gemm_strided_kernel" : "gemm_fp32_kernel"; break;
+        case STEP_GEMM_FP32: k = m->use_tf32 && gemm_strided_supported(1, st.M, st.N, st.K, m->ctx->sm_count) ? "gemm_strided_kernel" : "gemm_fp32_kernel"; break;
         case STEP_CONV_FP32: k = "conv2d_fp32_kernel"; break;
         case STEP_DEPTHWISE: k = st.dw_plan.variant >= 0 ? "depthwise3x3_tma_kernel" : "depthwise3x3_kernel"; break;
         case STEP_POOL: k = (st.g.Ho == 1 && st.g.Wo == 1 && st.g.fh == st.g.H && st.g.fw == st.g.W) ? "avg_pool_global_kernel" : "avg_pool_window_kernel"; break;

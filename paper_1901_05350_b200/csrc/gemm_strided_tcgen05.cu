@@ -20,6 +20,8 @@
 // of MMAs; sixteen loader warps per CTA were slower (2001^3: 297 us against 220), and so was fetching the next values before
 // this k-block's are stored, which takes twice the registers (2001^3: 275 us against 205).  64 products [199,64] . [64,199]:
 // 1179 us as 64 launches of the CUDA-core kernel, 18.6 us here; [64,1024] . [1024,101]: 201 us and 10.5 us.
+#include <algorithm>
+
 #include "common.cuh"
 #include "ptx_sm100.cuh"
 #include "umma_tile.cuh"
@@ -404,17 +406,26 @@ Choice choose(int64_t batches, int64_t M, int64_t N, int64_t K, int sm_count) {
     return best;
 }
 
+// One product over 16 terms or fewer, a single k-block of the CUDA-core kernel, takes what its tiles and their stores take:
+// there 128 x 128 tiles, here 128 x 64.  The CUDA cores are faster while an SM has one of the larger tiles at most (60 products
+// 5.0 to 7.3 us here and mostly 0.7 to 0.95 of that there: [1,3].[3,1] 5.1 and 4.4, [254,9].[9,3] 5.7 and 5.0, [16000,7].[7,13] 6.6
+// and 5.9; [20000,7].[7,9], 157 tiles, 7.6 and 9.7), and beyond that where the smaller tiles are 1.6 times as many or more
+// ([30000,7].[7,101] 15.3 and 12.0, [704,15].[15,6921] 19.8 and 18.0, [9000,7].[7,260] 13.7 and 12.9, but
+// [100000,7].[7,33] 21.7 and 28.4, [20000,7].[7,130] 15.2 and 16.3, [1000000,3].[3,1] 133 and 268).  55 products of 17 to 50 terms
+// take 0.5 to 0.9 of the time of the CUDA cores ([2,17].[17,5] 5.0 and 6.6, [3235,19].[19,7969] 75 and 107).  Batches have
+// one launch here and one per product there.
+bool short_sum_on_cuda_cores(int64_t M, int64_t N, int64_t K, int sm_count) {
+    if (K > 16) return false;
+    const int64_t wide = ((M + 127) / 128) * ((N + 127) / 128);
+    const int64_t narrow = std::min(((M + 127) / 128) * ((N + 63) / 64), ((N + 127) / 128) * ((M + 63) / 64));
+    return wide <= sm_count || 5 * narrow >= 8 * wide;
+}
+
 }  // namespace
 
-// One product over 16 terms or fewer stays on the CUDA cores, whose k-block is 16 wide and whose sums are exact to fp32 anyway:
-// 60 such products took 5.0 to 19.8 us here and 0.97 to 1.4 times less there ([1,3].[3,1] 5.1 and 4.4, [254,9].[9,3] 5.7 and
-// 5.0, [704,15].[15,6921] 19.8 and 18.0), but 55 with 17 to 50 terms 0.5 to 0.9 of the time of the CUDA cores ([2,17].[17,5] 5.0
-// and 6.6, [3235,19].[19,7969] 75 and 107). Batches have one launch here and one per product there.
-constexpr int64_t SHORT_SUM = 16;
-
-bool gemm_strided_supported(int64_t batches, int64_t M, int64_t N, int64_t K) {
+bool gemm_strided_supported(int64_t batches, int64_t M, int64_t N, int64_t K, int sm_count) {
     constexpr int64_t LIM = (1LL << 31) - 256;
-    if (batches == 1 && K <= SHORT_SUM) return false;
+    if (batches == 1 && short_sum_on_cuda_cores(M, N, K, sm_count)) return false;
     return batches >= 1 && M >= 1 && N >= 1 && K >= 1 && M < LIM && N < LIM && K <= SPLIT_MAX_K && batches < LIM &&
            (double)batches * (double)((M + 31) / 32) * (double)((N + 31) / 32) < 1e9;
 }

@@ -124,7 +124,7 @@ extern "C" tfjsb_status tfjsb_matmul_static_scratch(tfjsb_ctx* ctx, const tfjsb_
     // rows that are no multiples of 16 bytes, or FP32 mode: strided operand access, no scratch at all
     const int64_t a_rs = transpose_a ? 1 : K, a_cs = transpose_a ? M : 1;
     const int64_t b_rs = transpose_b ? 1 : N, b_cs = transpose_b ? K : 1;
-    if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(1, M, N, K)) {
+    if (ctx->math == TFJSB_MATH_TF32 && gemm_strided_supported(1, M, N, K, ctx->sm_count)) {
         if ((e = launch_gemm_strided(pa, a_rs, a_cs, pb, b_rs, b_cs, nullptr, TFJSB_ACT_NONE, pc, 1, M, N, K, ctx->sm_count,
                                      ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
             return cuda_fail(ctx, e, "strided gemm launch");
