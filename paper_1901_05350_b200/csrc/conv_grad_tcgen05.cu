@@ -31,6 +31,7 @@
 // order.  Bound by shared-memory bandwidth (about 1800 cycles per k-block with the lo half, 1000 without, against 768 /
 // 256 of MMAs).  [16,28,28,128], 3x3: 811 us with 32 x 32 tiles on CUDA cores, 40 us here (38 with one accumulator).
 // Pointwise, plain TF32, [32,56,56] 128 x 128: 36 + 36 us of transposes and 23 + 8 us of batched products, 25 + 6 us here.
+#include <algorithm>
 #include <cstdlib>
 
 #include "common.cuh"
@@ -721,12 +722,14 @@ static GradInputTiling grad_input_tiling(const ConvGeom& g, int64_t m_tiles, int
 }
 
 // Where a sample's sum is short, one CUDA-core thread per sample is the faster kernel.  In microseconds, fitted to both on
-// 110 shapes (4 to 64 output channels, windows up to 7 x 7, strides 1 to 3; 6 % of them still go to the slower one):
+// 145 shapes (4 to 64 output channels, windows up to 7 x 7, strides 1 to 3; 4 % of them still go to the slower one):
 //   here         3, and for each round of tiles 1.4 and 0.72 per k-block, of which a tap makes at least one however few its
 //                channels; parts of the K loop 2.5 more, several residue classes 1
 //   CUDA cores   2.5 and 0.42 per tap of a class, the chain of one thread; its samples x products at 0.2 to 1.7 per ps, the
-//                fewer the longer the filter rows that threads read apart
-// [15,8,8,20], 3x3, 8 channels: 11.3 us here and 7.6; [5,27,27,256]: 13.6 and 70; [35,108,108,4]: 174 and 75.
+//                fewer the longer the filter rows that threads read apart; strided, 2 ps a sample, also of those without a
+//                product; a strided 1x1, most of whose samples have none, 6.2 ps a sample and 0.6 per product
+// [15,8,8,20], 3x3, 8 channels: 11.3 us here and 7.6; [5,27,27,256]: 13.6 and 70; [35,108,108,4]: 174 and 75;
+// [4,224,224,64], 1x1 / 3, 4 channels: 28 and 85.
 bool conv2d_grad_input_preferred(const ConvGeom& g, int sm_count) {
     if (const char* env = getenv("TFJSB_GRAD_INPUT")) return atoi(env) != 0;  // for tests: 1 = this kernel wherever it can
     int q0h, q0w, Qh, Qw;
@@ -740,8 +743,9 @@ bool conv2d_grad_input_preferred(const ConvGeom& g, int sm_count) {
     const double per_us = g.C <= 8 && g.Co <= 16 ? 1.7e6 : g.Co <= 12 ? 1.0e6 : g.Co <= 16 || g.C <= 8 ? 0.52e6 : 0.22e6;
     const double class_taps = (double)((g.fh + g.sh - 1) / g.sh) * ((g.fw + g.sw - 1) / g.sw);
     // the threads of a warp are neighbouring channels: fewer than 32 of them and a strided window's taps diverge
-    const double chain = !strided ? 0.02 * products : (taps > 1 ? 0.08 * g.Co : 0) + (g.C < 32 ? 0.2 : 0.02) * taps;
-    return here <= 2.5 + 0.42 * class_taps + chain + samples * products * (strided ? 2 : 1) / per_us;
+    const double chain = !strided ? 0.02 * products : (taps > 1 ? 0.08 * g.Co : 0.07 * std::max<int64_t>(0, g.Co - 24)) + (g.C < 32 ? 0.2 : 0.02) * taps;
+    const double each = !strided ? products / per_us : taps > 1 ? 2 * products / per_us + 2e-6 : 0.6e-6 * products + 6.2e-6;
+    return here <= 2.5 + 0.42 * class_taps + chain + samples * each;
 }
 
 bool conv2d_grad_input_supported(const ConvGeom& g) {
