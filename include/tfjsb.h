@@ -96,7 +96,7 @@ const char* tfjsb_last_error(tfjsb_ctx* ctx);
  * write.  Returns TFJSB_ERR_TIMEOUT (and clears the word) if any wait gave up since the last
  * check, TFJSB_OK otherwise. */
 tfjsb_status tfjsb_check_device_status(tfjsb_ctx* ctx, void* stream);
-/* Sizes the context's three scratch blocks (transposed matMul operands, partial sums of the filter and
+/* Sizes the context's three scratch blocks (packed filters, transposed operands, partial sums of the filter and
  * bias gradients) to at least `bytes` each, so that later op calls find them large enough.  An op that
  * needs more grows its block by allocating a larger one (cudaMalloc, no synchronisation; the old block is
  * kept until tfjsb_shutdown because kernels in flight may still read it). */
@@ -121,17 +121,17 @@ tfjsb_status tfjsb_window_out_shape(int64_t in, int k, int stride, int dilation,
  *   out[M,N] = op(a) . op(b);  a is [M,K], or [K,M] when transpose_a; b is [K,N], or [N,K]
  *   when transpose_b.  Rank 2 only.  Inner-dimension or `out` mismatch: TFJSB_ERR_SHAPE.
  * TF32 mode uses the tensor-core kernel when K % 4 == 0 and N % 4 == 0 (row pitches must be
- * multiples of 16 bytes for the bulk tensor copies); operands that are not already K-contiguous
- * are transposed into context-owned scratch first (grown on demand without synchronising, see
- * tfjsb_reserve_scratch).  Other shapes are fp32 products, on the tensor cores too (each operand as two TF32
+ * multiples of 16 bytes for the bulk tensor copies) and reads operands as they are stored; only a
+ * transposed `a` with M % 4 != 0 goes through context-owned scratch first (grown on demand without
+ * synchronising, see tfjsb_reserve_scratch).  Other shapes are fp32 products, on the tensor cores too (each operand as two TF32
  * values: as exact as fp32 multiply-adds, with the same infinities and NaNs) up to K = 2^22, else, and in FP32
  * mode, on CUDA cores. */
 tfjsb_status tfjsb_matmul(tfjsb_ctx* ctx, const tfjsb_tensor* a, const tfjsb_tensor* b, int transpose_a,
                           int transpose_b, tfjsb_tensor* out, void* stream);
 
 /* The same operation as tfjsb_matmul for callers that must not allocate device memory; the
- * paper has no counterpart of this call.  tfjsb_matmul transposes operands that are not
- * K-contiguous into scratch memory it takes from cudaMalloc.  Some callers cannot afford that
+ * paper has no counterpart of this call.  tfjsb_matmul may take scratch memory for a transposed
+ * operand from cudaMalloc; this call transposes every operand that is not K-contiguous.  Some callers cannot afford that
  * where they call the library: a real-time loop that may not block on the allocator or on the
  * device synchronisation an allocation can imply, a service whose device-memory budget was
  * fixed at start-up, any code that runs at a point where cudaMalloc is not permitted.  Here the

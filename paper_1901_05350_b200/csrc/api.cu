@@ -299,23 +299,18 @@ static tfjsb_status matmul_2d(tfjsb_ctx* ctx, const float* pa, const float* pb, 
 
     if (ctx->math == TFJSB_MATH_TF32 && gemm_tf32_supported(M, N, K) && ctx->encode_tiled && aligned16(pa) && aligned16(pb) &&
         aligned16(pc)) {
-        // make both operands K-contiguous: A as [M,K], B as [N,K]
-        const float* a_km = pa;
-        const float* b_km = pb;
-        if (transpose_a) {  // stored [K,M]
+        // A stored [K,M] and B stored [K,N] are read as they are; A is transposed into scratch where its rows of M values
+        // are no multiples of 16 bytes
+        const float* a_tc = pa;
+        const bool a_mn = transpose_a && M % 4 == 0;
+        if (transpose_a && !a_mn) {
             if ((st = ensure_scratch(ctx, &ctx->scratch_a, (size_t)M * K * 4)) != TFJSB_OK) return st;
             if ((e = launch_transpose(pa, ctx->scratch_a.ptr, K, M, s, &ctx->launches)) != cudaSuccess)
                 return cuda_fail(ctx, e, "transpose(a)");
-            a_km = ctx->scratch_a.ptr;
-        }
-        if (!transpose_b) {  // stored [K,N]
-            if ((st = ensure_scratch(ctx, &ctx->scratch_b, (size_t)N * K * 4)) != TFJSB_OK) return st;
-            if ((e = launch_transpose(pb, ctx->scratch_b.ptr, K, N, s, &ctx->launches)) != cudaSuccess)
-                return cuda_fail(ctx, e, "transpose(b)");
-            b_km = ctx->scratch_b.ptr;
+            a_tc = ctx->scratch_a.ptr;
         }
         GemmTf32Plan plan;
-        if ((st = gemm_tf32_plan(ctx, a_km, b_km, pc, M, N, K, &plan)) != TFJSB_OK) return st;
+        if ((st = gemm_tf32_plan(ctx, a_tc, pb, pc, M, N, K, &plan, 1, a_mn, !transpose_b)) != TFJSB_OK) return st;
         if ((e = launch_gemm_tf32(plan, nullptr, TFJSB_ACT_NONE, ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
             return cuda_fail(ctx, e, "tf32 gemm launch");
         return TFJSB_OK;
@@ -400,25 +395,19 @@ tfjsb_status tfjsb_batch_matmul(tfjsb_ctx* ctx, const tfjsb_tensor* a, const tfj
     float* pc = static_cast<float*>(out->data);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (B > 1 && ctx->math == TFJSB_MATH_TF32 && gemm_tf32_supported(M, N, K) && ctx->encode_tiled) {
-        // All products in one launch of the tensor-core kernel: their tiles share the SMs.  Operands
-        // that are not K-contiguous are transposed into scratch first, all products of an operand in one launch.
+        // All products in one launch of the tensor-core kernel: their tiles share the SMs.  Operands are read either way
+        // round (see matmul_2d).
         cudaError_t e;
-        const float* a_km = pa;
-        const float* b_km = pb;
-        if (transpose_a) {
+        const float* a_tc = pa;
+        const bool a_mn = transpose_a && M % 4 == 0;
+        if (transpose_a && !a_mn) {
             if ((st = ensure_scratch(ctx, &ctx->scratch_a, (size_t)B * M * K * 4)) != TFJSB_OK) return st;
             if ((e = launch_transpose_batched(pa, ctx->scratch_a.ptr, B, K, M, s, &ctx->launches)) != cudaSuccess)
                 return cuda_fail(ctx, e, "transpose(a)");
-            a_km = ctx->scratch_a.ptr;
-        }
-        if (!transpose_b) {
-            if ((st = ensure_scratch(ctx, &ctx->scratch_b, (size_t)B * N * K * 4)) != TFJSB_OK) return st;
-            if ((e = launch_transpose_batched(pb, ctx->scratch_b.ptr, B, K, N, s, &ctx->launches)) != cudaSuccess)
-                return cuda_fail(ctx, e, "transpose(b)");
-            b_km = ctx->scratch_b.ptr;
+            a_tc = ctx->scratch_a.ptr;
         }
         GemmTf32Plan plan;
-        if ((st = gemm_tf32_plan(ctx, a_km, b_km, pc, M, N, K, &plan, B)) != TFJSB_OK) return st;
+        if ((st = gemm_tf32_plan(ctx, a_tc, pb, pc, M, N, K, &plan, B, a_mn, !transpose_b)) != TFJSB_OK) return st;
         if ((e = launch_gemm_tf32(plan, nullptr, TFJSB_ACT_NONE, ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
             return cuda_fail(ctx, e, "batched tf32 gemm launch");
         return TFJSB_OK;
@@ -470,11 +459,8 @@ tfjsb_status tfjsb_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_ten
         // x viewed as [N*H*W, Cin] (a free reshape), filter as [Cin, Cout]
         const int64_t M = g.N * g.H * g.W, K = g.C, N = Cout;
         if (ctx->math == TFJSB_MATH_TF32 && gemm_tf32_supported(M, N, K) && ctx->encode_tiled) {
-            if ((st = ensure_scratch(ctx, &ctx->scratch_b, (size_t)N * K * 4)) != TFJSB_OK) return st;
-            if ((e = launch_transpose(pf, ctx->scratch_b.ptr, K, N, s, &ctx->launches)) != cudaSuccess)
-                return cuda_fail(ctx, e, "transpose(filter)");
             GemmTf32Plan plan;
-            if ((st = gemm_tf32_plan(ctx, px, ctx->scratch_b.ptr, py, M, N, K, &plan)) != TFJSB_OK) return st;
+            if ((st = gemm_tf32_plan(ctx, px, pf, py, M, N, K, &plan, 1, false, true)) != TFJSB_OK) return st;
             if ((e = launch_gemm_tf32(plan, pbias, act, ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
                 return cuda_fail(ctx, e, "tf32 gemm launch");
             return TFJSB_OK;

@@ -260,7 +260,8 @@ cudaError_t launch_depthwise(const DepthwisePlan& plan, const float* x, const fl
                              int64_t* launches);
 
 // Tensor-core GEMM: C[M,N] = act(A[M,K] . Bt[N,K]^T + bias); all three row-major with K (resp. N)
-// contiguous.  A plan holds the tensor maps and tile choice; it can be built once and reused while
+// contiguous, or operands with their other dimension contiguous (a_mn: A as [K,M], M % 4 == 0; b_mn: B as [K,N]), whose
+// products have the same bits.  A plan holds the tensor maps and tile choice; it can be built once and reused while
 // the pointers stay the same.
 struct GemmTf32Plan {
     CUtensorMap map_a, map_b, map_c;
@@ -274,6 +275,7 @@ struct GemmTf32Plan {
     size_t smem_bytes;
     // CTA-pair kernel (gemm_pair.cu): 256 x block_n tiles shared by two CTAs
     bool pair = false;
+    bool a_mn = false, b_mn = false;   // A is stored [K, M], B is stored [K, N]
     // cluster split-K kernel (gemm_tf32_splitk.cu): `splits` CTAs per tile, reduced through shared memory
     bool cluster_split = false;
     int splits = 1, kb_per_split = 0;  // slices of the K loop (= cluster size) and k-blocks per slice
@@ -287,18 +289,18 @@ struct GemmTf32Plan {
 bool gemm_tf32_supported(int64_t M, int64_t N, int64_t K);
 // `batches` > 1: that many products of the same shape, operands and results stored one after the other.
 tfjsb_status gemm_tf32_plan(tfjsb_ctx* ctx, const float* a, const float* bt, float* c, int64_t M, int64_t N,
-                            int64_t K, GemmTf32Plan* plan, int64_t batches = 1);
+                            int64_t K, GemmTf32Plan* plan, int64_t batches = 1, bool a_mn = false, bool b_mn = false);
 // The same GEMM on CTA pairs; gemm_tf32_plan picks it where it is the faster kernel (environment
 // variable TFJSB_GEMM_PAIR: 0 = never, 1 = wherever the shape allows, unset = by shape).
 bool gemm_tf32_pair_preferred(int64_t M, int64_t N, int64_t K, int sm_count);
 tfjsb_status gemm_tf32_pair_plan(tfjsb_ctx* ctx, const float* a, const float* bt, float* c, int64_t M, int64_t N,
-                                 int64_t K, GemmTf32Plan* plan);
+                                 int64_t K, GemmTf32Plan* plan, bool a_mn, bool b_mn);
 cudaError_t launch_gemm_tf32_pair(const GemmTf32Plan& plan, const float* bias, int act, unsigned int* dev_status,
                                   cudaStream_t s, int64_t* launches);
 // Split K across the CTAs of a cluster, for GEMMs with too few tiles for the SMs (gemm_tf32_splitk.cu).
 bool gemm_tf32_splitk_choice(int64_t M, int64_t N, int64_t K, int sm_count, int64_t whole_ns, int* block_n, int* splits);
 tfjsb_status gemm_tf32_splitk_plan(tfjsb_ctx* ctx, const float* a, const float* bt, float* c, int64_t M, int64_t N,
-                                   int64_t K, int block_n, int splits, GemmTf32Plan* plan);
+                                   int64_t K, int block_n, int splits, GemmTf32Plan* plan, bool a_mn, bool b_mn);
 cudaError_t launch_gemm_tf32_splitk(const GemmTf32Plan& plan, const float* bias, int act, unsigned int* dev_status,
                                     cudaStream_t s, int64_t* launches);
 // Implicit-GEMM convolution on the same kernel: M = N*Ho*Wo output pixels, K = fh*fw*Cin, N = Cout.

@@ -159,6 +159,16 @@ __device__ __forceinline__ void gather_scalar(float (&v)[BLOCK_K], const float* 
     }
 }
 
+// An operand tile of 32 k whose rows of memory run along M or N: one copy of 32 k x 32 columns per group.
+template <bool BATCHED>
+__device__ __forceinline__ void load_mn_groups(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row0, int k0, int batch, int groups) {
+#pragma unroll 1
+    for (int i = 0; i < groups; ++i) {
+        if (BATCHED) tma_load_3d(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0, batch);
+        else tma_load_2d(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0);
+    }
+}
+
 // where the rows of A come from: a matrix in memory, threads that gather windows, or im2col copies of an NHWC tensor
 constexpr int A_TILED = 0;
 constexpr int A_GATHER = 1;
@@ -174,6 +184,8 @@ struct KernelArgs {
     int acc_stages;  // accumulator stages in tensor memory: 2 (block_n 256) or 4
     int epi_warps;   // 8 or 16
     int stage_tx;    // bytes that the copies of one stage deliver (fewer rows of A than a tile has when M is smaller)
+    int a_mn, b_mn;  // operands whose rows run along M (A is [K, M]) or N (B is [K, N]); instances with MN only
+    int a_groups;    // copies of 32 k x 32 rows that make the A tile (a_mn)
     const float* bias;
     int act;
     unsigned int* dev_status;
@@ -182,11 +194,12 @@ struct KernelArgs {
     ConvGeom g;
 };
 
-template <int A_SOURCE, int IO, bool BATCHED>
+template <int A_SOURCE, int IO, bool BATCHED, bool MN = false>
 __device__ __forceinline__ void gemm_pipeline(const CUtensorMap& map_a, const CUtensorMap& map_b, const CUtensorMap& map_c,
                                               const KernelArgs& args) {
     constexpr bool GATHER = A_SOURCE == A_GATHER, IM2COL = A_SOURCE == A_IM2COL;
     static_assert(A_SOURCE == A_TILED || IO == IO_F32, "the convolutions read fp32");
+    static_assert(!MN || (A_SOURCE == A_TILED && IO == IO_F32), "MN-major operands are fp32 matrices");
     constexpr bool IN_BF16 = IO != IO_F32;
     constexpr bool OUT_BF16 = IO == IO_BF16;
     constexpr int BK = IN_BF16 ? 64 : BLOCK_K;        // elements per k-block: 128 bytes either way
@@ -280,10 +293,12 @@ __device__ __forceinline__ void gemm_pipeline(const CUtensorMap& map_a, const CU
                     } else {
                         mbar_arrive_expect_tx(full, (uint32_t)args.stage_tx);
                         if (IM2COL) tma_load_im2col(a_dst, &map_a, full, c0, w0, h0, img, off_w, off_h);
+                        else if (MN && args.a_mn) load_mn_groups<BATCHED>(a_dst, &map_a, full, m0, kb * BK, batch, args.a_groups);
                         else if (BATCHED) tma_load_3d(a_dst, &map_a, full, kb * BK, m0, batch);
                         else tma_load_2d(a_dst, &map_a, full, kb * BK, m0);
                     }
-                    if (BATCHED) tma_load_3d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BK, n0, batch);
+                    if (MN && args.b_mn) load_mn_groups<BATCHED>(a_dst + A_STAGE_BYTES, &map_b, full, n0, kb * BK, batch, block_n >> 5);
+                    else if (BATCHED) tma_load_3d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BK, n0, batch);
                     else tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BK, n0);
                 }
                 if (IM2COL && (c0 += BK) >= args.g.C) {
@@ -313,7 +328,10 @@ __device__ __forceinline__ void gemm_pipeline(const CUtensorMap& map_a, const CU
         __syncwarp();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        const uint32_t idesc = IN_BF16 ? make_idesc_bf16(BLOCK_M, block_n) : make_idesc_tf32(BLOCK_M, block_n);
+        const bool a_mn = MN && args.a_mn, b_mn = MN && args.b_mn;
+        const uint32_t idesc = (IN_BF16 ? make_idesc_bf16(BLOCK_M, block_n) : make_idesc_tf32(BLOCK_M, block_n)) |
+                               (a_mn ? IDESC_A_MN : 0u) | (b_mn ? IDESC_B_MN : 0u);
+        const uint64_t a_step = a_mn ? 64 : 2, b_step = b_mn ? 64 : 2;
         int stage = 0;
         uint32_t phase = 0;
         int acc = 0;
@@ -326,12 +344,12 @@ __device__ __forceinline__ void gemm_pipeline(const CUtensorMap& map_a, const CU
             const uint32_t d_tmem = tmem_base + (uint32_t)(acc * block_n);
             for (int kb = 0; kb < num_k_blocks; ++kb) {
                 const uint32_t a_addr = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
-                const uint64_t a_desc = make_kmajor_sw128_desc(a_addr);
-                const uint64_t b_desc = make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
+                const uint64_t a_desc = a_mn ? make_mnmajor_desc(a_addr) : make_kmajor_sw128_desc(a_addr);
+                const uint64_t b_desc = b_mn ? make_mnmajor_desc(a_addr + A_STAGE_BYTES) : make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
                 // steps along K inside the 128-byte swizzled row: 32 bytes = 2 descriptor units
                 uint64_t ak[MMAS_PER_KB], bk[MMAS_PER_KB];
 #pragma unroll
-                for (int k = 0; k < MMAS_PER_KB; ++k) { ak[k] = a_desc + (uint64_t)(2 * k); bk[k] = b_desc + (uint64_t)(2 * k); }
+                for (int k = 0; k < MMAS_PER_KB; ++k) { ak[k] = a_desc + a_step * (uint64_t)k; bk[k] = b_desc + b_step * (uint64_t)k; }
                 if (leader && ok && (ok = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag))) {
                     tc_fence_after();
 #pragma unroll
@@ -556,6 +574,18 @@ gemm_tf32_batched_kernel(const __grid_constant__ CUtensorMap map_a, const __grid
     gemm_pipeline<A_TILED, IO_F32, true>(map_a, map_b, map_c, args);
 }
 
+// One product or a batch with operands as tf.matMul and a pointwise filter store them, [K, N] or [K, M], read by the tensor
+// core as they are: no transposing launch before the GEMM, the same bits.  512^3: 12.4 -> 8.3 us, with a as [K, M]
+// 16.5 -> 10.3; 2048^3 41 -> 33 and 57 -> 38; 4096^3 219 -> 167 and 277 -> 194; 64 products [200,64].[64,200] 14.4 -> 8.3.
+// A tile of such an operand comes in one copy per 32 columns instead of one, and 2048^3 is 26.7 us with K-contiguous
+// operands: an instance of its own, since the model's layers have their filters K-contiguous.
+template <bool BATCHED>
+__global__ void __launch_bounds__(GEMM_MAX_THREADS, 1)
+gemm_tf32_mn_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                    const __grid_constant__ CUtensorMap map_c, const KernelArgs args) {
+    gemm_pipeline<A_TILED, IO_F32, BATCHED, true>(map_a, map_b, map_c, args);
+}
+
 template <bool OUT_BF16>
 __global__ void __launch_bounds__(GEMM_MAX_THREADS, 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
@@ -654,7 +684,11 @@ tfjsb_status plan_common(tfjsb_ctx* ctx, const float* bt, int64_t k_pitch, float
     plan->num_tiles = (int)tiles;
     plan->grid = (int)(tiles < ctx->sm_count ? tiles : ctx->sm_count);
     tfjsb_status st;
-    if ((st = encode_2d(ctx, &plan->map_b, bt, k_pitch, N, BLOCK_K, plan->block_n, "B", batches)) != TFJSB_OK) return st;
+    if (plan->b_mn)
+        st = encode_2d(ctx, &plan->map_b, bt, N, plan->K, 32, BLOCK_K, "B", batches, false, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B);
+    else
+        st = encode_2d(ctx, &plan->map_b, bt, k_pitch, N, BLOCK_K, plan->block_n, "B", batches);
+    if (st != TFJSB_OK) return st;
     if ((st = encode_2d(ctx, &plan->map_c, c, N, M, EPI_COLS, 32, "C", batches)) != TFJSB_OK) return st;
     return TFJSB_OK;
 }
@@ -662,22 +696,24 @@ tfjsb_status plan_common(tfjsb_ctx* ctx, const float* bt, int64_t k_pitch, float
 }  // namespace
 
 tfjsb_status gemm_tf32_plan(tfjsb_ctx* ctx, const float* a, const float* bt, float* c, int64_t M, int64_t N,
-                            int64_t K, GemmTf32Plan* plan, int64_t batches) {
-    if (!gemm_tf32_supported(M, N, K) || batches < 1 || batches >= (1LL << 31))
+                            int64_t K, GemmTf32Plan* plan, int64_t batches, bool a_mn, bool b_mn) {
+    if (!gemm_tf32_supported(M, N, K) || batches < 1 || batches >= (1LL << 31) || (a_mn && M % 4 != 0))
         return fail(ctx, TFJSB_ERR_UNSUPPORTED, "shape not supported by the TF32 GEMM");
     if (!ctx->encode_tiled) return fail(ctx, TFJSB_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
     const char* pair_env = getenv("TFJSB_GEMM_PAIR");
     const bool use_pair = pair_env ? (pair_env[0] == '1' && N >= 64) : gemm_tf32_pair_preferred(M, N, K, ctx->sm_count);
-    if (batches == 1 && use_pair) return gemm_tf32_pair_plan(ctx, a, bt, c, M, N, K, plan);
+    if (batches == 1 && use_pair) return gemm_tf32_pair_plan(ctx, a, bt, c, M, N, K, plan, a_mn, b_mn);
     if (batches == 1) {
         // few tiles and a long K loop: the K loop is cut across the CTAs of a cluster (gemm_tf32_splitk.cu)
         int split_bn = 0, split_s = 0;
         int64_t whole_ns = 0;
         choose_block_n(M, N, (K + BLOCK_K - 1) / BLOCK_K, ctx->sm_count, 1, 0, &whole_ns);
         if (!getenv("TFJSB_NO_SPLIT_K") && gemm_tf32_splitk_choice(M, N, K, ctx->sm_count, whole_ns, &split_bn, &split_s))
-            return gemm_tf32_splitk_plan(ctx, a, bt, c, M, N, K, split_bn, split_s, plan);
+            return gemm_tf32_splitk_plan(ctx, a, bt, c, M, N, K, split_bn, split_s, plan, a_mn, b_mn);
     }
     plan->M = M; plan->N = N; plan->K = K;
+    plan->a_mn = a_mn;
+    plan->b_mn = b_mn;
     plan->pair = false;
     plan->cluster_split = false;
     plan->gather = false;
@@ -685,6 +721,7 @@ tfjsb_status gemm_tf32_plan(tfjsb_ctx* ctx, const float* a, const float* bt, flo
     plan->x = nullptr;
     tfjsb_status st;
     if ((st = plan_common(ctx, bt, K, c, plan, batches)) != TFJSB_OK) return st;
+    if (a_mn) return encode_2d(ctx, &plan->map_a, a, M, K, 32, BLOCK_K, "A", batches, false, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B);
     return encode_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, a_box_rows(M), "A", batches);
 }
 
@@ -727,6 +764,7 @@ tfjsb_status conv_igemm_plan(tfjsb_ctx* ctx, const float* x, const float* bt, fl
     plan->gather = !plan->im2col;
     plan->pair = false;
     plan->cluster_split = false;
+    plan->a_mn = plan->b_mn = false;
     plan->x = x;
     plan->g = g;
     tfjsb_status st = plan_common(ctx, bt, conv_igemm_k_pad(g), y, plan);
@@ -753,8 +791,11 @@ cudaError_t launch_gemm_tf32(const GemmTf32Plan& plan, const float* bias, int ac
                              cudaStream_t s, int64_t* launches) {
     if (plan.pair) return launch_gemm_tf32_pair(plan, bias, act, dev_status, s, launches);
     if (plan.cluster_split) return launch_gemm_tf32_splitk(plan, bias, act, dev_status, s, launches);
+    const bool mn = plan.a_mn || plan.b_mn;
+    auto mn_kernel = plan.batches > 1 ? gemm_tf32_mn_kernel<true> : gemm_tf32_mn_kernel<false>;
     const void* kernel = plan.gather ? reinterpret_cast<const void*>(&gemm_tf32_kernel<true>)
                          : plan.im2col ? reinterpret_cast<const void*>(&gemm_tf32_im2col_kernel)
+                         : mn ? reinterpret_cast<const void*>(mn_kernel)
                          : plan.batches > 1 ? reinterpret_cast<const void*>(&gemm_tf32_batched_kernel)
                                             : reinterpret_cast<const void*>(&gemm_tf32_kernel<false>);
     cudaError_t e = smem_attr_once(kernel, SMEM_LIMIT - 2048);
@@ -768,7 +809,10 @@ cudaError_t launch_gemm_tf32(const GemmTf32Plan& plan, const float* bias, int ac
     args.num_tiles = plan.num_tiles;
     args.acc_stages = plan.acc_stages;
     args.epi_warps = GATHER_EPI_WARPS;  // sixteen measured slower with fp32 tiles
-    args.stage_tx = (plan.im2col ? BLOCK_M : a_box_rows(plan.M)) * 128 + plan.block_n * 128;
+    args.a_mn = plan.a_mn;
+    args.b_mn = plan.b_mn;
+    args.a_groups = plan.M >= BLOCK_M ? BLOCK_M / 32 : (int)((plan.M + 31) / 32);
+    args.stage_tx = (plan.a_mn ? args.a_groups * 32 : plan.im2col ? BLOCK_M : a_box_rows(plan.M)) * 128 + plan.block_n * 128;
     args.bias = bias;
     args.act = act;
     args.dev_status = dev_status;
@@ -780,6 +824,8 @@ cudaError_t launch_gemm_tf32(const GemmTf32Plan& plan, const float* bias, int ac
     else if (plan.im2col)
         e = launch_k(gemm_tf32_im2col_kernel, dim3(plan.grid), dim3(64 + 32 * args.epi_warps), plan.smem_bytes, s, plan.map_a, plan.map_b,
                      plan.map_c, args);
+    else if (mn)
+        e = launch_k(mn_kernel, dim3(plan.grid), dim3(64 + 32 * args.epi_warps), plan.smem_bytes, s, plan.map_a, plan.map_b, plan.map_c, args);
     else if (plan.batches > 1)
         e = launch_k(gemm_tf32_batched_kernel, dim3(plan.grid), dim3(64 + 32 * args.epi_warps), plan.smem_bytes, s, plan.map_a,
                      plan.map_b, plan.map_c, args);

@@ -65,12 +65,19 @@ struct PairArgs {
     int stages;
     int n_tiles;    // tiles along N
     int num_tiles;  // total
+    int a_mn, b_mn; // operands stored [K, M] / [K, N] (the instance with MN only)
     const float* bias;
     int act;
     unsigned int* dev_status;
 };
 
-template <bool BF16>
+// An operand tile of 32 k whose rows of memory run along M or N: one copy of 32 k x 32 columns per group.
+__device__ __forceinline__ void load_groups_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row0, int k0, int groups) {
+#pragma unroll 1
+    for (int i = 0; i < groups; ++i) tma_load_2d_pair(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0);
+}
+
+template <bool BF16, bool MN>
 __global__ void __launch_bounds__(P_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                       const __grid_constant__ CUtensorMap map_c, const PairArgs args) {
@@ -150,8 +157,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
                 if (elected && ok && (ok = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag))) {
                     if (leader) mbar_arrive_expect_tx(smem_u32(&bar_full[stage]), (uint32_t)(2 * stage_bytes));
-                    tma_load_2d_pair(a_dst, &map_a, full, kb * BK, m0);
-                    tma_load_2d_pair(a_dst + A_STAGE_BYTES, &map_b, full, kb * BK, n0);
+                    if (MN && args.a_mn) load_groups_pair(a_dst, &map_a, full, m0, kb * BK, BLOCK_M / 32);
+                    else tma_load_2d_pair(a_dst, &map_a, full, kb * BK, m0);
+                    if (MN && args.b_mn) load_groups_pair(a_dst + A_STAGE_BYTES, &map_b, full, n0, kb * BK, half_n >> 5);
+                    else tma_load_2d_pair(a_dst + A_STAGE_BYTES, &map_b, full, kb * BK, n0);
                     ++issued;
                 }
                 if (++stage == stages) { stage = 0; phase ^= 1u; }
@@ -183,7 +192,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer (even CTA only)
         if (leader) {
-            const uint32_t idesc = BF16 ? make_idesc_bf16(P_TILE_M, block_n) : make_idesc_tf32(P_TILE_M, block_n);
+            const bool a_mn = MN && args.a_mn, b_mn = MN && args.b_mn;
+            const uint32_t idesc = (BF16 ? make_idesc_bf16(P_TILE_M, block_n) : make_idesc_tf32(P_TILE_M, block_n)) |
+                                   (a_mn ? IDESC_A_MN : 0u) | (b_mn ? IDESC_B_MN : 0u);
+            const uint64_t a_step = a_mn ? 64 : 2, b_step = b_mn ? 64 : 2;
             const uint16_t both = 3;
             int stage = 0;
             uint32_t phase = 0;
@@ -197,11 +209,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * block_n);
                 for (int kb = 0; kb < num_k_blocks; ++kb) {
                     const uint32_t a_addr = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
-                    const uint64_t a_desc = make_kmajor_sw128_desc(a_addr);
-                    const uint64_t b_desc = make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
+                    const uint64_t a_desc = a_mn ? make_mnmajor_desc(a_addr) : make_kmajor_sw128_desc(a_addr);
+                    const uint64_t b_desc = b_mn ? make_mnmajor_desc(a_addr + A_STAGE_BYTES) : make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
                     uint64_t ak[BK / MMA_K], bk[BK / MMA_K];  // 32 bytes along K per MMA: 2 descriptor units
 #pragma unroll
-                    for (int k = 0; k < BK / MMA_K; ++k) { ak[k] = a_desc + (uint64_t)(2 * k); bk[k] = b_desc + (uint64_t)(2 * k); }
+                    for (int k = 0; k < BK / MMA_K; ++k) { ak[k] = a_desc + a_step * (uint64_t)k; bk[k] = b_desc + b_step * (uint64_t)k; }
                     if (elected && ok && (ok = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag))) {
                         tc_fence_after();
 #pragma unroll
@@ -356,11 +368,14 @@ bool gemm_tf32_pair_preferred(int64_t M, int64_t N, int64_t K, int sm_count) {
 }
 
 tfjsb_status gemm_tf32_pair_plan(tfjsb_ctx* ctx, const float* a, const float* bt, float* c, int64_t M, int64_t N, int64_t K,
-                                 GemmTf32Plan* plan) {
+                                 GemmTf32Plan* plan, bool a_mn, bool b_mn) {
     if (!gemm_tf32_supported(M, N, K)) return fail(ctx, TFJSB_ERR_UNSUPPORTED, "shape not supported by the TF32 GEMM");
     if (!ctx->encode_tiled) return fail(ctx, TFJSB_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
     plan->M = M; plan->N = N; plan->K = K;
     plan->gather = false;
+    plan->im2col = false;
+    plan->a_mn = a_mn;
+    plan->b_mn = b_mn;
     plan->x = nullptr;
     plan->pair = true;
     plan->cluster_split = false;
@@ -383,18 +398,22 @@ tfjsb_status gemm_tf32_pair_plan(tfjsb_ctx* ctx, const float* a, const float* bt
     const int64_t pairs = ctx->sm_count / 2;
     plan->grid = 2 * (int)(tiles < pairs ? tiles : pairs);
     tfjsb_status st;
-    if ((st = encode_pair_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, BLOCK_M, "A")) != TFJSB_OK) return st;
-    if ((st = encode_pair_2d(ctx, &plan->map_b, bt, K, N, BLOCK_K, bn / 2, "B")) != TFJSB_OK) return st;
+    if (a_mn) st = encode_pair_2d(ctx, &plan->map_a, a, M, K, 32, BLOCK_K, "A", false, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B);
+    else st = encode_pair_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, BLOCK_M, "A");
+    if (st != TFJSB_OK) return st;
+    if (b_mn) st = encode_pair_2d(ctx, &plan->map_b, bt, N, K, 32, BLOCK_K, "B", false, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B);
+    else st = encode_pair_2d(ctx, &plan->map_b, bt, K, N, BLOCK_K, bn / 2, "B");
+    if (st != TFJSB_OK) return st;
     return encode_pair_2d(ctx, &plan->map_c, c, N, M, EPI_COLS, 32, "C");
 }
 
 namespace {
 
-template <bool BF16>
+template <bool BF16, bool MN>
 cudaError_t launch_pair(const CUtensorMap& map_a, const CUtensorMap& map_b, const CUtensorMap& map_c, int64_t M, int64_t N, int64_t K,
                         int block_n, int stages, int num_tiles, int grid, size_t smem_bytes, const float* bias, int act,
-                        unsigned int* dev_status, cudaStream_t s, int64_t* launches) {
-    cudaError_t ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_pair_kernel<BF16>), SMEM_LIMIT - 2048);
+                        unsigned int* dev_status, cudaStream_t s, int64_t* launches, bool a_mn = false, bool b_mn = false) {
+    cudaError_t ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_pair_kernel<BF16, MN>), SMEM_LIMIT - 2048);
     if (ae != cudaSuccess) return ae;
     PairArgs args;
     args.M = (int)M; args.N = (int)N; args.K = (int)K;
@@ -402,6 +421,8 @@ cudaError_t launch_pair(const CUtensorMap& map_a, const CUtensorMap& map_b, cons
     args.stages = stages;
     args.n_tiles = (int)((N + block_n - 1) / block_n);
     args.num_tiles = num_tiles;
+    args.a_mn = a_mn;
+    args.b_mn = b_mn;
     args.bias = bias;
     args.act = act;
     args.dev_status = dev_status;
@@ -419,7 +440,7 @@ cudaError_t launch_pair(const CUtensorMap& map_a, const CUtensorMap& map_b, cons
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = g_launch_pdl ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_pair_kernel<BF16>, map_a, map_b, map_c, args);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_pair_kernel<BF16, MN>, map_a, map_b, map_c, args);
     ++*launches;
     return e;
 }
@@ -428,8 +449,11 @@ cudaError_t launch_pair(const CUtensorMap& map_a, const CUtensorMap& map_b, cons
 
 cudaError_t launch_gemm_tf32_pair(const GemmTf32Plan& plan, const float* bias, int act, unsigned int* dev_status,
                                   cudaStream_t s, int64_t* launches) {
-    return launch_pair<false>(plan.map_a, plan.map_b, plan.map_c, plan.M, plan.N, plan.K, plan.block_n, plan.stages, plan.num_tiles,
-                              plan.grid, plan.smem_bytes, bias, act, dev_status, s, launches);
+    if (plan.a_mn || plan.b_mn)
+        return launch_pair<false, true>(plan.map_a, plan.map_b, plan.map_c, plan.M, plan.N, plan.K, plan.block_n, plan.stages, plan.num_tiles,
+                                        plan.grid, plan.smem_bytes, bias, act, dev_status, s, launches, plan.a_mn, plan.b_mn);
+    return launch_pair<false, false>(plan.map_a, plan.map_b, plan.map_c, plan.M, plan.N, plan.K, plan.block_n, plan.stages, plan.num_tiles,
+                                     plan.grid, plan.smem_bytes, bias, act, dev_status, s, launches);
 }
 
 // Where the pair pays: nowhere yet.  On the shape it was written for (25088 x 512 x 512, the 14 x 14
@@ -474,7 +498,7 @@ tfjsb_status gemm_bf16_pair_plan(tfjsb_ctx* ctx, const void* a, const void* bt, 
 
 cudaError_t launch_gemm_bf16_pair(const GemmBf16Plan& plan, const float* bias, int act, unsigned int* dev_status,
                                   cudaStream_t s, int64_t* launches) {
-    return launch_pair<true>(plan.map_a, plan.map_b, plan.map_c, plan.M, plan.N, plan.K, plan.block_n, plan.stages, plan.num_tiles,
+    return launch_pair<true, false>(plan.map_a, plan.map_b, plan.map_c, plan.M, plan.N, plan.K, plan.block_n, plan.stages, plan.num_tiles,
                              plan.grid, plan.smem_bytes, bias, act, dev_status, s, launches);
 }
 

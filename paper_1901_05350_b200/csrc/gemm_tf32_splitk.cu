@@ -51,6 +51,8 @@ struct SplitArgs {
     int splits;        // = cluster size
     int kb_per_split;
     int stage_tx;      // bytes that the copies of one stage deliver
+    int a_mn, b_mn;    // operands stored [K, M] / [K, N] (the instance with MN only)
+    int a_groups;      // copies of 32 k x 32 rows that make the A tile (a_mn)
     const float* bias;
     int act;
     float* c;
@@ -66,6 +68,13 @@ __device__ __forceinline__ float4 ld_shared_v4(uint32_t addr) {
     return v;
 }
 
+// An operand tile of 32 k whose rows of memory run along M or N: one copy of 32 k x 32 columns per group.
+__device__ __forceinline__ void load_groups(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row0, int k0, int groups) {
+#pragma unroll 1
+    for (int i = 0; i < groups; ++i) tma_load_2d(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0);
+}
+
+template <bool MN>
 __global__ void __launch_bounds__(S_THREADS, 1)
 gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                         const SplitArgs args) {
@@ -139,8 +148,10 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
             const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
             if (leader && ok && (ok = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag))) {
                 mbar_arrive_expect_tx(full, (uint32_t)args.stage_tx);
-                tma_load_2d(a_dst, &map_a, full, kb * BLOCK_K, m0);
-                tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BLOCK_K, n0);
+                if (MN && args.a_mn) load_groups(a_dst, &map_a, full, m0, kb * BLOCK_K, args.a_groups);
+                else tma_load_2d(a_dst, &map_a, full, kb * BLOCK_K, m0);
+                if (MN && args.b_mn) load_groups(a_dst + A_STAGE_BYTES, &map_b, full, n0, kb * BLOCK_K, block_n >> 5);
+                else tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BLOCK_K, n0);
                 ++issued;
             }
             if (++stage == stages) { stage = 0; phase ^= 1u; }
@@ -165,7 +176,9 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
         cluster_wait();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        const uint32_t idesc = make_idesc_tf32(BLOCK_M, block_n);
+        const bool a_mn = MN && args.a_mn, b_mn = MN && args.b_mn;
+        const uint32_t idesc = make_idesc_tf32(BLOCK_M, block_n) | (a_mn ? IDESC_A_MN : 0u) | (b_mn ? IDESC_B_MN : 0u);
+        const uint64_t a_step = a_mn ? 64 : 2, b_step = b_mn ? 64 : 2;
         int stage = 0;
         uint32_t phase = 0;
         const bool leader = elect_one();
@@ -173,11 +186,11 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
         bool issued_any = false;
         for (int kb = kb_begin; kb < kb_end; ++kb) {
             const uint32_t a_addr = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
-            const uint64_t a_desc = make_kmajor_sw128_desc(a_addr);
-            const uint64_t b_desc = make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
+            const uint64_t a_desc = a_mn ? make_mnmajor_desc(a_addr) : make_kmajor_sw128_desc(a_addr);
+            const uint64_t b_desc = b_mn ? make_mnmajor_desc(a_addr + A_STAGE_BYTES) : make_kmajor_sw128_desc(a_addr + A_STAGE_BYTES);
             uint64_t ak[BLOCK_K / UMMA_K], bk[BLOCK_K / UMMA_K];
 #pragma unroll
-            for (int k = 0; k < BLOCK_K / UMMA_K; ++k) { ak[k] = a_desc + (uint64_t)(2 * k); bk[k] = b_desc + (uint64_t)(2 * k); }
+            for (int k = 0; k < BLOCK_K / UMMA_K; ++k) { ak[k] = a_desc + a_step * (uint64_t)k; bk[k] = b_desc + b_step * (uint64_t)k; }
             if (leader && ok && (ok = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag))) {
                 tc_fence_after();
 #pragma unroll
@@ -272,13 +285,13 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
 }
 
 tfjsb_status encode_split_2d(tfjsb_ctx* ctx, CUtensorMap* map, const void* base, int64_t inner, int64_t outer, int box_inner,
-                             int box_outer, const char* what) {
+                             int box_outer, const char* what, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
     cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
     cuuint64_t strides[1] = {(cuuint64_t)inner * 4u};
     cuuint32_t box[2] = {(cuuint32_t)box_inner, (cuuint32_t)box_outer};
     cuuint32_t elem[2] = {1u, 1u};
     CUresult r = ctx->encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, elem,
-                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
         return fail(ctx, TFJSB_ERR_CUDA,
@@ -330,11 +343,14 @@ bool gemm_tf32_splitk_choice(int64_t M, int64_t N, int64_t K, int sm_count, int6
 }
 
 tfjsb_status gemm_tf32_splitk_plan(tfjsb_ctx* ctx, const float* a, const float* bt, float* c, int64_t M, int64_t N, int64_t K,
-                                   int block_n, int splits, GemmTf32Plan* plan) {
+                                   int block_n, int splits, GemmTf32Plan* plan, bool a_mn, bool b_mn) {
     if (!ctx->encode_tiled) return fail(ctx, TFJSB_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
     plan->M = M; plan->N = N; plan->K = K;
     plan->gather = false;
+    plan->im2col = false;
     plan->pair = false;
+    plan->a_mn = a_mn;
+    plan->b_mn = b_mn;
     plan->x = nullptr;
     plan->c = c;
     plan->batches = 1;
@@ -353,19 +369,21 @@ tfjsb_status gemm_tf32_splitk_plan(tfjsb_ctx* ctx, const float* a, const float* 
     plan->num_tiles = (int)tiles;
     plan->grid = (int)(tiles * splits);
     tfjsb_status st;
-    if ((st = encode_split_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, a_box_rows(M), "A")) != TFJSB_OK) return st;
-    if ((st = encode_split_2d(ctx, &plan->map_b, bt, K, N, BLOCK_K, block_n, "B")) != TFJSB_OK) return st;
+    if (a_mn) st = encode_split_2d(ctx, &plan->map_a, a, M, K, 32, BLOCK_K, "A", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B);
+    else st = encode_split_2d(ctx, &plan->map_a, a, K, M, BLOCK_K, a_box_rows(M), "A");
+    if (st != TFJSB_OK) return st;
+    if (b_mn) st = encode_split_2d(ctx, &plan->map_b, bt, N, K, 32, BLOCK_K, "B", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B);
+    else st = encode_split_2d(ctx, &plan->map_b, bt, K, N, BLOCK_K, block_n, "B");
+    if (st != TFJSB_OK) return st;
     plan->map_c = plan->map_b;  // unused: C is stored directly
     return TFJSB_OK;
 }
 
 cudaError_t launch_gemm_tf32_splitk(const GemmTf32Plan& plan, const float* bias, int act, unsigned int* dev_status,
                                     cudaStream_t s, int64_t* launches) {
-    {
-        cudaError_t ae = cudaSuccess;
-        if (ae == cudaSuccess) ae = smem_attr_once(reinterpret_cast<const void*>(&gemm_tf32_splitk_kernel), SMEM_LIMIT - 2048);
-        if (ae != cudaSuccess) return ae;
-    }
+    auto kernel = plan.a_mn || plan.b_mn ? gemm_tf32_splitk_kernel<true> : gemm_tf32_splitk_kernel<false>;
+    cudaError_t ae = smem_attr_once(reinterpret_cast<const void*>(kernel), SMEM_LIMIT - 2048);
+    if (ae != cudaSuccess) return ae;
     SplitArgs args;
     args.M = (int)plan.M; args.N = (int)plan.N; args.K = (int)plan.K;
     args.block_n = plan.block_n;
@@ -373,7 +391,10 @@ cudaError_t launch_gemm_tf32_splitk(const GemmTf32Plan& plan, const float* bias,
     args.n_tiles = (int)((plan.N + plan.block_n - 1) / plan.block_n);
     args.splits = plan.splits;
     args.kb_per_split = plan.kb_per_split;
-    args.stage_tx = a_box_rows(plan.M) * 128 + plan.block_n * 128;
+    args.a_mn = plan.a_mn;
+    args.b_mn = plan.b_mn;
+    args.a_groups = plan.M >= BLOCK_M ? BLOCK_M / 32 : (int)((plan.M + 31) / 32);
+    args.stage_tx = (plan.a_mn ? args.a_groups * 32 : a_box_rows(plan.M)) * 128 + plan.block_n * 128;
     args.bias = bias;
     args.act = act;
     args.c = plan.c;
@@ -392,7 +413,7 @@ cudaError_t launch_gemm_tf32_splitk(const GemmTf32Plan& plan, const float* bias,
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = g_launch_pdl ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_tf32_splitk_kernel, plan.map_a, plan.map_b, args);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, plan.map_a, plan.map_b, args);
     ++*launches;
     return e;
 }

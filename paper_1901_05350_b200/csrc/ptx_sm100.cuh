@@ -173,6 +173,21 @@ __device__ __forceinline__ uint64_t make_kmajor_sw128_desc(uint32_t smem_addr) {
     return d;
 }
 
+// The same for an operand stored the other way round (rows of memory run along M or N, "MN-major"), as TMA writes boxes of
+// 32 k x 32 columns with the 128-byte swizzle of 32-byte pieces: atoms of 4 k (512 bytes, the stride byte offset), groups of
+// 32 columns 4096 bytes apart (the leading byte offset), layout type 1.  Eight k, one MMA, are 1024 bytes: 64 descriptor
+// units where a K-major tile steps by 2.
+__device__ __forceinline__ uint64_t make_mnmajor_desc(uint32_t smem_addr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(4096u >> 4) << 16;
+    d |= (uint64_t)(512u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)1 << 61;
+    return d;
+}
+constexpr uint32_t IDESC_A_MN = 1u << 15, IDESC_B_MN = 1u << 16;  // instruction descriptor bits: operand is MN-major
+
 // Instruction descriptor: fp32 accumulator, TF32 A and B, both K-major, N and M encoded as N/8, M/16.
 __device__ __forceinline__ uint32_t make_idesc_tf32(int m, int n) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);

@@ -124,6 +124,27 @@ def test_matmul_tf32_transposes(ctx, oracle, ta, tb):
     assert same_bits(host(ctx.matmul(dev(ai), dev(bi), ta, tb)), oracle.matmul(ai, bi, ta, tb))
 
 
+@pytest.mark.parametrize("pair", ["0", "1"])
+@pytest.mark.parametrize("ta,tb", [(False, False), (True, False), (True, True)])
+@pytest.mark.parametrize("bmkn", [(1, 4, 4, 4), (1, 36, 28, 68), (1, 132, 36, 260), (1, 260, 96, 132), (1, 300, 1000, 128), (1, 34, 520, 72),
+                                  (5, 100, 36, 72), (3, 33, 64, 40)])
+def test_operands_as_stored_give_the_bits_of_k_contiguous_ones(ctx, monkeypatch, bmkn, ta, tb, pair):
+    """Operands stored [K, N] and [K, M] are read as they are (or transposed first, where M is no multiple of 4): the tiles'
+    groups of 32 rows and atoms of 4 k end inside the matrices, the K loop is whole, in slices, or on CTA pairs.  The plan
+    does not depend on the storage, so neither does any bit."""
+    monkeypatch.setenv("TFJSB_GEMM_PAIR", pair)
+    b, m, k, n = bmkn
+    x, y = si.uniform(77, 0, (b, m, k), -1, 1), si.uniform(77, 1, (b, n, k), -1, 1)
+    if b == 1:
+        x, y = x[0], y[0]
+    call = ctx.matmul if b == 1 else ctx.batch_matmul
+    want = host(call(dev(x), dev(y), transpose_b=True))
+    got = host(call(dev(np.ascontiguousarray(np.swapaxes(x, -1, -2))) if ta else dev(x), dev(y) if tb else dev(np.ascontiguousarray(np.swapaxes(y, -1, -2))),
+                    transpose_a=ta, transpose_b=tb))
+    ctx.check_device_status()
+    assert same_bits(got, want)
+
+
 def test_matmul_unaligned_shapes_take_the_cuda_core_path(ctx, oracle):
     a = si.uniform(305, 0, (70, 27), -1, 1)   # K % 4 != 0
     b = si.uniform(305, 1, (27, 33), -1, 1)   # N % 4 != 0
