@@ -13,7 +13,7 @@ using namespace tfjsb;
 
 namespace tfjsb {
 
-thread_local bool g_launch_pdl = false;
+thread_local bool g_launch_pdl = getenv("TFJSB_NO_PDL") == nullptr;
 
 tfjsb_status fail(tfjsb_ctx* ctx, tfjsb_status st, const std::string& msg) {
     if (ctx) ctx->last_error = msg;

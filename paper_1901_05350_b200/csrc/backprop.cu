@@ -10,6 +10,7 @@
 // in two steps, partial sums per slice of the pixels into scratch and then a sum over the slices in slice
 // order, so that the result does not depend on scheduling.
 #include "common.cuh"
+#include "ptx_sm100.cuh"
 
 namespace tfjsb {
 
@@ -30,8 +31,10 @@ __device__ __forceinline__ int source_of(int i, int p, int k, int d, int s, int 
 // thread = one input sample (n, iy, ix, ci), ci fastest; the dy row of a source pixel is the same address
 // for the threads of a pixel (a broadcast), the filter row f[tap, ci, :] is contiguous per thread.
 __global__ void __launch_bounds__(BP_THREADS)
-conv2d_backprop_input_kernel(const float* __restrict__ dy, const float* __restrict__ f, float* __restrict__ dx, ConvGeom g,
+conv2d_backprop_input_kernel(const float* dy, const float* f, float* __restrict__ dx, ConvGeom g,
                              int64_t total) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += stride) {
         const int ci = (int)(e % g.C);
@@ -49,7 +52,7 @@ conv2d_backprop_input_kernel(const float* __restrict__ dy, const float* __restri
                 if (ox < 0) continue;
                 const float* gp = dy + ((n * g.Ho + oy) * (int64_t)g.Wo + ox) * g.Co;
                 const float* fp = f + ((int64_t)(ky * g.fw + kx) * g.C + ci) * g.Co;
-                for (int co = 0; co < g.Co; ++co) acc = fmaf(__ldg(gp + co), __ldg(fp + co), acc);
+                for (int co = 0; co < g.Co; ++co) acc = fmaf(load_global(gp + co), load_global(fp + co), acc);
             }
         }
         dx[e] = acc;
@@ -60,8 +63,10 @@ conv2d_backprop_input_kernel(const float* __restrict__ dy, const float* __restri
 // Block = a 32 x 32 tile of (ci, co) for one tap and one slice of the output pixels; 32 pixels at a time go
 // through shared memory (x samples [32 pixels][32 ci], dy [32 pixels][32 co]); thread (tx = co, ty = ci).
 __global__ void __launch_bounds__(1024)
-conv2d_backprop_filter_partial_kernel(const float* __restrict__ x, const float* __restrict__ dy, float* __restrict__ partial,
+conv2d_backprop_filter_partial_kernel(const float* x, const float* dy, float* __restrict__ partial,
                                       ConvGeom g, int64_t pixels, int64_t pixels_per_slice, int ci_tiles, int co_tiles) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     __shared__ float xs[32][33];
     __shared__ float gs[32][33];
     int b = blockIdx.x;
@@ -86,8 +91,8 @@ conv2d_backprop_filter_partial_kernel(const float* __restrict__ x, const float* 
             const int64_t n = r / g.Ho;
             const int iy = oy * g.sh - g.pt + ky * g.dh, ix = ox * g.sw - g.pl + kx * g.dw;
             if (iy >= 0 && iy < g.H && ix >= 0 && ix < g.W && ci0 + tx < g.C)
-                xv = __ldg(x + ((n * g.H + iy) * (int64_t)g.W + ix) * g.C + ci0 + tx);
-            if (co0 + tx < g.Co) gv = __ldg(dy + p * g.Co + co0 + tx);
+                xv = load_global(x + ((n * g.H + iy) * (int64_t)g.W + ix) * g.C + ci0 + tx);
+            if (co0 + tx < g.Co) gv = load_global(dy + p * g.Co + co0 + tx);
         }
         xs[ty][tx] = xv;
         gs[ty][tx] = gv;
@@ -110,8 +115,10 @@ conv2d_backprop_filter_partial_kernel(const float* __restrict__ x, const float* 
 // 69 + 9 us (101 MB of dy; 22 us of multiply-adds); the 32 x 32 tiles per tap, 3 of 32 rows of each in use, took 3.3 ms.
 template <int CG>
 __global__ void __launch_bounds__(BP_THREADS)
-conv2d_backprop_small_filter_kernel(const float* __restrict__ x, const float* __restrict__ dy, float* __restrict__ partial, ConvGeom g,
+conv2d_backprop_small_filter_kernel(const float* x, const float* dy, float* __restrict__ partial, ConvGeom g,
                                     int64_t pixels, int64_t pixels_per_slice, int window) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     constexpr int PIX = 32, LANES = BP_THREADS / (8 * CG), CO = 4 * CG;
     constexpr int DY4 = PIX * CG / BP_THREADS;  // 16-byte pieces of dy per thread and step
     __shared__ __align__(16) float xs[2][PIX][32];
@@ -135,7 +142,7 @@ conv2d_backprop_small_filter_kernel(const float* __restrict__ x, const float* __
         for (int i = 0; i < PIX / 8; ++i) {
             const int iy = oy * g.sh - g.pt + off_y, ix = ox * g.sw - g.pl + off_x;
             xv[i] = p < p_end && e < window && iy >= 0 && iy < g.H && ix >= 0 && ix < g.W
-                        ? __ldg(x + ((n * g.H + iy) * (int64_t)g.W + ix) * g.C + ci) : 0.f;
+                        ? load_global(x + ((n * g.H + iy) * (int64_t)g.W + ix) * g.C + ci) : 0.f;
             p += 8;
             for (ox += 8; ox >= g.Wo; ox -= g.Wo)
                 if (++oy == g.Ho) { oy = 0; ++n; }
@@ -143,7 +150,7 @@ conv2d_backprop_small_filter_kernel(const float* __restrict__ x, const float* __
 #pragma unroll
         for (int i = 0; i < DY4; ++i) {
             const int j = tid + i * BP_THREADS, px = j / CG, c = co0 + 4 * (j % CG);
-            gv[i] = p0 + px < p_end && c < g.Co ? __ldg(reinterpret_cast<const float4*>(dy + (p0 + px) * g.Co + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            gv[i] = p0 + px < p_end && c < g.Co ? load_global(reinterpret_cast<const float4*>(dy + (p0 + px) * g.Co + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
     const int eg = (tid / CG) & 7, cg = tid % CG, lane = tid / (8 * CG);
@@ -210,7 +217,9 @@ conv2d_backprop_small_filter_kernel(const float* __restrict__ x, const float* __
 // flight per thread before that, took 24 + 26 us for [100352, 128] (51 MB); now 16 + 5 us with a cold cache.
 template <int V>
 __global__ void __launch_bounds__(1024)
-column_sums_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t rows, int64_t C, int64_t rows_per_slice) {
+column_sums_kernel(const float* in, float* __restrict__ out, int64_t rows, int64_t C, int64_t rows_per_slice) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     constexpr int UNROLL = 8;
     __shared__ float red[1024 * V];
     const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
@@ -231,8 +240,8 @@ column_sums_kernel(const float* __restrict__ in, float* __restrict__ out, int64_
 #pragma unroll
                 for (int v = 0; v < V; ++v) t[u][v] = 0.f;
                 if (row < r_end) {
-                    if (V == 4) *reinterpret_cast<float4*>(t[u]) = __ldg(reinterpret_cast<const float4*>(p + row * C));
-                    else t[u][0] = __ldg(p + row * C);
+                    if (V == 4) *reinterpret_cast<float4*>(t[u]) = load_global(reinterpret_cast<const float4*>(p + row * C));
+                    else t[u][0] = load_global(p + row * C);
                 }
             }
 #pragma unroll
@@ -260,8 +269,10 @@ column_sums_kernel(const float* __restrict__ in, float* __restrict__ out, int64_
 
 // ---- depthwise, gradient with respect to the input ---------------------------------------------------
 __global__ void __launch_bounds__(BP_THREADS)
-depthwise_backprop_input_kernel(const float* __restrict__ dy, const float* __restrict__ f, float* __restrict__ dx, ConvGeom g,
+depthwise_backprop_input_kernel(const float* dy, const float* f, float* __restrict__ dx, ConvGeom g,
                                 int64_t total) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += stride) {
         const int c = (int)(e % g.C);
@@ -279,7 +290,7 @@ depthwise_backprop_input_kernel(const float* __restrict__ dy, const float* __res
                 if (ox < 0) continue;
                 const float* gp = dy + ((n * g.Ho + oy) * (int64_t)g.Wo + ox) * g.Co + (int64_t)c * g.mult;
                 const float* fp = f + ((int64_t)(ky * g.fw + kx) * g.C + c) * g.mult;
-                for (int q = 0; q < g.mult; ++q) acc = fmaf(__ldg(gp + q), __ldg(fp + q), acc);
+                for (int q = 0; q < g.mult; ++q) acc = fmaf(load_global(gp + q), load_global(fp + q), acc);
             }
         }
         dx[e] = acc;
@@ -293,8 +304,10 @@ depthwise_backprop_input_kernel(const float* __restrict__ dy, const float* __res
 // the first use, feed 4 ROWS 16-byte stores.  Bound by memory (dx is four times dy).
 template <int ROWS>
 __global__ void __launch_bounds__(BP_THREADS)
-depthwise3x3_s2_backprop_input_kernel(const float* __restrict__ dy, const float* __restrict__ f, float* __restrict__ dx, ConvGeom g,
+depthwise3x3_s2_backprop_input_kernel(const float* dy, const float* f, float* __restrict__ dx, ConvGeom g,
                                       int tc, int c4_tiles) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int C4 = g.C >> 2;
     const int c4 = (blockIdx.x % c4_tiles) * tc + (threadIdx.x % tc);
     const int r = (blockIdx.x / c4_tiles) * (BP_THREADS / tc) + threadIdx.x / tc;
@@ -305,7 +318,7 @@ depthwise3x3_s2_backprop_input_kernel(const float* __restrict__ dy, const float*
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 w[9];
 #pragma unroll
-    for (int t = 0; t < 9; ++t) w[t] = __ldg(reinterpret_cast<const float4*>(f + (int64_t)t * g.C + c));
+    for (int t = 0; t < 9; ++t) w[t] = load_global(reinterpret_cast<const float4*>(f + (int64_t)t * g.C + c));
     const int64_t n = blockIdx.z;
     const float* gy = dy + n * (int64_t)g.Ho * g.Wo * g.C + c;
     float4 a[ROWS + 1], b[ROWS + 1];  // columns r - 1 and r of rows q0 - 1 .. q0 + ROWS - 1
@@ -314,8 +327,8 @@ depthwise3x3_s2_backprop_input_kernel(const float* __restrict__ dy, const float*
         const int oy = q0 - 1 + j;
         const bool row = oy >= 0 && oy < g.Ho;
         const float* p = gy + ((int64_t)oy * g.Wo + r) * g.C;
-        a[j] = row && r >= 1 && r - 1 < g.Wo ? __ldg(reinterpret_cast<const float4*>(p - g.C)) : zero;
-        b[j] = row && r < g.Wo ? __ldg(reinterpret_cast<const float4*>(p)) : zero;
+        a[j] = row && r >= 1 && r - 1 < g.Wo ? load_global(reinterpret_cast<const float4*>(p - g.C)) : zero;
+        b[j] = row && r < g.Wo ? load_global(reinterpret_cast<const float4*>(p)) : zero;
     }
     float* out = dx + n * (int64_t)g.H * g.W * g.C + c;
     // a filter that is not finite: only taps that meet an output pixel take part, where the zeros make NaNs of the others
@@ -330,8 +343,8 @@ depthwise3x3_s2_backprop_input_kernel(const float* __restrict__ dy, const float*
         for (int t = 0; t < 9; ++t) {
             const int oy = source_of(iy, g.pt, t / 3, 1, 2, g.Ho), ox = source_of(jx, g.pl, t % 3, 1, 2, g.Wo);
             if (oy < 0 || ox < 0) continue;
-            fma4_packed(v, __ldg(reinterpret_cast<const float4*>(gy + ((int64_t)oy * g.Wo + ox) * g.C)),
-                        __ldg(reinterpret_cast<const float4*>(f + (int64_t)t * g.C + c)));
+            fma4_packed(v, load_global(reinterpret_cast<const float4*>(gy + ((int64_t)oy * g.Wo + ox) * g.C)),
+                        load_global(reinterpret_cast<const float4*>(f + (int64_t)t * g.C + c)));
         }
         *reinterpret_cast<float4*>(out + ((int64_t)iy * g.W + jx) * g.C) = v;
     }
@@ -361,8 +374,10 @@ depthwise3x3_s2_backprop_input_kernel(const float* __restrict__ dy, const float*
 // Block = 32 output channels (tx) x 8 pixel lanes (ty) for one tap (blockIdx.z) and one slice of the
 // output pixels (blockIdx.y).
 __global__ void __launch_bounds__(BP_THREADS)
-depthwise_backprop_filter_partial_kernel(const float* __restrict__ x, const float* __restrict__ dy, float* __restrict__ partial,
+depthwise_backprop_filter_partial_kernel(const float* x, const float* dy, float* __restrict__ partial,
                                          ConvGeom g, int64_t pixels, int64_t pixels_per_slice) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     __shared__ float red[8][32];
     const int oc = blockIdx.x * 32 + threadIdx.x;
     const int tap = blockIdx.z;
@@ -379,7 +394,7 @@ depthwise_backprop_filter_partial_kernel(const float* __restrict__ x, const floa
             const int64_t n = r / g.Ho;
             const int iy = oy * g.sh - g.pt + ky * g.dh, ix = ox * g.sw - g.pl + kx * g.dw;
             if (iy >= 0 && iy < g.H && ix >= 0 && ix < g.W)
-                acc = fmaf(__ldg(x + ((n * g.H + iy) * (int64_t)g.W + ix) * g.C + c), __ldg(dy + p * g.Co + oc), acc);
+                acc = fmaf(load_global(x + ((n * g.H + iy) * (int64_t)g.W + ix) * g.C + c), load_global(dy + p * g.Co + oc), acc);
         }
     }
     red[threadIdx.y][threadIdx.x] = acc;
@@ -400,18 +415,30 @@ __device__ __forceinline__ float act_grad(float y, float dy, int act) {
     return pass ? dy : 0.f;
 }
 __global__ void __launch_bounds__(BP_THREADS)
-act_backprop_kernel(const float* __restrict__ y, const float* __restrict__ dy, float* __restrict__ dz, int64_t n, int act) {
+act_backprop_kernel(const float* y, const float* dy, float* __restrict__ dz, int64_t n, int act) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t n4 = n >> 2;
-    for (int64_t i = first; i < (n + 3) >> 2; i += stride) {
-        if (i == n4) {  // the last three values at most, by a thread of their own where there are enough
-            for (int64_t e = 4 * n4; e < n; ++e) dz[e] = act_grad(y[e], dy[e], act);
-            break;
+    const int64_t n4 = n >> 2, groups = (n + 3) >> 2;
+    constexpr int U = 2;  // groups per thread and pass, loaded before the first is stored
+    for (int64_t i = first; i < groups; i += U * stride) {
+        float4 v[U], g[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u * stride < n4) {
+                v[u] = reinterpret_cast<const float4*>(y)[i + u * stride];
+                g[u] = reinterpret_cast<const float4*>(dy)[i + u * stride];
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t at = i + u * stride;
+            if (at < n4)
+                reinterpret_cast<float4*>(dz)[at] = make_float4(act_grad(v[u].x, g[u].x, act), act_grad(v[u].y, g[u].y, act),
+                                                                act_grad(v[u].z, g[u].z, act), act_grad(v[u].w, g[u].w, act));
+            else if (at == n4)  // the last three values at most, by a thread of their own where there are enough
+                for (int64_t e = 4 * n4; e < n; ++e) dz[e] = act_grad(y[e], dy[e], act);
         }
-        const float4 v = reinterpret_cast<const float4*>(y)[i], g = reinterpret_cast<const float4*>(dy)[i];
-        reinterpret_cast<float4*>(dz)[i] =
-            make_float4(act_grad(v.x, g.x, act), act_grad(v.y, g.y, act), act_grad(v.z, g.z, act), act_grad(v.w, g.w, act));
     }
 }
 
@@ -433,9 +460,8 @@ int backprop_slices(int64_t rows, int sm_count) {
 cudaError_t launch_conv2d_backprop_input(const float* dy, const float* f, float* dx, const ConvGeom& g, int sm_count,
                                          cudaStream_t s, int64_t* launches) {
     const int64_t total = g.N * g.H * g.W * g.C;
-    conv2d_backprop_input_kernel<<<blocks_for(total, sm_count), BP_THREADS, 0, s>>>(dy, f, dx, g, total);
     ++*launches;
-    return cudaGetLastError();
+    return launch_k(conv2d_backprop_input_kernel, dim3(blocks_for(total, sm_count)), dim3(BP_THREADS), 0, s, dy, f, dx, g, total);
 }
 
 namespace {
@@ -457,10 +483,8 @@ cudaError_t launch_column_sums(const float* in, float* out, int64_t rows, int64_
     int ty = pow2_at_least((per + 7) / 8, 1024 / tx);
     if (ty * tx < 32) ty = 32 / tx;
     const dim3 grid((unsigned)((cols + tx - 1) / tx), (unsigned)slices), block(tx, ty);
-    if (vec) column_sums_kernel<4><<<grid, block, 0, s>>>(in, out, rows, C, per);
-    else column_sums_kernel<1><<<grid, block, 0, s>>>(in, out, rows, C, per);
     ++*launches;
-    return cudaGetLastError();
+    return launch_k(vec ? column_sums_kernel<4> : column_sums_kernel<1>, grid, block, 0, s, in, out, rows, C, per);
 }
 
 }  // namespace
@@ -500,14 +524,10 @@ cudaError_t launch_conv2d_small_filter(const float* x, const float* dy, float* d
     const int64_t pixels = g.N * g.Ho * g.Wo, per = ((pixels + slices - 1) / slices + 31) / 32 * 32;
     const int window = g.fh * g.fw * g.C;
     float* out = slices > 1 ? partial : df;
-    if (g.Co > 64)
-        conv2d_backprop_small_filter_kernel<32><<<dim3((unsigned)((g.Co + 127) / 128), (unsigned)slices), BP_THREADS, 0, s>>>(x, dy, out, g, pixels, per, window);
-    else if (g.Co > 32)
-        conv2d_backprop_small_filter_kernel<16><<<dim3(1, (unsigned)slices), BP_THREADS, 0, s>>>(x, dy, out, g, pixels, per, window);
-    else
-        conv2d_backprop_small_filter_kernel<8><<<dim3(1, (unsigned)slices), BP_THREADS, 0, s>>>(x, dy, out, g, pixels, per, window);
+    auto kernel = g.Co > 64 ? conv2d_backprop_small_filter_kernel<32> : g.Co > 32 ? conv2d_backprop_small_filter_kernel<16> : conv2d_backprop_small_filter_kernel<8>;
+    const unsigned tiles = g.Co > 64 ? (unsigned)((g.Co + 127) / 128) : 1u;
+    cudaError_t e = launch_k(kernel, dim3(tiles, (unsigned)slices), dim3(BP_THREADS), 0, s, x, dy, out, g, pixels, per, window);
     ++*launches;
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || slices <= 1) return e;
     return launch_sum_rows(partial, df, nullptr, slices, (int64_t)window * g.Co, 1, s, launches);
 }
@@ -520,10 +540,8 @@ cudaError_t launch_conv2d_backprop_filter(const float* x, const float* dy, float
     const int64_t blocks = (int64_t)g.fh * g.fw * ci_tiles * co_tiles;
     if (blocks >= (1LL << 31)) return cudaErrorInvalidConfiguration;
     const int64_t elems = (int64_t)g.fh * g.fw * g.C * g.Co;
-    conv2d_backprop_filter_partial_kernel<<<dim3((unsigned)blocks, (unsigned)slices), dim3(32, 32), 0, s>>>(
-        x, dy, slices > 1 ? partial : df, g, pixels, per, ci_tiles, co_tiles);
+    cudaError_t e = launch_k(conv2d_backprop_filter_partial_kernel, dim3((unsigned)blocks, (unsigned)slices), dim3(32, 32), 0, s, x, dy, slices > 1 ? partial : df, g, pixels, per, ci_tiles, co_tiles);
     ++*launches;
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || slices <= 1) return e;
     return launch_sum_rows(partial, df, nullptr, slices, elems, 1, s, launches);
 }
@@ -552,16 +570,13 @@ cudaError_t launch_depthwise_backprop_input(const float* dy, const float* f, flo
         const int64_t gx = (int64_t)c4_tiles * (((g.W + g.pl + 1) / 2 + cols - 1) / cols);
         const int gy = ((g.H + g.pt + 1) / 2 + ROWS - 1) / ROWS;
         if (gx <= 2147483647LL && gy <= 65535) {
-            depthwise3x3_s2_backprop_input_kernel<ROWS>
-                <<<dim3((unsigned)gx, (unsigned)gy, (unsigned)g.N), BP_THREADS, 0, s>>>(dy, f, dx, g, tc, c4_tiles);
             ++*launches;
-            return cudaGetLastError();
+            return launch_k(depthwise3x3_s2_backprop_input_kernel<ROWS>, dim3((unsigned)gx, (unsigned)gy, (unsigned)g.N), dim3(BP_THREADS), 0, s, dy, f, dx, g, tc, c4_tiles);
         }
     }
     const int64_t total = g.N * g.H * g.W * g.C;
-    depthwise_backprop_input_kernel<<<blocks_for(total, sm_count), BP_THREADS, 0, s>>>(dy, f, dx, g, total);
     ++*launches;
-    return cudaGetLastError();
+    return launch_k(depthwise_backprop_input_kernel, dim3(blocks_for(total, sm_count)), dim3(BP_THREADS), 0, s, dy, f, dx, g, total);
 }
 
 cudaError_t launch_depthwise_backprop_filter(const float* x, const float* dy, float* df, float* partial, int slices,
@@ -570,19 +585,16 @@ cudaError_t launch_depthwise_backprop_filter(const float* x, const float* dy, fl
     const int64_t per = (pixels + slices - 1) / slices;
     const int taps = g.fh * g.fw;
     if (taps > 65535 || slices > 65535) return cudaErrorInvalidConfiguration;
-    depthwise_backprop_filter_partial_kernel<<<dim3((unsigned)((g.Co + 31) / 32), (unsigned)slices, (unsigned)taps), dim3(32, 8), 0,
-                                               s>>>(x, dy, slices > 1 ? partial : df, g, pixels, per);
+    cudaError_t e = launch_k(depthwise_backprop_filter_partial_kernel, dim3((unsigned)((g.Co + 31) / 32), (unsigned)slices, (unsigned)taps), dim3(32, 8), 0, s, x, dy, slices > 1 ? partial : df, g, pixels, per);
     ++*launches;
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || slices <= 1) return e;
     return launch_sum_rows(partial, df, nullptr, slices, (int64_t)taps * g.Co, 1, s, launches);
 }
 
 cudaError_t launch_act_backprop(const float* y, const float* dy, float* dz, int64_t n, int act, int sm_count, cudaStream_t s,
                                 int64_t* launches) {
-    act_backprop_kernel<<<blocks_for((n + 3) / 4, sm_count), BP_THREADS, 0, s>>>(y, dy, dz, n, act);
     ++*launches;
-    return cudaGetLastError();
+    return launch_k(act_backprop_kernel, dim3(blocks_for((n + 3) / 4, sm_count)), dim3(BP_THREADS), 0, s, y, dy, dz, n, act);
 }
 
 }  // namespace tfjsb

@@ -151,7 +151,7 @@ __device__ __noinline__ float grad_input_in_fp32(const GradInputArgs& g, const G
         if (oy < 0 || oy >= g.Ho || ox < 0 || ox >= g.Wo) continue;
         const float* dy = g.dy + ((n * g.Ho + oy) * (long long)g.Wo + ox) * g.Cout;
         const float* f = g.f + ((long long)((r.a + jy * g.sh) * g.fw + r.b + jx * g.sw) * g.Cin + ci) * g.Cout;
-        for (int co = co0; co < min(co0 + BLOCK_K, g.Cout); ++co) acc = fmaf(__ldg(dy + co), __ldg(f + co), acc);
+        for (int co = co0; co < min(co0 + BLOCK_K, g.Cout); ++co) acc = fmaf(load_global(dy + co), load_global(f + co), acc);
         if (acc != acc) break;
     }
     return acc;
@@ -193,6 +193,8 @@ conv2d_grad_input_kernel(const __grid_constant__ CUtensorMap map_dy, const __gri
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    pdl_launch_dependents();
+    pdl_wait();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -412,7 +414,7 @@ __device__ __noinline__ float grad_filter_in_fp32(const GradFilterArgs& g, long 
         const long long row = p / g.Wo, n = row / g.Ho;
         const int iy = (int)(row - n * g.Ho) * g.sh + off_h, ix = (int)(p - row * g.Wo) * g.sw + off_w;
         const bool inside = iy >= 0 && iy < g.H && ix >= 0 && ix < g.W;
-        acc = fmaf(inside ? __ldg(g.x + ((n * g.H + iy) * (long long)g.W + ix) * g.Cin + ci) : 0.f, __ldg(g.dy + p * g.Cout + co), acc);
+        acc = fmaf(inside ? load_global(g.x + ((n * g.H + iy) * (long long)g.W + ix) * g.Cin + ci) : 0.f, load_global(g.dy + p * g.Cout + co), acc);
     }
     return acc;
 }
@@ -467,6 +469,8 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    pdl_launch_dependents();
+    pdl_wait();
 
     if (warp == 0) {
         if (lane == 0) {

@@ -61,7 +61,7 @@ __device__ __noinline__ float4 gradient_of_existing(const float* x, const float*
 
 template <int S, int ROWS, int D = 1, bool GRADIENT = false>
 __global__ void __launch_bounds__(DW_THREADS)
-depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ f, const float* __restrict__ bias,
+depthwise3x3_kernel(const float* x, const float* f, const float* bias,
                     int act, float* __restrict__ y, const __grid_constant__ ConvGeom g, int tc, int c4_tiles) {
     // block = tx_count output columns x tc channel quads
     const int C4 = g.C >> 2;
@@ -135,8 +135,8 @@ depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ f, co
         *reinterpret_cast<float4*>(y + ((n * g.Ho + oy) * (int64_t)g.Wo + ox) * g.Co + c) = gradient_of_existing(x, f, f_step, g, n, oy, ox, c);
 }
 
-__global__ void depthwise_generic_kernel(const float* __restrict__ x, const float* __restrict__ f,
-                                         const float* __restrict__ bias, int act, float* __restrict__ y,
+__global__ void depthwise_generic_kernel(const float* x, const float* f,
+                                         const float* bias, int act, float* __restrict__ y,
                                          ConvGeom g, int64_t n_out) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_out; i += stride) {
@@ -238,8 +238,8 @@ constexpr int DW_TMA_THREADS = DW_THREADS + 32;  // eight compute warps and the 
 // GRADIENT: the forward pass over dy that is the input gradient; `x` is the tensor itself, for filters that are not finite.
 template <int S, int TW, int R, int D = 1, int CB = DW_CB, bool NARROW = false, bool GRADIENT = false>
 __global__ void __launch_bounds__(DW_TMA_THREADS, 2)
-depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* __restrict__ x, const float* __restrict__ f,
-                        const float* __restrict__ bias, int act, void* __restrict__ y, int y_f32, const __grid_constant__ ConvGeom g,
+depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* x, const float* f,
+                        const float* bias, int act, void* __restrict__ y, int y_f32, const __grid_constant__ ConvGeom g,
                         const __grid_constant__ DwTiling t, unsigned int* dev_status) {
     using T = DwTile<S, TW, R, D, CB, NARROW>;
     extern __shared__ uint8_t dw_smem_raw[];
@@ -348,8 +348,8 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
             if (cb != loaded_cb) {
 #pragma unroll
                 for (int k = 0; k < 9; ++k)
-                    dw_tap(w[k], __ldg(reinterpret_cast<const float4*>(f + (int64_t)k * t.f_step + c)));
-                if (bias) b = __ldg(reinterpret_cast<const float4*>(bias + c));
+                    dw_tap(w[k], load_global(reinterpret_cast<const float4*>(f + (int64_t)k * t.f_step + c)));
+                if (bias) b = load_global(reinterpret_cast<const float4*>(bias + c));
                 if constexpr (GRADIENT) {
                     float4 nil = make_float4(0.f, 0.f, 0.f, 0.f);
                     const float4 zero = nil;

@@ -58,7 +58,7 @@ __device__ __noinline__ float sum_of_existing(const DgTensors& d, const DgTiling
             for (int ox = tx * TW; ox < min(d.Wo, (tx + 1) * TW); ++ox) {
                 const int iy = oy * S + off_y, ix = ox * S + off_x;
                 if (iy < 0 || iy >= d.H || ix < 0 || ix >= d.W) continue;
-                acc = fmaf(__ldg(d.x + ((n * d.H + iy) * d.W + ix) * C + c), __ldg(d.dy + ((n * d.Ho + oy) * d.Wo + ox) * C + c), acc);
+                acc = fmaf(load_global(d.x + ((n * d.H + iy) * d.W + ix) * C + c), load_global(d.dy + ((n * d.Ho + oy) * d.Wo + ox) * C + c), acc);
             }
         if (acc != acc) break;
     }
@@ -88,6 +88,8 @@ depthwise3x3_backprop_filter_kernel(const __grid_constant__ CUtensorMap map_x, c
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int first = blockIdx.x, step = gridDim.x;  // step is a multiple of the channel blocks
     const int my_tiles = first < t.num_tiles ? (t.num_tiles - first + step - 1) / step : 0;
     const int cb = first % t.c_blocks;
@@ -209,9 +211,8 @@ cudaError_t launch_instance(const DepthwiseGradPlan& p, float* out, unsigned int
     if (e != cudaSuccess) return e;
     const DgTiling t{p.tiles_x, p.tiles_y, p.c_blocks, p.stages, p.num_tiles};
     const DgTensors d{p.x, p.dy, p.g.H, p.g.W, p.g.Ho, p.g.Wo};
-    kernel<<<p.slices * p.c_blocks, DG_ALL_THREADS, (size_t)p.stages * p.stage_bytes + 128, s>>>(p.map_x, p.map_dy, out, p.g.C, p.g.pt,
-                                                                                                p.g.pl, t, d, dev_status);
-    return cudaGetLastError();
+    return launch_k(kernel, dim3(p.slices * p.c_blocks), dim3(DG_ALL_THREADS), (size_t)p.stages * p.stage_bytes + 128, s, p.map_x, p.map_dy,
+                    out, p.g.C, p.g.pt, p.g.pl, t, d, dev_status);
 }
 
 bool encode_nhwc(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int64_t n, int h, int w, int c, int box_h, int box_w) {

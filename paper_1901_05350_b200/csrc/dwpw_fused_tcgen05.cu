@@ -610,8 +610,8 @@ dwpw_fused_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
                     if (kb != loaded_kb) {
                         const int c = kb * BLOCK_K + c2 * 2;
 #pragma unroll
-                        for (int k = 0; k < 9; ++k) w[k] = __ldg(reinterpret_cast<const float2*>(args.dw_filter + (int64_t)k * args.C + c));
-                        if (args.dw_bias) b = __ldg(reinterpret_cast<const float2*>(args.dw_bias + c));
+                        for (int k = 0; k < 9; ++k) w[k] = load_global(reinterpret_cast<const float2*>(args.dw_filter + (int64_t)k * args.C + c));
+                        if (args.dw_bias) b = load_global(reinterpret_cast<const float2*>(args.dw_bias + c));
                         loaded_kb = kb;
                     }
                     // The operand stage first.  With two groups and a patch ring of three, this group did not wait for the

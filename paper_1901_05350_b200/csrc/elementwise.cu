@@ -16,38 +16,58 @@ inline int grid_for(int64_t work_items, int threads, int max_blocks) {
     return (int)b;
 }
 
+// The elementwise kernels take STRIDED items per thread and pass, a grid apart, and load all of them before they store the
+// first (add of 2 x 25.7 MB: 7.0 us, with one or two loads in flight per thread 8.3).
+constexpr int STRIDED = 4;
+
+// i % period, in 32 bits where they do (the 64-bit remainder is a hundred instructions)
+__device__ __forceinline__ int64_t wrap(int64_t i, int64_t period) {
+    return (uint64_t)i < (1ull << 32) && (uint64_t)period < (1ull << 32) ? (int64_t)((uint32_t)i % (uint32_t)period) : i % period;
+}
+
 // ---- bias + activation ----------------------------------------------------------------------
 // out[r, c] = act(x[r, c] + bias[c]).  float4 path: C % 4 == 0, so a float4 never straddles rows.
-__global__ void bias_act_vec4_kernel(const float4* __restrict__ x, const float* __restrict__ bias,
-                                     float4* __restrict__ y, int64_t n_vec, int C4, int act) {
+__global__ void bias_act_vec4_kernel(const float4* x, const float* bias, float4* y, int64_t n_vec, int C4, int act) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += stride) {
-        float4 v = x[i];
-        if (bias) {
-            const int c = (int)(i % C4) * 4;
-            const float4 b = *reinterpret_cast<const float4*>(bias + c);
-            v.x = v.x + b.x; v.y = v.y + b.y; v.z = v.z + b.z; v.w = v.w + b.w;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += STRIDED * stride) {
+        float4 v[STRIDED];
+#pragma unroll
+        for (int u = 0; u < STRIDED; ++u)
+            if (i + u * stride < n_vec) v[u] = x[i + u * stride];
+#pragma unroll
+        for (int u = 0; u < STRIDED; ++u) {
+            const int64_t at = i + u * stride;
+            if (at >= n_vec) break;
+            if (bias) {
+                const float4 b = load_global(reinterpret_cast<const float4*>(bias) + wrap(at, C4));
+                v[u].x = v[u].x + b.x; v[u].y = v[u].y + b.y; v[u].z = v[u].z + b.z; v[u].w = v[u].w + b.w;
+            }
+            v[u].x = apply_act(v[u].x, act); v[u].y = apply_act(v[u].y, act);
+            v[u].z = apply_act(v[u].z, act); v[u].w = apply_act(v[u].w, act);
+            y[at] = v[u];
         }
-        v.x = apply_act(v.x, act); v.y = apply_act(v.y, act);
-        v.z = apply_act(v.z, act); v.w = apply_act(v.w, act);
-        y[i] = v;
     }
 }
 
-__global__ void bias_act_scalar_kernel(const float* __restrict__ x, const float* __restrict__ bias,
-                                       float* __restrict__ y, int64_t n, int64_t C, int act) {
+__global__ void bias_act_scalar_kernel(const float* x, const float* bias, float* y, int64_t n, int64_t C, int act) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         float v = x[i];
-        if (bias) v = v + bias[i % C];
+        if (bias) v = v + bias[wrap(i, C)];
         y[i] = apply_act(v, act);
     }
 }
 
 // ---- avgPool ----------------------------------------------------------------------------------
 // One thread per output element, channel fastest (coalesced).  Padding never counts.
-__global__ void avg_pool_window_kernel(const float* __restrict__ x, float* __restrict__ y, ConvGeom g,
+__global__ void avg_pool_window_kernel(const float* x, float* __restrict__ y, ConvGeom g,
                                        int64_t n_out) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_out; i += stride) {
         const int c = (int)(i % g.C);
@@ -74,8 +94,10 @@ __global__ void avg_pool_window_kernel(const float* __restrict__ x, float* __res
 // ---- maxPool ----------------------------------------------------------------------------------
 // One thread per output element, channel fastest (coalesced).  Padding never takes part; max.NaN keeps
 // a NaN that is in the window.
-__global__ void max_pool_window_kernel(const float* __restrict__ x, float* __restrict__ y, ConvGeom g,
+__global__ void max_pool_window_kernel(const float* x, float* __restrict__ y, ConvGeom g,
                                        int64_t n_out) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_out; i += stride) {
         const int c = (int)(i % g.C);
@@ -106,7 +128,9 @@ __device__ __forceinline__ void max4_nan(float4& m, const float4& v) {
     asm("max.NaN.f32 %0, %0, %1;" : "+f"(m.z) : "f"(v.z));
     asm("max.NaN.f32 %0, %0, %1;" : "+f"(m.w) : "f"(v.w));
 }
-__global__ void max_pool_vec4_kernel(const float* __restrict__ x, float* __restrict__ y, ConvGeom g, int64_t n_out4) {
+__global__ void max_pool_vec4_kernel(const float* x, float* __restrict__ y, ConvGeom g, int64_t n_out4) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int C4 = g.C >> 2;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_out4; i += stride) {
@@ -120,9 +144,24 @@ __global__ void max_pool_vec4_kernel(const float* __restrict__ x, float* __restr
         const int iy0 = oy * g.sh - g.pt, ix0 = ox * g.sw - g.pl;
         const int ky0 = iy0 < 0 ? -iy0 : 0, ky1 = min(g.fh, g.H - iy0);
         const int kx0 = ix0 < 0 ? -ix0 : 0, kx1 = min(g.fw, g.W - ix0);
-        for (int ky = ky0; ky < ky1; ++ky) {
-            const float* row = x + ((n * g.H + iy0 + ky) * (int64_t)g.W + ix0) * g.C + c;
-            for (int kx = kx0; kx < kx1; ++kx) max4_nan(m, __ldg(reinterpret_cast<const float4*>(row + (int64_t)kx * g.C)));
+        if (g.fh <= 3 && g.fw <= 3) {
+            // the usual windows: all samples on their way before the first comparison; -inf where there is none
+            float4 v[3][3];
+#pragma unroll
+            for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx) {
+                    v[ky][kx] = m;
+                    if (ky >= ky0 && ky < ky1 && kx >= kx0 && kx < kx1)
+                        v[ky][kx] = load_global(reinterpret_cast<const float4*>(x + ((n * g.H + iy0 + ky) * (int64_t)g.W + ix0 + kx) * g.C + c));
+                }
+#pragma unroll
+            for (int k = 0; k < 9; ++k) max4_nan(m, v[k / 3][k % 3]);
+        } else {
+            for (int ky = ky0; ky < ky1; ++ky) {
+                const float* row = x + ((n * g.H + iy0 + ky) * (int64_t)g.W + ix0) * g.C + c;
+                for (int kx = kx0; kx < kx1; ++kx) max4_nan(m, load_global(reinterpret_cast<const float4*>(row + (int64_t)kx * g.C)));
+            }
         }
         *reinterpret_cast<float4*>(y + i * 4) = m;
     }
@@ -136,27 +175,40 @@ __device__ __forceinline__ float binary_op(float u, float v) {
 }
 // float4 path: n and b_len multiples of 4 (a float4 never straddles a period of b)
 template <int OP>
-__global__ void binary_vec4_kernel(const float4* __restrict__ a, const float4* __restrict__ b, float4* __restrict__ out,
-                                   int64_t n4, int64_t b_len4) {
+__global__ void binary_vec4_kernel(const float4* a, const float4* b, float4* out, int64_t n4, int64_t b_len4) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-        const float4 u = a[i];
-        const float4 v = b_len4 == n4 ? b[i] : __ldg(b + i % b_len4);
-        out[i] = make_float4(binary_op<OP>(u.x, v.x), binary_op<OP>(u.y, v.y), binary_op<OP>(u.z, v.z), binary_op<OP>(u.w, v.w));
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += STRIDED * stride) {
+        float4 u[STRIDED], v[STRIDED];
+#pragma unroll
+        for (int k = 0; k < STRIDED; ++k) {
+            const int64_t at = i + k * stride;
+            if (at >= n4) break;
+            u[k] = a[at];
+            v[k] = b[b_len4 == n4 ? at : wrap(at, b_len4)];
+        }
+#pragma unroll
+        for (int k = 0; k < STRIDED; ++k) {
+            if (i + k * stride >= n4) break;
+            out[i + k * stride] = make_float4(binary_op<OP>(u[k].x, v[k].x), binary_op<OP>(u[k].y, v[k].y), binary_op<OP>(u[k].z, v[k].z),
+                                              binary_op<OP>(u[k].w, v[k].w));
+        }
     }
 }
 template <int OP>
-__global__ void binary_scalar_kernel(const float* __restrict__ a, const float* __restrict__ b, float* __restrict__ out,
-                                     int64_t n, int64_t b_len) {
+__global__ void binary_scalar_kernel(const float* a, const float* b, float* out, int64_t n, int64_t b_len) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        out[i] = binary_op<OP>(a[i], b[i % b_len]);
+        out[i] = binary_op<OP>(a[i], b[wrap(i, b_len)]);
 }
 
 // Global pool: a block owns (image n, 128 consecutive channels).  Lane = 4 channels (one float4, so a
 // warp reads 512 contiguous bytes per position), the 8 warps stride over the H*W positions, partial
 // sums meet in shared memory.  C % 4 == 0.
-__global__ void avg_pool_global_vec4_kernel(const float* __restrict__ x, float* __restrict__ y, int HW, int C) {
+__global__ void avg_pool_global_vec4_kernel(const float* x, float* __restrict__ y, int HW, int C) {
     __shared__ float4 partial[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = (blockIdx.x * 32 + lane) * 4;
@@ -195,7 +247,7 @@ __global__ void avg_pool_global_vec4_kernel(const float* __restrict__ x, float* 
 }
 
 // The same with one channel per lane, for channel counts that are not multiples of 4.
-__global__ void avg_pool_global_kernel(const float* __restrict__ x, float* __restrict__ y, int HW, int C) {
+__global__ void avg_pool_global_kernel(const float* x, float* __restrict__ y, int HW, int C) {
     __shared__ float partial[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = blockIdx.x * 32 + lane;
@@ -230,7 +282,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // One block (kThreads) per row: max, then sum of exp(x - max), then the quotient.
-__global__ void softmax_rows_kernel(const float* __restrict__ x, float* __restrict__ y, int64_t cols) {
+__global__ void softmax_rows_kernel(const float* x, float* __restrict__ y, int64_t cols) {
     __shared__ float red[kThreads / 32];
     __shared__ float bcast;
     const float* xr = x + (int64_t)blockIdx.x * cols;
@@ -272,7 +324,9 @@ __global__ void softmax_rows_kernel(const float* __restrict__ x, float* __restri
 // ---- transpose --------------------------------------------------------------------------------
 // out[b, c, r] = in[b, r, c]: a 32 x 32 tile through shared memory per block.  The grid covers (columns, rows, matrices) and
 // walks on over rows and matrices beyond its limits.
-__global__ void transpose_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t batches, int64_t rows, int64_t cols) {
+__global__ void transpose_kernel(const float* in, float* __restrict__ out, int64_t batches, int64_t rows, int64_t cols) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     __shared__ float tile[32][33];
     const int64_t c0 = (int64_t)blockIdx.x * 32;
     for (int64_t b = blockIdx.z; b < batches; b += gridDim.z) {
@@ -296,7 +350,9 @@ __global__ void transpose_kernel(const float* __restrict__ in, float* __restrict
 // ---- filter packing for the implicit-GEMM convolution ------------------------------------------------
 // out[n, t * c_pad + c] = c < C ? f[t, c, n] : 0.  A 32 x 32 transpose through shared memory per block, so that both
 // sides are read and written in 128-byte runs.
-__global__ void pack_filter_kernel(const float* __restrict__ f, float* __restrict__ out, int64_t C, int64_t N, int64_t c_pad) {
+__global__ void pack_filter_kernel(const float* f, float* __restrict__ out, int64_t C, int64_t N, int64_t c_pad) {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     __shared__ float tile[32][33];
     const int64_t n0 = (int64_t)blockIdx.x * 32, t = blockIdx.z;
     for (int64_t c0 = (int64_t)blockIdx.y * 32; c0 < c_pad; c0 += (int64_t)gridDim.y * 32) {
@@ -320,24 +376,21 @@ cudaError_t launch_pack_filter(const float* f, float* out, int64_t taps, int64_t
     if (taps * N * c_pad == 0) return cudaSuccess;
     if (taps > 65535) return cudaErrorInvalidConfiguration;  // im2col copies have 128 x 128 at most
     const int64_t gy = (c_pad + 31) / 32;                    // the grid walks on where there are more
-    pack_filter_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)(gy < 65535 ? gy : 65535), (unsigned)taps), dim3(32, 8), 0, s>>>(f, out, C, N, c_pad);
     ++*launches;
-    return cudaGetLastError();
+    return launch_k(pack_filter_kernel, dim3((unsigned)((N + 31) / 32), (unsigned)(gy < 65535 ? gy : 65535), (unsigned)taps), dim3(32, 8), 0, s, f, out, C, N, c_pad);
 }
 
 cudaError_t launch_bias_act(const float* x, const float* bias, float* y, int64_t rows, int64_t C, int act,
                             cudaStream_t s, int64_t* launches) {
     const int64_t n = rows * C;
     if (n == 0) return cudaSuccess;
+    ++*launches;
     if (C % 4 == 0) {
         const int64_t n_vec = n / 4;
-        bias_act_vec4_kernel<<<grid_for(n_vec, kThreads, current_sm_count() * 16), kThreads, 0, s>>>(
-            reinterpret_cast<const float4*>(x), bias, reinterpret_cast<float4*>(y), n_vec, (int)(C / 4), act);
-    } else {
-        bias_act_scalar_kernel<<<grid_for(n, kThreads, current_sm_count() * 16), kThreads, 0, s>>>(x, bias, y, n, C, act);
+        return launch_k(bias_act_vec4_kernel, dim3(grid_for(n_vec, kThreads, current_sm_count() * 16)), dim3(kThreads), 0, s,
+                        reinterpret_cast<const float4*>(x), bias, reinterpret_cast<float4*>(y), n_vec, (int)(C / 4), act);
     }
-    ++*launches;
-    return cudaGetLastError();
+    return launch_k(bias_act_scalar_kernel, dim3(grid_for(n, kThreads, current_sm_count() * 16)), dim3(kThreads), 0, s, x, bias, y, n, C, act);
 }
 
 cudaError_t launch_avg_pool(const float* x, float* y, const ConvGeom& g, cudaStream_t s, int64_t* launches) {
@@ -345,43 +398,28 @@ cudaError_t launch_avg_pool(const float* x, float* y, const ConvGeom& g, cudaStr
     if (n_out == 0) return cudaSuccess;
     const bool global = g.Ho == 1 && g.Wo == 1 && g.fh == g.H && g.fw == g.W && g.pt == 0 && g.pl == 0 &&
                         g.N <= 65535;
-    if (global) {
-        cudaError_t e;
-        if (g.C % 4 == 0) {
-            dim3 grid((g.C / 4 + 31) / 32, (unsigned)g.N);
-            e = launch_k(avg_pool_global_vec4_kernel, grid, dim3(256), 0, s, x, y, g.H * g.W, g.C);
-        } else {
-            dim3 grid((g.C + 31) / 32, (unsigned)g.N);
-            e = launch_k(avg_pool_global_kernel, grid, dim3(256), 0, s, x, y, g.H * g.W, g.C);
-        }
-        ++*launches;
-        return e;
-    } else {
-        avg_pool_window_kernel<<<grid_for(n_out, kThreads, current_sm_count() * 16), kThreads, 0, s>>>(x, y, g, n_out);
-    }
     ++*launches;
-    return cudaGetLastError();
+    if (!global) return launch_k(avg_pool_window_kernel, dim3(grid_for(n_out, kThreads, current_sm_count() * 16)), dim3(kThreads), 0, s, x, y, g, n_out);
+    if (g.C % 4 == 0)
+        return launch_k(avg_pool_global_vec4_kernel, dim3((g.C / 4 + 31) / 32, (unsigned)g.N), dim3(256), 0, s, x, y, g.H * g.W, g.C);
+    return launch_k(avg_pool_global_kernel, dim3((g.C + 31) / 32, (unsigned)g.N), dim3(256), 0, s, x, y, g.H * g.W, g.C);
 }
 
 cudaError_t launch_max_pool(const float* x, float* y, const ConvGeom& g, cudaStream_t s, int64_t* launches) {
     const int64_t n_out = g.N * g.Ho * g.Wo * g.C;
     if (n_out == 0) return cudaSuccess;
-    if (g.C % 4 == 0)
-        max_pool_vec4_kernel<<<grid_for(n_out / 4, kThreads, current_sm_count() * 32), kThreads, 0, s>>>(x, y, g, n_out / 4);
-    else
-        max_pool_window_kernel<<<grid_for(n_out, kThreads, current_sm_count() * 16), kThreads, 0, s>>>(x, y, g, n_out);
     ++*launches;
-    return cudaGetLastError();
+    if (g.C % 4 == 0)
+        return launch_k(max_pool_vec4_kernel, dim3(grid_for(n_out / 4, kThreads, current_sm_count() * 32)), dim3(kThreads), 0, s, x, y, g, n_out / 4);
+    return launch_k(max_pool_window_kernel, dim3(grid_for(n_out, kThreads, current_sm_count() * 16)), dim3(kThreads), 0, s, x, y, g, n_out);
 }
 
 template <int OP>
 static cudaError_t launch_binary_op(const float* a, const float* b, float* out, int64_t n, int64_t b_len, cudaStream_t s) {
     if (n % 4 == 0 && b_len % 4 == 0)
-        binary_vec4_kernel<OP><<<grid_for(n / 4, kThreads, current_sm_count() * 16), kThreads, 0, s>>>(
-            reinterpret_cast<const float4*>(a), reinterpret_cast<const float4*>(b), reinterpret_cast<float4*>(out), n / 4, b_len / 4);
-    else
-        binary_scalar_kernel<OP><<<grid_for(n, kThreads, current_sm_count() * 16), kThreads, 0, s>>>(a, b, out, n, b_len);
-    return cudaGetLastError();
+        return launch_k(binary_vec4_kernel<OP>, dim3(grid_for(n / 4, kThreads, current_sm_count() * 16)), dim3(kThreads), 0, s,
+                        reinterpret_cast<const float4*>(a), reinterpret_cast<const float4*>(b), reinterpret_cast<float4*>(out), n / 4, b_len / 4);
+    return launch_k(binary_scalar_kernel<OP>, dim3(grid_for(n, kThreads, current_sm_count() * 16)), dim3(kThreads), 0, s, a, b, out, n, b_len);
 }
 
 cudaError_t launch_binary(int op, const float* a, const float* b, float* out, int64_t n, int64_t b_len, cudaStream_t s,
@@ -407,9 +445,8 @@ cudaError_t launch_transpose_batched(const float* in, float* out, int64_t batche
     if (rows == 0 || cols == 0 || batches == 0) return cudaSuccess;
     const int64_t gy = (rows + 31) / 32;
     const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)(gy < 65535 ? gy : 65535), (unsigned)(batches < 65535 ? batches : 65535));
-    transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(in, out, batches, rows, cols);
     ++*launches;
-    return cudaGetLastError();
+    return launch_k(transpose_kernel, grid, dim3(32, 8), 0, s, in, out, batches, rows, cols);
 }
 
 cudaError_t launch_transpose(const float* in, float* out, int64_t rows, int64_t cols, cudaStream_t s, int64_t* launches) {

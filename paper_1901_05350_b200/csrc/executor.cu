@@ -500,8 +500,9 @@ tfjsb_status capture_graph(tfjsb_model* m) {
 
 // Launches layer i (and, when it is fused with its successor, that one too); returns how many layers ran.
 struct PdlScope {
+    const bool before = g_launch_pdl;
     explicit PdlScope(bool on) { g_launch_pdl = on; }
-    ~PdlScope() { g_launch_pdl = false; }
+    ~PdlScope() { g_launch_pdl = before; }
 };
 
 cudaError_t launch_layers(tfjsb_model* m, int i, cudaStream_t s, int* consumed) {

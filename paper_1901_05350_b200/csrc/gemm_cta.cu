@@ -86,7 +86,7 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
 // Window and channel count known at compile time and fh*fw*Cin <= 32 (one k-block): no index
 // arithmetic is left at run time beyond three row pointers and six bounds flags.
 template <int FH, int FW, int CIN>
-__device__ __forceinline__ void gather_small(float (&v)[BLOCK_K], const float* __restrict__ xn, const ConvGeom& g,
+__device__ __forceinline__ void gather_small(float (&v)[BLOCK_K], const float* xn, const ConvGeom& g,
                                              int iy0, int ix0, bool live) {
     static_assert(FH * FW * CIN <= BLOCK_K, "one k-block only");
     const float* rowp[FH];
@@ -107,7 +107,7 @@ __device__ __forceinline__ void gather_small(float (&v)[BLOCK_K], const float* _
     for (int e = 0; e < BLOCK_K; ++e) {
         if (e < FH * FW * CIN) {
             const int ky = e / (FW * CIN), kx = (e / CIN) % FW, ci = e % CIN;
-            v[e] = (vy[ky] && vx[kx]) ? __ldg(rowp[ky] + kx * dwc + ci) : 0.0f;
+            v[e] = (vy[ky] && vx[kx]) ? load_global(rowp[ky] + kx * dwc + ci) : 0.0f;
         } else {
             v[e] = 0.0f;
         }
@@ -115,7 +115,7 @@ __device__ __forceinline__ void gather_small(float (&v)[BLOCK_K], const float* _
 }
 
 // Cin % 4 == 0: four consecutive k share a tap, so each quad is one float4 load.
-__device__ __forceinline__ void gather_vec4(float (&v)[BLOCK_K], const float* __restrict__ xn, const ConvGeom& g,
+__device__ __forceinline__ void gather_vec4(float (&v)[BLOCK_K], const float* xn, const ConvGeom& g,
                                             int iy0, int ix0, bool live, int k0, int k_total) {
     int tap = k0 / g.C;
     int ci = k0 - tap * g.C;
@@ -126,7 +126,7 @@ __device__ __forceinline__ void gather_vec4(float (&v)[BLOCK_K], const float* __
         float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
         const int iy = iy0 + ky * g.dh, ix = ix0 + kx * g.dw;
         if (live && k0 + e < k_total && iy >= 0 && iy < g.H && ix >= 0 && ix < g.W)
-            q = __ldg(reinterpret_cast<const float4*>(xn + ((int64_t)iy * g.W + ix) * g.C + ci));
+            q = load_global(reinterpret_cast<const float4*>(xn + ((int64_t)iy * g.W + ix) * g.C + ci));
         v[e] = q.x; v[e + 1] = q.y; v[e + 2] = q.z; v[e + 3] = q.w;
         ci += 4;
         if (ci == g.C) { ci = 0; if (++kx == g.fw) { kx = 0; ++ky; } }
@@ -134,7 +134,7 @@ __device__ __forceinline__ void gather_vec4(float (&v)[BLOCK_K], const float* __
 }
 
 // Any window and channel count: a pointer walks the tap, re-based when the tap column or row changes.
-__device__ __forceinline__ void gather_scalar(float (&v)[BLOCK_K], const float* __restrict__ xn, const ConvGeom& g,
+__device__ __forceinline__ void gather_scalar(float (&v)[BLOCK_K], const float* xn, const ConvGeom& g,
                                               int iy0, int ix0, bool live, int k0, int k_total) {
     int tap = k0 / g.C;
     int ci = k0 - tap * g.C;
@@ -146,7 +146,7 @@ __device__ __forceinline__ void gather_scalar(float (&v)[BLOCK_K], const float* 
     const int left = k_total - k0;
 #pragma unroll
     for (int e = 0; e < BLOCK_K; ++e) {
-        v[e] = (ok && e < left) ? __ldg(p) : 0.0f;
+        v[e] = (ok && e < left) ? load_global(p) : 0.0f;
         ++p;
         if (++ci == g.C) {
             ci = 0;

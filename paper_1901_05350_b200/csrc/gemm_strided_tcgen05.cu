@@ -70,14 +70,14 @@ struct Fetch {
             const bool ok = k0 + lane < K;
             const float* at = base + k0 + lane;
 #pragma unroll
-            for (int i = 0; i < ROWS / 8; ++i) v[i] = ok ? __ldg(at + (long long)min(r0 + w + 8 * i, last) * s.row_stride) : 0.f;
+            for (int i = 0; i < ROWS / 8; ++i) v[i] = ok ? load_global(at + (long long)min(r0 + w + 8 * i, last) * s.row_stride) : 0.f;
         } else {                // lane = row of block i, k = 4 w + e; rows are contiguous
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int k = k0 + 4 * w + e;
                 const float* at = base + (long long)k * s.k_stride;
 #pragma unroll
-                for (int i = 0; i < ROWS / 32; ++i) v[4 * i + e] = k < K ? __ldg(at + min(r0 + 32 * i + lane, last)) : 0.f;
+                for (int i = 0; i < ROWS / 32; ++i) v[4 * i + e] = k < K ? load_global(at + min(r0 + 32 * i + lane, last)) : 0.f;
             }
         }
     }
@@ -108,7 +108,7 @@ struct Fetch {
 // One element over k0 .. k1 by fp32 multiply-adds.
 __device__ __noinline__ float sum_in_fp32(const float* p, const float* q, int p_step, int q_step, int k0, int k1) {
     float acc = 0.f;
-    for (int k = k0; k < k1 && acc == acc; ++k) acc = fmaf(__ldg(p + (long long)k * p_step), __ldg(q + (long long)k * q_step), acc);
+    for (int k = k0; k < k1 && acc == acc; ++k) acc = fmaf(load_global(p + (long long)k * p_step), load_global(q + (long long)k * q_step), acc);
     return acc;
 }
 
@@ -300,7 +300,7 @@ gemm_strided_kernel(const StridedArgs g) {
         const uint32_t at_step = (uint32_t)((row_step * PITCH + col_step) * 4);
         // the bias is either one value per thread or walked along
         const bool one_bias = g.bias != nullptr && along_p == (g.bias_p != 0);
-        const float b0 = one_bias && live ? __ldg(g.bias + (along_p ? p : q)) : 0.f;
+        const float b0 = one_bias && live ? load_global(g.bias + (along_p ? p : q)) : 0.f;
         const float* bias = g.bias != nullptr && !one_bias ? g.bias + (along_p ? q0 : p0 + r0) : nullptr;
 #pragma unroll 4
         for (int i = along_p ? col : row; i < (live ? limit : 0); i += step, at += at_step, out += out_step) {
@@ -317,7 +317,7 @@ gemm_strided_kernel(const StridedArgs g) {
                 for (int s = 1; s < GS_MAX_CLUSTER; ++s)
                     if (s < g.splits) v += part[s];
             }
-            if (g.bias) v += bias ? __ldg(bias + i) : b0;
+            if (g.bias) v += bias ? load_global(bias + i) : b0;
             *out = apply_act(v, g.act);
         }
     }

@@ -262,7 +262,7 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
             const int grow = m0 + (int)rank * rows_per + i, gcol = n0 + ch * EPI_COLS + 4 * j;
             const bool live = grow < args.M && gcol < args.N;   // N % 4 == 0: a quad is all in or all out
             float4 bq = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (args.bias != nullptr && live) bq = __ldg(reinterpret_cast<const float4*>(args.bias + gcol));
+            if (args.bias != nullptr && live) bq = load_global(reinterpret_cast<const float4*>(args.bias + gcol));
             const uint32_t piece = partial_base + (uint32_t)((i * chunks + ch) * 128) + (uint32_t)((j ^ (i & 7)) << 4);
             const uint32_t slice_pitch = (uint32_t)(rows_per * chunks * 128);
             float4 v = ld_shared_v4(piece);

@@ -29,7 +29,7 @@ inline int a_box_rows(int64_t M) { return M >= BLOCK_M ? BLOCK_M : (int)((M + 7)
 // activation, and the swizzled store into the staging slab the bulk tensor store reads from
 // (16-byte chunk j of row `lane` lives at chunk j ^ (lane % 8): the 128-byte swizzle).
 template <int ACT>
-__device__ __forceinline__ void stage_chunk(const uint32_t (&r)[32], const float* __restrict__ bias, int cols_left,
+__device__ __forceinline__ void stage_chunk(const uint32_t (&r)[32], const float* bias, int cols_left,
                                             uint32_t row_addr, int lane) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -37,7 +37,7 @@ __device__ __forceinline__ void stage_chunk(const uint32_t (&r)[32], const float
         v.x = __uint_as_float(r[4 * j + 0]); v.y = __uint_as_float(r[4 * j + 1]);
         v.z = __uint_as_float(r[4 * j + 2]); v.w = __uint_as_float(r[4 * j + 3]);
         if (bias != nullptr && 4 * j < cols_left) {  // N % 4 == 0: a quad is all in or all out
-            const float4 b = __ldg(reinterpret_cast<const float4*>(bias + 4 * j));
+            const float4 b = load_global(reinterpret_cast<const float4*>(bias + 4 * j));
             v.x = v.x + b.x; v.y = v.y + b.y; v.z = v.z + b.z; v.w = v.w + b.w;
         }
         v.x = apply_act_t<ACT>(v.x); v.y = apply_act_t<ACT>(v.y);
@@ -126,7 +126,7 @@ __device__ __forceinline__ uint32_t make_idesc_bf16(int m, int n) {
 // and the store into the staging slab in the 64-byte swizzle the bulk tensor store expects (rows of
 // 64 bytes; 16-byte piece j of row r lives at piece j ^ ((r / 2) % 4)).
 template <int ACT>
-__device__ __forceinline__ void stage_chunk_bf16(const uint32_t (&r)[32], const float* __restrict__ bias, int cols_left,
+__device__ __forceinline__ void stage_chunk_bf16(const uint32_t (&r)[32], const float* bias, int cols_left,
                                                  uint32_t slab, int lane) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -134,8 +134,8 @@ __device__ __forceinline__ void stage_chunk_bf16(const uint32_t (&r)[32], const 
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(r[8 * j + e]);
         if (bias != nullptr && 8 * j < cols_left) {  // N % 8 == 0: a group of eight is all in or all out
-            const float4 b0 = __ldg(reinterpret_cast<const float4*>(bias + 8 * j));
-            const float4 b1 = __ldg(reinterpret_cast<const float4*>(bias + 8 * j + 4));
+            const float4 b0 = load_global(reinterpret_cast<const float4*>(bias + 8 * j));
+            const float4 b1 = load_global(reinterpret_cast<const float4*>(bias + 8 * j + 4));
             v[0] += b0.x; v[1] += b0.y; v[2] += b0.z; v[3] += b0.w;
             v[4] += b1.x; v[5] += b1.y; v[6] += b1.z; v[7] += b1.w;
         }

@@ -198,3 +198,78 @@ def test_a_call_that_fails_is_not_made_twice(ctx, tfjsb, monkeypatch, call):
             model.run(dev(x), out=wrong)
     assert e.value.status_name == "SHAPE" and str(e.value)
     model.close()
+
+
+def test_op_calls_one_after_another_see_each_others_results(ctx):
+    """Each kernel is launched while the one before drains and waits for it before it reads or writes anything: chains of
+    dependent small and large calls through two buffers, and calls that overwrite what the call before reads."""
+    import torch
+
+    one = {n: torch.ones(n, device="cuda") for n in (64, 1 << 20)}
+    for n, o in one.items():
+        bufs = [torch.zeros(n, device="cuda") for _ in range(2)]
+        for i in range(200):
+            ctx.binary("add", bufs[i % 2], o, out=bufs[(i + 1) % 2])
+        assert float(bufs[0].min()) == 200.0 == float(bufs[0].max())
+    x, w = torch.ones(256, 64, device="cuda"), torch.ones(64, 256, device="cuda")
+    y, z = torch.empty(256, 256, device="cuda"), torch.empty(256, 256, device="cuda")
+    for i in range(50):
+        ctx.matmul(x, w, out=y)                                # 64 everywhere ...
+        ctx.binary("mul", y, y, out=z)                         # ... squared
+        total = ctx.bias_backprop(z)
+    ctx.check_device_status()
+    assert float(z.min()) == 4096.0 == float(z.max())
+    assert float(total.min()) == 256 * 4096.0 == float(total.max())
+
+
+def test_op_calls_captured_on_two_streams_that_join(ctx):
+    import torch
+
+    x, w, b = torch.rand(64, 96, device="cuda"), torch.rand(96, 40, device="cuda"), torch.rand(40, device="cuda")
+
+    def work(side):
+        main = torch.cuda.current_stream()
+        z = torch.zeros(64, 40, device="cuda")
+        a = ctx.binary("add", ctx.matmul(x, w), b)
+        z.add_(a)                                              # another library's kernel in between
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            s = ctx.bias_act(ctx.binary("mul", z, a), act="relu6")
+        c = ctx.binary("sub", z, b)
+        main.wait_stream(side)
+        return ctx.binary("add", c, s)
+
+    side = torch.cuda.Stream()
+    want = work(side).clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = work(side)
+    for _ in range(20):
+        got.zero_()
+        graph.replay()
+        assert torch.equal(got, want)
+    ctx.check_device_status()
+
+
+@pytest.mark.parametrize("n", [4 * 2368 * 256 - 4, 4 * 2368 * 256 + 4, 16 * 2368 * 256, 16 * 2368 * 256 + 8, 36 * 2368 * 256 + 12, 8 * 2368 * 256 + 3])
+def test_elementwise_passes_of_several_items_per_thread(ctx, n):
+    """Sizes at which the last pass of a grid of 2368 x 256 threads (and of any other) holds none, some or all of its items."""
+    import torch
+
+    x, y, b = torch.randn(n, device="cuda"), torch.randn(n, device="cuda"), torch.randn(4, device="cuda")
+    assert torch.equal(ctx.binary("add", x, y), x + y)
+    assert torch.equal(ctx.act_backprop(x, y, "relu"), torch.where(x > 0, y, torch.zeros_like(y)))
+    if n % 4 == 0:
+        r = x.view(n // 4, 4)
+        assert torch.equal(ctx.binary("mul", r, b), r * b)
+        assert torch.equal(ctx.bias_act(r, b, act="relu"), torch.relu(r + b))
+
+
+@pytest.mark.parametrize("window", [(1, 3), (3, 1), (2, 3), (3, 3), (4, 2)])
+def test_max_pool_of_quads_at_the_window_sizes_around_the_unrolled_one(ctx, oracle, window):
+    x = si.uniform(91, 0, (2, 7, 6, 8), -1, 1)
+    x[0, 3, 2, 1] = np.nan
+    x[1, 0, 0, 2] = -np.inf
+    for strides in ((1, 1), (2, 2)):
+        got = host(ctx.max_pool(dev(x), window, strides, "same"))
+        assert same_bits_or_both_nan(got, oracle.max_pool(x, window, strides, "same"))
