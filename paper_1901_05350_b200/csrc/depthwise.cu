@@ -417,31 +417,28 @@ struct DwVariant {
     {S, TW, DwTile<S, TW, R, D, CB, NARROW>::TH, DwTile<S, TW, R, D, CB, NARROW>::STAGE_BYTES,    \
      DwTile<S, TW, R, D, CB, NARROW>::STAGE_STRIDE, CB}
 constexpr DwVariant kDwVariants[] = {
-    // fp32, 32 channels per tile.  Seven rows per thread for every stride-1 image wider than 8 (seven divides the
-    // heights of the usual networks, and against four rows per thread it measured [128,56,56,128] 84.0 -> 77.2 us,
-    // [128,28,28,256] 41.5 -> 39.2 us, [128,112,112,32] no change)
+    // fp32, 32 channels per tile
     DW_VARIANT(1, 16, 7, 1, 32, false),   // 0: stride 1
-    DW_VARIANT(1, 8, 2, 1, 32, false),    // 1: stride 1, images up to 8 wide
+    DW_VARIANT(1, 8, 2, 1, 32, false),    // 1: stride 1, 8 x 8 outputs
     DW_VARIANT(2, 16, 2, 1, 32, false),   // 2: stride 2
     DW_VARIANT(2, 8, 2, 1, 32, false),    // 3: stride 2, 8 outputs wide
     DW_VARIANT(1, 16, 4, 2, 32, false),   // 4: stride 1, dilation 2
     DW_VARIANT(1, 16, 4, 4, 32, false),   // 5: stride 1, dilation 4
     // fp32, 64 channels per tile (256-byte lines): half as many box rows for the copy unit per byte moved
-    DW_VARIANT(1, 16, 7, 1, 64, false),   // 6: stride 1
-    DW_VARIANT(1, 8, 4, 1, 64, false),    // 7: stride 1, images up to 8 wide (a whole 7 x 7 image per tile)
-    DW_VARIANT(2, 8, 2, 1, 64, false),    // 8: stride 2, 8 outputs wide
+    DW_VARIANT(1, 8, 4, 1, 64, false),    // 6: stride 1, 8 x 8 outputs (a whole 7 x 7 image per tile)
+    DW_VARIANT(2, 8, 2, 1, 64, false),    // 7: stride 2, 8 outputs wide
     // bfloat16 storage: the same tiles on 2-byte values, 64 channels (one 128-byte line) then 32
-    DW_VARIANT(1, 16, 7, 1, 64, true),    // 9
-    DW_VARIANT(1, 8, 4, 1, 64, true),     // 10
-    DW_VARIANT(2, 16, 2, 1, 64, true),    // 11
-    DW_VARIANT(2, 8, 2, 1, 64, true),     // 12
-    DW_VARIANT(1, 16, 7, 1, 32, true),    // 13
-    DW_VARIANT(1, 8, 2, 1, 32, true),     // 14
-    DW_VARIANT(2, 16, 2, 1, 32, true),    // 15
-    DW_VARIANT(2, 8, 2, 1, 32, true),     // 16
+    DW_VARIANT(1, 16, 7, 1, 64, true),    // 8
+    DW_VARIANT(1, 8, 4, 1, 64, true),     // 9
+    DW_VARIANT(2, 16, 2, 1, 64, true),    // 10
+    DW_VARIANT(2, 8, 2, 1, 64, true),     // 11
+    DW_VARIANT(1, 16, 7, 1, 32, true),    // 12
+    DW_VARIANT(1, 8, 2, 1, 32, true),     // 13
+    DW_VARIANT(2, 16, 2, 1, 32, true),    // 14
+    DW_VARIANT(2, 8, 2, 1, 32, true),     // 15
 };
 #undef DW_VARIANT
-constexpr int DW_FIRST_NARROW = 9;
+constexpr int DW_FIRST_NARROW = 8;
 constexpr int DW_SMEM_BUDGET = 113 * 1024;  // two CTAs per SM
 
 template <int S, int TW, int R, int D = 1, int CB = DW_CB, bool NARROW = false>
@@ -469,17 +466,16 @@ cudaError_t launch_tma_variant(const DepthwisePlan& plan, const float* x, const 
         DW_CASE(3, 2, 8, 2, 1, 32, false);
         DW_CASE(4, 1, 16, 4, 2, 32, false);
         DW_CASE(5, 1, 16, 4, 4, 32, false);
-        DW_CASE(6, 1, 16, 7, 1, 64, false);
-        DW_CASE(7, 1, 8, 4, 1, 64, false);
-        DW_CASE(8, 2, 8, 2, 1, 64, false);
-        DW_CASE(9, 1, 16, 7, 1, 64, true);
-        DW_CASE(10, 1, 8, 4, 1, 64, true);
-        DW_CASE(11, 2, 16, 2, 1, 64, true);
-        DW_CASE(12, 2, 8, 2, 1, 64, true);
-        DW_CASE(13, 1, 16, 7, 1, 32, true);
-        DW_CASE(14, 1, 8, 2, 1, 32, true);
-        DW_CASE(15, 2, 16, 2, 1, 32, true);
-        DW_CASE(16, 2, 8, 2, 1, 32, true);
+        DW_CASE(6, 1, 8, 4, 1, 64, false);
+        DW_CASE(7, 2, 8, 2, 1, 64, false);
+        DW_CASE(8, 1, 16, 7, 1, 64, true);
+        DW_CASE(9, 1, 8, 4, 1, 64, true);
+        DW_CASE(10, 2, 16, 2, 1, 64, true);
+        DW_CASE(11, 2, 8, 2, 1, 64, true);
+        DW_CASE(12, 1, 16, 7, 1, 32, true);
+        DW_CASE(13, 1, 8, 2, 1, 32, true);
+        DW_CASE(14, 2, 16, 2, 1, 32, true);
+        DW_CASE(15, 2, 8, 2, 1, 32, true);
         default: return cudaErrorInvalidValue;
     }
 #undef DW_CASE
@@ -507,15 +503,22 @@ tfjsb_status depthwise_plan(tfjsb_ctx* ctx, const void* x, const ConvGeom& g, De
     if (dilated) v = g.dh == 2 ? 4 : 5;
     else if (narrow) v = DW_FIRST_NARROW + (g.C % 64 == 0 ? 0 : 4) + (g.sh == 1 ? (g.Wo <= 8 ? 1 : 0) : (wide8 ? 3 : 2));
     else {
-        v = g.sh == 1 ? (g.Wo <= 8 ? 1 : 0) : (g.Wo <= 8 ? 3 : 2);
-        // 64-channel tiles where the channel count allows.  Measured at batch 128: [112,112,64] stride 2
-        // 90.1 -> 86.9 us, [7,7,1024] 19.5 -> 15.4 us, the 14 x 14 x 512 layers unchanged; the stride-2 form is
-        // 8 outputs wide, so it is taken only where that wastes fewer columns than the 16-wide 32-channel one
-        // ([28,28,256] stride 2 ran 27.3 -> 29.1 us with it).
-        if (g.C % 64 == 0) {
-            if (g.sh == 1) v = v == 0 ? 6 : 7;
-            else if (wide8) v = 8;
-        }
+        // Stride 1.  8 x 8 tiles of 32 channels while an SM would not have one of 64: a short layer takes what one tile takes
+        // (copy, rows, stores), and its rows per thread are 2 instead of 4 or 7 ([1,56,56,128] 4.1 -> 3.0 us, [1,14,14,512]
+        // 3.3 -> 2.9, [4,14,14,512] 3.8 -> 3.2; against 16 x 7 tiles, as all below).  They also read DRAM faster where the
+        // tensors do not stay in L2 and a pixel is 512 bytes or less ([128,56,56,128] 73.4 -> 66.3, [100,112,112,64] 116 -> 100;
+        // but [128,28,28,256] 36.7 and 39.6).  Otherwise 8 x 8 of 64 channels, whose edges waste less than those of 16 x 7
+        // ([8,17,17,512] 5.9 -> 4.6, [32,56,56,128] 18.8 -> 17.1, [128,14,14,512] 18.1 either way, [128,28,28,256] 36.7 -> 37.1).
+        // Channels that are no multiple of 64: 8 x 8 up to 24 tiles per SM ([8,112,112,32] 6.8 -> 6.0, [16,112,112,32] 9.7 -> 9.2),
+        // then 16 x 14 ([32,112,112,32] 17.8 and 18.7 with 8 x 8).
+        const int64_t tiles8 = g.N * ((g.Wo + 7) / 8) * ((g.Ho + 7) / 8);
+        const bool beyond_l2 = (double)g.N * g.H * g.W * g.C * 8.0 > 1.5e8;  // both tensors
+        if (g.sh == 1 && g.C % 64 == 0) v = tiles8 * (g.C / 64) < ctx->sm_count || (g.C <= 128 && beyond_l2) ? 1 : 6;
+        else if (g.sh == 1) v = g.Wo <= 8 || tiles8 * ((g.C + DW_CB - 1) / DW_CB) <= 24 * (int64_t)ctx->sm_count ? 1 : 0;
+        // stride 2: 64-channel tiles are 8 outputs wide, so they are taken only where that wastes fewer columns than the
+        // 16-wide 32-channel ones ([128,112,112,64] 90.1 -> 86.9 us; [128,28,28,256] ran 27.3 -> 29.1 with them)
+        else if (g.C % 64 == 0 && wide8) v = 7;
+        else v = g.Wo <= 8 ? 3 : 2;
     }
     const DwVariant& d = kDwVariants[v];
     const cuuint64_t eb = narrow ? 2u : 4u;

@@ -151,3 +151,14 @@ def test_depthwise_shifted_delta_taps_on_gpu(ctx):
                         iy, ix = oy * stride - before + ky, ox * stride - before + kx
                         want = x[0, iy, ix] if (0 <= iy < size and 0 <= ix < size) else np.zeros(C, np.float32)
                         assert np.array_equal(y[0, oy, ox], want)
+
+
+@pytest.mark.parametrize("case", [(1, 14, 14, 128), (2, 9, 8, 64), (3, 17, 33, 64), (18, 17, 17, 128), (1, 8, 40, 96), (1, 7, 7, 192), (40, 74, 70, 32)])
+def test_depthwise_3x3_tiles(ctx, oracle, case):
+    """Stride 1: 8 x 8 tiles of 32 channels and of 64, and 16 x 14 of 32, which the number of tiles chooses between, with rows
+    and columns left over."""
+    N, H, W, C = case
+    x, f, b = si.uniform(341, 0, (N, H, W, C), 0, 6), si.normal(341, 1, (3, 3, C, 1), 0, 0.5), si.normal(341, 2, (C,), 0, 0.1)
+    got = host(ctx.depthwise_conv2d(dev(x), dev(f), (1, 1), "same", bias=dev(b), act="relu6"))
+    ctx.check_device_status()
+    assert rel_fro(got, oracle.depthwise_conv2d(x, f, (1, 1), "same", bias=b, act="relu6")) <= 1e-6
