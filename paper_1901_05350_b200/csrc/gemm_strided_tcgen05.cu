@@ -43,6 +43,7 @@ struct Side {
     const float* ptr;
     int row_stride, k_stride;
     int rows;
+    int quads;  // K-contiguous, and every row starts on 16 bytes: four k per load
     long long batch_stride;
 };
 
@@ -66,23 +67,46 @@ struct Fetch {
     // Rows past the last are read as the last one: their results are not stored.  k past K must be zero.
     __device__ __forceinline__ void load(const Side& s, const float* base, int r0, int k0, int K, int w, int lane) {
         const int last = s.rows - 1;
-        if (s.k_stride == 1) {  // lane = k, row w + 8 i
+        if (s.quads) {                 // lane = 4 k of one of four rows, row 32 i + 4 w + lane / 8
+            const bool ok = k0 + 4 * (lane & 7) < K;  // K % 4 == 0
+            const float* at = base + k0 + 4 * (lane & 7);
+#pragma unroll
+            for (int i = 0; i < ROWS / 32; ++i) {
+                float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (ok) q = __ldg(reinterpret_cast<const float4*>(at + (long long)min(r0 + 32 * i + 4 * w + (lane >> 3), last) * s.row_stride));
+                v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
+            }
+        } else if (s.k_stride == 1) {  // lane = k, row w + 8 i
             const bool ok = k0 + lane < K;
             const float* at = base + k0 + lane;
 #pragma unroll
-            for (int i = 0; i < ROWS / 8; ++i) v[i] = ok ? load_global(at + (long long)min(r0 + w + 8 * i, last) * s.row_stride) : 0.f;
+            for (int i = 0; i < ROWS / 8; ++i) v[i] = ok ? __ldg(at + (long long)min(r0 + w + 8 * i, last) * s.row_stride) : 0.f;
         } else {                // lane = row of block i, k = 4 w + e; rows are contiguous
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int k = k0 + 4 * w + e;
                 const float* at = base + (long long)k * s.k_stride;
 #pragma unroll
-                for (int i = 0; i < ROWS / 32; ++i) v[4 * i + e] = k < K ? load_global(at + min(r0 + 32 * i + lane, last)) : 0.f;
+                for (int i = 0; i < ROWS / 32; ++i) v[4 * i + e] = k < K ? __ldg(at + min(r0 + 32 * i + lane, last)) : 0.f;
             }
         }
     }
-    __device__ __forceinline__ void store(bool k_contiguous, uint32_t tile, uint32_t lo_offset, int w, int lane) const {
-        if (k_contiguous) {
+    // four k of one row in every 32
+    __device__ __forceinline__ void store_quads(uint32_t at, uint32_t lo_offset) const {
+#pragma unroll
+        for (int i = 0; i < ROWS / 32; ++i) {
+            float hi[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) tf32_split(v[4 * i + e], hi[e], lo[e]);
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + (uint32_t)i * 4096u), "f"(hi[0]), "f"(hi[1]), "f"(hi[2]), "f"(hi[3]) : "memory");
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + lo_offset + (uint32_t)i * 4096u), "f"(lo[0]), "f"(lo[1]), "f"(lo[2]), "f"(lo[3]) : "memory");
+        }
+    }
+    __device__ __forceinline__ void store(const Side& s, uint32_t tile, uint32_t lo_offset, int w, int lane) const {
+        if (s.quads) {
+            const int row = 4 * w + (lane >> 3);
+            store_quads(tile + (uint32_t)(row * 128 + (((lane ^ row) & 7) << 4)), lo_offset);
+        } else if (s.k_stride == 1) {
             const uint32_t at = tile + (uint32_t)(w * 128 + (((lane >> 2) ^ w) << 4) + (lane & 3) * 4);
 #pragma unroll
             for (int i = 0; i < ROWS / 8; ++i) {
@@ -92,15 +116,7 @@ struct Fetch {
                 asm volatile("st.shared.f32 [%0], %1;" ::"r"(at + lo_offset + (uint32_t)i * 1024u), "f"(lo) : "memory");
             }
         } else {
-            const uint32_t at = tile + (uint32_t)(lane * 128 + ((w ^ (lane & 7)) << 4));
-#pragma unroll
-            for (int i = 0; i < ROWS / 32; ++i) {
-                float hi[4], lo[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) tf32_split(v[4 * i + e], hi[e], lo[e]);
-                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + (uint32_t)i * 4096u), "f"(hi[0]), "f"(hi[1]), "f"(hi[2]), "f"(hi[3]) : "memory");
-                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + lo_offset + (uint32_t)i * 4096u), "f"(lo[0]), "f"(lo[1]), "f"(lo[2]), "f"(lo[3]) : "memory");
-            }
+            store_quads(tile + (uint32_t)(lane * 128 + ((w ^ (lane & 7)) << 4)), lo_offset);
         }
     }
 };
@@ -108,7 +124,7 @@ struct Fetch {
 // One element over k0 .. k1 by fp32 multiply-adds.
 __device__ __noinline__ float sum_in_fp32(const float* p, const float* q, int p_step, int q_step, int k0, int k1) {
     float acc = 0.f;
-    for (int k = k0; k < k1 && acc == acc; ++k) acc = fmaf(load_global(p + (long long)k * p_step), load_global(q + (long long)k * q_step), acc);
+    for (int k = k0; k < k1 && acc == acc; ++k) acc = fmaf(__ldg(p + (long long)k * p_step), load_global(q + (long long)k * q_step), acc);
     return acc;
 }
 
@@ -206,7 +222,6 @@ gemm_strided_kernel(const StridedArgs g) {
         const int w = warp - 1;
         const float* pb = g.p.ptr + batch * g.p.batch_stride;
         const float* qb = g.q.ptr + batch * g.q.batch_stride;
-        const bool p_k = g.p.k_stride == 1, q_k = g.q.k_stride == 1;
         bool ok = true;
         Fetch<BLOCK_M> fp;
         Fetch<BN> fq;
@@ -229,8 +244,8 @@ gemm_strided_kernel(const StridedArgs g) {
             const bool got = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag);
             if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
             const uint32_t hi = base + (uint32_t)(stage * STAGE_BYTES);
-            fp.store(p_k, hi, OPERANDS, w, lane);
-            fq.store(q_k, hi + A_STAGE_BYTES, OPERANDS, w, lane);
+            fp.store(g.p, hi, OPERANDS, w, lane);
+            fq.store(g.q, hi + A_STAGE_BYTES, OPERANDS, w, lane);
             if (kb == add_at) {  // before the next values are fetched: it wants their registers
                 add(false);
                 add_at += g.segment;
@@ -300,7 +315,7 @@ gemm_strided_kernel(const StridedArgs g) {
         const uint32_t at_step = (uint32_t)((row_step * PITCH + col_step) * 4);
         // the bias is either one value per thread or walked along
         const bool one_bias = g.bias != nullptr && along_p == (g.bias_p != 0);
-        const float b0 = one_bias && live ? load_global(g.bias + (along_p ? p : q)) : 0.f;
+        const float b0 = one_bias && live ? __ldg(g.bias + (along_p ? p : q)) : 0.f;
         const float* bias = g.bias != nullptr && !one_bias ? g.bias + (along_p ? q0 : p0 + r0) : nullptr;
 #pragma unroll 4
         for (int i = along_p ? col : row; i < (live ? limit : 0); i += step, at += at_step, out += out_step) {
@@ -317,7 +332,7 @@ gemm_strided_kernel(const StridedArgs g) {
                 for (int s = 1; s < GS_MAX_CLUSTER; ++s)
                     if (s < g.splits) v += part[s];
             }
-            if (g.bias) v += bias ? load_global(bias + i) : b0;
+            if (g.bias) v += bias ? __ldg(bias + i) : b0;
             *out = apply_act(v, g.act);
         }
     }
@@ -435,7 +450,10 @@ cudaError_t launch_gemm_strided(const float* a, int64_t a_rs, int64_t a_ks, cons
                                 unsigned int* dev_status, cudaStream_t s, int64_t* launches) {
     if (M == 0 || N == 0 || batches == 0) return cudaSuccess;
     const Choice ch = choose(batches, M, N, K, sm_count);
-    const Side sa{a, (int)a_rs, (int)a_ks, (int)M, M * K}, sb{b, (int)b_cs, (int)b_ks, (int)N, K * N};
+    const bool aligned = K % 4 == 0 && (batches == 1 || (M * K % 4 == 0 && K * N % 4 == 0));
+    const bool a_quads = aligned && a_ks == 1 && a_rs % 4 == 0 && (reinterpret_cast<uintptr_t>(a) & 15u) == 0;
+    const bool b_quads = aligned && b_ks == 1 && b_cs % 4 == 0 && (reinterpret_cast<uintptr_t>(b) & 15u) == 0;
+    const Side sa{a, (int)a_rs, (int)a_ks, (int)M, a_quads, M * K}, sb{b, (int)b_cs, (int)b_ks, (int)N, b_quads, K * N};
     StridedArgs g{};
     g.p = ch.swap ? sb : sa;
     g.q = ch.swap ? sa : sb;
