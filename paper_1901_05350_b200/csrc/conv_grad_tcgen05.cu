@@ -24,13 +24,12 @@
 // lane and not an elected thread of a converged warp issued the MMAs).
 //
 // Filter gradient, conv2d_grad_filter_kernel.  df[(tap, ci), co] = sum over pixels: the summed index is the row of
-// both x and dy, so both landed tiles ([32 pixels][32 channels] groups: im2col or matrix boxes) are transposed into
-// operand tiles by the eight converter warps: 4x4 blocks through registers, on diagonals of the group so that the
-// 16-byte reads and writes are both free of bank conflicts under the 128-byte swizzle.  M = four (tap, 32-channel)
+// both x and dy, so a landed group ([32 pixels][32 channels]: an im2col or matrix box, with the swizzle of 32-byte pieces) is
+// an MN-major operand as it is, and its halves are elementwise functions of it.  hi is rounded here, in place: left as copied,
+// cut, it is 2.7e-7 off where rounded it is 2.2e-7 ([16,28,28,128], 3x3; 33.6 us).  M = four (tap, 32-channel)
 // groups, N = 32..128 channels of dy, one (M tile, N tile, slice of the pixels) per CTA, partial sums added in slice
-// order.  Bound by shared-memory bandwidth (about 1800 cycles per k-block with the lo half, 1000 without, against 768 /
-// 256 of MMAs).  [16,28,28,128], 3x3: 811 us with 32 x 32 tiles on CUDA cores, 40 us here (38 with one accumulator).
-// Pointwise, plain TF32, [32,56,56] 128 x 128: 36 + 36 us of transposes and 23 + 8 us of batched products, 25 + 6 us here.
+// order.  Per k-block at block_n 128, 32 KB landed, read and split and 96 KB read by the MMAs: 1500 cycles of shared memory
+// (768 of MMAs); without the lo half a copy and 256 cycles of MMAs.
 #include <algorithm>
 #include <cstdlib>
 
@@ -395,7 +394,7 @@ struct GradFilterArgs {
     int taps, fw, sh, sw, dh, dw, pt, pl, Ho, Wo;
     int c_blocks;   // 32-channel blocks of x
     int groups;     // taps * c_blocks
-    int n_tiles, block_n, raw_stages, op_stages;
+    int n_tiles, block_n, stages;
     int pixel_blocks, blocks_per_slice;  // blocks of 32 pixels
     int m_tiles;
     int segment;    // k-blocks per accumulator of the large products
@@ -424,19 +423,18 @@ __global__ void __launch_bounds__(CG_THREADS, 1)
 conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_dy,
                           const __grid_constant__ CUtensorMap map_out, const __grid_constant__ GradFilterArgs g) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bar_raw_full[CG_MAX_STAGES], bar_raw_empty[CG_MAX_STAGES];
-    __shared__ __align__(8) uint64_t bar_op_full[CG_MAX_STAGES], bar_op_empty[CG_MAX_STAGES];
+    __shared__ __align__(8) uint64_t bar_full[CG_MAX_STAGES], bar_split[CG_MAX_STAGES], bar_empty[CG_MAX_STAGES];
     __shared__ __align__(8) uint64_t bar_acc_full[2], bar_acc_empty[2], bar_drain;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag_s;
     volatile int* abort_flag = &abort_flag_s;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b_groups = g.block_n >> 5;
-    const int raw_bytes = (4 + b_groups) * GROUP_BYTES;  // A groups, then B groups; an operand stage has the same size
-    const uint32_t epi_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t raw_base = epi_base + EPI_WARPS * EPI_SLAB_BYTES;
-    const uint32_t op_base = raw_base + (uint32_t)(g.raw_stages * raw_bytes);
+    const int raw_bytes = (4 + b_groups) * GROUP_BYTES;  // A groups, then B groups; SPLIT: their lo halves behind them
     constexpr int HALVES = SPLIT ? 2 : 1;
+    const uint32_t epi_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t stage_base = epi_base + EPI_WARPS * EPI_SLAB_BYTES;
+    auto stage_addr = [&](int s) { return stage_base + (uint32_t)(s * HALVES * raw_bytes); };
 
     int unit = blockIdx.x;
     const int nt = unit % g.n_tiles;
@@ -447,13 +445,10 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
     const int kbs = max(0, min(g.blocks_per_slice, g.pixel_blocks - pb0));  // never zero: the host makes no empty slice
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < g.raw_stages; ++s) {
-            mbar_init(smem_u32(&bar_raw_full[s]), 1);
-            mbar_init(smem_u32(&bar_raw_empty[s]), CVT_WARPS);
-        }
-        for (int s = 0; s < g.op_stages; ++s) {
-            mbar_init(smem_u32(&bar_op_full[s]), CVT_WARPS);
-            mbar_init(smem_u32(&bar_op_empty[s]), 1);
+        for (int s = 0; s < g.stages; ++s) {
+            mbar_init(smem_u32(&bar_full[s]), 1);
+            mbar_init(smem_u32(&bar_split[s]), CVT_WARPS);
+            mbar_init(smem_u32(&bar_empty[s]), 1);
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&bar_acc_full[s]), 1);
@@ -487,8 +482,8 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
             uint32_t phase = 0;
             bool ok = true;
             for (int kb = 0; kb < kbs; ++kb) {
-                if (!bounded_wait(smem_u32(&bar_raw_empty[stage]), phase ^ 1u, abort_flag)) { ok = false; break; }
-                const uint32_t full = smem_u32(&bar_raw_full[stage]), dst = raw_base + (uint32_t)(stage * raw_bytes);
+                if (!bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag)) { ok = false; break; }
+                const uint32_t full = smem_u32(&bar_full[stage]), dst = stage_addr(stage);
                 const int p0 = (pb0 + kb) * 32;
                 mbar_arrive_expect_tx(full, (uint32_t)((live_groups + b_groups) * GROUP_BYTES));
                 const int row = p0 / g.Wo, img = row / g.Ho;
@@ -501,16 +496,16 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
                 }
                 for (int i = 0; i < b_groups; ++i) tma_load_2d(dst + (4 + i) * GROUP_BYTES, &map_dy, full, n0 + i * 32, p0);
                 ++filled;
-                if (++stage == g.raw_stages) { stage = 0; phase ^= 1u; }
+                if (++stage == g.stages) { stage = 0; phase ^= 1u; }
             }
             if (!ok) {
                 give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
-                for (int k = filled > g.raw_stages ? filled - g.raw_stages : 0; k < filled; ++k)
-                    drain(smem_u32(&bar_raw_full[k % g.raw_stages]), (uint32_t)((k / g.raw_stages) & 1), g.dev_status);
+                for (int k = filled > g.stages ? filled - g.stages : 0; k < filled; ++k)
+                    drain(smem_u32(&bar_full[k % g.stages]), (uint32_t)((k / g.stages) & 1), g.dev_status);
             }
         }
     } else if (warp == 1) {
-        const uint32_t idesc = make_idesc_tf32(BLOCK_M, g.block_n);
+        const uint32_t idesc = make_idesc_tf32(BLOCK_M, g.block_n) | IDESC_A_MN | IDESC_B_MN;
         const uint32_t small = tmem + (uint32_t)(2 * g.block_n);
         int stage = 0, acc = 0, in_seg = 0;
         uint32_t phase = 0, acc_phase = 0;
@@ -519,24 +514,30 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
         for (int kb = 0; kb < kbs; ++kb) {
             if (SPLIT && in_seg == 0 && leader && ok) ok = bounded_wait(smem_u32(&bar_acc_empty[acc]), acc_phase ^ 1u, abort_flag);
             const uint32_t large = tmem + (uint32_t)(acc * g.block_n);
-            const uint32_t hi = op_base + (uint32_t)(stage * HALVES * raw_bytes), lo = hi + (uint32_t)raw_bytes;
-            const uint64_t ah = make_kmajor_sw128_desc(hi), bh = make_kmajor_sw128_desc(hi + A_STAGE_BYTES);
-            const uint64_t al = make_kmajor_sw128_desc(lo), bl = make_kmajor_sw128_desc(lo + A_STAGE_BYTES);
-            if (leader && ok && (ok = bounded_wait(smem_u32(&bar_op_full[stage]), phase, abort_flag))) {
+            const uint32_t hi = stage_addr(stage), lo = hi + (uint32_t)raw_bytes;
+            uint64_t ah[4], bh[4], al[4], bl[4];  // eight pixels per MMA
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                ah[k] = make_mnmajor_desc(hi) + (uint64_t)(64 * k);
+                bh[k] = make_mnmajor_desc(hi + A_STAGE_BYTES) + (uint64_t)(64 * k);
+                al[k] = make_mnmajor_desc(lo) + (uint64_t)(64 * k);
+                bl[k] = make_mnmajor_desc(lo + A_STAGE_BYTES) + (uint64_t)(64 * k);
+            }
+            if (leader && ok && (ok = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag) &&
+                                      (!SPLIT || bounded_wait(smem_u32(&bar_split[stage]), phase, abort_flag)))) {
                 tc_fence_after();
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const uint64_t o = (uint64_t)(2 * k);
-                    tc_mma_tf32(large, ah + o, bh + o, idesc, ((SPLIT ? in_seg : kb) | k) != 0 ? 1u : 0u);
+                    tc_mma_tf32(large, ah[k], bh[k], idesc, ((SPLIT ? in_seg : kb) | k) != 0 ? 1u : 0u);
                     if (SPLIT) {
-                        tc_mma_tf32(small, ah + o, bl + o, idesc, (kb | k) != 0 ? 1u : 0u);
-                        tc_mma_tf32(small, al + o, bh + o, idesc, 1u);
+                        tc_mma_tf32(small, ah[k], bl[k], idesc, (kb | k) != 0 ? 1u : 0u);
+                        tc_mma_tf32(small, al[k], bh[k], idesc, 1u);
                     }
                 }
                 issued = true;
-                tc_commit(smem_u32(&bar_op_empty[stage]));
+                tc_commit(smem_u32(&bar_empty[stage]));
             }
-            if (++stage == g.op_stages) { stage = 0; phase ^= 1u; }
+            if (++stage == g.stages) { stage = 0; phase ^= 1u; }
             if (kb + 1 == kbs || (SPLIT && ++in_seg == g.segment)) {
                 if (leader && ok) tc_commit(smem_u32(&bar_acc_full[acc]));
                 in_seg = 0;
@@ -599,55 +600,33 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
             if (lane == 0) tma_store_wait_all();
             __syncwarp();
         }
-    } else {
-        const int w = warp - 2 - EPI_WARPS;
-        const int l = lane & 7, sub = lane >> 3;
-        int rs = 0, os = 0;
-        uint32_t rphase = 0, ophase = 0;
+    } else if (SPLIT) {
+        const uint32_t mine = (uint32_t)(threadIdx.x - (2 + EPI_WARPS) * 32) * 16u;
+        int stage = 0;
+        uint32_t phase = 0;
         for (int kb = 0; kb < kbs; ++kb) {
-            const bool got = bounded_wait(smem_u32(&bar_raw_full[rs]), rphase, abort_flag) &&
-                             bounded_wait(smem_u32(&bar_op_empty[os]), ophase ^ 1u, abort_flag);
+            const bool got = bounded_wait(smem_u32(&bar_full[stage]), phase, abort_flag);
             if (!__all_sync(0xffffffffu, got)) {
                 if (lane == 0) give_up(abort_flag, g.dev_status, DEV_STATUS_TIMEOUT_PRODUCER);
                 break;
             }
-            const uint32_t raw = raw_base + (uint32_t)(rs * raw_bytes), hi = op_base + (uint32_t)(os * HALVES * raw_bytes);
-            for (int step = w; step < 2 * (4 + b_groups); step += CVT_WARPS) {
-                const int grp = step >> 1;
-                if (grp >= live_groups && grp < 4) continue;  // rows that nothing reads
-                // eight lanes: pixel quad l and channel quad l ^ base, so that neither the reads (slot q ^ pixel % 8) nor
-                // the writes (slot l ^ channel % 8) of the eight meet in a bank
-                const int q = l ^ ((step & 1) * 4 + sub);
-                float4 v[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int px = 4 * l + i;
-                    v[i] = lds4(raw + (uint32_t)(grp * GROUP_BYTES + px * 128 + ((q ^ (px & 7)) << 4)));
-                }
-                const float* f = reinterpret_cast<const float*>(v);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int row = 4 * q + e;
-                    const uint32_t at = (uint32_t)(grp * GROUP_BYTES + row * 128 + ((l ^ (row & 7)) << 4));
-                    if (SPLIT) {
-                        float large[4], small[4];
-#pragma unroll
-                        for (int p = 0; p < 4; ++p) tf32_split(f[4 * p + e], large[p], small[p]);
-                        sts4(hi + at, large[0], large[1], large[2], large[3]);
-                        sts4(hi + (uint32_t)raw_bytes + at, small[0], small[1], small[2], small[3]);
-                    } else {
-                        sts4(hi + at, f[e], f[4 + e], f[8 + e], f[12 + e]);
-                    }
-                }
+            const uint32_t src = stage_addr(stage) + mine, dst = src + (uint32_t)raw_bytes;
+            // 256 threads x 16 bytes: a group of 32 pixels x 32 channels per step
+#pragma unroll 4
+            for (int o = 0; o < raw_bytes; o += CVT_WARPS * 512) {
+                const float4 v = lds4(src + (uint32_t)o);
+                float hi[4], lo[4];
+                tf32_split(v.x, hi[0], lo[0]);
+                tf32_split(v.y, hi[1], lo[1]);
+                tf32_split(v.z, hi[2], lo[2]);
+                tf32_split(v.w, hi[3], lo[3]);
+                sts4(src + (uint32_t)o, hi[0], hi[1], hi[2], hi[3]);
+                sts4(dst + (uint32_t)o, lo[0], lo[1], lo[2], lo[3]);
             }
             fence_async_smem();
             __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(smem_u32(&bar_raw_empty[rs]));
-                mbar_arrive(smem_u32(&bar_op_full[os]));
-            }
-            if (++rs == g.raw_stages) { rs = 0; rphase ^= 1u; }
-            if (++os == g.op_stages) { os = 0; ophase ^= 1u; }
+            if (lane == 0) mbar_arrive(smem_u32(&bar_split[stage]));
+            if (++stage == g.stages) { stage = 0; phase ^= 1u; }
         }
     }
     tc_fence_before();
@@ -660,7 +639,8 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
 
 constexpr int CG_SMEM = SMEM_LIMIT - 1024;  // beside the barriers
 
-tfjsb_status encode(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int rank, const int64_t* dims, const uint32_t* box, const char* what) {
+tfjsb_status encode(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int rank, const int64_t* dims, const uint32_t* box, const char* what,
+                    CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
     cuuint64_t d[3], st[2];
     cuuint32_t b[3], elem[3] = {1u, 1u, 1u};
     cuuint64_t pitch = 4;
@@ -671,19 +651,19 @@ tfjsb_status encode(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int ran
         if (i + 1 < rank) st[i] = pitch;
     }
     CUresult r = ctx->encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), d, st, b, elem,
-                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(ctx, TFJSB_ERR_CUDA, std::string("cuTensorMapEncodeTiled failed for ") + what + " (CUresult " + std::to_string((int)r) + ")");
     return TFJSB_OK;
 }
 
 tfjsb_status encode_im2col(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int64_t n, int h, int w, int c, const int lower[2],
-                           const int upper[2], int sw, int sh, int pixels, const char* what) {
+                           const int upper[2], int sw, int sh, int pixels, const char* what, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
     cuuint64_t d[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
     cuuint64_t st[3] = {(cuuint64_t)c * 4, (cuuint64_t)w * c * 4, (cuuint64_t)h * w * c * 4};
     cuuint32_t elem[4] = {1u, (cuuint32_t)sw, (cuuint32_t)sh, 1u};
     CUresult r = ctx->encode_im2col(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(base), d, st, lower, upper, 32,
-                                    (cuuint32_t)pixels, elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                    (cuuint32_t)pixels, elem, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(ctx, TFJSB_ERR_CUDA, std::string("cuTensorMapEncodeIm2col failed for ") + what + " (CUresult " + std::to_string((int)r) + ")");
     return TFJSB_OK;
@@ -858,9 +838,8 @@ tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float*
     slices = (a.pixel_blocks + a.blocks_per_slice - 1) / a.blocks_per_slice;
     a.segment = split_segment((int64_t)a.blocks_per_slice * 32);
     const int raw_bytes = (4 + a.block_n / 32) * GROUP_BYTES, halves = split ? 2 : 1;
-    a.op_stages = split ? 2 : 3;
-    a.raw_stages = (CG_SMEM - 1024 - EPI_WARPS * EPI_SLAB_BYTES - a.op_stages * halves * raw_bytes) / raw_bytes;
-    if (a.raw_stages > CG_MAX_STAGES) a.raw_stages = CG_MAX_STAGES;
+    a.stages = (CG_SMEM - 1024 - EPI_WARPS * EPI_SLAB_BYTES) / (halves * raw_bytes);
+    if (a.stages > CG_MAX_STAGES) a.stages = CG_MAX_STAGES;
     tfjsb_status st;
     float* out = df;
     if (slices > 1) {
@@ -871,20 +850,20 @@ tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float*
     const uint32_t box[3] = {32u, 32u, 1u};
     if (a.tiled) {
         const int64_t d[2] = {g.C, pixels};
-        if ((st = encode(ctx, &map_x, x, 2, d, box, "x")) != TFJSB_OK) return st;
+        if ((st = encode(ctx, &map_x, x, 2, d, box, "x", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) != TFJSB_OK) return st;
     } else {
         const int lower[2] = {-g.pl, -g.pt};
         const int upper[2] = {(g.Wo - 1) * g.sw - g.pl - (g.W - 1), (g.Ho - 1) * g.sh - g.pt - (g.H - 1)};
-        if ((st = encode_im2col(ctx, &map_x, x, g.N, g.H, g.W, g.C, lower, upper, g.sw, g.sh, 32, "x")) != TFJSB_OK) return st;
+        if ((st = encode_im2col(ctx, &map_x, x, g.N, g.H, g.W, g.C, lower, upper, g.sw, g.sh, 32, "x", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) != TFJSB_OK) return st;
     }
     const int64_t dd[2] = {g.Co, pixels}, od[3] = {g.Co, g.C, slices * a.taps};
-    if ((st = encode(ctx, &map_dy, dy, 2, dd, box, "dy")) != TFJSB_OK) return st;
+    if ((st = encode(ctx, &map_dy, dy, 2, dd, box, "dy", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) != TFJSB_OK) return st;
     if ((st = encode(ctx, &map_out, out, 3, od, box, "the filter gradient")) != TFJSB_OK) return st;
     auto kernel = split ? conv2d_grad_filter_kernel<true> : conv2d_grad_filter_kernel<false>;
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kernel), CG_SMEM);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "shared-memory limit");
-    const size_t smem = 1024 + (size_t)EPI_WARPS * EPI_SLAB_BYTES + (size_t)(a.raw_stages + a.op_stages * halves) * raw_bytes;
-    if ((e = launch_k(kernel, dim3((unsigned)(units * slices)), dim3(CG_THREADS), smem, s, map_x, map_dy, map_out, a)) != cudaSuccess)
+    const size_t smem = 1024 + (size_t)EPI_WARPS * EPI_SLAB_BYTES + (size_t)a.stages * halves * raw_bytes;
+    if ((e = launch_k(kernel, dim3((unsigned)(units * slices)), dim3(split ? CG_THREADS : CG_THREADS - CVT_WARPS * 32), smem, s, map_x, map_dy, map_out, a)) != cudaSuccess)
         return cuda_fail(ctx, e, "conv2d_grad_filter launch");
     ++ctx->launches;
     if (slices > 1 && (e = launch_sum_rows(out, df, nullptr, slices, elems, 1, s, &ctx->launches)) != cudaSuccess)
