@@ -60,14 +60,14 @@ struct StridedArgs {
 };
 
 // What one loader thread fetches of a k-block of ROWS rows, and where it stores it.
-template <int ROWS>
+template <int ROWS, bool QUADS>
 struct Fetch {
     float v[ROWS / 8];
 
     // Rows past the last are read as the last one: their results are not stored.  k past K must be zero.
     __device__ __forceinline__ void load(const Side& s, const float* base, int r0, int k0, int K, int w, int lane) {
         const int last = s.rows - 1;
-        if (s.quads) {                 // lane = 4 k of one of four rows, row 32 i + 4 w + lane / 8
+        if (QUADS && s.quads) {        // lane = 4 k of one of four rows, row 32 i + 4 w + lane / 8
             const bool ok = k0 + 4 * (lane & 7) < K;  // K % 4 == 0
             const float* at = base + k0 + 4 * (lane & 7);
 #pragma unroll
@@ -103,7 +103,7 @@ struct Fetch {
         }
     }
     __device__ __forceinline__ void store(const Side& s, uint32_t tile, uint32_t lo_offset, int w, int lane) const {
-        if (s.quads) {
+        if (QUADS && s.quads) {
             const int row = 4 * w + (lane >> 3);
             store_quads(tile + (uint32_t)(row * 128 + (((lane ^ row) & 7) << 4)), lo_offset);
         } else if (s.k_stride == 1) {
@@ -128,7 +128,8 @@ __device__ __noinline__ float sum_in_fp32(const float* p, const float* q, int p_
     return acc;
 }
 
-template <int BN>
+// QUADS: an operand has rows of whole quads (an instance of its own: the code for them cost the others 7 %)
+template <int BN, bool QUADS>
 __global__ void __launch_bounds__(GS_THREADS, 2)
 gemm_strided_kernel(const StridedArgs g) {
     constexpr int OPERANDS = A_STAGE_BYTES + BN * 128;  // hi (or lo) of one stage
@@ -223,8 +224,8 @@ gemm_strided_kernel(const StridedArgs g) {
         const float* pb = g.p.ptr + batch * g.p.batch_stride;
         const float* qb = g.q.ptr + batch * g.q.batch_stride;
         bool ok = true;
-        Fetch<BLOCK_M> fp;
-        Fetch<BN> fq;
+        Fetch<BLOCK_M, QUADS> fp;
+        Fetch<BN, QUADS> fq;
         fp.load(g.p, pb, p0, kb0 * BLOCK_K, g.K, w, lane);
         fq.load(g.q, qb, q0, kb0 * BLOCK_K, g.K, w, lane);
         // the sum: the two warps of a lane quadrant take 32 columns each
@@ -350,7 +351,7 @@ gemm_strided_kernel(const StridedArgs g) {
 
 template <int BN>
 cudaError_t launch_instance(StridedArgs a, int64_t tiles, cudaStream_t s) {
-    auto kernel = gemm_strided_kernel<BN>;
+    auto kernel = a.p.quads || a.q.quads ? gemm_strided_kernel<BN, true> : gemm_strided_kernel<BN, false>;
     constexpr int STAGE_BYTES = (A_STAGE_BYTES + BN * 128) * 2;
     constexpr int LIMIT = 110 * 1024;  // two CTAs per SM
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kernel), LIMIT);
