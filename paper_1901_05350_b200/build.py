@@ -37,6 +37,7 @@ SOURCES = [
     "backprop.cu",
     "depthwise_grad.cu",
     "conv_grad_tcgen05.cu",
+    "conv_patch_tcgen05.cu",
     "gemm_strided_tcgen05.cu",
     "chain_cluster.cu",
 ]

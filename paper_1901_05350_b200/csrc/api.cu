@@ -476,6 +476,8 @@ tfjsb_status tfjsb_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_ten
         return TFJSB_OK;
     }
     if (ctx->math == TFJSB_MATH_TF32 && conv_igemm_supported(g) && ctx->encode_tiled) {
+        if (!conv_patch_supported(g) && conv_patch_input_preferred(g, ctx->sm_count))
+            return run_conv_patch_input(ctx, px, pf, pbias, act, py, g, s);
         // implicit GEMM on the tensor cores: the filter is packed [Cout, k_pad] into scratch first
         g.gather_only = scratch_is_short(ctx->scratch_b, (size_t)Cout * conv_igemm_k_pad(g) * 4, s);
         const int64_t k_pad = conv_igemm_k_pad(g);
@@ -687,6 +689,8 @@ tfjsb_status tfjsb_conv2d_backprop_input(tfjsb_ctx* ctx, const tfjsb_tensor* dy,
         return e == cudaSuccess ? TFJSB_OK : cuda_fail(ctx, e, "cudaMemsetAsync");
     }
     const bool pointwise = g.fh == 1 && g.fw == 1 && g.sh == 1 && g.sw == 1;
+    if (ctx->math == TFJSB_MATH_TF32 && ctx->encode_tiled && conv_patch_gradient_preferred(g, ctx->sm_count))
+        return run_conv_patch_gradient(ctx, pg, pf, pdx, g, s);
     if (ctx->math == TFJSB_MATH_TF32 && ctx->encode_tiled && conv2d_grad_input_supported(g) &&
         (pointwise ? !gemm_tf32_supported(g.N * g.H * g.W, g.C, g.Co) : conv2d_grad_input_preferred(g, ctx->sm_count)))
         return run_conv2d_grad_input(ctx, pg, pf, pdx, g, s);

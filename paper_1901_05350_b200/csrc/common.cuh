@@ -393,6 +393,12 @@ bool conv2d_grad_input_preferred(const ConvGeom& g, int sm_count);  // to the CU
 tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float* f, float* dx, const ConvGeom& g, cudaStream_t s);
 bool conv2d_grad_filter_supported(const ConvGeom& g);
 tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float* dy, float* df, const ConvGeom& g, bool split, cudaStream_t s);
+// conv2d 3x3 with stride 1 from input patches (conv_patch_tcgen05.cu): the forward pass with TF32 operands, f as it is stored,
+// and the input gradient with fp32 accuracy; `g` is the forward geometry of both.
+bool conv_patch_input_preferred(const ConvGeom& g, int sm_count);
+tfjsb_status run_conv_patch_input(tfjsb_ctx* ctx, const float* x, const float* f, const float* bias, int act, float* y, const ConvGeom& g, cudaStream_t s);
+bool conv_patch_gradient_preferred(const ConvGeom& g, int sm_count);
+tfjsb_status run_conv_patch_gradient(tfjsb_ctx* ctx, const float* dy, const float* f, float* dx, const ConvGeom& g, cudaStream_t s);
 // Pipelined filter gradient of the 3x3 depthwise convolution (depthwise_grad.cu); depthwise_grad_plan says whether the
 // shape is one of its own.  `partial` holds slices * 9 * C floats (unused when slices == 1).
 struct DepthwiseGradPlan {

@@ -432,3 +432,48 @@ def test_fused_depthwise_pointwise_block(ctx, oracle, monkeypatch, case):
     assert same_bits(host(model.run(dev(xi))), oracle.run_model(layers, xi))
     ctx.check_device_status()
     model.close()
+
+
+# N, H, W, Cin, Cout, pad: 3x3, stride 1, A tiles from patches of 16 x 8 output pixels
+PATCH_CASES = [
+    (1, 16, 8, 32, 32, "same"),      # one whole tile, one channel block
+    (1, 5, 3, 16, 4, "same"),        # smaller than a tile, half a channel block
+    (2, 17, 9, 36, 68, "same"),      # one row and one column more than a tile; ragged channels
+    (1, 33, 24, 64, 64, "valid"),    # no padding; the filter stays in shared memory
+    (1, 20, 20, 40, 300, "same"),    # several column tiles
+    (3, 14, 14, 128, 256, "same"),   # filter tiles through a ring
+    (40, 9, 9, 64, 64, "same"),      # several tiles per CTA
+    (2, 40, 70, 32, 96, "same"),     # an odd number of 32-column chunks per tile
+]
+
+
+@pytest.mark.parametrize("case", PATCH_CASES)
+def test_conv2d_from_patches(ctx, oracle, monkeypatch, case):
+    N, H, W, Cin, Cout, pad = case
+    fh = fw = 3
+    d = 1
+    monkeypatch.setenv("TFJSB_CONV_PATCH", "1")
+    x, f, b = si.small_integers(331, 0, (N, H, W, Cin), -3, 3), si.small_integers(331, 1, (fh, fw, Cin, Cout), -3, 3), si.small_integers(331, 2, (Cout,), -9, 9)
+    for act in ("none", "relu6"):
+        got = host(ctx.conv2d(dev(x), dev(f), (1, 1), pad, (d, d), bias=dev(b), act=act))
+        ctx.check_device_status()
+        assert same_bits(got + 0.0, oracle.conv2d(x, f, (1, 1), pad, (d, d), bias=b, act=act) + 0.0)
+    x, f = si.uniform(332, 0, x.shape, -1, 1), si.normal(332, 1, f.shape, 0, 0.2)
+    got = host(ctx.conv2d(dev(x), dev(f), (1, 1), pad, (d, d)))
+    assert rel_fro(got, oracle.conv2d(x, f, (1, 1), pad, (d, d))) <= TF32_TOL
+    # operands as the tensor core reads them: fp32 sums over up to 1000 products, cut at every MMA (7e-9 of the result each)
+    assert rel_fro(got, oracle.conv2d(x, f, (1, 1), pad, (d, d), operand="tf32_rz")) <= MATCHED_TOL
+
+
+@pytest.mark.parametrize("case", [(1, 130, 36, 65), (1, 127, 4, 3), (1, 33, 100, 201), (3, 50, 64, 51), (5, 199, 68, 70), (3, 9, 20, 7), (1, 64, 1024, 101)])
+def test_unaligned_products_with_rows_of_whole_quads(ctx, oracle, case):
+    """K a multiple of 4 and N odd: K-contiguous operands are fetched four k at a time, of a batch only where every product
+    starts on 16 bytes, and the last k-block ends inside a row of tiles."""
+    b, m, k, n = case
+    for ta, tb in ((False, True), (False, False), (True, True)):
+        x, y = si.uniform(333, 0, (b, m, k), -1, 1), si.uniform(333, 1, (b, k, n), -1, 1)
+        want = np.einsum("bmk,bkn->bmn", x.astype(np.float64), y.astype(np.float64))
+        xs, ys = np.ascontiguousarray(np.swapaxes(x, 1, 2)) if ta else x, np.ascontiguousarray(np.swapaxes(y, 1, 2)) if tb else y
+        got = host(ctx.batch_matmul(dev(xs), dev(ys), ta, tb)) if b > 1 else host(ctx.matmul(dev(xs[0]), dev(ys[0]), ta, tb))[None]
+        ctx.check_device_status()
+        assert rel_fro(got, want) <= 1.8e-8 * max(k, 32) ** 0.5 + 1.2e-7  # fp32 multiply-adds, and the operands' split

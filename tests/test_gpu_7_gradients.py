@@ -410,3 +410,31 @@ def test_gradients_in_a_capture_without_scratch(tfjsb, oracle):
         assert same_bits(host(a) + 0.0, b + 0.0)
     del graph, got
     own.close()
+
+
+@pytest.mark.parametrize("case", [(1, 16, 8, 32, 32, "same"), (1, 5, 3, 4, 16, "same"), (2, 17, 9, 36, 68, "same"), (1, 33, 24, 64, 64, "valid"),
+                                  (1, 20, 20, 300, 40, "same"), (2, 14, 14, 128, 512, "same"), (30, 9, 20, 64, 32, "same")])
+def test_conv2d_input_gradient_from_patches(ctx, oracle, monkeypatch, case):
+    """Stride 1, tiles of 16 x 8 samples: taps last to first, the forward padding's complement, parts of the K loop."""
+    N, H, W, Cin, Cout, pad = case
+    fh, fw, d = 3, 3, 1
+    monkeypatch.setenv("TFJSB_CONV_PATCH", "1")
+    Ho, Wo = geometry(oracle, H, W, fh, fw, 1, d, pad)
+    shape, args = (N, H, W, Cin), ((1, 1), pad, (d, d))
+    f, g = si.small_integers(99, 1, (fh, fw, Cin, Cout), -3, 3), si.small_integers(99, 2, (N, Ho, Wo, Cout), -3, 3)
+    got = host(ctx.conv2d_backprop_input(shape, dev(f), dev(g), *args))
+    ctx.check_device_status()
+    assert same_bits(got + 0.0, oracle.conv2d_backprop_input(shape, f, g, *args) + 0.0)
+    f, g = si.normal(99, 3, f.shape, 0, 0.2), si.normal(99, 4, g.shape, 0, 1)
+    got = host(ctx.conv2d_backprop_input(shape, dev(f), dev(g), *args))
+    # fp32 multiply-adds in order, 1.8e-8 sqrt(K), the operands' split, the oracle's rounding
+    assert rel_fro(got, oracle.conv2d_backprop_input(shape, f, g, *args)) <= 1.8e-8 * (fh * fw * Cout) ** 0.5 + 1.2e-7
+    # infinities and NaNs as fp32 multiply-adds give them, at the border too
+    f, g = plant_specials(f, 6, (0, f.size - 1), False), plant_specials(g, 7, (0, g.size - 1), False)
+    got = host(ctx.conv2d_backprop_input(shape, dev(f), dev(g), *args))
+    ctx.set_math("fp32")
+    try:
+        want = host(ctx.conv2d_backprop_input(shape, dev(f), dev(g), *args))
+    finally:
+        ctx.set_math("tf32")
+    assert same_classes(got, want)
