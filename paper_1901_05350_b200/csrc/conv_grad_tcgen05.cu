@@ -28,8 +28,10 @@
 // an MN-major operand as it is, and its halves are elementwise functions of it.  hi is rounded here, in place: left as copied,
 // cut, it is 2.7e-7 off where rounded it is 2.2e-7 ([16,28,28,128], 3x3; 33.6 us).  M = four (tap, 32-channel)
 // groups, N = 32..128 channels of dy, one (M tile, N tile, slice of the pixels) per CTA, partial sums added in slice
-// order.  Per k-block at block_n 128, 32 KB landed, read and split and 96 KB read by the MMAs: 1500 cycles of shared memory
-// (768 of MMAs); without the lo half a copy and 256 cycles of MMAs.
+// order.  Per k-block at block_n 128, 32 KB landed and read, 64 KB of halves written and 96 KB read by the MMAs are 1750 cycles
+// of shared memory (768 of MMAs); without the lo half the copy and 256 cycles of MMAs.  Against tiles transposed by the
+// converter warps: [16,28,28,128], 3x3, 38.5 -> 36 us, [4,14,14,512] of 512 34 -> 32; pointwise, plain TF32, [32,56,56]
+// 128 x 128 31 -> 26.5 with the sum of the parts, [64,14,14] 512 x 512 53 -> 46.
 #include <algorithm>
 #include <cstdlib>
 

@@ -1,8 +1,8 @@
 // tfjsb_matmul_static_scratch: tfjsb_matmul for callers that must not allocate device memory.
 //
-// The tensor-core matMul needs both operands K-contiguous, so an operand that is stored the
-// other way round is first transposed into scratch memory.  tfjsb_matmul takes that scratch
-// from cudaMalloc (growing it on demand).  Some callers cannot do that where they call the
+// This call makes both operands K-contiguous: one that is stored the other way round is first
+// transposed into scratch memory.  tfjsb_matmul, which reads most operands as they are stored, takes
+// such scratch from cudaMalloc (growing it on demand).  Some callers cannot do that where they call the
 // library: a real-time loop that may not take the allocator's lock or the device
 // synchronisation an allocation can imply, a service whose device-memory budget was fixed at
 // start-up, any code that runs at a point where cudaMalloc is not permitted.  For them the
