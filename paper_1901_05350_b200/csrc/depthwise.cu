@@ -436,6 +436,7 @@ constexpr DwVariant kDwVariants[] = {
     DW_VARIANT(1, 8, 2, 1, 32, true),     // 13
     DW_VARIANT(2, 16, 2, 1, 32, true),    // 14
     DW_VARIANT(2, 8, 2, 1, 32, true),     // 15
+    DW_VARIANT(1, 16, 7, 1, 64, false),   // 16: fp32, stride 1, 16 x 7 outputs of 64 channels
 };
 #undef DW_VARIANT
 constexpr int DW_FIRST_NARROW = 8;
@@ -476,6 +477,7 @@ cudaError_t launch_tma_variant(const DepthwisePlan& plan, const float* x, const 
         DW_CASE(13, 1, 8, 2, 1, 32, true);
         DW_CASE(14, 2, 16, 2, 1, 32, true);
         DW_CASE(15, 2, 8, 2, 1, 32, true);
+        DW_CASE(16, 1, 16, 7, 1, 64, false);
         default: return cudaErrorInvalidValue;
     }
 #undef DW_CASE
@@ -499,22 +501,32 @@ tfjsb_status depthwise_plan(tfjsb_ctx* ctx, const void* x, const ConvGeom& g, De
     if (narrow && (dilated || g.C % 8 != 0)) return TFJSB_OK;  // 16-byte row pitches; no dilated instances in this format
     // the 8-wide stride-2 tile where it wastes fewer columns than the 16-wide one
     const bool wide8 = g.Wo <= 8 || (g.Wo + 7) / 8 * 8 < (g.Wo + 15) / 16 * 16;
+    const int64_t tiles8 = g.N * ((g.Wo + 7) / 8) * ((g.Ho + 7) / 8);  // of 8 x 8 outputs
+    const int64_t blocks32 = (g.C + DW_CB - 1) / DW_CB;
     int v;
     if (dilated) v = g.dh == 2 ? 4 : 5;
-    else if (narrow) v = DW_FIRST_NARROW + (g.C % 64 == 0 ? 0 : 4) + (g.sh == 1 ? (g.Wo <= 8 ? 1 : 0) : (wide8 ? 3 : 2));
+    else if (narrow) {
+        v = DW_FIRST_NARROW + (g.C % 64 == 0 ? 0 : 4) + (g.sh == 1 ? (g.Wo <= 8 ? 1 : 0) : (wide8 ? 3 : 2));
+        // short layers as in fp32 storage below, also of other channel counts up to 6 tiles per SM (a whole model at batch 1, 2 and 4:
+        // 124.3 -> 120.2 us, 125.8 -> 124.0, 132.8 -> 129.9; at batch 16 in every layer 169.6 -> 180)
+        if (g.sh == 1 && (g.C % 64 == 0 ? tiles8 * (g.C / 64) < ctx->sm_count : tiles8 * blocks32 < 6 * (int64_t)ctx->sm_count)) v = DW_FIRST_NARROW + 5;
+    }
     else {
         // Stride 1.  8 x 8 tiles of 32 channels while an SM would not have one of 64: a short layer takes what one tile takes
         // (copy, rows, stores), and its rows per thread are 2 instead of 4 or 7 ([1,56,56,128] 4.1 -> 3.0 us, [1,14,14,512]
         // 3.3 -> 2.9, [4,14,14,512] 3.8 -> 3.2; against 16 x 7 tiles, as all below).  They also read DRAM faster where the
         // tensors do not stay in L2 and a pixel is 512 bytes or less ([128,56,56,128] 73.4 -> 66.3, [100,112,112,64] 116 -> 100;
-        // but [128,28,28,256] 36.7 and 39.6).  Otherwise 8 x 8 of 64 channels, whose edges waste less than those of 16 x 7
-        // ([8,17,17,512] 5.9 -> 4.6, [32,56,56,128] 18.8 -> 17.1, [128,14,14,512] 18.1 either way, [128,28,28,256] 36.7 -> 37.1).
+        // but [128,28,28,256] 36.7 and 39.6).  Otherwise 8 x 8 of 64 channels where they take fewer rounds of two tiles per SM, at half
+        // the time of one of 16 x 7 ([8,17,17,512] 5.9 -> 4.6, [32,56,56,128] 18.8 -> 17.1, [64,14,14,512] 9.5 -> 9.1), else
+        // 16 x 7 ([128,28,28,256] 36.7 and 37.1, [32,14,14,512] 6.1 and 6.2).
         // Channels that are no multiple of 64: 8 x 8 up to 24 tiles per SM ([8,112,112,32] 6.8 -> 6.0, [16,112,112,32] 9.7 -> 9.2),
         // then 16 x 14 ([32,112,112,32] 17.8 and 18.7 with 8 x 8).
-        const int64_t tiles8 = g.N * ((g.Wo + 7) / 8) * ((g.Ho + 7) / 8);
         const bool beyond_l2 = (double)g.N * g.H * g.W * g.C * 8.0 > 1.5e8;  // both tensors
-        if (g.sh == 1 && g.C % 64 == 0) v = tiles8 * (g.C / 64) < ctx->sm_count || (g.C <= 128 && beyond_l2) ? 1 : 6;
-        else if (g.sh == 1) v = g.Wo <= 8 || tiles8 * ((g.C + DW_CB - 1) / DW_CB) <= 24 * (int64_t)ctx->sm_count ? 1 : 0;
+        const int64_t pair = 2 * (int64_t)ctx->sm_count;
+        const int64_t rounds8 = (tiles8 * (g.C / 64) + pair - 1) / pair;
+        const int64_t rounds16 = (g.N * ((g.Wo + 15) / 16) * ((g.Ho + 6) / 7) * (g.C / 64) + pair - 1) / pair;
+        if (g.sh == 1 && g.C % 64 == 0) v = tiles8 * (g.C / 64) < ctx->sm_count || (g.C <= 128 && beyond_l2) ? 1 : rounds8 < 2 * rounds16 ? 6 : 16;
+        else if (g.sh == 1) v = g.Wo <= 8 || tiles8 * blocks32 <= 24 * (int64_t)ctx->sm_count ? 1 : 0;
         // stride 2: 64-channel tiles are 8 outputs wide, so they are taken only where that wastes fewer columns than the
         // 16-wide 32-channel ones ([128,112,112,64] 90.1 -> 86.9 us; [128,28,28,256] ran 27.3 -> 29.1 with them)
         else if (g.C % 64 == 0 && wide8) v = 7;
