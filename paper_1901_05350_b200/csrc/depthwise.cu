@@ -510,8 +510,7 @@ tfjsb_status depthwise_plan(tfjsb_ctx* ctx, const void* x, const ConvGeom& g, De
         // short layers as in fp32 storage below, also of other channel counts up to 6 tiles per SM (a whole model at batch 1, 2 and 4:
         // 124.3 -> 120.2 us, 125.8 -> 124.0, 132.8 -> 129.9; at batch 16 in every layer 169.6 -> 180)
         if (g.sh == 1 && (g.C % 64 == 0 ? tiles8 * (g.C / 64) < ctx->sm_count : tiles8 * blocks32 < 6 * (int64_t)ctx->sm_count)) v = DW_FIRST_NARROW + 5;
-    }
-    else {
+    } else {
         // Stride 1.  8 x 8 tiles of 32 channels while an SM would not have one of 64: a short layer takes what one tile takes
         // (copy, rows, stores), and its rows per thread are 2 instead of 4 or 7 ([1,56,56,128] 4.1 -> 3.0 us, [1,14,14,512]
         // 3.3 -> 2.9, [4,14,14,512] 3.8 -> 3.2; against 16 x 7 tiles, as all below).  They also read DRAM faster where the
