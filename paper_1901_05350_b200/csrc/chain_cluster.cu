@@ -58,17 +58,7 @@ __device__ __forceinline__ void cluster_sync() {
     cluster_arrive();
     cluster_wait();
 }
-// Activations are written by other blocks of the cluster during the kernel: never through the read-only path.
-__device__ __forceinline__ float4 ld_act4(const float* p) {
-    float4 v;
-    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ float ld_act(const float* p) {
-    float v;
-    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
+// Activations are written by other blocks of the cluster during the kernel: ld_global, never the read-only path.
 // `bytes` (a multiple of 16) to shared memory, counted on `bar`.
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const float* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
@@ -337,7 +327,7 @@ __device__ __forceinline__ void block_depthwise(const ChainOp& o, const BlockWor
 #pragma unroll
                 for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
-                    for (int kx = 0; kx < 3; ++kx) x[3 * ky + kx] = ld_act4(src + ky * tap_row + kx * tap_col);
+                    for (int kx = 0; kx < 3; ++kx) x[3 * ky + kx] = ld_global4(src + ky * tap_row + kx * tap_col);
 #pragma unroll
                 for (int k = 0; k < 9; ++k) fma4_packed(v[0], x[k], f[k * quads]);
             } else {
@@ -345,7 +335,7 @@ __device__ __forceinline__ void block_depthwise(const ChainOp& o, const BlockWor
                 for (int ky = 0; ky < 3; ++ky) {
                     float4 x[R + 2];
 #pragma unroll
-                    for (int j = 0; j < R + 2; ++j) x[j] = ld_act4(src + ky * in_row + j * C);
+                    for (int j = 0; j < R + 2; ++j) x[j] = ld_global4(src + ky * in_row + j * C);
 #pragma unroll
                     for (int kx = 0; kx < 3; ++kx) {
                         const float4 tap = f[(3 * ky + kx) * quads];
@@ -415,9 +405,9 @@ __device__ __forceinline__ void stem(const ChainOp& o, const float* in, float* o
         if (u == rank) {
             for (int j = tid; j < 32 * ldf; j += THREADS) {
                 const int k = div_by(j, o.by_pieces), c = j - k * ldf;
-                f_sm[j] = k < 27 && c < Co ? __ldg(o.f1 + k * Co + c) : 0.f;
+                f_sm[j] = k < 27 && c < Co ? load_fixed(o.f1 + k * Co + c) : 0.f;
             }
-            if (tid < Co) f_sm[32 * ldf + tid] = o.b1 ? __ldg(o.b1 + tid) : 0.f;
+            if (tid < Co) f_sm[32 * ldf + tid] = o.b1 ? load_fixed(o.b1 + tid) : 0.f;
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         block_sync();
@@ -457,7 +447,7 @@ __device__ __forceinline__ void pool(const ChainOp& o, int64_t image, const floa
     for (int q = rank * WARPS + (threadIdx.x >> 5); q < (o.C >> 2); q += cs * WARPS) {
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int p = lane; p < M; p += 32) {
-            const float4 v = ld_act4(in + p * o.C + 4 * q);
+            const float4 v = ld_global4(in + p * o.C + 4 * q);
             s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
         }
 #pragma unroll
@@ -486,14 +476,14 @@ __device__ __forceinline__ void load_dense(const ChainOp& o, float4 (&w)[DENSE_A
     const float* src = o.f1 + min(n0 + 4 * (int)(threadIdx.x & 15), o.Co - 4);
     const int share = threadIdx.x >> 4, last = o.C - 1, Co = o.Co;
 #pragma unroll
-    for (int j = 0; j < DENSE_AHEAD; ++j) w[j] = __ldg(reinterpret_cast<const float4*>(src + (int64_t)min(k0 + share + j * DENSE_SHARES, last) * Co));
+    for (int j = 0; j < DENSE_AHEAD; ++j) w[j] = load_fixed(reinterpret_cast<const float4*>(src + (int64_t)min(k0 + share + j * DENSE_SHARES, last) * Co));
 }
 __device__ __forceinline__ void dense(const ChainOp& o, float4 (&w)[DENSE_AHEAD], int64_t image, const float* in, float* out, float* x_sm, float* red,
                                       int rank, int cs) {
     const int q = threadIdx.x & 15, share = threadIdx.x >> 4, Co = o.Co, C = o.C;
     const int padded = (C + DENSE_AHEAD * DENSE_SHARES - 1) / (DENSE_AHEAD * DENSE_SHARES) * (DENSE_AHEAD * DENSE_SHARES);
     for (int k = 4 * threadIdx.x; k < padded; k += 4 * THREADS)
-        *reinterpret_cast<float4*>(x_sm + k) = k < C ? ld_act4(in + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4*>(x_sm + k) = k < C ? ld_global4(in + k) : make_float4(0.f, 0.f, 0.f, 0.f);
     block_sync();
     for (int n0 = rank * 64; n0 < Co; n0 += cs * 64) {
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -509,7 +499,7 @@ __device__ __forceinline__ void dense(const ChainOp& o, float4 (&w)[DENSE_AHEAD]
         *reinterpret_cast<float4*>(red + share * 64 + 4 * q) = s;
         block_sync();
         if (threadIdx.x < 64 && n0 + (int)threadIdx.x < Co) {
-            float v = o.b1 ? __ldg(o.b1 + n0 + threadIdx.x) : 0.f;
+            float v = o.b1 ? load_fixed(o.b1 + n0 + threadIdx.x) : 0.f;
 #pragma unroll
             for (int k = 0; k < DENSE_SHARES; ++k) v += red[k * 64 + threadIdx.x];
             v = bounded(v, o.lo2, o.hi2);
@@ -529,11 +519,11 @@ __device__ __forceinline__ void softmax(const ChainOp& o, const float* in, float
 #pragma unroll
     for (int k = 0; k < HELD; ++k) {
         const int j = threadIdx.x + k * THREADS;
-        x[k] = j < o.Co ? ld_act(in + j) : -INFINITY;
+        x[k] = j < o.Co ? ld_global(in + j) : -INFINITY;
     }
 #pragma unroll
     for (int k = 0; k < HELD; ++k) top = fmaxf(top, x[k]);
-    for (int j = threadIdx.x + HELD * THREADS; j < o.Co; j += THREADS) top = fmaxf(top, ld_act(in + j));
+    for (int j = threadIdx.x + HELD * THREADS; j < o.Co; j += THREADS) top = fmaxf(top, ld_global(in + j));
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
     if (lane == 0) red[warp] = top;
@@ -547,7 +537,7 @@ __device__ __forceinline__ void softmax(const ChainOp& o, const float* in, float
         x[k] = (int)threadIdx.x + k * THREADS < o.Co ? expf(x[k] - top) : 0.f;
         sum += x[k];
     }
-    for (int j = threadIdx.x + HELD * THREADS; j < o.Co; j += THREADS) sum += expf(ld_act(in + j) - top);
+    for (int j = threadIdx.x + HELD * THREADS; j < o.Co; j += THREADS) sum += expf(ld_global(in + j) - top);
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
     if (lane == 0) red[WARPS + warp] = sum;
@@ -560,7 +550,7 @@ __device__ __forceinline__ void softmax(const ChainOp& o, const float* in, float
         const int j = threadIdx.x + k * THREADS;
         if (j < o.Co) out[j] = x[k] / sum;
     }
-    for (int j = threadIdx.x + HELD * THREADS; j < o.Co; j += THREADS) out[j] = expf(ld_act(in + j) - top) / sum;
+    for (int j = threadIdx.x + HELD * THREADS; j < o.Co; j += THREADS) out[j] = expf(ld_global(in + j) - top) / sum;
 }
 
 // The end of the layer before.

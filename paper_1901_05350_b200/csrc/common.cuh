@@ -163,6 +163,21 @@ extern thread_local bool g_launch_pdl;
 // while the kernel runs).
 template <typename T>
 __device__ __forceinline__ T load_global(const T* p) { return *p; }
+// The other kind, for what nothing writes while any kernel runs that reads it: a model's filters and biases.
+template <typename T>
+__device__ __forceinline__ T load_fixed(const T* p) { return __ldg(p); }
+// load_global as an instruction that stays where it is written, for loops that load ahead with few registers to spare (the
+// strided GEMM's loaders spill 16 to 40 bytes with load_global and nothing with these).
+__device__ __forceinline__ float ld_global(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_global4(const float* p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
 
 template <typename... KArgs, typename... Args>
 cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {

@@ -74,21 +74,21 @@ struct Fetch {
 #pragma unroll
             for (int i = 0; i < ROWS / 32; ++i) {
                 float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (ok) q = __ldg(reinterpret_cast<const float4*>(at + (long long)min(r0 + 32 * i + 4 * w + (lane >> 3), last) * s.row_stride));
+                if (ok) q = ld_global4(at + (long long)min(r0 + 32 * i + 4 * w + (lane >> 3), last) * s.row_stride);
                 v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
             }
         } else if (s.k_stride == 1) {  // lane = k, row w + 8 i
             const bool ok = k0 + lane < K;
             const float* at = base + k0 + lane;
 #pragma unroll
-            for (int i = 0; i < ROWS / 8; ++i) v[i] = ok ? __ldg(at + (long long)min(r0 + w + 8 * i, last) * s.row_stride) : 0.f;
+            for (int i = 0; i < ROWS / 8; ++i) v[i] = ok ? ld_global(at + (long long)min(r0 + w + 8 * i, last) * s.row_stride) : 0.f;
         } else {                // lane = row of block i, k = 4 w + e; rows are contiguous
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int k = k0 + 4 * w + e;
                 const float* at = base + (long long)k * s.k_stride;
 #pragma unroll
-                for (int i = 0; i < ROWS / 32; ++i) v[4 * i + e] = k < K ? __ldg(at + min(r0 + 32 * i + lane, last)) : 0.f;
+                for (int i = 0; i < ROWS / 32; ++i) v[4 * i + e] = k < K ? ld_global(at + min(r0 + 32 * i + lane, last)) : 0.f;
             }
         }
     }
@@ -125,7 +125,7 @@ struct Fetch {
 // One element over k0 .. k1 by fp32 multiply-adds.
 __device__ __noinline__ float sum_in_fp32(const float* p, const float* q, int p_step, int q_step, int k0, int k1) {
     float acc = 0.f;
-    for (int k = k0; k < k1 && acc == acc; ++k) acc = fmaf(__ldg(p + (long long)k * p_step), load_global(q + (long long)k * q_step), acc);
+    for (int k = k0; k < k1 && acc == acc; ++k) acc = fmaf(ld_global(p + (long long)k * p_step), ld_global(q + (long long)k * q_step), acc);
     return acc;
 }
 
@@ -317,7 +317,7 @@ gemm_strided_kernel(const StridedArgs g) {
         const uint32_t at_step = (uint32_t)((row_step * PITCH + col_step) * 4);
         // the bias is either one value per thread or walked along
         const bool one_bias = g.bias != nullptr && along_p == (g.bias_p != 0);
-        const float b0 = one_bias && live ? __ldg(g.bias + (along_p ? p : q)) : 0.f;
+        const float b0 = one_bias && live ? ld_global(g.bias + (along_p ? p : q)) : 0.f;
         const float* bias = g.bias != nullptr && !one_bias ? g.bias + (along_p ? q0 : p0 + r0) : nullptr;
 #pragma unroll 4
         for (int i = along_p ? col : row; i < (live ? limit : 0); i += step, at += at_step, out += out_step) {
@@ -334,7 +334,7 @@ gemm_strided_kernel(const StridedArgs g) {
                 for (int s = 1; s < GS_MAX_CLUSTER; ++s)
                     if (s < g.splits) v += part[s];
             }
-            if (g.bias) v += bias ? __ldg(bias + i) : b0;
+            if (g.bias) v += bias ? ld_global(bias + i) : b0;
             *out = apply_act(v, g.act);
         }
     }

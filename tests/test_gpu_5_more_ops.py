@@ -222,6 +222,35 @@ def test_op_calls_one_after_another_see_each_others_results(ctx):
     assert float(total.min()) == 256 * 4096.0 == float(total.max())
 
 
+@pytest.mark.parametrize("tb", [False, True])
+@pytest.mark.parametrize("shape", [(64, 1024, 101), (300, 36, 65), (8, 19, 1003)])
+def test_unaligned_products_between_updates_of_their_operand(ctx, shape, tb):
+    """Operands that are written again and again, two buffers in turn: a product's blocks may be on an SM that has read the
+    older values of its buffer, and all the same the bits are those of calls with a synchronisation after each."""
+    import torch
+
+    m, k, n = shape
+    x, step = torch.rand(m, k, device="cuda"), torch.rand(n, k, device="cuda") if tb else torch.rand(k, n, device="cuda")
+    first = torch.rand_like(step)
+
+    def calls(wait):
+        w, out = [first.clone(), torch.empty_like(first)], torch.empty(100, m, n, device="cuda")
+        torch.cuda.synchronize()
+        for i in range(100):
+            ctx.matmul(x, w[i % 2], transpose_b=tb, out=out[i])
+            if wait:
+                torch.cuda.synchronize()
+            ctx.binary("sub", w[i % 2], step, out=w[(i + 1) % 2])
+            if wait:
+                torch.cuda.synchronize()
+        return out
+
+    want = calls(True)
+    for _ in range(3):
+        assert torch.equal(calls(False), want)
+    ctx.check_device_status()
+
+
 def test_op_calls_captured_on_two_streams_that_join(ctx):
     import torch
 
