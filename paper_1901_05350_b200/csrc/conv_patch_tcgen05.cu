@@ -665,6 +665,7 @@ bool conv_patch_gradient_preferred(const ConvGeom& g, int sm_count) {
     const ConvGeom b = transposed(g);
     if (!shape_ok(b) || !patch_tiling(b, true, sm_count, &t) || (int64_t)PC_TAPS * t.c_blocks * 32 > SPLIT_MAX_K) return false;
     if (const char* env = getenv("TFJSB_CONV_PATCH")) return atoi(env) != 0;
+    if (getenv("TFJSB_GRAD_INPUT")) return false;  // which decides between the two kernels for any window
     int64_t patches, rows;
     tile_rounds(b, t, sm_count, &patches, &rows);
     return b.Co % 128 == 0 && t.pixel_tiles >= 8 && 5 * patches <= 6 * rows;

@@ -438,3 +438,27 @@ def test_conv2d_input_gradient_from_patches(ctx, oracle, monkeypatch, case):
     finally:
         ctx.set_math("tf32")
     assert same_classes(got, want)
+
+
+def test_the_input_gradient_switch_decides_where_patches_would_run(ctx, monkeypatch):
+    """Sums of the three kernels differ in order, so in the last bits: 0 is the kernel of the fp32 mode, 1 the one that runs
+    without patches, unset the patches, which the same shape takes by rule."""
+    shape, f, g = (8, 14, 14, 128), dev(si.normal(101, 1, (3, 3, 128, 32), 0, 0.2)), dev(si.normal(101, 2, (8, 14, 14, 32), 0, 1))
+    monkeypatch.setenv("TFJSB_CONV_PATCH", "1")
+    patches = host(ctx.conv2d_backprop_input(shape, f, g))
+    monkeypatch.setenv("TFJSB_CONV_PATCH", "0")
+    monkeypatch.setenv("TFJSB_GRAD_INPUT", "1")
+    any_window = host(ctx.conv2d_backprop_input(shape, f, g))
+    monkeypatch.delenv("TFJSB_CONV_PATCH")
+    ctx.set_math("fp32")
+    try:
+        cuda_cores = host(ctx.conv2d_backprop_input(shape, f, g))
+    finally:
+        ctx.set_math("tf32")
+    assert not same_bits(patches, any_window) and not same_bits(patches, cuda_cores) and not same_bits(any_window, cuda_cores)
+    assert same_bits(host(ctx.conv2d_backprop_input(shape, f, g)), any_window)
+    monkeypatch.setenv("TFJSB_GRAD_INPUT", "0")
+    assert same_bits(host(ctx.conv2d_backprop_input(shape, f, g)), cuda_cores)
+    monkeypatch.delenv("TFJSB_GRAD_INPUT")
+    assert same_bits(host(ctx.conv2d_backprop_input(shape, f, g)), patches)
+    ctx.check_device_status()
