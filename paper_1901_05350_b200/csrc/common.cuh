@@ -331,6 +331,7 @@ cudaError_t launch_gemm_tf32_splitk(const GemmTf32Plan& plan, const float* bias,
 // 32: each tap for itself where A comes by im2col loads, the whole window otherwise).
 bool conv_igemm_supported(const ConvGeom& g);
 bool conv_igemm_uses_im2col(const ConvGeom& g);
+double conv_im2col_us(const ConvGeom& g, int sm_count);  // estimate of the filter packing and the im2col kernel
 int64_t conv_igemm_k_pad(const ConvGeom& g);
 cudaError_t launch_pack_conv_filter(const float* f, float* out, const ConvGeom& g, cudaStream_t s, int64_t* launches);
 tfjsb_status conv_igemm_plan(tfjsb_ctx* ctx, const float* x, const float* bt, float* y, const ConvGeom& g,
@@ -404,6 +405,7 @@ cudaError_t launch_depthwise_backprop_filter(const float* x, const float* dy, fl
 // Gradients of conv2d on the tensor cores (conv_grad_tcgen05.cu).  fp32 results: operands as two TF32 values each, except
 // the filter gradient with `split` false, which reads them as TF32.  Scratch for partial sums is the context's.
 bool conv2d_grad_input_supported(const ConvGeom& g);
+double conv2d_grad_input_us(const ConvGeom& g, int sm_count);  // estimate for stride 1, to compare it with patches
 bool conv2d_grad_input_preferred(const ConvGeom& g, int sm_count);  // to the CUDA-core kernel (TFJSB_GRAD_INPUT=1: always)
 tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float* f, float* dx, const ConvGeom& g, cudaStream_t s);
 bool conv2d_grad_filter_supported(const ConvGeom& g);

@@ -707,6 +707,15 @@ static GradInputTiling grad_input_tiling(const ConvGeom& g, int64_t m_tiles, int
     return t;
 }
 
+// The kernel below at stride 1 with 3x3 windows of 16 channels or more, fitted like the patch kernel's estimate and to the same
+// shapes (conv_patch_tcgen05.cu; nine in ten within 10 %): per round an epilogue and k-blocks.
+double conv2d_grad_input_us(const ConvGeom& g, int sm_count) {
+    const GradInputTiling t = grad_input_tiling(g, (g.N * g.H * g.W + BLOCK_M - 1) / BLOCK_M, sm_count);
+    const double round = t.block_n == 32 ? 2.6 : t.block_n == 64 ? 3.8 : 5.8, kb = t.block_n == 32 ? 0.62 : t.block_n == 64 ? 0.65 : 0.77;
+    const double rounds = (double)((t.tiles * t.splits + sm_count - 1) / sm_count), out_mb = (double)g.N * g.H * g.W * g.C * 4e-6;
+    return 4.5 + rounds * (round + kb * ((t.kbs + t.splits - 1) / t.splits)) + (t.splits > 1 ? 1.0 + t.splits * out_mb : 0.0);
+}
+
 // Where a sample's sum is short, one CUDA-core thread per sample is the faster kernel.  In microseconds, fitted to both on
 // 145 shapes (4 to 64 output channels, windows up to 7 x 7, strides 1 to 3; 4 % of them still go to the slower one):
 //   here         3, and for each round of tiles 1.4 and 0.72 per k-block, of which a tap makes at least one however few its

@@ -519,7 +519,7 @@ struct PatchTiling {
     int block_n = 0, splits = 1, patch_stages = 0, b_stages = 0, c_blocks = 0, n_tiles = 0;
     bool resident = false;
     int64_t pixel_tiles = 0, tiles = 0;
-    double cycles = 0;  // estimate, to choose between widths and kernels only
+    double us = 0;  // estimate, to choose between widths and kernels only
 };
 
 bool rings_fit(PatchTiling* t, bool split) {
@@ -538,24 +538,34 @@ bool rings_fit(PatchTiling* t, bool split) {
     return t->patch_stages * patch < room && t->b_stages >= 2;
 }
 
+// What a launch takes, in microseconds, fitted to 500 shapes of 7 to 224 squared, 16 to 512 channels each way, 1 to 64 images, all
+// widths (nine in ten within 7 %): a start, and for every round of tiles an epilogue and its k-blocks, of 32 channels of one tap.
+struct PatchCost {
+    double round, kb;
+};
+constexpr PatchCost kRing[] = {{0.45, 0.215}, {0.55, 0.221}, {1.3, 0.24}, {2.55, 0.386}};  // 32, 64, 128, 256 columns
+constexpr PatchCost kResident[] = {{0.0, 0.205}, {0.0, 0.205}, {0.0, 0.245}};              // the filter stays in shared memory
+constexpr PatchCost kSplit[] = {{2.9, 0.54}, {3.6, 0.60}, {6.4, 0.69}};                    // SPLIT
+
 bool patch_tiling(const ConvGeom& g, bool split, int sms, PatchTiling* best) {
     PatchTiling t;
     t.c_blocks = (g.C + BLOCK_K - 1) / BLOCK_K;
     t.pixel_tiles = g.N * ((g.Ho + PC_TH - 1) / PC_TH) * ((g.Wo + PC_TW - 1) / PC_TW);
+    const double out_mb = (double)g.N * g.Ho * g.Wo * g.Co * 4e-6;
     bool any = false;
-    for (int bn : {32, 64, 128, 256}) {
-        if (split && bn > 128) break;
+    for (int i = 0; i < (split ? 3 : 4); ++i) {
+        const int bn = 32 << i;
         t.block_n = bn;
         t.n_tiles = (g.Co + bn - 1) / bn;
         t.tiles = t.pixel_tiles * t.n_tiles;
         t.splits = 1;
         if (split && 2 * t.tiles <= sms) t.splits = (int)std::min<int64_t>(std::min<int64_t>(sms / t.tiles, t.c_blocks), 16);
         if (rings_fit(&t, split)) {
-            // a k-block: the MMAs and their operands' way through shared memory, or the issuing loop
-            const double kb = split ? std::max(500.0, 9.0 * bn + 60) : std::max(210.0, 2.0 * bn);
+            const PatchCost c = split ? kSplit[i] : t.resident ? kResident[i] : kRing[i];
             const int64_t rounds = (t.tiles * t.splits + sms - 1) / sms;
-            t.cycles = rounds * (double)((t.c_blocks + t.splits - 1) / t.splits) * PC_TAPS * kb + rounds * 8.0 * bn + 6000 + (t.splits > 1 ? 4000 : 0);
-            if (!any || t.cycles < best->cycles) *best = t;
+            const int kbs = (t.c_blocks + t.splits - 1) / t.splits * PC_TAPS;
+            t.us = (!split && t.resident ? 5.2 : 4.7) + rounds * (c.round + c.kb * kbs) + (t.splits > 1 ? 0.7 + t.splits * out_mb : 0.0);
+            if (!any || t.us < best->us) *best = t;
             any = true;
         }
         if (bn >= g.Co) break;
@@ -631,24 +641,21 @@ ConvGeom transposed(const ConvGeom& g) {
 
 }  // namespace
 
-// Rounds of tiles over the SMs: of 16 x 8 pixels, which leave some of an image's edges empty, and of 128 pixels in a row, as the
-// im2col kernels take them.
-static void tile_rounds(const ConvGeom& g, const PatchTiling& t, int sms, int64_t* patches, int64_t* rows) {
-    *patches = (t.tiles * t.splits + sms - 1) / sms;
-    *rows = ((g.N * g.Ho * g.Wo + BLOCK_M - 1) / BLOCK_M * t.n_tiles + sms - 1) / sms;
-}
+// By how much the estimate of this kernel has to be the lower one: both are a few percent off.  On 500 other shapes than those
+// that the estimates were fitted to
+//   forward   153 are taken, at 0.90 of the time of the im2col kernel and its filter packing on average, the worst at 1.04
+//             ([64,112,112,32] -> 32: 108 and 84 us, [1,224,224,16] -> 16: 12.9 and 10.9, [16,28,28,128] -> 128: 15.6 and 15.2; not
+//             taken, images that tiles of 16 x 8 fill badly: [63,28,28,128] -> 256: 50 and 69, [9,135,135,72] -> 64: 63 and 68)
+//   gradient  132, at 0.87, the worst at 1.04 (most where im2col tiles have the K loop in fewer parts: [4,14,14,512] of 512 91.6 and
+//             39.7, but also [16,28,28,128] of 128: 38.3 and 37.1, [2,172,172,128] of 96: 109 and 99; not taken: [61,28,28,128]
+//             of 120: 106 and 125, [63,8,8,256] of 312: 66 and 73, [32,56,56,64] of 64: 103 and 108)
+constexpr double PC_AHEAD = 0.95;
 
-// Where this kernel is the faster one, of 17 shapes measured against im2col copies.  Forward: up to 128 channels, a whole number
-// of column tiles, and no more than a fifth more rounds ([64,112,112,32] -> 32: 108 and 84 us, [1,224,224,16] -> 16: 12.9 and
-// 10.9, [32,56,56,64] -> 64: 31.7 and 30.0, [16,28,28,128] -> 128: 16.4 and 15.4, packing the filter included there; but
-// [64,28,28,64] -> 64: 19.7 and 20.2, four rounds for three, [30,20,20,24] -> 40: 8.2 and 9.2, [8,28,28,256] -> 256: 23.3 and 24.6).
 bool conv_patch_input_preferred(const ConvGeom& g, int sm_count) {
     PatchTiling t;
     if (!shape_ok(g) || !patch_tiling(g, false, sm_count, &t)) return false;
     if (const char* env = getenv("TFJSB_CONV_PATCH")) return atoi(env) != 0;  // for tests: 1 = wherever it can, 0 = never
-    int64_t patches, rows;
-    tile_rounds(g, t, sm_count, &patches, &rows);
-    return g.C <= 128 && (g.Co <= 32 || g.Co % t.block_n == 0) && 5 * patches <= 6 * rows;
+    return t.us < PC_AHEAD * conv_im2col_us(g, sm_count);
 }
 
 tfjsb_status run_conv_patch_input(tfjsb_ctx* ctx, const float* x, const float* f, const float* bias, int act, float* y, const ConvGeom& g, cudaStream_t s) {
@@ -657,18 +664,13 @@ tfjsb_status run_conv_patch_input(tfjsb_ctx* ctx, const float* x, const float* f
     return launch(ctx, x, f, bias, act, y, g, false, t, s);
 }
 
-// The gradient: input channels in whole tiles of 128 and eight pixel tiles or more ([4,14,14,512] of 512: 92.8 and 40.3 us,
-// [16,7,7,256] of 256: 31.5 and 25.7, [16,28,28,128] of 128: 39.7 and 37.4, [2,56,56,128] of 128: 32.8 and 31.7; but
-// [32,56,56,64] of 64: 104 and 109, [1,14,14,256] of 256: 14.3 and 15.8, [30,20,20,24] of 40: 18.3 and 30.9).
 bool conv_patch_gradient_preferred(const ConvGeom& g, int sm_count) {
     PatchTiling t;
     const ConvGeom b = transposed(g);
     if (!shape_ok(b) || !patch_tiling(b, true, sm_count, &t) || (int64_t)PC_TAPS * t.c_blocks * 32 > SPLIT_MAX_K) return false;
     if (const char* env = getenv("TFJSB_CONV_PATCH")) return atoi(env) != 0;
     if (getenv("TFJSB_GRAD_INPUT")) return false;  // which decides between the two kernels for any window
-    int64_t patches, rows;
-    tile_rounds(b, t, sm_count, &patches, &rows);
-    return b.Co % 128 == 0 && t.pixel_tiles >= 8 && 5 * patches <= 6 * rows;
+    return conv2d_grad_input_preferred(g, sm_count) && t.us < PC_AHEAD * conv2d_grad_input_us(g, sm_count);
 }
 
 tfjsb_status run_conv_patch_gradient(tfjsb_ctx* ctx, const float* dy, const float* f, float* dx, const ConvGeom& g, cudaStream_t s) {

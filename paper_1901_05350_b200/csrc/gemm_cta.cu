@@ -663,12 +663,14 @@ bool gemm_tf32_supported(int64_t M, int64_t N, int64_t K) {
            K < (1LL << 31) - 256 && ((M + BLOCK_M - 1) / BLOCK_M) * ((N + 31) / 32) < (1LL << 31);
 }
 
+// an im2col copy delivers a pixel's 128 bytes in about five cycles; the gathering threads need about twice as long
+constexpr int IM2COL_KB_NS = 330, GATHER_KB_NS = 600;
+
 namespace {
 
 // tile choice, pipeline depth and the B / C tensor maps shared by the GEMM and the convolution
 tfjsb_status plan_common(tfjsb_ctx* ctx, const float* bt, int64_t k_pitch, float* c, GemmTf32Plan* plan, int64_t batches = 1) {
-    // an im2col copy delivers a pixel's 128 bytes in about five cycles; the gathering threads need about twice as long
-    const int min_kb_ns = plan->im2col ? 330 : plan->gather ? 600 : 0;
+    const int min_kb_ns = plan->im2col ? IM2COL_KB_NS : plan->gather ? GATHER_KB_NS : 0;
     const int64_t M = plan->M, N = plan->N;
     plan->batches = batches;
     plan->block_n = choose_block_n(M, N, (k_pitch + BLOCK_K - 1) / BLOCK_K, ctx->sm_count, batches, min_kb_ns);
@@ -732,6 +734,18 @@ bool conv_igemm_uses_im2col(const ConvGeom& g) {
     const int64_t upper_w = (int64_t)(g.Wo - 1) * g.sw - g.pl - (g.W - 1), upper_h = (int64_t)(g.Ho - 1) * g.sh - g.pt - (g.H - 1);
     return !g.gather_only && !conv_patch_supported(g) && g.C % 4 == 0 && g.C >= 16 && g.sh <= 8 && g.sw <= 8 && (int64_t)(g.fh - 1) * g.dh <= 127 && (int64_t)(g.fw - 1) * g.dw <= 127 &&
            g.pl <= 127 && g.pt <= 127 && upper_w >= -128 && upper_w <= 127 && upper_h >= -128 && upper_h <= 127;
+}
+
+// Fitted to the same 500 shapes as the patch kernel's estimate (conv_patch_tcgen05.cu; nine in ten within 7 %), for the width that
+// the planner takes.  A k-block measures 180 ns at 32 columns to 300 at 256, what the table has for copied tiles less 20, where
+// the planner counts 330.
+double conv_im2col_us(const ConvGeom& g, int sm_count) {
+    const int64_t M = g.N * g.Ho * g.Wo, kbs = (int64_t)g.fh * g.fw * ((g.C + BLOCK_K - 1) / BLOCK_K);
+    const int width = choose_block_n(M, g.Co, kbs, sm_count, 1, IM2COL_KB_NS);
+    const TileCost* t = kTileCosts;
+    while (t->width != width) ++t;
+    const int64_t tiles = (M + BLOCK_M - 1) / BLOCK_M * ((g.Co + width - 1) / width), rounds = (tiles + sm_count - 1) / sm_count;
+    return 6.2 + 1e-3 * rounds * (t->epilogue_ns + kbs * (t->kb_ns - 20)) + 2e-6 * g.fh * g.fw * g.C * g.Co;  // packing: 0.5 us per MB
 }
 
 int64_t conv_igemm_k_pad(const ConvGeom& g) {

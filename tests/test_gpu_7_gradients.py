@@ -443,7 +443,7 @@ def test_conv2d_input_gradient_from_patches(ctx, oracle, monkeypatch, case):
 def test_the_input_gradient_switch_decides_where_patches_would_run(ctx, monkeypatch):
     """Sums of the three kernels differ in order, so in the last bits: 0 is the kernel of the fp32 mode, 1 the one that runs
     without patches, unset the patches, which the same shape takes by rule."""
-    shape, f, g = (8, 14, 14, 128), dev(si.normal(101, 1, (3, 3, 128, 32), 0, 0.2)), dev(si.normal(101, 2, (8, 14, 14, 32), 0, 1))
+    shape, f, g = (4, 14, 14, 512), dev(si.normal(101, 1, (3, 3, 512, 512), 0, 0.2)), dev(si.normal(101, 2, (4, 14, 14, 512), 0, 1))
     monkeypatch.setenv("TFJSB_CONV_PATCH", "1")
     patches = host(ctx.conv2d_backprop_input(shape, f, g))
     monkeypatch.setenv("TFJSB_CONV_PATCH", "0")
@@ -461,4 +461,28 @@ def test_the_input_gradient_switch_decides_where_patches_would_run(ctx, monkeypa
     assert same_bits(host(ctx.conv2d_backprop_input(shape, f, g)), cuda_cores)
     monkeypatch.delenv("TFJSB_GRAD_INPUT")
     assert same_bits(host(ctx.conv2d_backprop_input(shape, f, g)), patches)
+    ctx.check_device_status()
+
+
+@pytest.mark.parametrize("case,forward,gradient", [((63, 28, 28, 128, 256), False, None), ((2, 56, 56, 64, 64), True, None), ((61, 28, 28, 128, 120), None, False),
+                                                   ((42, 7, 7, 128, 128), None, False), ((9, 8, 8, 512, 112), None, True)])
+def test_which_3x3_convolutions_run_from_patches(ctx, monkeypatch, case, forward, gradient):
+    """By estimate.  Images that 16 x 8 pixels divide badly took up to 1.7 times as long from patches; the bits, sums in
+    another order, show which kernel ran."""
+    import torch
+
+    N, H, W, Cin, Cout = case
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    x, f, g = (torch.randn(shape, generator=gen, device="cuda") for shape in ((N, H, W, Cin), (3, 3, Cin, Cout), (N, H, W, Cout)))
+    for call, taken in ((lambda: ctx.conv2d(x, f), forward), (lambda: ctx.conv2d_backprop_input(x.shape, f, g), gradient)):
+        if taken is None:
+            continue
+        monkeypatch.delenv("TFJSB_CONV_PATCH", raising=False)
+        chosen = call()
+        monkeypatch.setenv("TFJSB_CONV_PATCH", "1")
+        patches = call()
+        monkeypatch.setenv("TFJSB_CONV_PATCH", "0")
+        copies = call()
+        assert not torch.equal(patches, copies)
+        assert torch.equal(chosen, patches if taken else copies)
     ctx.check_device_status()
