@@ -128,6 +128,11 @@ __device__ __forceinline__ void max4_nan(float4& m, const float4& v) {
     asm("max.NaN.f32 %0, %0, %1;" : "+f"(m.z) : "f"(v.z));
     asm("max.NaN.f32 %0, %0, %1;" : "+f"(m.w) : "f"(v.w));
 }
+// W: windows of up to W x W, all samples on their way before the first comparison, -inf where there is none; 0: any window, one
+// sample after the other (ld_global: with loads that the compiler may move, 5 x 5 over [32,55,55,172] takes 146 us, 117 so).
+// [32,55,55,172]: 3 x 3 / 2 22.6 us with W = 0 and 17.6 with W = 3, 2 x 2 / 2 16.5 and 10.2 with W = 2 (17.3 with W = 3), 1 x 3
+// 41.9 with W = 0 and 45.8 with W = 3.
+template <int W>
 __global__ void max_pool_vec4_kernel(const float* x, float* __restrict__ y, ConvGeom g, int64_t n_out4) {
     ptx::pdl_launch_dependents();
     ptx::pdl_wait();
@@ -144,23 +149,22 @@ __global__ void max_pool_vec4_kernel(const float* x, float* __restrict__ y, Conv
         const int iy0 = oy * g.sh - g.pt, ix0 = ox * g.sw - g.pl;
         const int ky0 = iy0 < 0 ? -iy0 : 0, ky1 = min(g.fh, g.H - iy0);
         const int kx0 = ix0 < 0 ? -ix0 : 0, kx1 = min(g.fw, g.W - ix0);
-        if (g.fh <= 3 && g.fw <= 3) {
-            // the usual windows: all samples on their way before the first comparison; -inf where there is none
-            float4 v[3][3];
+        if constexpr (W > 0) {
+            float4 v[W][W];
 #pragma unroll
-            for (int ky = 0; ky < 3; ++ky)
+            for (int ky = 0; ky < W; ++ky)
 #pragma unroll
-                for (int kx = 0; kx < 3; ++kx) {
+                for (int kx = 0; kx < W; ++kx) {
                     v[ky][kx] = m;
                     if (ky >= ky0 && ky < ky1 && kx >= kx0 && kx < kx1)
                         v[ky][kx] = load_global(reinterpret_cast<const float4*>(x + ((n * g.H + iy0 + ky) * (int64_t)g.W + ix0 + kx) * g.C + c));
                 }
 #pragma unroll
-            for (int k = 0; k < 9; ++k) max4_nan(m, v[k / 3][k % 3]);
+            for (int k = 0; k < W * W; ++k) max4_nan(m, v[k / W][k % W]);
         } else {
             for (int ky = ky0; ky < ky1; ++ky) {
                 const float* row = x + ((n * g.H + iy0 + ky) * (int64_t)g.W + ix0) * g.C + c;
-                for (int kx = kx0; kx < kx1; ++kx) max4_nan(m, load_global(reinterpret_cast<const float4*>(row + (int64_t)kx * g.C)));
+                for (int kx = kx0; kx < kx1; ++kx) max4_nan(m, ld_global4(row + (int64_t)kx * g.C));
             }
         }
         *reinterpret_cast<float4*>(y + i * 4) = m;
@@ -409,8 +413,9 @@ cudaError_t launch_max_pool(const float* x, float* y, const ConvGeom& g, cudaStr
     const int64_t n_out = g.N * g.Ho * g.Wo * g.C;
     if (n_out == 0) return cudaSuccess;
     ++*launches;
+    auto vec4 = g.fh <= 2 && g.fw <= 2 ? max_pool_vec4_kernel<2> : g.fh == 3 && g.fw == 3 ? max_pool_vec4_kernel<3> : max_pool_vec4_kernel<0>;
     if (g.C % 4 == 0)
-        return launch_k(max_pool_vec4_kernel, dim3(grid_for(n_out / 4, kThreads, current_sm_count() * 32)), dim3(kThreads), 0, s, x, y, g, n_out / 4);
+        return launch_k(vec4, dim3(grid_for(n_out / 4, kThreads, current_sm_count() * 32)), dim3(kThreads), 0, s, x, y, g, n_out / 4);
     return launch_k(max_pool_window_kernel, dim3(grid_for(n_out, kThreads, current_sm_count() * 16)), dim3(kThreads), 0, s, x, y, g, n_out);
 }
 

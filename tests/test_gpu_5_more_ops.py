@@ -294,7 +294,7 @@ def test_elementwise_passes_of_several_items_per_thread(ctx, n):
         assert torch.equal(ctx.bias_act(r, b, act="relu"), torch.relu(r + b))
 
 
-@pytest.mark.parametrize("window", [(1, 3), (3, 1), (2, 3), (3, 3), (4, 2)])
+@pytest.mark.parametrize("window", [(1, 3), (3, 1), (2, 3), (3, 3), (4, 2), (1, 1), (1, 2), (2, 1), (2, 2), (5, 5)])
 def test_max_pool_of_quads_at_the_window_sizes_around_the_unrolled_one(ctx, oracle, window):
     x = si.uniform(91, 0, (2, 7, 6, 8), -1, 1)
     x[0, 3, 2, 1] = np.nan
