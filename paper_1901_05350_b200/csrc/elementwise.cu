@@ -63,10 +63,12 @@ __global__ void bias_act_scalar_kernel(const float* x, const float* bias, float*
 }
 
 // ---- avgPool ----------------------------------------------------------------------------------
+// The pools over windows let the next kernel start as they end, not before: blocks of it that wait beside the last ones of a
+// pool that is two waves of small blocks are spread unevenly over the SMs (one avgPool 3 x 3 after another, [64,112,112,64]
+// 812 us with an early start, 787 without; [8,33,35,36] / 2 5.0 and 3.5).
 // One thread per output element, channel fastest (coalesced).  Padding never counts.
 __global__ void avg_pool_window_kernel(const float* x, float* __restrict__ y, ConvGeom g,
                                        int64_t n_out) {
-    ptx::pdl_launch_dependents();
     ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_out; i += stride) {
@@ -96,7 +98,6 @@ __global__ void avg_pool_window_kernel(const float* x, float* __restrict__ y, Co
 // a NaN that is in the window.
 __global__ void max_pool_window_kernel(const float* x, float* __restrict__ y, ConvGeom g,
                                        int64_t n_out) {
-    ptx::pdl_launch_dependents();
     ptx::pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_out; i += stride) {
@@ -134,7 +135,6 @@ __device__ __forceinline__ void max4_nan(float4& m, const float4& v) {
 // 41.9 with W = 0 and 45.8 with W = 3.
 template <int W>
 __global__ void max_pool_vec4_kernel(const float* x, float* __restrict__ y, ConvGeom g, int64_t n_out4) {
-    ptx::pdl_launch_dependents();
     ptx::pdl_wait();
     const int C4 = g.C >> 2;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
