@@ -209,6 +209,11 @@ __global__ void binary_scalar_kernel(const float* a, const float* b, float* out,
         out[i] = binary_op<OP>(a[i], b[wrap(i, b_len)]);
 }
 
+// Global pools of more positions than this (2 us) are launched after the kernel before: early, their blocks, fewer than SMs as a
+// rule, are put several to an SM and share its bandwidth for as long as they run ([34,45,45,336], 102 blocks, 16.5 us and 37.6;
+// [59,79,79,64] 45 and 101; after a pointwise convolution of 100352 pixels the pair 76 and 155).
+constexpr int SHORT_POOL = 256;
+
 // Global pool: a block owns (image n, 128 consecutive channels).  Lane = 4 channels (one float4, so a
 // warp reads 512 contiguous bytes per position), the 8 warps stride over the H*W positions, partial
 // sums meet in shared memory.  C % 4 == 0.
@@ -217,7 +222,7 @@ __global__ void avg_pool_global_vec4_kernel(const float* x, float* __restrict__ 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = (blockIdx.x * 32 + lane) * 4;
     const int64_t n = blockIdx.y;
-    ptx::pdl_launch_dependents();
+    if (HW <= SHORT_POOL) ptx::pdl_launch_dependents();
     ptx::pdl_wait();
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (c < C) {
@@ -256,12 +261,20 @@ __global__ void avg_pool_global_kernel(const float* x, float* __restrict__ y, in
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = blockIdx.x * 32 + lane;
     const int64_t n = blockIdx.y;
-    ptx::pdl_launch_dependents();
+    if (HW <= SHORT_POOL) ptx::pdl_launch_dependents();
     ptx::pdl_wait();
     float acc = 0.0f;
     if (c < C) {
         const float* base = x + n * (int64_t)HW * C + c;
-        for (int p = warp; p < HW; p += 8) acc += base[(int64_t)p * C];
+        int p = warp;
+        for (; p + 56 < HW; p += 64) {  // eight loads in flight
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = load_global(base + (int64_t)(p + 8 * u) * C);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc += v[u];
+        }
+        for (; p < HW; p += 8) acc += load_global(base + (int64_t)p * C);
     }
     partial[warp][lane] = acc;
     __syncthreads();
@@ -404,9 +417,9 @@ cudaError_t launch_avg_pool(const float* x, float* y, const ConvGeom& g, cudaStr
                         g.N <= 65535;
     ++*launches;
     if (!global) return launch_k(avg_pool_window_kernel, dim3(grid_for(n_out, kThreads, current_sm_count() * 16)), dim3(kThreads), 0, s, x, y, g, n_out);
-    if (g.C % 4 == 0)
-        return launch_k(avg_pool_global_vec4_kernel, dim3((g.C / 4 + 31) / 32, (unsigned)g.N), dim3(256), 0, s, x, y, g.H * g.W, g.C);
-    return launch_k(avg_pool_global_kernel, dim3((g.C + 31) / 32, (unsigned)g.N), dim3(256), 0, s, x, y, g.H * g.W, g.C);
+    auto global_kernel = g.C % 4 == 0 ? avg_pool_global_vec4_kernel : avg_pool_global_kernel;
+    const dim3 grid(g.C % 4 == 0 ? (g.C / 4 + 31) / 32 : (g.C + 31) / 32, (unsigned)g.N);
+    return launch_k_if(g.H * g.W <= SHORT_POOL, global_kernel, grid, dim3(256), 0, s, x, y, g.H * g.W, g.C);
 }
 
 cudaError_t launch_max_pool(const float* x, float* y, const ConvGeom& g, cudaStream_t s, int64_t* launches) {

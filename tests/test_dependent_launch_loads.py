@@ -19,7 +19,7 @@ def sources():
 
 
 def launched_early(text):
-    return re.search(r"\blaunch_k\(|ProgrammaticStreamSerialization", text) is not None
+    return re.search(r"\blaunch_k(_if)?\(|ProgrammaticStreamSerialization", text) is not None
 
 
 @pytest.mark.parametrize("name,text", [(n, t) for n, t in sources() if n.endswith(".cu") and launched_early(t)], ids=lambda v: v if v.endswith(".cu") else "")

@@ -53,6 +53,16 @@ def test_avg_pool_parity(ctx, oracle, case):
     np.testing.assert_allclose(got, want, rtol=0, atol=2e-5)
 
 
+@pytest.mark.parametrize("C", [3, 130, 132])
+@pytest.mark.parametrize("hw", [(1, 57), (7, 9), (8, 8), (16, 16), (1, 257), (23, 29)])
+def test_global_pools_of_few_and_many_positions(ctx, oracle, hw, C):
+    """Short ones are launched while the kernel before runs, longer ones after it; the eight warps' shares are whole batches of
+    loads, more or fewer.  The pool reads what the call before writes."""
+    x = si.uniform(113, 0, (3, *hw, C), 0, 6)
+    got = host(ctx.avg_pool(ctx.binary("add", dev(x), dev(x)), hw, hw))
+    np.testing.assert_allclose(got, oracle.avg_pool(x + x, hw, hw, "valid"), rtol=0, atol=4e-5)  # sums of 667 values up to 12
+
+
 @pytest.mark.parametrize("shape", [(1, 1000), (128, 1000), (7, 33), (3, 5, 17), (4097,), (2, 2, 2, 300)])
 def test_softmax_parity(ctx, oracle, shape):
     x = si.normal(104, 0, shape, 0, 3)
