@@ -63,7 +63,7 @@ def test_global_pools_of_few_and_many_positions(ctx, oracle, hw, C):
     np.testing.assert_allclose(got, oracle.avg_pool(x + x, hw, hw, "valid"), rtol=0, atol=4e-5)  # sums of 667 values up to 12
 
 
-@pytest.mark.parametrize("shape", [(1, 1000), (128, 1000), (7, 33), (3, 5, 17), (4097,), (2, 2, 2, 300)])
+@pytest.mark.parametrize("shape", [(1, 1000), (128, 1000), (7, 33), (3, 5, 17), (4097,), (2, 2, 2, 300), (3, 4096)])
 def test_softmax_parity(ctx, oracle, shape):
     x = si.normal(104, 0, shape, 0, 3)
     got = host(ctx.softmax(dev(x)))
