@@ -290,7 +290,10 @@ depthwise_backprop_input_kernel(const float* dy, const float* f, float* __restri
                 if (ox < 0) continue;
                 const float* gp = dy + ((n * g.Ho + oy) * (int64_t)g.Wo + ox) * g.Co + (int64_t)c * g.mult;
                 const float* fp = f + ((int64_t)(ky * g.fw + kx) * g.C + c) * g.mult;
-                for (int q = 0; q < g.mult; ++q) acc = fmaf(load_global(gp + q), load_global(fp + q), acc);
+                // the first apart: with it in the loop the taps' loads come one after the other (5 x 5 over [8,56,56,64] 147 us
+                // for 120, and 136 with read-only loads)
+                acc = fmaf(load_global(gp), load_global(fp), acc);
+                for (int q = 1; q < g.mult; ++q) acc = fmaf(load_global(gp + q), load_global(fp + q), acc);
             }
         }
         dx[e] = acc;
