@@ -527,6 +527,7 @@ tfjsb_status tfjsb_depthwise_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const
     if (numel(out) == 0) return TFJSB_OK;
     DepthwisePlan plan;
     if ((st = depthwise_plan(ctx, static_cast<const float*>(x->data), g, &plan)) != TFJSB_OK) return st;
+    plan.next_early = false;
     cudaError_t e = launch_depthwise(plan, static_cast<const float*>(x->data), static_cast<const float*>(filter->data),
                                      bias ? static_cast<const float*>(bias->data) : nullptr, act,
                                      static_cast<float*>(out->data), g, ctx->dev_status,
@@ -794,6 +795,7 @@ tfjsb_status tfjsb_depthwise_conv2d_backprop_input(tfjsb_ctx* ctx, const tfjsb_t
         const ConvGeom t = depthwise_backprop_geometry(g);
         DepthwisePlan plan;
         if ((st = depthwise_plan(ctx, dy->data, t, &plan)) != TFJSB_OK) return st;
+        plan.next_early = false;
         e = launch_depthwise(plan, static_cast<const float*>(dy->data), static_cast<const float*>(filter->data), nullptr,
                              TFJSB_ACT_NONE, static_cast<float*>(dx->data), t, ctx->dev_status, static_cast<cudaStream_t>(stream),
                              &ctx->launches);

@@ -217,6 +217,7 @@ struct DwTiling {
     int tiles_x, tiles_y, c_blocks, stages;
     long long num_tiles;
     int f_step;  // from one tap of the filter to the next: C, or -C with f at the last tap (the taps reversed)
+    int next_early;  // see DepthwisePlan
 };
 
 template <int S, int TW, int R, int D = 1, int CB = DW_CB, bool NARROW = false>
@@ -264,7 +265,7 @@ depthwise3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const float* 
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
     }
     __syncthreads();
-    ptx::pdl_launch_dependents();
+    if (t.next_early) ptx::pdl_launch_dependents();
     ptx::pdl_wait();  // the input is the previous kernel's output
 
     const int num_tiles = (int)t.num_tiles;
@@ -451,7 +452,7 @@ cudaError_t launch_tma_instance(const DepthwisePlan& plan, const float* x, const
     }
     cudaError_t ae = smem_attr_once(reinterpret_cast<const void*>(kernel), DW_SMEM_BUDGET);
     if (ae != cudaSuccess) return ae;
-    DwTiling t{plan.tiles_x, plan.tiles_y, plan.c_blocks, plan.stages, (long long)plan.num_tiles, g.reversed ? -g.C : g.C};
+    DwTiling t{plan.tiles_x, plan.tiles_y, plan.c_blocks, plan.stages, (long long)plan.num_tiles, g.reversed ? -g.C : g.C, plan.next_early};
     if (g.reversed) f += 8 * (int64_t)g.C;
     return launch_k(kernel, dim3(plan.grid), dim3(DW_TMA_THREADS), plan.smem_bytes, s, plan.map_x, x, f, bias, act, y,
                     y_f32 ? 1 : 0, g, t, dev_status);
