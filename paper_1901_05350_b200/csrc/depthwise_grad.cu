@@ -88,8 +88,7 @@ depthwise3x3_backprop_filter_kernel(const __grid_constant__ CUtensorMap map_x, c
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    ptx::pdl_launch_dependents();
-    ptx::pdl_wait();
+    ptx::pdl_wait();  // (the next kernel starts as this one ends: two CTAs fit an SM, see DepthwisePlan)
     const int first = blockIdx.x, step = gridDim.x;  // step is a multiple of the channel blocks
     const int my_tiles = first < t.num_tiles ? (t.num_tiles - first + step - 1) / step : 0;
     const int cb = first % t.c_blocks;
