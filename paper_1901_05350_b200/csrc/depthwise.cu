@@ -443,6 +443,19 @@ constexpr DwVariant kDwVariants[] = {
 constexpr int DW_FIRST_NARROW = 8;
 constexpr int DW_SMEM_BUDGET = 113 * 1024;  // two CTAs per SM
 
+// What a stride-1 layer in fp32 storage takes, in microseconds, fitted to the same shapes (nine in ten within 15 %): a start, the rounds
+// of two tiles per SM, begun and on average, and what of both tensors does not stay in L2.
+struct DwTileCost {
+    double start, round, part, mb;
+};
+constexpr DwTileCost kDw8x8x64{3.1, 0.51, 0.44, 0.119}, kDw16x7x64{2.9, 0.78, 0.98, 0.081};
+constexpr DwTileCost kDw8x8x32{3.1, 0.65, 0.03, 0.030}, kDw16x14x32{2.8, 1.05, 0.88, 0.063};
+double tiles_us(const DwTileCost& c, int64_t tiles, const ConvGeom& g, int sm_count) {
+    const int64_t pair = 2 * (int64_t)sm_count;
+    const double mb = (double)g.N * g.H * g.W * g.C * 8e-6 - 120;
+    return c.start + c.round * (double)((tiles + pair - 1) / pair) + c.part * (double)tiles / pair + (mb > 0 ? c.mb * mb : 0);
+}
+
 template <int S, int TW, int R, int D = 1, int CB = DW_CB, bool NARROW = false>
 cudaError_t launch_tma_instance(const DepthwisePlan& plan, const float* x, const float* f, const float* bias, int act, void* y, bool y_f32,
                                 const ConvGeom& g, unsigned int* dev_status, cudaStream_t s) {
@@ -512,25 +525,31 @@ tfjsb_status depthwise_plan(tfjsb_ctx* ctx, const void* x, const ConvGeom& g, De
         // 124.3 -> 120.2 us, 125.8 -> 124.0, 132.8 -> 129.9; at batch 16 in every layer 169.6 -> 180)
         if (g.sh == 1 && (g.C % 64 == 0 ? tiles8 * (g.C / 64) < ctx->sm_count : tiles8 * blocks32 < 6 * (int64_t)ctx->sm_count)) v = DW_FIRST_NARROW + 5;
     } else {
-        // Stride 1.  8 x 8 tiles of 32 channels while an SM would not have one of 64: a short layer takes what one tile takes
+        // Stride 1.  8 x 8 tiles of 32 channels while an SM would not have one tile: a short layer takes what one tile takes
         // (copy, rows, stores), and its rows per thread are 2 instead of 4 or 7 ([1,56,56,128] 4.1 -> 3.0 us, [1,14,14,512]
-        // 3.3 -> 2.9, [4,14,14,512] 3.8 -> 3.2; against 16 x 7 tiles, as all below).  They also read DRAM faster where the
-        // tensors do not stay in L2 and a pixel is 512 bytes or less ([128,56,56,128] 73.4 -> 66.3, [100,112,112,64] 116 -> 100;
-        // but [128,28,28,256] 36.7 and 39.6).  Otherwise 8 x 8 of 64 channels where they take fewer rounds of two tiles per SM, at half
-        // the time of one of 16 x 7 ([8,17,17,512] 5.9 -> 4.6, [32,56,56,128] 18.8 -> 17.1, [64,14,14,512] 9.5 -> 9.1), else
-        // 16 x 7 ([128,28,28,256] 36.7 and 37.1, [32,14,14,512] 6.1 and 6.2).
-        // Channels that are no multiple of 64: 8 x 8 up to 24 tiles per SM ([8,112,112,32] 6.8 -> 6.0, [16,112,112,32] 9.7 -> 9.2),
-        // then 16 x 14 ([32,112,112,32] 17.8 and 18.7 with 8 x 8).
+        // 3.3 -> 2.9; against 16 x 7 tiles, as all below).  They also read DRAM faster where the tensors do not stay in L2 and a
+        // pixel is 512 bytes or less ([128,56,56,128] 73.4 -> 66.3, [100,112,112,64] 116 -> 100).  Otherwise the tiles of earlier
+        // planning, 16 x 7 of 64 channels and 16 x 14 of 32, unless 8 x 8 of as many channels are 5 % ahead by the estimates:
+        // of 360 shapes, 32 to 1024 channels of 7 to 128 squared, 10 more than 2 % slower than without 8 x 8, 0.98 of the time on
+        // average.  ([32,56,56,128] 18.8 -> 17.1, [8,17,17,512] 5.9 -> 4.6; but [18,68,68,512] would be 66.4 for 55.8,
+        // [40,10,10,768] 9.5 for 7.3, [54,13,13,424] 10.0 for 7.9.)
         const bool beyond_l2 = (double)g.N * g.H * g.W * g.C * 8.0 > 1.5e8;  // both tensors
-        const int64_t pair = 2 * (int64_t)ctx->sm_count;
-        const int64_t rounds8 = (tiles8 * (g.C / 64) + pair - 1) / pair;
-        const int64_t rounds16 = (g.N * ((g.Wo + 15) / 16) * ((g.Ho + 6) / 7) * (g.C / 64) + pair - 1) / pair;
-        if (g.sh == 1 && g.C % 64 == 0) v = tiles8 * (g.C / 64) < ctx->sm_count || (g.C <= 128 && beyond_l2) ? 1 : rounds8 < 2 * rounds16 ? 6 : 16;
-        else if (g.sh == 1) v = g.Wo <= 8 || tiles8 * blocks32 <= 24 * (int64_t)ctx->sm_count ? 1 : 0;
-        // stride 2: 64-channel tiles are 8 outputs wide, so they are taken only where that wastes fewer columns than the
-        // 16-wide 32-channel ones ([128,112,112,64] 90.1 -> 86.9 us; [128,28,28,256] ran 27.3 -> 29.1 with them)
-        else if (g.C % 64 == 0 && wide8) v = 7;
-        else v = g.Wo <= 8 ? 3 : 2;
+        const bool whole64 = g.C % 64 == 0;
+        const int64_t blocks = whole64 ? g.C / 64 : blocks32;
+        const int64_t wide = g.N * ((g.Wo + 15) / 16) * ((g.Ho + (whole64 ? 6 : 13)) / (whole64 ? 7 : 14)) * blocks;
+        auto ahead = [&](const DwTileCost& narrow_tiles, const DwTileCost& wide_tiles) {
+            return tiles_us(narrow_tiles, tiles8 * blocks, g, ctx->sm_count) < 0.95 * tiles_us(wide_tiles, wide, g, ctx->sm_count);
+        };
+        if (g.sh == 1 && whole64) {
+            if (tiles8 * blocks < ctx->sm_count || (g.C <= 128 && beyond_l2)) v = 1;
+            else v = g.Wo <= 8 || ahead(kDw8x8x64, kDw16x7x64) ? 6 : 16;
+        } else if (g.sh == 1) {
+            v = g.Wo <= 8 || tiles8 * blocks < ctx->sm_count || ahead(kDw8x8x32, kDw16x14x32) ? 1 : 0;
+        } else {
+            // stride 2: 64-channel tiles are 8 outputs wide, so they are taken only where that wastes fewer columns than the
+            // 16-wide 32-channel ones ([128,112,112,64] 90.1 -> 86.9 us; [128,28,28,256] ran 27.3 -> 29.1 with them)
+            v = whole64 && wide8 ? 7 : g.Wo <= 8 ? 3 : 2;
+        }
     }
     const DwVariant& d = kDwVariants[v];
     const cuuint64_t eb = narrow ? 2u : 4u;
