@@ -311,6 +311,7 @@ static tfjsb_status matmul_2d(tfjsb_ctx* ctx, const float* pa, const float* pb, 
         }
         GemmTf32Plan plan;
         if ((st = gemm_tf32_plan(ctx, a_tc, pb, pc, M, N, K, &plan, 1, a_mn, !transpose_b)) != TFJSB_OK) return st;
+        plan.next_early = false;
         if ((e = launch_gemm_tf32(plan, nullptr, TFJSB_ACT_NONE, ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
             return cuda_fail(ctx, e, "tf32 gemm launch");
         return TFJSB_OK;
@@ -408,6 +409,7 @@ tfjsb_status tfjsb_batch_matmul(tfjsb_ctx* ctx, const tfjsb_tensor* a, const tfj
         }
         GemmTf32Plan plan;
         if ((st = gemm_tf32_plan(ctx, a_tc, pb, pc, M, N, K, &plan, B, a_mn, !transpose_b)) != TFJSB_OK) return st;
+        plan.next_early = false;
         if ((e = launch_gemm_tf32(plan, nullptr, TFJSB_ACT_NONE, ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
             return cuda_fail(ctx, e, "batched tf32 gemm launch");
         return TFJSB_OK;
@@ -461,6 +463,7 @@ tfjsb_status tfjsb_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_ten
         if (ctx->math == TFJSB_MATH_TF32 && gemm_tf32_supported(M, N, K) && ctx->encode_tiled) {
             GemmTf32Plan plan;
             if ((st = gemm_tf32_plan(ctx, px, pf, py, M, N, K, &plan, 1, false, true)) != TFJSB_OK) return st;
+            plan.next_early = false;
             if ((e = launch_gemm_tf32(plan, pbias, act, ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
                 return cuda_fail(ctx, e, "tf32 gemm launch");
             return TFJSB_OK;
@@ -754,6 +757,7 @@ tfjsb_status tfjsb_conv2d_backprop_filter(tfjsb_ctx* ctx, const tfjsb_tensor* x,
             GemmTf32Plan plan;
             float* target = B > 1 ? ctx->scratch_c.ptr : pdf;
             if ((st = gemm_tf32_plan(ctx, ctx->scratch_a.ptr, ctx->scratch_b.ptr, target, g.C, g.Co, Ms, &plan, B)) != TFJSB_OK) return st;
+            plan.next_early = false;
             if ((e = launch_gemm_tf32(plan, nullptr, TFJSB_ACT_NONE, ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
                 return cuda_fail(ctx, e, "tf32 gemm launch");
             if (B > 1 && (e = launch_sum_rows(ctx->scratch_c.ptr, pdf, nullptr, B, (int64_t)g.C * g.Co, 1, s, &ctx->launches)) != cudaSuccess)

@@ -304,6 +304,7 @@ struct GemmTf32Plan {
     // cluster split-K kernel (gemm_tf32_splitk.cu): `splits` CTAs per tile, reduced through shared memory
     bool cluster_split = false;
     int splits = 1, kb_per_split = 0;  // slices of the K loop (= cluster size) and k-blocks per slice
+    bool next_early = true;            // of the cluster kernel, whose CTAs may share an SM: see DepthwisePlan
     float* c = nullptr;                // C, which that kernel stores directly
     // implicit-GEMM convolution: A is gathered from x by the kernel instead of copied, or copied by im2col loads
     bool gather = false;

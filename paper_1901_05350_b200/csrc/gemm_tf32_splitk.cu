@@ -53,6 +53,7 @@ struct SplitArgs {
     int stage_tx;      // bytes that the copies of one stage deliver
     int a_mn, b_mn;    // operands stored [K, M] / [K, N] (the instance with MN only)
     int a_groups;      // copies of 32 k x 32 rows that make the A tile (a_mn)
+    int next_early;    // see GemmTf32Plan
     const float* bias;
     int act;
     float* c;
@@ -133,7 +134,7 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
     // partners.  Each thread completes it (cluster_wait) where it next needs it: warps 2-5 before
     // their first remote store, warps 0-1 at the end of their role, before arriving at the second barrier.
     cluster_arrive();
-    pdl_launch_dependents();
+    if (args.next_early) pdl_launch_dependents();
     pdl_wait();
 
     if (warp == 0) {
@@ -248,6 +249,7 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
     }
 
     // ---------------------------------------------------------------- reduction of this CTA's band
+    if (!args.next_early) pdl_launch_dependents();
     tc_fence_before();
     __syncthreads();
     cluster_arrive();   // this CTA's stores into its partners' shared memory are done ...
@@ -395,6 +397,7 @@ cudaError_t launch_gemm_tf32_splitk(const GemmTf32Plan& plan, const float* bias,
     args.b_mn = plan.b_mn;
     args.a_groups = plan.M >= BLOCK_M ? BLOCK_M / 32 : (int)((plan.M + 31) / 32);
     args.stage_tx = (plan.a_mn ? args.a_groups * 32 : a_box_rows(plan.M)) * 128 + plan.block_n * 128;
+    args.next_early = plan.next_early;
     args.bias = bias;
     args.act = act;
     args.c = plan.c;

@@ -116,6 +116,7 @@ extern "C" tfjsb_status tfjsb_matmul_static_scratch(tfjsb_ctx* ctx, const tfjsb_
         }
         GemmTf32Plan plan;
         tfjsb_status st = gemm_tf32_plan(ctx, a_km, b_km, pc, M, N, K, &plan);
+        plan.next_early = false;
         if (st != TFJSB_OK) return st;
         if ((e = launch_gemm_tf32(plan, nullptr, TFJSB_ACT_NONE, ctx->dev_status, s, &ctx->launches)) != cudaSuccess)
             return cuda_fail(ctx, e, "tf32 gemm launch");
