@@ -426,21 +426,21 @@ constexpr DwVariant kDwVariants[] = {
     DW_VARIANT(1, 16, 4, 2, 32, false),   // 4: stride 1, dilation 2
     DW_VARIANT(1, 16, 4, 4, 32, false),   // 5: stride 1, dilation 4
     // fp32, 64 channels per tile (256-byte lines): half as many box rows for the copy unit per byte moved
-    DW_VARIANT(1, 8, 4, 1, 64, false),    // 6: stride 1, 8 x 8 outputs (a whole 7 x 7 image per tile)
-    DW_VARIANT(2, 8, 2, 1, 64, false),    // 7: stride 2, 8 outputs wide
+    DW_VARIANT(1, 16, 7, 1, 64, false),   // 6: stride 1
+    DW_VARIANT(1, 8, 4, 1, 64, false),    // 7: stride 1, 8 x 8 outputs (a whole 7 x 7 image per tile)
+    DW_VARIANT(2, 8, 2, 1, 64, false),    // 8: stride 2, 8 outputs wide
     // bfloat16 storage: the same tiles on 2-byte values, 64 channels (one 128-byte line) then 32
-    DW_VARIANT(1, 16, 7, 1, 64, true),    // 8
-    DW_VARIANT(1, 8, 4, 1, 64, true),     // 9
-    DW_VARIANT(2, 16, 2, 1, 64, true),    // 10
-    DW_VARIANT(2, 8, 2, 1, 64, true),     // 11
-    DW_VARIANT(1, 16, 7, 1, 32, true),    // 12
-    DW_VARIANT(1, 8, 2, 1, 32, true),     // 13
-    DW_VARIANT(2, 16, 2, 1, 32, true),    // 14
-    DW_VARIANT(2, 8, 2, 1, 32, true),     // 15
-    DW_VARIANT(1, 16, 7, 1, 64, false),   // 16: fp32, stride 1, 16 x 7 outputs of 64 channels
+    DW_VARIANT(1, 16, 7, 1, 64, true),    // 9
+    DW_VARIANT(1, 8, 4, 1, 64, true),     // 10
+    DW_VARIANT(2, 16, 2, 1, 64, true),    // 11
+    DW_VARIANT(2, 8, 2, 1, 64, true),     // 12
+    DW_VARIANT(1, 16, 7, 1, 32, true),    // 13
+    DW_VARIANT(1, 8, 2, 1, 32, true),     // 14
+    DW_VARIANT(2, 16, 2, 1, 32, true),    // 15
+    DW_VARIANT(2, 8, 2, 1, 32, true),     // 16
 };
 #undef DW_VARIANT
-constexpr int DW_FIRST_NARROW = 8;
+constexpr int DW_FIRST_NARROW = 9, DW_LAST = 16;
 constexpr int DW_SMEM_BUDGET = 113 * 1024;  // two CTAs per SM
 
 // What a stride-1 layer in fp32 storage takes, in microseconds, fitted to the same shapes (nine in ten within 15 %): a start, the rounds
@@ -481,17 +481,17 @@ cudaError_t launch_tma_variant(const DepthwisePlan& plan, const float* x, const 
         DW_CASE(3, 2, 8, 2, 1, 32, false);
         DW_CASE(4, 1, 16, 4, 2, 32, false);
         DW_CASE(5, 1, 16, 4, 4, 32, false);
-        DW_CASE(6, 1, 8, 4, 1, 64, false);
-        DW_CASE(7, 2, 8, 2, 1, 64, false);
-        DW_CASE(8, 1, 16, 7, 1, 64, true);
-        DW_CASE(9, 1, 8, 4, 1, 64, true);
-        DW_CASE(10, 2, 16, 2, 1, 64, true);
-        DW_CASE(11, 2, 8, 2, 1, 64, true);
-        DW_CASE(12, 1, 16, 7, 1, 32, true);
-        DW_CASE(13, 1, 8, 2, 1, 32, true);
-        DW_CASE(14, 2, 16, 2, 1, 32, true);
-        DW_CASE(15, 2, 8, 2, 1, 32, true);
-        DW_CASE(16, 1, 16, 7, 1, 64, false);
+        DW_CASE(6, 1, 16, 7, 1, 64, false);
+        DW_CASE(7, 1, 8, 4, 1, 64, false);
+        DW_CASE(8, 2, 8, 2, 1, 64, false);
+        DW_CASE(9, 1, 16, 7, 1, 64, true);
+        DW_CASE(10, 1, 8, 4, 1, 64, true);
+        DW_CASE(11, 2, 16, 2, 1, 64, true);
+        DW_CASE(12, 2, 8, 2, 1, 64, true);
+        DW_CASE(13, 1, 16, 7, 1, 32, true);
+        DW_CASE(14, 1, 8, 2, 1, 32, true);
+        DW_CASE(15, 2, 16, 2, 1, 32, true);
+        DW_CASE(16, 2, 8, 2, 1, 32, true);
         default: return cudaErrorInvalidValue;
     }
 #undef DW_CASE
@@ -542,14 +542,20 @@ tfjsb_status depthwise_plan(tfjsb_ctx* ctx, const void* x, const ConvGeom& g, De
         };
         if (g.sh == 1 && whole64) {
             if (tiles8 * blocks < ctx->sm_count || (g.C <= 128 && beyond_l2)) v = 1;
-            else v = g.Wo <= 8 || ahead(kDw8x8x64, kDw16x7x64) ? 6 : 16;
+            else v = g.Wo <= 8 || ahead(kDw8x8x64, kDw16x7x64) ? 7 : 6;
         } else if (g.sh == 1) {
             v = g.Wo <= 8 || tiles8 * blocks < ctx->sm_count || ahead(kDw8x8x32, kDw16x14x32) ? 1 : 0;
         } else {
             // stride 2: 64-channel tiles are 8 outputs wide, so they are taken only where that wastes fewer columns than the
             // 16-wide 32-channel ones ([128,112,112,64] 90.1 -> 86.9 us; [128,28,28,256] ran 27.3 -> 29.1 with them)
-            v = whole64 && wide8 ? 7 : g.Wo <= 8 ? 3 : 2;
+            v = whole64 && wide8 ? 8 : g.Wo <= 8 ? 3 : 2;
         }
+    }
+    if (const char* env = dilated ? nullptr : getenv("TFJSB_DW_TILES")) {  // for tests: this instance, or an error
+        v = atoi(env);
+        const bool of_format = narrow ? v >= DW_FIRST_NARROW && v <= DW_LAST : v >= 0 && v < DW_FIRST_NARROW && v != 4 && v != 5;
+        if (!of_format || kDwVariants[v].S != g.sh || (kDwVariants[v].cb == 64 && g.C % 64 != 0))
+            return fail(ctx, TFJSB_ERR_UNSUPPORTED, "TFJSB_DW_TILES names no instance for this layer");
     }
     const DwVariant& d = kDwVariants[v];
     const cuuint64_t eb = narrow ? 2u : 4u;

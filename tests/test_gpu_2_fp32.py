@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 
 import seeded_inputs as si
-from helpers import dev, host, rel_fro, same_bits
+from helpers import dev, host, plant_specials, rel_fro, same_bits, same_classes
 
 pytestmark = pytest.mark.gpu
 
@@ -155,10 +155,40 @@ def test_depthwise_shifted_delta_taps_on_gpu(ctx):
 
 @pytest.mark.parametrize("case", [(1, 14, 14, 128), (2, 9, 8, 64), (3, 17, 33, 64), (18, 17, 17, 128), (1, 8, 40, 96), (1, 7, 7, 192), (40, 74, 70, 32)])
 def test_depthwise_3x3_tiles(ctx, oracle, case):
-    """Stride 1: 8 x 8 tiles of 32 channels and of 64, and 16 x 14 of 32, which the number of tiles chooses between, with rows
-    and columns left over."""
+    """Stride 1, the tiles that the planner chooses, with rows and columns left over."""
     N, H, W, C = case
     x, f, b = si.uniform(341, 0, (N, H, W, C), 0, 6), si.normal(341, 1, (3, 3, C, 1), 0, 0.5), si.normal(341, 2, (C,), 0, 0.1)
     got = host(ctx.depthwise_conv2d(dev(x), dev(f), (1, 1), "same", bias=dev(b), act="relu6"))
     ctx.check_device_status()
     assert rel_fro(got, oracle.depthwise_conv2d(x, f, (1, 1), "same", bias=b, act="relu6")) <= 1e-6
+
+
+RAGGED_64 = [(2, 21, 37, 128), (3, 13, 20, 64), (3, 7, 7, 192), (2, 11, 6, 64), (40, 9, 17, 128)]  # the last: several tiles per CTA
+RAGGED_32 = [(2, 21, 37, 40), (3, 13, 20, 96), (3, 7, 7, 36), (1, 9, 40, 32), (60, 15, 17, 68)]
+
+
+@pytest.mark.parametrize("instance,stride,case", [(v, 1, c) for v in (6, 7) for c in RAGGED_64] + [(v, 1, c) for v in (0, 1) for c in RAGGED_32 + RAGGED_64[:2]] +
+                         [(8, 2, c) for c in RAGGED_64] + [(v, 2, c) for v in (2, 3) for c in RAGGED_32])
+def test_every_depthwise_tile(ctx, oracle, monkeypatch, instance, stride, case):
+    """Each instance of the pipelined kernel in fp32 storage on sizes that its tiles do not divide, whichever the planner takes there:
+    the forward pass and, at stride 1, the input gradient, also with a filter that is not finite."""
+    monkeypatch.setenv("TFJSB_DW_TILES", str(instance))
+    N, H, W, C = case
+    x, f = si.small_integers(342, 0, (N, H, W, C), -8, 8), si.small_integers(342, 1, (3, 3, C, 1), -8, 8)
+    assert same_bits(host(ctx.depthwise_conv2d(dev(x), dev(f), (stride, stride), "same")), oracle.depthwise_conv2d(x, f, (stride, stride), "same"))
+    if stride == 1:
+        got = host(ctx.depthwise_conv2d_backprop_input(x.shape, dev(f), dev(x)))
+        assert same_bits(got + 0.0, oracle.depthwise_conv2d_backprop_input(x.shape, f, x, (1, 1), "same") + 0.0)
+        f, g = plant_specials(si.normal(343, 1, f.shape, 0, 0.3), 6, (0, f.size - 1)), si.normal(343, 2, x.shape, 0, 0.5)
+        got = host(ctx.depthwise_conv2d_backprop_input(x.shape, dev(f), dev(g)))
+        assert same_classes(got, oracle.depthwise_conv2d_backprop_input(x.shape, f, g, (1, 1), "same"))
+    ctx.check_device_status()
+
+
+def test_a_depthwise_tile_that_does_not_fit_is_refused(ctx, tfjsb, monkeypatch):
+    x, f = si.uniform(344, 0, (1, 9, 9, 40), -1, 1), si.uniform(344, 1, (3, 3, 40, 1), -1, 1)
+    for instance in ("6", "2", "9", "17", "-1"):  # 64 channels, stride 2, bfloat16 storage, none
+        monkeypatch.setenv("TFJSB_DW_TILES", instance)
+        with pytest.raises(tfjsb.TfjsbError) as e:
+            ctx.depthwise_conv2d(dev(x), dev(f))
+        assert e.value.status_name == "UNSUPPORTED"

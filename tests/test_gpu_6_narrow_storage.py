@@ -364,7 +364,7 @@ def test_depthwise_as_last_layer_narrow_writes_fp32(ctx, oracle):
 
 
 NARROW_DEPTHWISE = [
-    # N, H, W, C, stride: one case per instance of the pipelined depthwise kernel in the narrow format
+    # N, H, W, C, stride: the pipelined depthwise kernel in the narrow format, tiles as the planner takes them
     (2, 21, 37, 128, 1),   # 64-channel tiles, large stride-1 image, ragged tiles both ways
     (3, 13, 20, 64, 1),    # 9..14 rows: two tiles down
     (3, 7, 7, 192, 1),     # whole 7 x 7 image per tile, three channel blocks
@@ -551,3 +551,12 @@ def test_narrow_mode_rejects_layers_it_does_not_have(ctx, tfjsb):
     assert e.value.status_name == "UNSUPPORTED"
     # the context is left in its default mode and still builds the default model
     ctx.model(layers, x.shape).close()
+
+
+@pytest.mark.parametrize("instance,case", [(v, c) for v in (9, 10) for c in NARROW_DEPTHWISE[:4]] + [(v, c) for v in (11, 12) for c in NARROW_DEPTHWISE[4:6]] +
+                         [(v, c) for v in (13, 14) for c in NARROW_DEPTHWISE[6:9] + NARROW_DEPTHWISE[:2]] +
+                         [(v, c) for v in (15, 16) for c in NARROW_DEPTHWISE[9:11]])
+def test_every_narrow_depthwise_tile(ctx, oracle, monkeypatch, instance, case):
+    """Each instance in this format, whichever the planner takes for these sizes."""
+    monkeypatch.setenv("TFJSB_DW_TILES", str(instance))
+    test_depthwise_pipelined_kernel_narrow(ctx, oracle, case)
