@@ -455,7 +455,7 @@ cudaError_t launch_gemm_strided(const float* a, int64_t a_rs, int64_t a_ks, cons
                                 unsigned int* dev_status, cudaStream_t s, int64_t* launches) {
     if (M == 0 || N == 0 || batches == 0) return cudaSuccess;
     const Choice ch = choose(batches, M, N, K, sm_count);
-    const bool aligned = K % 4 == 0 && (batches == 1 || (M * K % 4 == 0 && K * N % 4 == 0));
+    const bool aligned = K % 4 == 0;  // and so are the products of a batch
     const bool a_quads = aligned && a_ks == 1 && a_rs % 4 == 0 && (reinterpret_cast<uintptr_t>(a) & 15u) == 0;
     const bool b_quads = aligned && b_ks == 1 && b_cs % 4 == 0 && (reinterpret_cast<uintptr_t>(b) & 15u) == 0;
     const Side sa{a, (int)a_rs, (int)a_ks, (int)M, a_quads, M * K}, sb{b, (int)b_cs, (int)b_ks, (int)N, b_quads, K * N};

@@ -361,7 +361,8 @@ IM2COL_CASES = [
 
 
 @pytest.mark.parametrize("case", IM2COL_CASES)
-def test_conv2d_im2col_copies(ctx, oracle, case):
+def test_conv2d_im2col_copies(ctx, oracle, monkeypatch, case):
+    monkeypatch.setenv("TFJSB_CONV_PATCH", "0")  # which would take some of these
     N, H, W, Cin, fh, fw, Cout, strides, pad, dil = case
     K = fh * fw * Cin
     xi = si.small_integers(315, 0, (N, H, W, Cin), -4, 4)   # |sums| <= 16 K < 2^24: exact in any order
@@ -455,7 +456,9 @@ def test_conv2d_from_patches(ctx, oracle, monkeypatch, case):
     monkeypatch.setenv("TFJSB_CONV_PATCH", "1")
     x, f, b = si.small_integers(331, 0, (N, H, W, Cin), -3, 3), si.small_integers(331, 1, (fh, fw, Cin, Cout), -3, 3), si.small_integers(331, 2, (Cout,), -9, 9)
     for act in ("none", "relu6"):
+        before = ctx.launch_count
         got = host(ctx.conv2d(dev(x), dev(f), (1, 1), pad, (d, d), bias=dev(b), act=act))
+        assert ctx.launch_count == before + 1  # the other kernels for these shapes pack the filter first
         ctx.check_device_status()
         assert same_bits(got + 0.0, oracle.conv2d(x, f, (1, 1), pad, (d, d), bias=b, act=act) + 0.0)
     x, f = si.uniform(332, 0, x.shape, -1, 1), si.normal(332, 1, f.shape, 0, 0.2)
@@ -465,10 +468,10 @@ def test_conv2d_from_patches(ctx, oracle, monkeypatch, case):
     assert rel_fro(got, oracle.conv2d(x, f, (1, 1), pad, (d, d), operand="tf32_rz")) <= MATCHED_TOL
 
 
-@pytest.mark.parametrize("case", [(1, 130, 36, 65), (1, 127, 4, 3), (1, 33, 100, 201), (3, 50, 64, 51), (5, 199, 68, 70), (3, 9, 20, 7), (1, 64, 1024, 101)])
+@pytest.mark.parametrize("case", [(1, 130, 36, 65), (1, 127, 4, 3), (1, 33, 100, 201), (3, 50, 64, 51), (5, 199, 68, 70), (3, 9, 20, 7), (1, 64, 1024, 101), (3, 50, 63, 51)])
 def test_unaligned_products_with_rows_of_whole_quads(ctx, oracle, case):
-    """K a multiple of 4 and N odd: K-contiguous operands are fetched four k at a time, of a batch only where every product
-    starts on 16 bytes, and the last k-block ends inside a row of tiles."""
+    """K a multiple of 4 and N odd: K-contiguous operands are fetched four k at a time, of a batch too, whose products then
+    start on 16 bytes, and the last k-block ends inside a row of tiles.  Beside them a batch whose K is no multiple of 4."""
     b, m, k, n = case
     for ta, tb in ((False, True), (False, False), (True, True)):
         x, y = si.uniform(333, 0, (b, m, k), -1, 1), si.uniform(333, 1, (b, k, n), -1, 1)

@@ -427,6 +427,11 @@ def test_conv2d_input_gradient_from_patches(ctx, oracle, monkeypatch, case):
     assert same_bits(got + 0.0, oracle.conv2d_backprop_input(shape, f, g, *args) + 0.0)
     f, g = si.normal(99, 3, f.shape, 0, 0.2), si.normal(99, 4, g.shape, 0, 1)
     got = host(ctx.conv2d_backprop_input(shape, dev(f), dev(g), *args))
+    if Cout > 32:  # sums over channels first and taps second, not the other way round: other bits than the other kernel's
+        with monkeypatch.context() as m:
+            m.setenv("TFJSB_CONV_PATCH", "0")
+            m.setenv("TFJSB_GRAD_INPUT", "1")
+            assert not same_bits(got, host(ctx.conv2d_backprop_input(shape, dev(f), dev(g), *args)))
     # fp32 multiply-adds in order, 1.8e-8 sqrt(K), the operands' split, the oracle's rounding
     assert rel_fro(got, oracle.conv2d_backprop_input(shape, f, g, *args)) <= 1.8e-8 * (fh * fw * Cout) ** 0.5 + 1.2e-7
     # infinities and NaNs as fp32 multiply-adds give them, at the border too
@@ -486,3 +491,13 @@ def test_which_3x3_convolutions_run_from_patches(ctx, monkeypatch, case, forward
         assert not torch.equal(patches, copies)
         assert torch.equal(chosen, patches if taken else copies)
     ctx.check_device_status()
+
+
+@pytest.mark.parametrize("patches", ["0", "1"])
+def test_long_sums_of_both_input_gradient_kernels(ctx, oracle, monkeypatch, patches):
+    """4608 products: the bound of fp32 multiply-adds in order, as for the other shapes above."""
+    monkeypatch.setenv("TFJSB_CONV_PATCH", patches)
+    f, g = si.normal(97, 1, (3, 3, 512, 512), 0, float(np.sqrt(2.0 / 4608))), si.normal(97, 2, (4, 14, 14, 512), 0, 1)
+    got = host(ctx.conv2d_backprop_input((4, 14, 14, 512), dev(f), dev(g), (1, 1), "same"))
+    ctx.check_device_status()
+    assert rel_fro(got, oracle.conv2d_backprop_input((4, 14, 14, 512), f, g, (1, 1), "same")) <= 1.8e-8 * 4608 ** 0.5 + 2.5e-8
