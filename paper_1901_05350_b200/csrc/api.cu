@@ -479,7 +479,7 @@ tfjsb_status tfjsb_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_ten
         return TFJSB_OK;
     }
     if (ctx->math == TFJSB_MATH_TF32 && conv_igemm_supported(g) && ctx->encode_tiled) {
-        if (!conv_patch_supported(g) && conv_patch_input_preferred(g, ctx->sm_count))
+        if (!conv_small_window_supported(g) && conv_patch_input_preferred(g, ctx->sm_count))
             return run_conv_patch_input(ctx, px, pf, pbias, act, py, g, s);
         // implicit GEMM on the tensor cores: the filter is packed [Cout, k_pad] into scratch first
         g.gather_only = scratch_is_short(ctx->scratch_b, (size_t)Cout * conv_igemm_k_pad(g) * 4, s);
@@ -487,9 +487,9 @@ tfjsb_status tfjsb_conv2d(tfjsb_ctx* ctx, const tfjsb_tensor* x, const tfjsb_ten
         if ((st = ensure_scratch(ctx, &ctx->scratch_b, (size_t)Cout * k_pad * 4)) != TFJSB_OK) return st;
         if ((e = launch_pack_conv_filter(pf, ctx->scratch_b.ptr, g, s, &ctx->launches)) != cudaSuccess)
             return cuda_fail(ctx, e, "filter packing");
-        if (conv_patch_supported(g) && !getenv("TFJSB_NO_PATCH_CONV")) {
+        if (conv_small_window_supported(g) && !getenv("TFJSB_NO_PATCH_CONV")) {
             DwPwPlan pplan;
-            if ((st = conv_patch_plan(ctx, px, ctx->scratch_b.ptr, py, g, &pplan)) != TFJSB_OK) return st;
+            if ((st = conv_small_window_plan(ctx, px, ctx->scratch_b.ptr, py, g, &pplan)) != TFJSB_OK) return st;
             if ((e = launch_dwpw_fused(pplan, nullptr, nullptr, TFJSB_ACT_NONE, pbias, act, ctx->dev_status, s,
                                        &ctx->launches)) != cudaSuccess)
                 return cuda_fail(ctx, e, "patch conv2d launch");

@@ -413,6 +413,9 @@ bool conv2d_grad_input_preferred(const ConvGeom& g, int sm_count);  // to the CU
 tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float* f, float* dx, const ConvGeom& g, cudaStream_t s);
 bool conv2d_grad_filter_supported(const ConvGeom& g);
 tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float* dy, float* df, const ConvGeom& g, bool split, cudaStream_t s);
+// A row-major fp32 tensor of up to four dimensions, innermost first, copied in boxes (conv_grad_tcgen05.cu).
+tfjsb_status encode_tile_map(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int rank, const int64_t* dims, const uint32_t* box, const char* what,
+                             CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B);
 // conv2d 3x3 with stride 1 from input patches (conv_patch_tcgen05.cu): the forward pass with TF32 operands, f as it is stored,
 // and the input gradient with fp32 accuracy; `g` is the forward geometry of both.
 bool conv_patch_input_preferred(const ConvGeom& g, int sm_count);
@@ -465,8 +468,8 @@ tfjsb_status dwpw_fused_plan(tfjsb_ctx* ctx, const void* x, const float* bt, voi
 // conv2d with fh*fw*Cin <= 32 on the same kernel (input patch by bulk tensor copy, im2col in shared
 // memory); `bt` is the filter packed [Cout, 32].  Launched with launch_dwpw_fused (pw_bias / pw_act = the
 // convolution's bias and activation; the depthwise arguments are ignored).
-bool conv_patch_supported(const ConvGeom& g);
-tfjsb_status conv_patch_plan(tfjsb_ctx* ctx, const float* x, const float* bt, void* y, const ConvGeom& g, DwPwPlan* plan,
+bool conv_small_window_supported(const ConvGeom& g);
+tfjsb_status conv_small_window_plan(tfjsb_ctx* ctx, const float* x, const float* bt, void* y, const ConvGeom& g, DwPwPlan* plan,
                              bool y_bf16 = false);
 cudaError_t launch_dwpw_fused(const DwPwPlan& plan, const float* dw_filter, const float* dw_bias, int dw_act,
                               const float* pw_bias, int pw_act, unsigned int* dev_status, cudaStream_t s,

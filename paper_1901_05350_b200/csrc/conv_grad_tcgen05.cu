@@ -51,32 +51,6 @@ constexpr int CG_THREADS = (2 + EPI_WARPS + CVT_WARPS) * 32;
 constexpr int CG_MAX_STAGES = 4;
 constexpr int GROUP_BYTES = 4096;  // 32 pixels x 32 channels
 
-__device__ __forceinline__ float4 lds4(uint32_t a) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, float w) {
-    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
-}
-
-// Raises the abort flag; the first role to do so reports the reason.
-__device__ __forceinline__ void give_up(volatile int* abort_flag, unsigned int* dev_status, unsigned int code) {
-    if (!*abort_flag) {
-        *abort_flag = 1;
-        atomicOr(dev_status, code);
-    }
-}
-// Waits (bounded) until the phase has completed, whatever the abort flag says.
-__device__ __forceinline__ void drain(uint32_t bar, uint32_t parity, unsigned int* dev_status) {
-    const unsigned long long t0 = global_ns();
-    while (!mbar_try_wait(bar, parity)) {
-        if (global_ns() - t0 > WAIT_LIMIT_NS) {
-            atomicOr(dev_status, DEV_STATUS_TIMEOUT_DRAIN);
-            break;
-        }
-    }
-}
 __device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -641,24 +615,6 @@ conv2d_grad_filter_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
 
 constexpr int CG_SMEM = SMEM_LIMIT - 1024;  // beside the barriers
 
-tfjsb_status encode(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int rank, const int64_t* dims, const uint32_t* box, const char* what,
-                    CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
-    cuuint64_t d[3], st[2];
-    cuuint32_t b[3], elem[3] = {1u, 1u, 1u};
-    cuuint64_t pitch = 4;
-    for (int i = 0; i < rank; ++i) {
-        d[i] = (cuuint64_t)dims[i];
-        b[i] = box[i];
-        pitch *= d[i];
-        if (i + 1 < rank) st[i] = pitch;
-    }
-    CUresult r = ctx->encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), d, st, b, elem,
-                                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(ctx, TFJSB_ERR_CUDA, std::string("cuTensorMapEncodeTiled failed for ") + what + " (CUresult " + std::to_string((int)r) + ")");
-    return TFJSB_OK;
-}
-
 tfjsb_status encode_im2col(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int64_t n, int h, int w, int c, const int lower[2],
                            const int upper[2], int sw, int sh, int pixels, const char* what, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
     cuuint64_t d[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
@@ -674,6 +630,24 @@ tfjsb_status encode_im2col(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, 
 bool corner_ok(int64_t v) { return v >= -128 && v <= 127; }
 
 }  // namespace
+
+tfjsb_status encode_tile_map(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int rank, const int64_t* dims, const uint32_t* box, const char* what,
+                             CUtensorMapSwizzle swizzle) {
+    cuuint64_t d[4], st[3];
+    cuuint32_t b[4], elem[4] = {1u, 1u, 1u, 1u};
+    cuuint64_t pitch = 4;
+    for (int i = 0; i < rank; ++i) {
+        d[i] = (cuuint64_t)dims[i];
+        b[i] = box[i];
+        pitch *= d[i];
+        if (i + 1 < rank) st[i] = pitch;
+    }
+    CUresult r = ctx->encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), d, st, b, elem,
+                                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(ctx, TFJSB_ERR_CUDA, std::string("cuTensorMapEncodeTiled failed for ") + what + " (CUresult " + std::to_string((int)r) + ")");
+    return TFJSB_OK;
+}
 
 // u / s of the first sample along one dimension, and how many values it takes
 static void grad_rows(int size, int pad, int s, int* q0, int* count) {
@@ -793,7 +767,7 @@ tfjsb_status run_conv2d_grad_input(tfjsb_ctx* ctx, const float* dy, const float*
     if ((st = encode_im2col(ctx, &map_dy, dy, g.N, g.Ho, g.Wo, g.Co, lower, upper, 1, 1, BLOCK_M, "dy")) != TFJSB_OK) return st;
     const int64_t fd[3] = {g.Co, g.C, (int64_t)g.fh * g.fw};
     const uint32_t fb[3] = {32u, (uint32_t)a.block_n, 1u};
-    if ((st = encode(ctx, &map_f, f, 3, fd, fb, "the filter")) != TFJSB_OK) return st;
+    if ((st = encode_tile_map(ctx, &map_f, f, 3, fd, fb, "the filter")) != TFJSB_OK) return st;
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(&conv2d_grad_input_kernel), CG_SMEM);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "shared-memory limit");
     const size_t smem = 1024 + (size_t)EPI_WARPS * EPI_SLAB_BYTES + (size_t)a.stages * stage_bytes;
@@ -861,15 +835,15 @@ tfjsb_status run_conv2d_grad_filter(tfjsb_ctx* ctx, const float* x, const float*
     const uint32_t box[3] = {32u, 32u, 1u};
     if (a.tiled) {
         const int64_t d[2] = {g.C, pixels};
-        if ((st = encode(ctx, &map_x, x, 2, d, box, "x", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) != TFJSB_OK) return st;
+        if ((st = encode_tile_map(ctx, &map_x, x, 2, d, box, "x", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) != TFJSB_OK) return st;
     } else {
         const int lower[2] = {-g.pl, -g.pt};
         const int upper[2] = {(g.Wo - 1) * g.sw - g.pl - (g.W - 1), (g.Ho - 1) * g.sh - g.pt - (g.H - 1)};
         if ((st = encode_im2col(ctx, &map_x, x, g.N, g.H, g.W, g.C, lower, upper, g.sw, g.sh, 32, "x", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) != TFJSB_OK) return st;
     }
     const int64_t dd[2] = {g.Co, pixels}, od[3] = {g.Co, g.C, slices * a.taps};
-    if ((st = encode(ctx, &map_dy, dy, 2, dd, box, "dy", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) != TFJSB_OK) return st;
-    if ((st = encode(ctx, &map_out, out, 3, od, box, "the filter gradient")) != TFJSB_OK) return st;
+    if ((st = encode_tile_map(ctx, &map_dy, dy, 2, dd, box, "dy", CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) != TFJSB_OK) return st;
+    if ((st = encode_tile_map(ctx, &map_out, out, 3, od, box, "the filter gradient")) != TFJSB_OK) return st;
     auto kernel = split ? conv2d_grad_filter_kernel<true> : conv2d_grad_filter_kernel<false>;
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kernel), CG_SMEM);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "shared-memory limit");

@@ -126,32 +126,6 @@ __device__ __forceinline__ void mma_words(uint32_t d_tmem, uint32_t a_lo, uint32
         : "memory");
 }
 
-__device__ __forceinline__ float4 lds4(uint32_t a) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, float w) {
-    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
-}
-// Raises the abort flag; the first role to do so reports the reason.
-__device__ __forceinline__ void give_up(volatile int* abort_flag, unsigned int* dev_status, unsigned int code) {
-    if (!*abort_flag) {
-        *abort_flag = 1;
-        atomicOr(dev_status, code);
-    }
-}
-// Waits (bounded) until the phase has completed, whatever the abort flag says.
-__device__ __forceinline__ void drain(uint32_t bar, uint32_t parity, unsigned int* dev_status) {
-    const unsigned long long t0 = global_ns();
-    while (!mbar_try_wait(bar, parity)) {
-        if (global_ns() - t0 > WAIT_LIMIT_NS) {
-            atomicOr(dev_status, DEV_STATUS_TIMEOUT_DRAIN);
-            break;
-        }
-    }
-}
-
 // One result of a tile once more by fp32 multiply-adds, over the samples that exist (in the copied patches those outside the
 // image are zeros, which an infinite filter value turns into NaN).
 __device__ __noinline__ float patch_conv_in_fp32(const PatchConvArgs& g, const PatchTile& r, int oy, int ox, int co) {
@@ -495,23 +469,6 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     }
 }
 
-tfjsb_status encode(tfjsb_ctx* ctx, CUtensorMap* map, const float* base, int rank, const int64_t* dims, const uint32_t* box,
-                    CUtensorMapSwizzle swizzle, const char* what) {
-    cuuint64_t d[4], st[3];
-    cuuint32_t b[4], elem[4] = {1u, 1u, 1u, 1u};
-    cuuint64_t pitch = 4;
-    for (int i = 0; i < rank; ++i) {
-        d[i] = (cuuint64_t)dims[i];
-        b[i] = box[i];
-        pitch *= d[i];
-        if (i + 1 < rank) st[i] = pitch;
-    }
-    CUresult r = ctx->encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), d, st, b, elem,
-                                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(ctx, TFJSB_ERR_CUDA, std::string("cuTensorMapEncodeTiled failed for ") + what + " (CUresult " + std::to_string((int)r) + ")");
-    return TFJSB_OK;
-}
-
 constexpr int PC_SMEM = SMEM_LIMIT - 2048;  // beside the barriers
 
 // Tile width, rings and shared memory for a geometry (as the sum is written above: of the input gradient, the transposed one).
@@ -605,9 +562,9 @@ tfjsb_status launch(tfjsb_ctx* ctx, const float* x, const float* w, const float*
     const uint32_t xb[4] = {32u, (uint32_t)PC_PW, (uint32_t)PC_PH, 1u}, yb[4] = {32u, 8u, 4u, 1u};
     const int64_t wd[3] = {split ? g.C : g.Co, split ? g.Co : g.C, PC_TAPS};
     const uint32_t wb[3] = {32u, split ? (uint32_t)t.block_n : 32u, 1u};
-    if ((st = encode(ctx, &map_x, x, 4, xd, xb, CU_TENSOR_MAP_SWIZZLE_128B, "x")) != TFJSB_OK) return st;
-    if ((st = encode(ctx, &map_w, w, 3, wd, wb, split ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B, "the filter")) != TFJSB_OK) return st;
-    if ((st = encode(ctx, &map_y, out, 4, yd, yb, CU_TENSOR_MAP_SWIZZLE_128B, "y")) != TFJSB_OK) return st;
+    if ((st = encode_tile_map(ctx, &map_x, x, 4, xd, xb, "x")) != TFJSB_OK) return st;
+    if ((st = encode_tile_map(ctx, &map_w, w, 3, wd, wb, "the filter", split ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) != TFJSB_OK) return st;
+    if ((st = encode_tile_map(ctx, &map_y, out, 4, yd, yb, "y")) != TFJSB_OK) return st;
     auto kernel = split ? conv_patch_kernel<true> : conv_patch_kernel<false>;
     cudaError_t e = smem_attr_once(reinterpret_cast<const void*>(kernel), PC_SMEM);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "shared-memory limit");

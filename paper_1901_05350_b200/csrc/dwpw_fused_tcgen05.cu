@@ -783,7 +783,7 @@ tfjsb_status dwpw_fused_plan(tfjsb_ctx* ctx, const void* x, const float* bt, voi
 // conv2d whose whole im2col row fits one k-block (fh*fw*Cin <= 32, e.g. the 3x3x3 stem): the input
 // patch of an 8 x 16 pixel tile comes in by one 3-D bulk tensor copy over x viewed as
 // [N, H, W*Cin] and the compute warps only rearrange it into the A operand.
-bool conv_patch_supported(const ConvGeom& g) {
+bool conv_small_window_supported(const ConvGeom& g) {
     const int64_t k = (int64_t)g.fh * g.fw * g.C;
     const int64_t row_floats = (((int64_t)(F_TW - 1) * g.sw + g.fw) * g.C + 3) / 4 * 4;
     const int64_t rows = (int64_t)(F_TH - 1) * g.sh + g.fh;
@@ -794,11 +794,11 @@ bool conv_patch_supported(const ConvGeom& g) {
            g.N < (1LL << 31);
 }
 
-tfjsb_status conv_patch_plan(tfjsb_ctx* ctx, const float* x, const float* bt, void* y, const ConvGeom& g, DwPwPlan* plan,
+tfjsb_status conv_small_window_plan(tfjsb_ctx* ctx, const float* x, const float* bt, void* y, const ConvGeom& g, DwPwPlan* plan,
                              bool y_bf16) {
     if (y_bf16 && g.Co % 8 != 0) return fail(ctx, TFJSB_ERR_UNSUPPORTED, "a bfloat16 output needs a channel count that is a multiple of 8");
     plan->y_bf16 = y_bf16;
-    if (!conv_patch_supported(g)) return fail(ctx, TFJSB_ERR_UNSUPPORTED, "shape not supported by the patch convolution kernel");
+    if (!conv_small_window_supported(g)) return fail(ctx, TFJSB_ERR_UNSUPPORTED, "shape not supported by the patch convolution kernel");
     if (!ctx->encode_tiled) return fail(ctx, TFJSB_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
     plan->conv = true;
     plan->wide_epi = false;

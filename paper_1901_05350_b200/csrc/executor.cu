@@ -157,7 +157,7 @@ tfjsb_status bind_step(tfjsb_model* m, Step& st, const float* in, float* out) {
         st.plan_built = true;
     }
     if (st.kind == STEP_CONV_TF32 && (changed || !st.plan_built)) {
-        tfjsb_status rc = st.conv_patch ? conv_patch_plan(m->ctx, in, st.filter_km, out, st.g, &st.fused_plan)
+        tfjsb_status rc = st.conv_patch ? conv_small_window_plan(m->ctx, in, st.filter_km, out, st.g, &st.fused_plan)
                                         : conv_igemm_plan(m->ctx, in, st.filter_km, out, st.g, &st.plan);
         if (rc != TFJSB_OK) return rc;
         st.plan_built = true;
@@ -169,7 +169,7 @@ tfjsb_status bind_step(tfjsb_model* m, Step& st, const float* in, float* out) {
         st.plan_built = true;
     }
     if (st.kind == STEP_CONV_NARROW && st.conv_patch && (changed || !st.plan_built)) {
-        tfjsb_status rc = conv_patch_plan(m->ctx, in, st.filter_km, out, st.g, &st.fused_plan, true);
+        tfjsb_status rc = conv_small_window_plan(m->ctx, in, st.filter_km, out, st.g, &st.fused_plan, true);
         if (rc != TFJSB_OK) return rc;
         st.plan_built = true;
     }
@@ -716,7 +716,7 @@ tfjsb_status tfjsb_model_create(tfjsb_ctx* ctx, const tfjsb_layer_desc* layers, 
                 return bail(TFJSB_ERR_INVALID_ARG, where + "unknown layer kind");
         }
         if (step.kind == STEP_CONV_TF32) {
-            step.conv_patch = conv_patch_supported(step.g) && !getenv("TFJSB_NO_PATCH_CONV");
+            step.conv_patch = conv_small_window_supported(step.g) && !getenv("TFJSB_NO_PATCH_CONV");
             // filter [fh*fw*Cin, Cout] -> [Cout, k_pad] once, on the device
             const int64_t k_pad = conv_igemm_k_pad(step.g);
             if ((st = dev_alloc(m, (size_t)(k_pad * step.g.Co), &step.filter_km)) != TFJSB_OK) return bail(st, ctx->last_error);
@@ -777,7 +777,7 @@ tfjsb_status tfjsb_model_create(tfjsb_ctx* ctx, const tfjsb_layer_desc* layers, 
             // rounds the fp32 image as it builds the operand tile, multiplies in TF32 (exact for bfloat16
             // values) and stores bfloat16.
             if (sp.kind == STEP_CONV_NARROW && sp.in_f32 && sp.out_bf16 && !sp.is_dense && sp.g.Co % 8 == 0 &&
-                conv_patch_supported(sp.g) && !getenv("TFJSB_NO_PATCH_CONV")) {
+                conv_small_window_supported(sp.g) && !getenv("TFJSB_NO_PATCH_CONV")) {
                 const int64_t k_pad = conv_igemm_k_pad(sp.g);
                 if ((st = dev_alloc(m, (size_t)(k_pad * sp.g.Co), &sp.filter_km)) != TFJSB_OK) return bail(st, ctx->last_error);
                 cudaError_t e = launch_pack_conv_filter(sp.filter, sp.filter_km, sp.g, 0, &ctx->launches);

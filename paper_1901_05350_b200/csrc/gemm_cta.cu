@@ -159,16 +159,6 @@ __device__ __forceinline__ void gather_scalar(float (&v)[BLOCK_K], const float* 
     }
 }
 
-// An operand tile of 32 k whose rows of memory run along M or N: one copy of 32 k x 32 columns per group.
-template <bool BATCHED>
-__device__ __forceinline__ void load_mn_groups(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row0, int k0, int batch, int groups) {
-#pragma unroll 1
-    for (int i = 0; i < groups; ++i) {
-        if (BATCHED) tma_load_3d(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0, batch);
-        else tma_load_2d(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0);
-    }
-}
-
 // where the rows of A come from: a matrix in memory, threads that gather windows, or im2col copies of an NHWC tensor
 constexpr int A_TILED = 0;
 constexpr int A_GATHER = 1;
@@ -732,7 +722,7 @@ tfjsb_status gemm_tf32_plan(tfjsb_ctx* ctx, const float* a, const float* bt, flo
 // packs the taps, is the faster one.
 bool conv_igemm_uses_im2col(const ConvGeom& g) {
     const int64_t upper_w = (int64_t)(g.Wo - 1) * g.sw - g.pl - (g.W - 1), upper_h = (int64_t)(g.Ho - 1) * g.sh - g.pt - (g.H - 1);
-    return !g.gather_only && !conv_patch_supported(g) && g.C % 4 == 0 && g.C >= 16 && g.sh <= 8 && g.sw <= 8 && (int64_t)(g.fh - 1) * g.dh <= 127 && (int64_t)(g.fw - 1) * g.dw <= 127 &&
+    return !g.gather_only && !conv_small_window_supported(g) && g.C % 4 == 0 && g.C >= 16 && g.sh <= 8 && g.sw <= 8 && (int64_t)(g.fh - 1) * g.dh <= 127 && (int64_t)(g.fw - 1) * g.dw <= 127 &&
            g.pl <= 127 && g.pt <= 127 && upper_w >= -128 && upper_w <= 127 && upper_h >= -128 && upper_h <= 127;
 }
 

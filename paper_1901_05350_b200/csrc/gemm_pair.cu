@@ -71,7 +71,7 @@ struct PairArgs {
     unsigned int* dev_status;
 };
 
-// An operand tile of 32 k whose rows of memory run along M or N: one copy of 32 k x 32 columns per group.
+// load_mn_groups with copies that the even CTA counts.
 __device__ __forceinline__ void load_groups_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row0, int k0, int groups) {
 #pragma unroll 1
     for (int i = 0; i < groups; ++i) tma_load_2d_pair(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0);

@@ -69,12 +69,6 @@ __device__ __forceinline__ float4 ld_shared_v4(uint32_t addr) {
     return v;
 }
 
-// An operand tile of 32 k whose rows of memory run along M or N: one copy of 32 k x 32 columns per group.
-__device__ __forceinline__ void load_groups(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row0, int k0, int groups) {
-#pragma unroll 1
-    for (int i = 0; i < groups; ++i) tma_load_2d(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0);
-}
-
 template <bool MN>
 __global__ void __launch_bounds__(S_THREADS, 1)
 gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
@@ -149,9 +143,9 @@ gemm_tf32_splitk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_
             const uint32_t a_dst = stage_base + (uint32_t)stage * (uint32_t)stage_bytes;
             if (leader && ok && (ok = bounded_wait(smem_u32(&bar_empty[stage]), phase ^ 1u, abort_flag))) {
                 mbar_arrive_expect_tx(full, (uint32_t)args.stage_tx);
-                if (MN && args.a_mn) load_groups(a_dst, &map_a, full, m0, kb * BLOCK_K, args.a_groups);
+                if (MN && args.a_mn) load_mn_groups<false>(a_dst, &map_a, full, m0, kb * BLOCK_K, 0, args.a_groups);
                 else tma_load_2d(a_dst, &map_a, full, kb * BLOCK_K, m0);
-                if (MN && args.b_mn) load_groups(a_dst + A_STAGE_BYTES, &map_b, full, n0, kb * BLOCK_K, block_n >> 5);
+                if (MN && args.b_mn) load_mn_groups<false>(a_dst + A_STAGE_BYTES, &map_b, full, n0, kb * BLOCK_K, 0, block_n >> 5);
                 else tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, full, kb * BLOCK_K, n0);
                 ++issued;
             }

@@ -117,6 +117,44 @@ __device__ __forceinline__ void add_segment(uint32_t large, uint32_t small, uint
     ptx::tc_st_wait();
 }
 
+// ---- shared memory, time-outs, copies ---------------------------------------------------------------
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, float w) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+
+// Raises the abort flag; the first role to do so reports the reason.
+__device__ __forceinline__ void give_up(volatile int* abort_flag, unsigned int* dev_status, unsigned int code) {
+    if (!*abort_flag) {
+        *abort_flag = 1;
+        atomicOr(dev_status, code);
+    }
+}
+// Waits (bounded) until the phase has completed, whatever the abort flag says.
+__device__ __forceinline__ void drain(uint32_t bar, uint32_t parity, unsigned int* dev_status) {
+    const unsigned long long t0 = ptx::global_ns();
+    while (!ptx::mbar_try_wait(bar, parity)) {
+        if (ptx::global_ns() - t0 > ptx::WAIT_LIMIT_NS) {
+            atomicOr(dev_status, DEV_STATUS_TIMEOUT_DRAIN);
+            break;
+        }
+    }
+}
+
+// An operand tile of 32 k whose rows of memory run along M or N: one copy of 32 k x 32 columns per group.
+template <bool BATCHED>
+__device__ __forceinline__ void load_mn_groups(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row0, int k0, int batch, int groups) {
+#pragma unroll 1
+    for (int i = 0; i < groups; ++i) {
+        if (BATCHED) ptx::tma_load_3d(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0, batch);
+        else ptx::tma_load_2d(dst + (uint32_t)i * 4096u, map, bar, row0 + 32 * i, k0);
+    }
+}
+
 // ---- bfloat16 storage ------------------------------------------------------------------------------
 // Instruction descriptor: fp32 accumulator, bfloat16 A and B (format 1), both K-major.
 __device__ __forceinline__ uint32_t make_idesc_bf16(int m, int n) {
