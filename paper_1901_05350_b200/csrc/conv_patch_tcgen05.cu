@@ -25,7 +25,7 @@
 //
 // SPLIT (gradients): fp32 accuracy from TF32 products as in conv_grad_tcgen05.cu: every operand tile has a lo tile beside it,
 // made by warps 12-23 (four for patches, eight for filter tiles), three products per 8 of k, large products summed in
-// segments.  A patch is split once and not once per tap.
+// segments.  A patch is split once and not once per tap.  24 warps leave a thread 80 registers; it spills 124 bytes.
 // Every wait is bounded (ptx_sm100.cuh).
 #include <algorithm>
 #include <cstdlib>
@@ -392,12 +392,13 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
                 const int col0 = n0 + ch * EPI_COLS;
                 if (lane == 0) tma_store_wait_read<0>();
                 __syncwarp();
-                const float* bias = g.bias != nullptr ? g.bias + col0 : nullptr;
+                const float* bias = !SPLIT && g.bias != nullptr ? g.bias + col0 : nullptr;
                 const uint32_t row_addr = slab + (uint32_t)lane * 128u;
-                if (g.act == TFJSB_ACT_RELU6) stage_chunk<TFJSB_ACT_RELU6>(u, bias, g.Co - col0, row_addr, lane);
+                if (SPLIT) stage_chunk<TFJSB_ACT_NONE>(u, nullptr, 0, row_addr, lane);  // a gradient has neither
+                else if (g.act == TFJSB_ACT_RELU6) stage_chunk<TFJSB_ACT_RELU6>(u, bias, g.Co - col0, row_addr, lane);
                 else if (g.act == TFJSB_ACT_RELU) stage_chunk<TFJSB_ACT_RELU>(u, bias, g.Co - col0, row_addr, lane);
                 else stage_chunk<TFJSB_ACT_NONE>(u, bias, g.Co - col0, row_addr, lane);
-                if (SPLIT) {  // no bias, no activation
+                if (SPLIT) {
                     const int oy = row0 + (lane >> 3), ox = r.x0() + (lane & 7);
                     bool odd = false;
 #pragma unroll
