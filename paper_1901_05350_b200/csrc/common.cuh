@@ -156,6 +156,10 @@ int current_sm_count();
 // TMEM allocation) and the launch itself overlap.  Between kernels of op calls this saves 1 to 3 us (eleven small ops
 // 61 -> 38 us, a block's forward and backward pass 229 -> 210, one 512^3 matMul after another 8.4 -> 7.3).
 // On unless TFJSB_NO_PDL is set; the executor switches it by the model's setting while it enqueues one.
+// What starts early is put where there is room and not one block to an SM, so it costs more than it saves where blocks of either
+// kernel run long and share SMs.  Long reductions of few blocks are therefore launched after the kernel before (launch_k_if:
+// global pools, softmax), and kernels of small blocks, or of two CTAs to an SM, that another such kernel may follow say
+// pdl_launch_dependents() late or not at all, in which case the next one starts as they end.
 extern thread_local bool g_launch_pdl;
 
 // A load of what the kernel before may still be writing when this one starts: an ordinary one, also through pointers to
@@ -167,7 +171,8 @@ __device__ __forceinline__ T load_global(const T* p) { return *p; }
 template <typename T>
 __device__ __forceinline__ T load_fixed(const T* p) { return __ldg(p); }
 // load_global as an instruction that stays where it is written, for loops that load ahead with few registers to spare (the
-// strided GEMM's loaders spill 16 to 40 bytes with load_global and nothing with these).
+// strided GEMM's loaders spill 16 to 40 bytes with load_global and nothing with these) or whose loads the compiler spreads out
+// (max and global pools).
 __device__ __forceinline__ float ld_global(const float* p) {
     float v;
     asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));

@@ -20,7 +20,7 @@
 // One thread issues everything, and every instruction around its MMAs counts: the nine taps are unrolled, an operand is the low
 // word of its descriptor, worked out by the converged warp, and tiles are stepped without divisions (with the window as a loop
 // and descriptors inside the elected thread's branch a tap took 880 cycles).
-// What bounds it: two to four patches in flight per SM and the copies and stores of single pixels; [32,56,56,64] -> 64 takes 435
+// What bounds it: two to four patches in flight per SM and the copies and stores of single pixels; [64,56,56,64] -> 64 takes 372
 // cycles a tap where its MMAs take 196.
 //
 // SPLIT (gradients): fp32 accuracy from TF32 products as in conv_grad_tcgen05.cu: every operand tile has a lo tile beside it,
