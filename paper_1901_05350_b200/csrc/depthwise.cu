@@ -528,23 +528,28 @@ tfjsb_status depthwise_plan(tfjsb_ctx* ctx, const void* x, const ConvGeom& g, De
         // Stride 1.  8 x 8 tiles of 32 channels while an SM would not have one tile: a short layer takes what one tile takes
         // (copy, rows, stores), and its rows per thread are 2 instead of 4 or 7 ([1,56,56,128] 4.1 -> 3.0 us, [1,14,14,512]
         // 3.3 -> 2.9; against 16 x 7 tiles, as all below).  They also read DRAM faster where the tensors do not stay in L2 and a
-        // pixel is 512 bytes or less ([128,56,56,128] 73.4 -> 66.3, [100,112,112,64] 116 -> 100).  Otherwise the tiles of earlier
-        // planning, 16 x 7 of 64 channels and 16 x 14 of 32, unless 8 x 8 of as many channels are 5 % ahead by the estimates:
-        // of 360 shapes, 32 to 1024 channels of 7 to 128 squared, 10 more than 2 % slower than without 8 x 8, 0.98 of the time on
-        // average.  ([32,56,56,128] 18.8 -> 17.1, [8,17,17,512] 5.9 -> 4.6; but [18,68,68,512] would be 66.4 for 55.8,
-        // [40,10,10,768] 9.5 for 7.3, [54,13,13,424] 10.0 for 7.9.)
+        // pixel is 512 bytes or less ([128,56,56,128] 73.4 -> 66.3, [100,112,112,64] 116 -> 100).  Otherwise 16 x 7 of 64 channels,
+        // unless 8 x 8 of 64 are 3 % ahead by the estimates, or up to 3 % behind while both tensors stay in L2 and the rounds of two
+        // tiles per SM, at half the time of one of 16 x 7, are fewer, where models gain more than calls ([32,56,56,128]
+        // 18.8 -> 17.1, [8,17,17,512] 5.9 -> 4.6; but [18,68,68,512] would be 66.4 for 55.8, [40,10,10,768] 9.5 for 7.3).
+        // Channels that are no multiple of 64: 16 x 14 of 32, unless 8 x 8 of 32 are ahead, by up to 24 tiles per SM for whole blocks of
+        // 32 ([8,112,112,32] 6.8 -> 6.0, [16,112,112,32] 9.7 -> 9.2, [32,112,112,32] 17.8 and 18.7) and by the estimates for others
+        // ([54,13,13,424] would be 10.0 for 7.9).
+        // Of 360 shapes, 32 to 1024 channels of 7 to 128 squared, 29 are 2 to 8 % slower than without 8 x 8, three of them by more than
+        // 0.4 us; 0.975 of the time on average.
         const bool beyond_l2 = (double)g.N * g.H * g.W * g.C * 8.0 > 1.5e8;  // both tensors
         const bool whole64 = g.C % 64 == 0;
-        const int64_t blocks = whole64 ? g.C / 64 : blocks32;
+        const int64_t blocks = whole64 ? g.C / 64 : blocks32, pair = 2 * (int64_t)ctx->sm_count;
         const int64_t wide = g.N * ((g.Wo + 15) / 16) * ((g.Ho + (whole64 ? 6 : 13)) / (whole64 ? 7 : 14)) * blocks;
-        auto ahead = [&](const DwTileCost& narrow_tiles, const DwTileCost& wide_tiles) {
-            return tiles_us(narrow_tiles, tiles8 * blocks, g, ctx->sm_count) < 0.95 * tiles_us(wide_tiles, wide, g, ctx->sm_count);
-        };
+        const double ratio = tiles_us(whole64 ? kDw8x8x64 : kDw8x8x32, tiles8 * blocks, g, ctx->sm_count) /
+                             tiles_us(whole64 ? kDw16x7x64 : kDw16x14x32, wide, g, ctx->sm_count);
         if (g.sh == 1 && whole64) {
+            const bool fewer_rounds = (tiles8 * blocks + pair - 1) / pair < 2 * ((wide + pair - 1) / pair);
             if (tiles8 * blocks < ctx->sm_count || (g.C <= 128 && beyond_l2)) v = 1;
-            else v = g.Wo <= 8 || ahead(kDw8x8x64, kDw16x7x64) ? 7 : 6;
+            else v = g.Wo <= 8 || ratio < 0.97 || (!beyond_l2 && fewer_rounds && ratio < 1.03) ? 7 : 6;
         } else if (g.sh == 1) {
-            v = g.Wo <= 8 || tiles8 * blocks < ctx->sm_count || ahead(kDw8x8x32, kDw16x14x32) ? 1 : 0;
+            const bool ahead = g.C % DW_CB == 0 ? tiles8 * blocks <= 24 * (int64_t)ctx->sm_count : tiles8 * blocks < ctx->sm_count || ratio < 0.97;
+            v = g.Wo <= 8 || ahead ? 1 : 0;
         } else {
             // stride 2: 64-channel tiles are 8 outputs wide, so they are taken only where that wastes fewer columns than the
             // 16-wide 32-channel ones ([128,112,112,64] 90.1 -> 86.9 us; [128,28,28,256] ran 27.3 -> 29.1 with them)
