@@ -36,9 +36,8 @@ __device__ __forceinline__ void stage_chunk(const uint32_t (&r)[32], const float
         float4 v;
         v.x = __uint_as_float(r[4 * j + 0]); v.y = __uint_as_float(r[4 * j + 1]);
         v.z = __uint_as_float(r[4 * j + 2]); v.w = __uint_as_float(r[4 * j + 3]);
-        // (ld_global: where they stand; loads that the compiler may move take bfloat16 models 0.2 to 0.6 % longer)
         if (bias != nullptr && 4 * j < cols_left) {  // N % 4 == 0: a quad is all in or all out
-            const float4 b = ld_global4(bias + 4 * j);
+            const float4 b = load_global(reinterpret_cast<const float4*>(bias + 4 * j));
             v.x = v.x + b.x; v.y = v.y + b.y; v.z = v.z + b.z; v.w = v.w + b.w;
         }
         v.x = apply_act_t<ACT>(v.x); v.y = apply_act_t<ACT>(v.y);
@@ -173,8 +172,8 @@ __device__ __forceinline__ void stage_chunk_bf16(const uint32_t (&r)[32], const 
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(r[8 * j + e]);
         if (bias != nullptr && 8 * j < cols_left) {  // N % 8 == 0: a group of eight is all in or all out
-            const float4 b0 = ld_global4(bias + 8 * j);
-            const float4 b1 = ld_global4(bias + 8 * j + 4);
+            const float4 b0 = load_global(reinterpret_cast<const float4*>(bias + 8 * j));
+            const float4 b1 = load_global(reinterpret_cast<const float4*>(bias + 8 * j + 4));
             v[0] += b0.x; v[1] += b0.y; v[2] += b0.z; v[3] += b0.w;
             v[4] += b1.x; v[5] += b1.y; v[6] += b1.z; v[7] += b1.w;
         }
